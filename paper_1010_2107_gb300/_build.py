@@ -22,7 +22,8 @@ FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", 
          "--expt-relaxed-constexpr", "-I", OUT]
 # Headers the run-time compiled kernels (rtc.cu) are built from, embedded in
 # the library as text under the names their #include lines use.
-RTC_HEADERS = [("common.cuh", os.path.join(CSRC, "common.cuh")),
+RTC_HEADERS = [("col_hist.cuh", os.path.join(CSRC, "col_hist.cuh")),
+               ("common.cuh", os.path.join(CSRC, "common.cuh")),
                ("integrands.cuh", os.path.join(CSRC, "integrands.cuh")),
                ("kernels.h", os.path.join(CSRC, "kernels.h")),
                ("sample_kernel.cuh", os.path.join(CSRC, "sample_kernel.cuh")),

@@ -94,15 +94,14 @@ struct vegas_ctx {
   uint64_t ncubes = 1, nc = 0;
   int strat = 0;
   gv::KernelEntry ke{};
+  const void* col = nullptr;  // the column-histogram kernel of this shape, or null
   int sm_count = 0;
-  // launch geometry
-  int threads = 256, ctas_per_sm_req = 0, ctas = 0, lanes = 1, lanes_req = 0, occ = 0;
-  int cap = 16;  // histogram bucket capacity (see sample_kernel.cuh)
-  int ctas_nb = 0;      // CTAs of a pass without the per-bin histogram
-  size_t smem_nb = 0;   // and its dynamic shared memory
+  // launch geometry: threads per CTA asked for (0: automatic) and CTAs per SM
+  int threads_req = 0, ctas_per_sm_req = 0;
+  int cap = 0;  // histogram bucket capacity (see sample_kernel.cuh; 0: column histogram)
   int ppt = 1, ppt_req = 0, ppt_min = 1;  // points per thread per histogram tile
   bool small_cap = false;                 // tile capacity policy (gv::choose_tile)
-  size_t smem = 0;
+  gv::PassShape pass_bins, pass_nobins;   // passes with and without the per-bin sums
   // device buffers
   double* d_edges = nullptr;
   double2* d_tab64 = nullptr;
@@ -112,7 +111,6 @@ struct vegas_ctx {
   double* d_part_tot = nullptr;
   int part_rows = 0;
   double* d_bins = nullptr;
-  double* d_tot = nullptr;
   double* d_cubes = nullptr;
   double* d_cube_max = nullptr;  // [G] max(0, largest w) per cube, integration phase
   bool have_max = false;         // a bases_integrate has recorded the maxima
@@ -397,61 +395,117 @@ __global__ void k_spring_compact(const uint32_t* counts, uint32_t chunk, int d, 
   for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) ot[off + i] = st[src + i];
 }
 
-vegas_status configure_launch(vegas_ctx* c) {
-  const int d = c->cfg.ndim, N = c->cfg.nbins;
-  // Histogram tile (gv::choose_tile): points per thread between gathers and
-  // bucket capacity, against the CTAs per SM each leaves resident.
-  cudaError_t e = cudaSuccess;
-  auto occ_of = [&](int cap, int) -> int {
-    const size_t smem = c->ke.smem(d, N, cap);
+// Shape of the column-histogram pass (col_hist.cuh) for `threads` threads per
+// CTA, or, when 0, for the count that keeps most warps resident (the columns'
+// shared memory bounds them) and, on equal terms, the widest CTA (fewest
+// partial rows); a small pass takes narrower CTAs until every SM has one.
+// False when fewer than kColMinWarps warps would be resident: the columns of
+// many bins are too large and bucketed tiles are the better form (measured at
+// 4M points in 8 dimensions: 64 bins and below columns, see DESIGN).
+constexpr int kColMinWarps = 8;
+bool shape_col(const void* fn, const gv::KernelEntry& ke, int d, int N, int sm_count, int threads, int per_sm_req,
+               uint64_t ncubes, uint64_t nc, uint64_t ncall, int64_t max_rows, gv::PassShape* out, cudaError_t* e) {
+  static const int kAuto[] = {512, 384, 256, 192, 128, 64};
+  int best_t = 0, best_occ = 0;
+  const int one[] = {threads};
+  const int* list = threads > 0 ? one : kAuto;
+  const int n = threads > 0 ? 1 : (int)(sizeof kAuto / sizeof kAuto[0]);
+  for (int i = 0; i < n; ++i) {
+    const size_t smem = ke.smem_col(d, N, list[i] / 32);
+    if (smem + 2048 > 227 * 1024) continue;  // (2 KB: the kernel's static shared memory)
+    if ((*e = gv_raise_smem_limit(fn, smem)) != cudaSuccess) return false;
     int o = 0;
-    if (e != cudaSuccess || smem > 227 * 1024) return 0;
-    e = gv_raise_smem_limit(c->ke.sample, smem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, c->ke.sample, c->threads, smem);
-    return e == cudaSuccess ? o : 0;
-  };
-  int occ_cap = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_cap, c->ke.sample, c->threads, 0);
-  if (e != cudaSuccess) return c->fail(VEGAS_ECUDA, "launch configuration: %s", cudaGetErrorString(e));
-  const gv::TileShape t = gv::choose_tile(c->threads, N, c->ppt_req, c->ppt_min, occ_cap, occ_of, c->small_cap);
-  if (e != cudaSuccess) return c->fail(VEGAS_ECUDA, "launch configuration: %s", cudaGetErrorString(e));
-  if (t.occ < 1) return c->fail(VEGAS_EINVAL, "sampling kernel does not fit: %d threads, %d points per thread",
-                                c->threads, t.ppt);
-  // the limit covers the chosen size (it only grows: see gv_raise_smem_limit)
-  c->smem = c->ke.smem(d, N, t.cap);
-  e = gv_raise_smem_limit(c->ke.sample, c->smem);
-  if (e != cudaSuccess) return c->fail(VEGAS_ECUDA, "launch configuration: %s", cudaGetErrorString(e));
-  c->cap = t.cap;
-  c->ppt = t.ppt;
-  const int occ = t.occ;
-  c->occ = occ;
-  const int per_sm = c->ctas_per_sm_req > 0 ? std::min(c->ctas_per_sm_req, occ) : occ;
-  const int64_t cap_ctas = (int64_t)c->sm_count * per_sm;
-  uint64_t units;
-  if (c->strat) {
-    // lanes per hypercube: the best balance of rounds and chain length
-    int L = gv::choose_lanes(c->ncubes, c->nc, c->threads, cap_ctas);
-    if (c->lanes_req > 0) L = std::min<int>(c->lanes_req, (int)std::min<uint64_t>(32, c->nc));
-    int Lp = 1;
-    while (2 * Lp <= L) Lp *= 2;
-    c->lanes = Lp;
-    units = c->ncubes * (uint64_t)Lp;
-  } else {
-    c->lanes = 1;
-    units = (uint64_t)c->cfg.ncall;
+    if ((*e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, fn, list[i], smem)) != cudaSuccess) return false;
+    if (per_sm_req > 0) o = std::min(o, per_sm_req);
+    if (o * list[i] > best_occ * best_t) {
+      best_t = list[i];
+      best_occ = o;
+    }
   }
-  int64_t ctas = (int64_t)((units + c->threads - 1) / c->threads);
-  c->ctas = (int)std::max<int64_t>(1, std::min<int64_t>(ctas, cap_ctas));
+  if (best_occ * best_t < 32 * kColMinWarps && threads == 0) return false;
+  if (best_occ < 1) return false;
+  const int pif = d <= 8 ? 2 : 1;
+  if (threads == 0 && ncubes == 1) {
+    const uint64_t per = (ncall + (uint64_t)sm_count * pif - 1) / ((uint64_t)sm_count * pif);
+    if (per < (uint64_t)best_t) {
+      best_t = (int)std::max<uint64_t>(64, (per + 31) / 32 * 32);
+      best_occ = 1;
+    }
+  }
+  out->fn = fn;
+  out->threads = best_t;
+  out->occ = best_occ;
+  out->smem = ke.smem_col(d, N, best_t / 32);
+  const int64_t most = std::min<int64_t>((int64_t)sm_count * best_occ, max_rows);
+  out->lanes = ncubes > 1 ? gv::balanced_lanes(ncubes, nc, best_t, sm_count, pif) : 1;
+  const uint64_t units = ncubes > 1 ? ncubes * (uint64_t)out->lanes : ncall;
+  out->ctas = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)((units + best_t - 1) / best_t), most));
+  return true;
+}
+
+vegas_status configure_launch(vegas_ctx* c) {
+  const int threads = c->threads_req > 0 ? c->threads_req : 256;
+  const int d = c->cfg.ndim, N = c->cfg.nbins;
+  gv::PassShape &pb = c->pass_bins, &pn = c->pass_nobins;
+  const bool strat = c->strat != 0;
+  cudaError_t e = cudaSuccess;
+  auto ctas_for = [&](int lanes, int t, int64_t most) {
+    const uint64_t units = strat ? c->ncubes * (uint64_t)lanes : (uint64_t)c->cfg.ncall;
+    return (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)((units + t - 1) / t), most));
+  };
+  int per_sm = 1;
+  if (c->col && c->ppt_req == 0 &&
+      shape_col(c->col, c->ke, d, N, c->sm_count, c->threads_req, c->ctas_per_sm_req, c->ncubes, c->nc,
+                (uint64_t)c->cfg.ncall, INT64_MAX, &pb, &e)) {
+    c->cap = 0;
+    c->ppt = d <= 8 ? 2 : 1;
+    per_sm = std::max(1, pb.occ);
+  } else {
+    // Histogram tile (gv::choose_tile): points per thread between gathers and
+    // bucket capacity, against the CTAs per SM each leaves resident.
+    auto occ_of = [&](int cap, int) -> int {
+      const size_t smem = c->ke.smem(d, N, cap);
+      int o = 0;
+      if (e != cudaSuccess || smem > 227 * 1024) return 0;
+      e = gv_raise_smem_limit(c->ke.sample, smem);
+      if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, c->ke.sample, threads, smem);
+      return e == cudaSuccess ? o : 0;
+    };
+    int occ_cap = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_cap, c->ke.sample, threads, 0);
+    if (e != cudaSuccess) return c->fail(VEGAS_ECUDA, "launch configuration: %s", cudaGetErrorString(e));
+    const gv::TileShape t = gv::choose_tile(threads, N, c->ppt_req, c->ppt_min, occ_cap, occ_of, c->small_cap);
+    if (e != cudaSuccess) return c->fail(VEGAS_ECUDA, "launch configuration: %s", cudaGetErrorString(e));
+    if (t.occ < 1) return c->fail(VEGAS_EINVAL, "sampling kernel does not fit: %d threads, %d points per thread",
+                                  threads, t.ppt);
+    pb.fn = c->ke.sample;
+    pb.threads = threads;
+    pb.occ = t.occ;
+    // the limit covers the chosen size (it only grows: see gv_raise_smem_limit)
+    pb.smem = c->ke.smem(d, N, t.cap);
+    e = gv_raise_smem_limit(c->ke.sample, pb.smem);
+    if (e != cudaSuccess) return c->fail(VEGAS_ECUDA, "launch configuration: %s", cudaGetErrorString(e));
+    c->cap = t.cap;
+    c->ppt = t.ppt;
+    per_sm = c->ctas_per_sm_req > 0 ? std::min(c->ctas_per_sm_req, t.occ) : t.occ;
+    const int64_t most = (int64_t)c->sm_count * per_sm;
+    pb.lanes = strat ? gv::choose_lanes(c->ncubes, c->nc, threads, most) : 1;
+    pb.ctas = ctas_for(pb.lanes, threads, most);
+  }
   // passes without the per-bin histogram (no refinement) need only the
   // grid table and constants in shared memory: more CTAs may be resident
-  c->smem_nb = c->ke.smem_nobins(d, N);
+  pn.fn = c->ke.sample;
+  pn.threads = threads;
+  pn.smem = c->ke.smem_nobins(d, N);
   int occ_nb = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_nb, c->ke.sample, c->threads, c->smem_nb);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_nb, c->ke.sample, threads, pn.smem);
   if (e != cudaSuccess) return c->fail(VEGAS_ECUDA, "launch configuration: %s", cudaGetErrorString(e));
-  occ_nb = std::max(occ_nb, per_sm);
   if (c->ctas_per_sm_req > 0) occ_nb = std::min(occ_nb, std::max(c->ctas_per_sm_req, per_sm));
-  c->ctas_nb = (int)std::max<int64_t>(1, std::min<int64_t>(ctas, (int64_t)c->sm_count * occ_nb));
-  const int rows = std::max(c->ctas, c->ctas_nb);
+  pn.occ = std::max(occ_nb, 1);
+  const int64_t most_nb = (int64_t)c->sm_count * pn.occ;
+  pn.lanes = strat ? gv::balanced_lanes(c->ncubes, c->nc, threads, c->sm_count, c->ppt_min) : 1;
+  pn.ctas = ctas_for(pn.lanes, threads, most_nb);
+  const int rows = std::max(pb.ctas, pn.ctas);
   if (rows > c->part_rows) {
     if (c->d_part_bins) cudaFree(c->d_part_bins);
     if (c->d_part_tot) cudaFree(c->d_part_tot);
@@ -468,12 +522,13 @@ vegas_status configure_launch(vegas_ctx* c) {
 
 gv::SampleArgs sample_args(const vegas_ctx* c, int it_override, bool nobins = false) {
   gv::SampleArgs A{};
+  const gv::PassShape& ps = nobins ? c->pass_nobins : c->pass_bins;
   A.nobins = nobins;
   A.d = c->cfg.ndim;
   A.N = c->cfg.nbins;
   A.g = c->g;
   A.ybits = c->ybits;
-  A.lanes = c->lanes;
+  A.lanes = ps.lanes;
   A.cap = c->cap;
   A.ppt = c->ppt;
   A.strat = c->strat;
@@ -496,7 +551,7 @@ gv::SampleArgs sample_args(const vegas_ctx* c, int it_override, bool nobins = fa
   A.inv_gb_f = (float)(1.0 / gb);
   A.inv_nc = c->nc > 0 ? 1.0 / (double)c->nc : 0.0;
   A.inv_nc1 = c->nc > 1 ? 1.0 / (double)(c->nc - 1) : 0.0;
-  A.nparts = nobins ? c->ctas_nb : c->ctas;
+  A.nparts = ps.ctas;
   A.tab = c->prec == VG_FP64 ? (const void*)c->d_tab64 : (const void*)c->d_tab32;
   A.dparams = c->d_derived;
   A.st = c->d_st;
@@ -511,7 +566,7 @@ gv::FinArgs fin_args(const vegas_ctx* c, int refine, int record, bool nobins = f
   F.d = c->cfg.ndim;
   F.N = c->cfg.nbins;
   F.nobins = nobins;
-  F.nparts = nobins ? c->ctas_nb : c->ctas;
+  F.nparts = (nobins ? c->pass_nobins : c->pass_bins).ctas;
   F.strat = c->strat;
   F.refine = refine;
   F.record = record;
@@ -523,7 +578,6 @@ gv::FinArgs fin_args(const vegas_ctx* c, int refine, int record, bool nobins = f
   F.part_bins = c->d_part_bins;
   F.part_tot = c->d_part_tot;
   F.bins = c->d_bins;
-  F.tot = c->d_tot;
   F.edges = c->d_edges;
   F.tab64 = c->d_tab64;
   F.tab32 = c->d_tab32;
@@ -540,8 +594,8 @@ vegas_status launch_pass(vegas_ctx* c, int it_override, int refine, int record, 
   gv::SampleArgs A = sample_args(c, it_override, nobins);
   if (record_max) A.cube_max = c->d_cube_max;
   void* args[] = {&A};
-  CK(c, cudaLaunchKernel(c->ke.sample, dim3(nobins ? c->ctas_nb : c->ctas), dim3(c->threads), args,
-                         nobins ? c->smem_nb : c->smem, c->stream));
+  const gv::PassShape& ps = nobins ? c->pass_nobins : c->pass_bins;
+  CK(c, cudaLaunchKernel(ps.fn, dim3(ps.ctas), dim3(ps.threads), args, ps.smem, c->stream));
   gv::FinArgs F = fin_args(c, refine, record, nobins);
   CK(c, gv_launch_finish(&F, c->stream));
   return VEGAS_OK;
@@ -704,6 +758,14 @@ bool spec_shape(int d, int dm, int ybits, int g, int N) {
   return d == dm && ybits == 24 && (g & (g - 1)) == 0 && (int64_t)g * N <= 256;
 }
 
+// The column-histogram kernel of a shape (the divisions of spec_shape with
+// any d up to the compile-time bound; the exact one where d equals it), or
+// null.
+const void* pick_col(const gv::KernelEntry& ke, int d, int ybits, int g, int N) {
+  if (!spec_shape(ke.dm, ke.dm, ybits, g, N)) return nullptr;
+  return d == ke.dm ? ke.sample_col_exact : ke.sample_col;
+}
+
 // Second half of every constructor, for a context whose integrand, kernel
 // entry and constants are set: device buffers, launch shape, uniform grid.
 vegas_status finish_create(vegas_ctx* c, vegas_ctx** out) {
@@ -716,6 +778,7 @@ vegas_status finish_create(vegas_ctx* c, vegas_ctx** out) {
     c->ppt_min = c->ke.spec_ppt_min;
     if (c->ke.grad_spec) c->ke.grad = c->ke.grad_spec;
   }
+  c->col = pick_col(c->ke, d, c->ybits, c->g, N);
   auto bail = [&](vegas_status st) {
     g_thread_err = c->err;
     vegas_destroy(c);
@@ -728,6 +791,9 @@ vegas_status finish_create(vegas_ctx* c, vegas_ctx** out) {
   e = gv_prepare_aux_kernels();
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(c->ke.sample, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             (int)cudaSharedmemCarveoutMaxShared);
+  if (e == cudaSuccess && c->col)
+    e = cudaFuncSetAttribute(c->col, cudaFuncAttributePreferredSharedMemoryCarveout,
                              (int)cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return bail(c->fail(VEGAS_ECUDA, "kernel attributes: %s", cudaGetErrorString(e)));
   if (cfg->stream) {
@@ -749,7 +815,6 @@ vegas_status finish_create(vegas_ctx* c, vegas_ctx** out) {
   if (!st) st = alloc((void**)&c->d_tab32, sizeof(float2) * d * N);
   if (!st) st = alloc((void**)&c->d_derived, sizeof c->derived + sizeof(double));  // + the output scale
   if (!st) st = alloc((void**)&c->d_bins, sizeof(double) * 2 * d * N);
-  if (!st) st = alloc((void**)&c->d_tot, sizeof(double) * gv::kTotCols);
   if (!st && c->strat) st = alloc((void**)&c->d_cubes, sizeof(double) * 2 * G);
   if (!st) st = alloc((void**)&c->d_cube_max, sizeof(double) * G);
   if (!st) st = alloc((void**)&c->d_st, sizeof(GState));
@@ -802,7 +867,6 @@ void vegas_destroy(vegas_ctx* c) {
   cudaFree(c->d_part_bins);
   cudaFree(c->d_part_tot);
   cudaFree(c->d_bins);
-  cudaFree(c->d_tot);
   cudaFree(c->d_cubes);
   cudaFree(c->d_cube_max);
   for (void* p : {(void*)c->d_q, (void*)c->d_mt, (void*)c->d_mt32, (void*)c->d_guide, (void*)c->d_bmax, (void*)c->d_bsum, (void*)c->d_prefix, (void*)c->d_meta, (void*)c->d_stage_x, (void*)c->d_stage_t,
@@ -1281,12 +1345,12 @@ vegas_status vegas_set_launch(vegas_ctx* c, int threads, int ctas_per_sm) {
     return c->fail(VEGAS_EINVAL, "threads must be a multiple of 32 in 64..%d", fa.maxThreadsPerBlock);
   if (ctas_per_sm < 0) return c->fail(VEGAS_EINVAL, "ctas_per_sm < 0");
   CK(c, cudaStreamSynchronize(c->stream));
-  const int t0 = c->threads, p0 = c->ctas_per_sm_req;
-  c->threads = threads;
+  const int t0 = c->threads_req, p0 = c->ctas_per_sm_req;
+  c->threads_req = threads;
   c->ctas_per_sm_req = ctas_per_sm;
   vegas_status st = configure_launch(c);
   if (st) {
-    c->threads = t0;
+    c->threads_req = t0;
     c->ctas_per_sm_req = p0;
     configure_launch(c);
   }
@@ -1374,9 +1438,9 @@ vegas_status vegas_get_tile(vegas_ctx* c, int* points_per_thread, int* cap) {
 
 vegas_status vegas_get_launch(vegas_ctx* c, int* threads, int* ctas, int* ctas_per_sm) {
   if (!c) return thread_fail(VEGAS_EINVAL, "ctx is NULL");
-  if (threads) *threads = c->threads;
-  if (ctas) *ctas = c->ctas;
-  if (ctas_per_sm) *ctas_per_sm = c->occ;
+  if (threads) *threads = c->pass_bins.threads;
+  if (ctas) *ctas = c->pass_bins.ctas;
+  if (ctas_per_sm) *ctas_per_sm = c->pass_bins.occ;
   return VEGAS_OK;
 }
 
@@ -1441,6 +1505,7 @@ vegas_status profile_passes(vegas_ctx* c, int n_pass, bool nobins, double* ms) {
   cudaEvent_t ev[3];
   for (int i = 0; i < 3; ++i) CK(c, cudaEventCreate(&ev[i]));
   double acc[3] = {0, 0, 0};
+  const gv::PassShape& ps = nobins ? c->pass_nobins : c->pass_bins;
   cudaError_t e = cudaSuccess;
   for (int p = 0; p < n_pass && e == cudaSuccess; ++p) {
     gv::SampleArgs A = sample_args(c, (int)(it & 0x7FFFFFFFu), nobins);
@@ -1448,8 +1513,7 @@ vegas_status profile_passes(vegas_ctx* c, int n_pass, bool nobins, double* ms) {
     gv::FinArgs F = fin_args(c, 0, 0, nobins);
     e = cudaEventRecord(ev[0], c->stream);
     if (!e)
-      e = cudaLaunchKernel(c->ke.sample, dim3(nobins ? c->ctas_nb : c->ctas), dim3(c->threads), args,
-                           nobins ? c->smem_nb : c->smem, c->stream);
+      e = cudaLaunchKernel(ps.fn, dim3(ps.ctas), dim3(ps.threads), args, ps.smem, c->stream);
     if (!e) e = cudaEventRecord(ev[1], c->stream);
     if (!e) e = gv_launch_finish(&F, c->stream);
     if (!e) e = cudaEventRecord(ev[2], c->stream);
@@ -1601,31 +1665,12 @@ extern "C" vegas_status vegas_eval_noalloc(const vegas_config* cfg, const vegas_
 
   // Launch shape (as for a context) with the CTA count bounded by the rows
   // of partial sums that fit in the scratch array.
-  const int threads = 256;
-  auto occ_of = [&](int cap, int) -> int {
-    const size_t sm = ke.smem(d, N, cap);
-    int o = 0;
-    if (e != cudaSuccess || sm > 227 * 1024) return 0;
-    e = gv_raise_smem_limit(ke.sample, sm);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, ke.sample, threads, sm);
-    return e == cudaSuccess ? o : 0;
-  };
-  int occ_cap = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_cap, ke.sample, threads, 0);
-  const gv::TileShape t = e == cudaSuccess ? gv::choose_tile(threads, N, 0, ppt_min, occ_cap, occ_of) : gv::TileShape{1, 4, 0};
-  if (e != cudaSuccess) return thread_fail(VEGAS_ECUDA, "launch configuration: %s", cudaGetErrorString(e));
-  if (t.occ < 1) return thread_fail(VEGAS_EINVAL, "sampling kernel does not fit in shared memory");
-  const int ppt = t.ppt, cap = t.cap, occ = t.occ;
-  const size_t smem = ke.smem(d, N, cap);
-  e = gv_raise_smem_limit(ke.sample, smem);
-  if (e != cudaSuccess) return thread_fail(VEGAS_ECUDA, "launch configuration: %s", cudaGetErrorString(e));
   const int dN = d * N;
   const size_t off_st = 0;
   const size_t off_dp = align256(off_st + sizeof(GState));
   const size_t off_t64 = align256(off_dp + sizeof(double) * (gv::kNumDerived + 1));
   const size_t off_t32 = align256(off_t64 + sizeof(double2) * dN);
-  const size_t off_tot = align256(off_t32 + sizeof(float2) * dN);
-  const size_t off_rows = align256(off_tot + sizeof(double) * gv::kTotCols);
+  const size_t off_rows = align256(off_t32 + sizeof(float2) * dN);
   const size_t row_bytes = sizeof(double) * (2 * (size_t)dN + gv::kTotCols);
   const int64_t max_rows = off_rows < kNoAllocScratchBytes ? (int64_t)((kNoAllocScratchBytes - off_rows - 512) / row_bytes) : 0;
   if (max_rows < 1)
@@ -1633,14 +1678,37 @@ extern "C" vegas_status vegas_eval_noalloc(const vegas_config* cfg, const vegas_
                        kNoAllocScratchBytes);
   const uint64_t nc = (uint64_t)cfg->ncall / G;
   const int strat = G > 1;
-  const int64_t cap_ctas = (int64_t)sms * occ;
-  int L = 1;
-  uint64_t units = (uint64_t)cfg->ncall;
-  if (strat) {
-    L = gv::choose_lanes(G, nc, threads, std::min<int64_t>(cap_ctas, max_rows));
-    units = G * (uint64_t)L;
+  gv::PassShape ps;
+  int ppt = d <= 8 ? 2 : 1, cap = 0;
+  const void* col = pick_col(ke, d, ybits, g, N);
+  if (!col || !shape_col(col, ke, d, N, sms, 0, 0, G, nc, (uint64_t)cfg->ncall, max_rows, &ps, &e)) {
+    const int threads = 256;
+    auto occ_of = [&](int cp, int) -> int {
+      const size_t sm = ke.smem(d, N, cp);
+      int o = 0;
+      if (e != cudaSuccess || sm > 227 * 1024) return 0;
+      e = gv_raise_smem_limit(ke.sample, sm);
+      if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, ke.sample, threads, sm);
+      return e == cudaSuccess ? o : 0;
+    };
+    int occ_cap = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_cap, ke.sample, threads, 0);
+    const gv::TileShape t = e == cudaSuccess ? gv::choose_tile(threads, N, 0, ppt_min, occ_cap, occ_of) : gv::TileShape{1, 4, 0};
+    if (e != cudaSuccess) return thread_fail(VEGAS_ECUDA, "launch configuration: %s", cudaGetErrorString(e));
+    if (t.occ < 1) return thread_fail(VEGAS_EINVAL, "sampling kernel does not fit in shared memory");
+    ppt = t.ppt;
+    cap = t.cap;
+    ps.fn = ke.sample;
+    ps.threads = threads;
+    ps.smem = ke.smem(d, N, cap);
+    e = gv_raise_smem_limit(ke.sample, ps.smem);
+    const int64_t most = std::min<int64_t>((int64_t)sms * t.occ, max_rows);
+    ps.lanes = strat ? gv::choose_lanes(G, nc, threads, most) : 1;
+    const uint64_t units = strat ? G * (uint64_t)ps.lanes : (uint64_t)cfg->ncall;
+    ps.ctas = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)((units + threads - 1) / threads), most));
   }
-  const int ctas = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)((units + threads - 1) / threads), cap_ctas, max_rows}));
+  if (e != cudaSuccess) return thread_fail(VEGAS_ECUDA, "launch configuration: %s", cudaGetErrorString(e));
+  const int ctas = ps.ctas;
   double* part_tot = reinterpret_cast<double*>(scratch + off_rows);
   double* part_bins = reinterpret_cast<double*>(scratch + align256(off_rows + sizeof(double) * gv::kTotCols * ctas));
   GState* st = reinterpret_cast<GState*>(scratch + off_st);
@@ -1664,7 +1732,7 @@ extern "C" vegas_status vegas_eval_noalloc(const vegas_config* cfg, const vegas_
   A.N = N;
   A.g = g;
   A.ybits = ybits;
-  A.lanes = L;
+  A.lanes = ps.lanes;
   A.cap = cap;
   A.ppt = ppt;
   A.strat = strat;
@@ -1694,7 +1762,7 @@ extern "C" vegas_status vegas_eval_noalloc(const vegas_config* cfg, const vegas_
   A.part_tot = part_tot;
   A.cubes = nullptr;
   void* args[] = {&A};
-  e = cudaLaunchKernel(ke.sample, dim3(ctas), dim3(threads), args, smem, s);
+  e = cudaLaunchKernel(ps.fn, dim3(ctas), dim3(ps.threads), args, ps.smem, s);
   gv::FinArgs F{};
   F.d = d;
   F.N = N;
@@ -1710,7 +1778,6 @@ extern "C" vegas_status vegas_eval_noalloc(const vegas_config* cfg, const vegas_
   F.part_bins = part_bins;
   F.part_tot = part_tot;
   F.bins = out;
-  F.tot = reinterpret_cast<double*>(scratch + off_tot);
   F.edges = nullptr;
   F.tab64 = reinterpret_cast<double2*>(scratch + off_t64);
   F.tab32 = reinterpret_cast<float2*>(scratch + off_t32);

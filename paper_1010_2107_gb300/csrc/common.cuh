@@ -213,7 +213,6 @@ struct GState {
   double ph1_I, ph1_sigma, ph1_chi2;
   int ph1_iters, ph1_stopped;
   long long ph1_nonfinite, ph1_samples;
-  unsigned arrive[kMaxDim + 1];  // block arrivals per group of k_finish (reset by the last)
   double hist[kMaxHist][2];
 };
 
@@ -248,7 +247,7 @@ struct SampleArgs {
   const void* tab;         // [d][N] (e_k, Delta_k) in the kernel precision
   const double* dparams;   // derived integrand constants
   GState* st;              // the sampling kernel latches st->live
-  void* part_bins;         // [2 d N][nparts]: double, or float (hi, lo) pairs (FP32 forms)
+  void* part_bins;         // [nparts][2 d N]: double, or float (hi, lo) pairs (FP32 forms)
   double* part_tot;        // [kTotCols][nparts]
   void* cubes;             // [ncubes]: double (sum w, sum w^2), or float (hi, lo, hi, lo)
   double* cube_max;        // [ncubes] running max(0, largest w) (integration phase), or null
@@ -267,7 +266,6 @@ struct FinArgs {
   const void* part_bins;
   const double* part_tot;
   double* bins;            // [2][d][N] reduced, scaled
-  double* tot;             // [kTotCols] reduced, scaled
   double* edges;           // [d][N+1]
   double2* tab64;          // [d][N]
   float2* tab32;           // [d][N]

@@ -1,13 +1,14 @@
 // finalize.cu -- steps 4-6 of Sec. 2.1 after the sampling pass, all on the
 // GPU in FP64 (the paper ran them on the host, Sec. 2.2), in one launch:
 //   k_finish    fixed-order reduction of the per-CTA partial rows into the
-//               per-bin sums S1, S2 and the iteration totals (one warp per
-//               column; lanes stride the rows, then an xor butterfly); the
-//               last block of each axis then runs the grid optimisation
-//               (Lepage 1978: smoothing, log-compression with exponent
-//               alpha, rebinning to equal weight) and the last block of the
-//               totals the iteration estimate, the inverse-variance
+//               per-bin sums S1, S2 and the iteration totals; one cluster of
+//               CTAs per axis, whose first CTA then runs the grid
+//               optimisation (Lepage 1978: smoothing, log-compression with
+//               exponent alpha, rebinning to equal weight), and one CTA that
+//               forms the iteration estimate, the inverse-variance
 //               combination, chi^2 and the ACC test.
+#include <cooperative_groups.h>
+
 #include <map>
 #include <mutex>
 #include <utility>
@@ -18,37 +19,15 @@
 
 namespace gv {
 
-// Fixed-order sum of one column of per-CTA partials by one warp (lanes
-// stride the rows, eight loads in flight, then an xor butterfly); compensated
-// FP32 pairs or doubles.  Returns the sum on every lane.
-__device__ double column_sum(const FinArgs& F, int col, int lane) {
-  const int dN = F.d * F.N, np = F.nparts;
-  if (col < 2 * dN && F.pair32) {
-    const float2* p = reinterpret_cast<const float2*>(F.part_bins) + (size_t)col * np;
-    fpair acc{0.f, 0.f};
-    int r = lane;
-    for (; r + 7 * 32 < np; r += 8 * 32) {
-      float2 v[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = __ldcg(p + r + 32 * j);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) comp_merge(acc, fpair{v[j].x, v[j].y});
-    }
-    for (; r < np; r += 32) {
-      const float2 v = __ldcg(p + r);
-      comp_merge(acc, fpair{v.x, v.y});
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      fpair o;
-      o.hi = __shfl_xor_sync(0xffffffffu, acc.hi, off);
-      o.lo = __shfl_xor_sync(0xffffffffu, acc.lo, off);
-      comp_merge(acc, o);
-    }
-    return comp_value(acc);
-  }
-  const double* src = col < 2 * dN ? reinterpret_cast<const double*>(F.part_bins) + (size_t)col * np
-                                   : F.part_tot + (size_t)(col - 2 * dN) * np;
+// CTAs per cluster of k_finish: an axis's partial rows are shared out over
+// this many SMs.
+constexpr int kFinishCluster = 8;
+// Thread slices per column within a CTA, at most.
+constexpr int kFinishSlices = 8;
+
+// Sum of one per-CTA totals column by one warp (lanes stride the rows, eight
+// loads in flight, then a fixed xor butterfly); every lane gets the sum.
+__device__ double total_column(const double* src, int np, int lane) {
   double acc = 0.0;
   int r = lane;
   for (; r + 7 * 32 < np; r += 8 * 32) {
@@ -64,25 +43,83 @@ __device__ double column_sum(const FinArgs& F, int col, int lane) {
   return acc;
 }
 
-// Refinement of axis a from its S2 column sums, which other blocks of this
-// launch wrote: read past L1 into shared memory first.  One thread per bin
-// (whole warps) takes part; the other warps leave.
-__device__ void refine_axis(const FinArgs& F, int a) {
-  __shared__ double s2[kMaxBins];
-  const int N = F.N;
-  const Team t{min((int)blockDim.x, (N + 31) / 32 * 32)};
-  if ((int)threadIdx.x >= t.n) return;
-  const double* src = F.bins + (size_t)F.d * N + (size_t)a * N;
-  for (int k = threadIdx.x; k < N; k += t.n) s2[k] = __ldcg(src + k);
-  t.sync();
-  refine_axis_core(s2, F.edges + (size_t)a * (N + 1), F.tab64 + (size_t)a * N, F.tab32 + (size_t)a * N, N,
-                   F.alpha, t);
+// A partial sum of the rows: a compensated FP32 pair or a double.
+__device__ __forceinline__ void psum_add(fpair& a, const float2& v) { comp_merge(a, fpair{v.x, v.y}); }
+__device__ __forceinline__ void psum_add(double& a, const double& v) { a += v; }
+__device__ __forceinline__ void psum_merge(fpair& a, const fpair& b) { comp_merge(a, b); }
+__device__ __forceinline__ void psum_merge(double& a, const double& b) { a += b; }
+__device__ __forceinline__ double psum_value(const fpair& a) { return comp_value(a); }
+__device__ __forceinline__ double psum_value(const double& a) { return a; }
+__device__ __forceinline__ void psum_zero(fpair& a) { a = fpair{0.f, 0.f}; }
+__device__ __forceinline__ void psum_zero(double& a) { a = 0.0; }
+
+// The 2N columns (S1 then S2) of axis a over the rows of this cluster: CTA
+// `rank` takes rows rank, rank + 8, ..., its threads the columns, in
+// nsl slices of those rows; the slices, then the CTAs, are merged in order
+// by the cluster's first CTA.  The rows are stored [CTA][2 d N], so a warp
+// reads consecutive columns of a row.  V: stored element, S: running sum.
+// Returns in the first CTA's s2[] the scaled S2 sums.
+template <typename V, typename S>
+__device__ __forceinline__ void reduce_axis(const FinArgs& F, int a, unsigned rank, S* buf, double* s2) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int N = F.N, dN = F.d * N, C = 2 * N, np = F.nparts, T = kFinishThreads;
+  const int nsl = min(kFinishSlices, max(1, T / C));
+  const int j = threadIdx.x % C, sl = threadIdx.x / C;  // column and slice (C <= T: one column per thread)
+  const size_t stride = 2 * (size_t)dN;
+  for (int c = C <= T ? j : (int)threadIdx.x; c < C && sl < nsl; c += C <= T ? C : T) {
+    const int slice = C <= T ? sl : 0;
+    const V* src = reinterpret_cast<const V*>(F.part_bins) + (c < N ? a * N + c : dN + a * N + (c - N));
+    const int step = kFinishCluster * nsl;
+    int r = (int)rank + kFinishCluster * slice;
+    S acc;
+    psum_zero(acc);
+    for (; r + 7 * step < np; r += 8 * step) {
+      V v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = __ldcg(src + (size_t)(r + u * step) * stride);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) psum_add(acc, v[u]);
+    }
+    V v[8];
+    int m = 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (r + u * step < np) {
+        v[u] = __ldcg(src + (size_t)(r + u * step) * stride);
+        m = u + 1;
+      }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (u < m) psum_add(acc, v[u]);
+    buf[slice * C + c] = acc;
+  }
+  __syncthreads();
+  for (int c = threadIdx.x; c < C && nsl > 1; c += T) {
+    S acc = buf[c];
+    for (int q = 1; q < nsl; ++q) psum_merge(acc, buf[q * C + c]);
+    buf[c] = acc;
+  }
+  cl.sync();
+  if (rank == 0) {
+    const double sc = *F.scale;
+    for (int c = threadIdx.x; c < C; c += T) {
+      S q[kFinishCluster];
+#pragma unroll
+      for (int k = 0; k < kFinishCluster; ++k) q[k] = cl.map_shared_rank(buf, k)[c];
+#pragma unroll
+      for (int k = 1; k < kFinishCluster; ++k) psum_merge(q[0], q[k]);
+      const double v = psum_value(q[0]) * (c < N ? sc : sc * sc);
+      F.bins[c < N ? a * N + c : dN + a * N + (c - N)] = v;
+      if (c >= N) s2[c - N] = v;
+    }
+  }
+  cl.sync();  // the first CTA has read the others' sums; s2 is complete
 }
 
 // Step 6 for the pass, by one full warp (lane 0 writes the state).
-__device__ void record_iteration(const FinArgs& F) {
+__device__ void record_iteration(const FinArgs& F, const double* t) {
   GState* st = F.st;
-  const double* t = F.tot;
   const int lane = threadIdx.x & 31;
   double I, var;
   if (F.strat) {
@@ -132,56 +169,49 @@ __device__ void record_iteration(const FinArgs& F) {
   }
 }
 
-// Steps 4-6 after a sampling pass in one launch.  Blocks come in groups:
-// group a < d reduces the 2N columns (S1, S2) of axis a, one warp per
-// column, and the last of its blocks to finish (an arrival counter, after
-// a memory fence) refines axis a; the final group reduces the iteration
-// totals and records the iteration.  No block waits for another: the last
-// arrival does the dependent work.  `live` was latched by the sampling
-// kernel of this pass and the ACC test below writes only `done`.
-__global__ void __launch_bounds__(kFinishThreads) k_finish(const FinArgs F) {
+// Steps 4-6 after a sampling pass in one launch.  Cluster a < d reduces the
+// 2N columns (S1, S2) of axis a and its first CTA refines the axis; the last
+// cluster's first CTA reduces the iteration totals and records the
+// iteration.  No block waits for another cluster.  `live` was latched by the
+// sampling kernel of this pass and the ACC test below writes only `done`.
+//
+// Bound by latency: the rows are read once (dgauss8: 152 rows of 6.4 KB)
+// with every load of a thread in flight, the merge crosses the SMs through
+// distributed shared memory, without a memory fence and an arrival counter,
+// and what remains is the dependent FP64 chain of the refinement.
+__global__ void __cluster_dims__(kFinishCluster, 1, 1) __launch_bounds__(kFinishThreads) k_finish(const FinArgs F) {
+  __shared__ __align__(16) unsigned char buf[kFinishThreads * 16 > 2 * kMaxBins * 8 ? kFinishThreads * 16 : 2 * kMaxBins * 8];
+  __shared__ double s2[kMaxBins];
+  __shared__ double tot[kTotCols];
   GState* st = F.st;
-  if (!st->live) return;
-  const int wpb = kFinishThreads / 32, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int N = F.N, dN = F.d * N;
-  const int bpa = (2 * N + wpb - 1) / wpb;  // blocks per axis
-  const int b = blockIdx.x;
-  // without per-bin sums only the totals block is launched
-  const int group = (!F.nobins && b < F.d * bpa) ? b / bpa : F.d;
+  if (!st->live) return;  // (uniform over the launch)
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned rank = blockIdx.x % kFinishCluster;
+  const int group = F.nobins ? F.d : (int)(blockIdx.x / kFinishCluster);
   if (group < F.d) {
-    const int a = group, i = (b - a * bpa) * wpb + warp;  // column of the axis, 0 .. 2N
-    if (i < 2 * N) {
-      const int col = i < N ? a * N + i : dN + a * N + (i - N);
-      const double v = column_sum(F, col, lane);
-      const double sc = *F.scale;
-      if (lane == 0) F.bins[col] = v * (i < N ? sc : sc * sc);
-    }
-  } else if (warp < kTotCols) {
+    if (F.pair32)
+      reduce_axis<float2, fpair>(F, group, rank, reinterpret_cast<fpair*>(buf), s2);
+    else
+      reduce_axis<double, double>(F, group, rank, reinterpret_cast<double*>(buf), s2);
+    if (rank != 0 || !F.refine) return;
+    // one thread per bin (whole warps) refines; the other warps leave
+    const int N = F.N, a = group;
+    const Team t{min((int)blockDim.x, (N + 31) / 32 * 32)};
+    if ((int)threadIdx.x >= t.n) return;
+    refine_axis_core(s2, F.edges + (size_t)a * (N + 1), F.tab64 + (size_t)a * N, F.tab32 + (size_t)a * N, N,
+                     F.alpha, t);
+    return;
+  }
+  if (rank != 0) return;
+  if (warp < 5) {
     const int q = warp;
-    if (q < 5) {
-      const double v = column_sum(F, 2 * dN + q, lane);
-      const double s1 = *F.scale;
-      const double sc = (q == TOT_SW || q == TOT_SI) ? s1 : (q == TOT_NONFINITE ? 1.0 : s1 * s1);
-      if (lane == 0) F.tot[q] = v * sc;
-    }
-  }
-  // arrival: the group's last block continues
-  __shared__ int last;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const int n = group < F.d ? bpa : 1;
-    last = atomicAdd(&st->arrive[group], 1u) == (unsigned)(n - 1);
-    if (last) st->arrive[group] = 0;  // ready for the next pass
+    const double v = total_column(F.part_tot + (size_t)q * F.nparts, F.nparts, lane);
+    const double s1 = *F.scale;
+    const double sc = (q == TOT_SW || q == TOT_SI) ? s1 : (q == TOT_NONFINITE ? 1.0 : s1 * s1);
+    if (lane == 0) tot[q] = v * sc;
   }
   __syncthreads();
-  if (!last) return;
-  __threadfence();
-  if (group < F.d) {
-    if (F.refine && !F.nobins) refine_axis(F, group);
-  } else if (threadIdx.x < 32) {
-    record_iteration(F);
-  }
+  if (warp == 0) record_iteration(F, tot);
 }
 
 // Column sums of a [ncols][nrows] partial block (one warp per column,
@@ -278,8 +308,7 @@ cudaError_t gv_raise_smem_limit(const void* fn, size_t bytes) {
 }
 
 cudaError_t gv_launch_finish(const gv::FinArgs* F, cudaStream_t s) {
-  const int wpb = gv::kFinishThreads / 32;
-  const int blocks = F->nobins ? 1 : F->d * ((2 * F->N + wpb - 1) / wpb) + 1;
+  const int blocks = gv::kFinishCluster * (F->nobins ? 1 : F->d + 1);
   gv::k_finish<<<blocks, gv::kFinishThreads, 0, s>>>(*F);
   return cudaGetLastError();
 }

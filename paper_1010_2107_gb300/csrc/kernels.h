@@ -21,6 +21,10 @@ struct KernelEntry {
   const void* sample;                 // k_sample<T, DM, F, ACC, YB, false> (any d <= DM)
   const void* sample_spec;            // k_sample<..., true>: d == DM, 24-bit, power-of-two
                                       // divisions with g N <= 256; may be null
+  const void* sample_col;             // k_sample_col<DM, F, false>: the FP32 form with 24-bit words,
+                                      // column histogram (any d <= DM, the divisions of sample_spec); or null
+  const void* sample_col_exact;       // k_sample_col<DM, F, true>: d == DM
+  size_t (*smem_col)(int d, int N, int nwarps);  // their dynamic shared memory
   const void* dump;                   // k_dump<T, DM, F>
   size_t (*smem)(int d, int N, int cap);  // dynamic shared memory of `sample`
                                           // with bucket capacity cap
@@ -72,6 +76,15 @@ bool derive_params(int kind, int d, const double* p, double* dv, double* scale, 
 int rtc_user_entry(const char* source, int prec, int ybits, int d, bool spec, KernelEntry* out, std::string* why);
 // The same compile without loading (no device needed); the result is cached.
 int rtc_user_compile(const char* source, int prec, int ybits, int d, bool spec, std::string* why);
+
+// Launch shape of one kind of sampling pass.
+struct PassShape {
+  const void* fn = nullptr;
+  int ctas = 0, threads = 256;
+  int lanes = 1;    // lanes per hypercube (stratified sampling)
+  int occ = 0;      // CTAs per SM
+  size_t smem = 0;  // dynamic shared memory
+};
 
 // Histogram tile of a sampling kernel: ppt points per thread between two
 // gathers, bucket capacity cap per (axis, bin), and the CTAs per SM that
@@ -147,6 +160,32 @@ inline int choose_lanes(uint64_t G, uint64_t nc, int threads, int64_t ctas) {
   int L = 1;
   while (L < 32 && (uint64_t)(2 * L) <= nc && G * (uint64_t)L < 4 * (uint64_t)ctas * (uint64_t)threads) L *= 2;
   return L;
+}
+
+// Lanes per hypercube where a tile's crowding does not matter (the column
+// histogram, passes without a histogram): the power of two L <= min(32, nc)
+// of least cost.  A CTA of `threads` threads takes the G L lanes in rounds;
+// a round costs a lane's points (in steps of `pif`) and, in eighths of a
+// point, 0.6 per level of the group's butterfly and 3 for the cube's own
+// totals; an SM runs its share of the rounds, and about one more while its
+// last CTAs leave it partly idle.  (Measured, us per pass at 2^22 points:
+// dgauss8, 65 536 cubes of 64, L = 4, 8, 16, 32: 66, 60.5, 63.5, 70.5 with
+// columns and 52, 48, 52, 61 without; wmunu, 32 768 of 128: 72, 73, 66, 70
+// and 61, 62, 57, 61.  The rule takes 8 and 16.)
+inline int balanced_lanes(uint64_t G, uint64_t nc, int threads, int sms, int pif) {
+  int best = 1;
+  double least = 0.0;
+  for (int L = 1, lg = 0; L <= 32 && (uint64_t)L <= nc; L *= 2, ++lg) {
+    const uint64_t rounds = (G * (uint64_t)L + threads - 1) / threads, per_sm = (rounds + sms - 1) / sms;
+    uint64_t pts = (nc + L - 1) / L;
+    pts = (pts + pif - 1) / pif * pif;
+    const double cost = (double)(per_sm + 1) * (8.0 * (double)pts + 0.6 * lg + 3.0);
+    if (L == 1 || cost < least) {
+      least = cost;
+      best = L;
+    }
+  }
+  return best;
 }
 
 #endif  // __CUDACC_RTC__

@@ -83,7 +83,7 @@ const Nvrtc* nvrtc(std::string* why) {
 }
 
 // Kernels of one program: which are built and their names.
-enum { K_SAMPLE = 0, K_SPRING = 1, K_DUMP = 2, K_COUNT = 3 };
+enum { K_SAMPLE = 0, K_SPRING = 1, K_DUMP = 2, K_COL = 3, K_COUNT = 4 };
 
 struct Shape {
   int prec, ybits, d;
@@ -98,6 +98,10 @@ static_assert(kPairPoints<float, 8, true> && !kPairPoints<float, 9, true> && !kP
               "pair rule of the specialised sampling kernel");
 int spec_ppt_min(const Shape& s) { return s.spec && s.prec != VG_FP64 && s.d <= 8 ? 2 : 1; }
 
+// Kernels of a shape's program: the column-histogram kernel exists for the
+// specialised FP32 form with compensated sums.
+int kernel_count(const Shape& s) { return s.spec && s.prec == VG_FP32_ACCCOMP ? K_COUNT : K_COL; }
+
 // Template arguments (T, ACC) of the precision.
 const char* type_of(int prec) { return prec == VG_FP64 ? "double" : "float"; }
 int acc_of(int prec) { return prec == VG_FP64 ? 0 : (prec == VG_FP32_ACC64 ? 1 : 2); }
@@ -109,6 +113,8 @@ std::string name_expr(int k, const Shape& s) {
     case K_SAMPLE:
       return "&gv::k_sample<" + T + ", " + D + ", gv::UserIntegrand, " + std::to_string(acc_of(s.prec)) + ", " + Y +
              ", " + sp + ">";
+    case K_COL:
+      return "&gv::k_sample_col<" + D + ", gv::UserIntegrand, true>";
     case K_SPRING:
       return "&gv::k_spring<" + T + ", " + D + ", gv::UserIntegrand, " + Y + ", " + sp + ">";
     default:
@@ -165,7 +171,7 @@ int compile(const char* source, const Shape& s, Compiled* out, std::string* why)
     if (*p) nvrtc(nullptr)->destroy(p);
   });
   std::string exprs[K_COUNT];
-  for (int k = 0; k < K_COUNT; ++k) {
+  for (int k = 0; k < kernel_count(s); ++k) {
     exprs[k] = name_expr(k, s);
     if ((r = api->add_name(prog, exprs[k].c_str())) != NVRTC_SUCCESS) {
       *why = std::string("nvrtcAddNameExpression: ") + api->err(r);
@@ -196,7 +202,7 @@ int compile(const char* source, const Shape& s, Compiled* out, std::string* why)
     *why = std::string("nvrtcGetCUBIN: ") + api->err(r);
     return VEGAS_ECUDA;
   }
-  for (int k = 0; k < K_COUNT; ++k) {
+  for (int k = 0; k < kernel_count(s); ++k) {
     const char* low = nullptr;
     if ((r = api->lowered(prog, exprs[k].c_str(), &low)) != NVRTC_SUCCESS || !low) {
       *why = "nvrtcGetLoweredName failed for " + exprs[k];
@@ -206,6 +212,18 @@ int compile(const char* source, const Shape& s, Compiled* out, std::string* why)
   }
   return VEGAS_OK;
 }
+
+// Shared memory of the column-histogram kernel: its layout depends on the
+// compile-time bound, here the dimension itself.
+template <int D>
+size_t col_smem_upto(int d, int N, int nwarps) {
+  if constexpr (D > kMaxDim) {
+    return 0;
+  } else {
+    return d == D ? ColSmem<D, true>::total(d, N, nwarps) : col_smem_upto<D + 1>(d, N, nwarps);
+  }
+}
+size_t col_smem_user(int d, int N, int nwarps) { return col_smem_upto<1>(d, N, nwarps); }
 
 std::string cache_key(const char* source, const Shape& s) {
   return std::to_string(s.prec) + "," + std::to_string(s.ybits) + "," + std::to_string(s.d) + "," +
@@ -278,7 +296,7 @@ int rtc_user_entry(const char* source, int prec, int ybits, int d, bool spec, Ke
     return VEGAS_ECUDA;
   }
   cudaKernel_t k[K_COUNT] = {};
-  for (int i = 0; i < K_COUNT && e == cudaSuccess; ++i) e = cudaLibraryGetKernel(&k[i], lib, c->lowered[i].c_str());
+  for (int i = 0; i < kernel_count(s) && e == cudaSuccess; ++i) e = cudaLibraryGetKernel(&k[i], lib, c->lowered[i].c_str());
   if (e != cudaSuccess) {
     cudaLibraryUnload(lib);
     *why = std::string("cudaLibraryGetKernel: ") + cudaGetErrorString(e);
@@ -290,6 +308,8 @@ int rtc_user_entry(const char* source, int prec, int ybits, int d, bool spec, Ke
   ke.spring = (const void*)k[K_SPRING];
   ke.spring_spec = s.spec ? ke.spring : nullptr;
   ke.dump = (const void*)k[K_DUMP];
+  ke.sample_col_exact = (const void*)k[K_COL];
+  ke.smem_col = &col_smem_user;
   ke.smem = prec == VG_FP64 ? &sample_smem_bytes<double, 0>
                             : (prec == VG_FP32_ACC64 ? &sample_smem_bytes<float, 1> : &sample_smem_bytes<float, 2>);
   ke.smem_nobins = prec == VG_FP64 ? &sample_smem_nobins<double, 0>

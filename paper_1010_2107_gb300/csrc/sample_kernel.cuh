@@ -22,6 +22,7 @@ template <class A, class B> struct conditional<false, A, B> { using type = B; };
 #include <type_traits>
 #endif
 
+#include "col_hist.cuh"
 #include "common.cuh"
 #include "integrands.cuh"
 #include "kernels.h"
@@ -376,6 +377,55 @@ __device__ __forceinline__ fpair warp_sum(fpair p) {
   return p;
 }
 
+// Step 4 of one hypercube from its compensated sums: the cube mean m = C1 /
+// nc and variance (C2 / nc - m^2) / (nc - 1) into the totals, in FP32 with
+// the square formed exactly (FMA) and the pairs kept, and the cube's sums.
+__device__ __forceinline__ void cube_totals(const SampleArgs& A, uint32_t c, const fpair& c1, const fpair& c2,
+                                            fpair (&tp)[4]) {
+  const float inv = (float)A.inv_nc, inv1 = (float)A.inv_nc1;
+  const float mh = c1.hi * inv, ml = c1.lo * inv;
+  const float sq = mh * mh;
+  const float sqe = fmaf(mh, mh, -sq) + 2.0f * mh * ml;
+  const float e2h = c2.hi * inv, e2l = c2.lo * inv;
+  float v = ((e2h - sq) + (e2l - sqe)) * inv1;
+  if (!(v > 0.f)) v = 0.f;
+  comp_merge(tp[0], c1);
+  comp_merge(tp[1], c2);
+  comp_add(tp[2], mh);
+  comp_add(tp[2], ml);
+  comp_add(tp[3], v);
+  if (A.cubes) reinterpret_cast<float4*>(A.cubes)[c] = make_float4(c1.hi, c1.lo, c2.hi, c2.lo);
+}
+
+// The CTA's totals (compensated pairs per thread) into its column of
+// part_tot: fixed butterflies, then the warps in order.
+__device__ __forceinline__ void store_totals(const SampleArgs& A, const fpair (&tp)[4], int nonfinite) {
+  __shared__ double wnf[32];
+  __shared__ fpair wpair[32][4];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const fpair v = warp_sum(tp[q]);
+    if (lane == 0) wpair[warp][q] = v;
+  }
+  int nf = nonfinite;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) nf += __shfl_xor_sync(0xffffffffu, nf, off);
+  if (lane == 0) wnf[warp] = (double)nf;
+  __syncthreads();
+  if (tid < 5) {
+    double acc = 0.0;
+    if (tid < 4) {
+      fpair p{0.f, 0.f};
+      for (int w = 0; w < nw; ++w) comp_merge(p, wpair[w][tid]);
+      acc = comp_value(p);
+    } else {
+      for (int w = 0; w < nw; ++w) acc += wnf[w];
+    }
+    A.part_tot[(size_t)tid * A.nparts + blockIdx.x] = acc;
+  }
+}
+
 // Threads per CTA a sampling kernel may be launched with: the specialised
 // kernels up to 512 (larger tiles for many cells), the general ones 256
 // (their register budget).
@@ -615,22 +665,7 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>) k_sample(const Sample
             comp_merge(c2, o2);
           }
           if (live && gl == 0) {
-            // cube mean m = C1 / nc and variance (C2 / nc - m^2) / (nc - 1),
-            // in FP32 with the square formed exactly (FMA) and the pairs kept
-            const float inv = (float)A.inv_nc, inv1 = (float)A.inv_nc1;
-            const float mh = c1.hi * inv, ml = c1.lo * inv;
-            const float sq = mh * mh;
-            const float sqe = fmaf(mh, mh, -sq) + 2.0f * mh * ml;
-            const float e2h = c2.hi * inv, e2l = c2.lo * inv;
-            float v = ((e2h - sq) + (e2l - sqe)) * inv1;
-            if (!(v > 0.f)) v = 0.f;
-            comp_merge(tp[0], c1);
-            comp_merge(tp[1], c2);
-            comp_add(tp[2], mh);
-            comp_add(tp[2], ml);
-            comp_add(tp[3], v);
-            if (A.cubes)
-              reinterpret_cast<float4*>(A.cubes)[c] = make_float4(c1.hi, c1.lo, c2.hi, c2.lo);
+            cube_totals(A, c, c1, c2, tp);
           }
         } else {
           double c1 = p1, c2 = p2;
@@ -664,25 +699,20 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>) k_sample(const Sample
 
   // Partial row of this CTA: histogram cells (FP64, or compensated FP32
   // pairs) including the overflow cells, then the totals.
-  const int np = A.nparts, row = blockIdx.x;
+  const int row = blockIdx.x;
   for (int i = tid; bins && i < 2 * dN; i += blockDim.x) {
     if constexpr (COMP) {
       const fpair p = hist.pair(i);
-      reinterpret_cast<float2*>(A.part_bins)[(size_t)i * np + row] = make_float2(p.hi, p.lo);
+      reinterpret_cast<float2*>(A.part_bins)[(size_t)row * 2 * dN + i] = make_float2(p.hi, p.lo);
     } else {
-      reinterpret_cast<double*>(A.part_bins)[(size_t)i * np + row] = hist.value(i);
+      reinterpret_cast<double*>(A.part_bins)[(size_t)row * 2 * dN + i] = hist.value(i);
     }
   }
 
-  __shared__ double wsum[32][5];
-  __shared__ fpair wpair[32][4];
   if constexpr (COMP) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const fpair v = warp_sum(tp[q]);
-      if (lane == 0) wpair[warp][q] = v;
-    }
+    store_totals(A, tp, nonfinite);
   } else {
+    __shared__ double wsum[32][5];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       double v = t[q];
@@ -690,23 +720,231 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>) k_sample(const Sample
       for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
       if (lane == 0) wsum[warp][q] = v;
     }
-  }
-  int nf = nonfinite;
+    int nf = nonfinite;
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) nf += __shfl_xor_sync(0xffffffffu, nf, off);
-  if (lane == 0) wsum[warp][4] = (double)nf;
-  __syncthreads();
-  if (tid < 5) {
-    double acc = 0.0;
-    if (COMP && tid < 4) {
-      fpair p{0.f, 0.f};
-      for (int w = 0; w < nw; ++w) comp_merge(p, wpair[w][tid]);
-      acc = comp_value(p);
-    } else {
+    for (int off = 16; off > 0; off >>= 1) nf += __shfl_xor_sync(0xffffffffu, nf, off);
+    if (lane == 0) wsum[warp][4] = (double)nf;
+    __syncthreads();
+    if (tid < 5) {
+      double acc = 0.0;
       for (int w = 0; w < nw; ++w) acc += wsum[w][tid];
+      A.part_tot[(size_t)tid * A.nparts + row] = acc;
     }
-    A.part_tot[(size_t)tid * np + row] = acc;
   }
+}
+
+// ---------------------------------------------------------------------------
+// The sampling pass with the column histogram (col_hist.cuh): the FP32 form
+// with compensated sums, 24-bit words and a power-of-two number of
+// hypercube divisions with g N <= 256, in passes that keep the per-bin sums.
+// EXACT: d equals the compile-time bound DM; otherwise any d <= DM.
+// The points, weights and totals are those of k_sample (same samples per
+// thread, same arithmetic); only the per-bin sums are formed differently.
+// ---------------------------------------------------------------------------
+// Points per thread in flight: two up to 8 dimensions (registers).
+template <int DM>
+constexpr int kColPif = DM <= 8 ? 2 : 1;
+
+// One point as make_point's specialised form computes it (the same bits),
+// with the bins packed in bytes; slot(a) is called once per axis.
+template <int DM, bool EXACT, class SLOT>
+__device__ __forceinline__ float col_point(const SampleArgs& A, int d, uint32_t it, uint32_t s, const int (&cd)[DM],
+                                           const float2* tab, float (&x)[DM], uint32_t (&kb)[(DM + 3) / 4],
+                                           SLOT slot) {
+  const float Nf = (float)A.N;
+  const int sh = 24 + A.g_log2;
+  float J = 1.f;
+  uint4 w4 = make_uint4(0, 0, 0, 0);
+#pragma unroll
+  for (int q = 0; q < (DM + 3) / 4; ++q) kb[q] = 0u;
+#pragma unroll
+  for (int a = 0; a < DM; ++a)
+    if (EXACT || a < d) {
+      if ((a & 3) == 0) w4 = philox4x32_10(make_uint4(s, (uint32_t)(a >> 2), it, A.instance), A.ks);
+      const uint32_t u = pick(w4, a & 3);
+      const uint32_t t = __funnelshift_r(u, (uint32_t)cd[a], 8) * (uint32_t)A.N;
+      const uint32_t k = t >> sh;
+      const float fr = __uint_as_float(__funnelshift_r(t << (32 - sh), 0x7Fu, 9)) - 1.0f;
+      const float2 e = tab[a * A.N + (int)k];
+      x[a] = fmaf(fr, e.y, e.x);
+      J *= Nf * e.y;
+      kb[a >> 2] |= k << (8 * (a & 3));
+      slot(a);
+    }
+  return J;
+}
+
+// Shared memory of k_sample_col: grid table, integrand constants, then each
+// warp's columns and staging area.
+template <int DM, bool EXACT>
+struct ColSmem {
+  using C = ColHist<DM, EXACT, kColPif<DM>>;
+  static __host__ __device__ size_t params(int dN) { return (size_t)dN * sizeof(float2); }
+  static __host__ __device__ size_t warps(int dN) { return (params(dN) + kNumDerived * sizeof(float) + 15) & ~size_t(15); }
+  static __host__ __device__ size_t total(int d, int N, int nwarps) {
+    return warps(d * N) + (size_t)nwarps * C::warp_bytes(d, N);
+  }
+};
+
+template <int DM, template <typename, int> class F, bool EXACT>
+__global__ void __launch_bounds__(512, 1) k_sample_col(const SampleArgs A) {
+  constexpr int PIF = kColPif<DM>;
+  constexpr int KW = (DM + 3) / 4;
+  using C = ColHist<DM, EXACT, PIF>;
+  using L = ColSmem<DM, EXACT>;
+  const int stop = A.st->done;
+  if (blockIdx.x == 0 && threadIdx.x == 0) A.st->live = !stop;
+  if (stop) return;
+  const uint32_t it = A.it_override >= 0 ? (uint32_t)A.it_override : A.st->it;
+  const int d = EXACT ? DM : A.d, N = A.N, dN = d * N;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+
+  extern __shared__ __align__(16) unsigned char smem[];
+  float2* tab = reinterpret_cast<float2*>(smem);
+  float* P = reinterpret_cast<float*>(smem + L::params(dN));
+  unsigned char* columns = smem + L::warps(dN);
+  const size_t warp_bytes = C::warp_bytes(d, N);
+  C hist;
+  hist.bind(columns + warp * warp_bytes, d, N, lane);
+  const float2* gtab = reinterpret_cast<const float2*>(A.tab);
+  for (int i = tid; i < dN; i += blockDim.x) tab[i] = gtab[i];
+  for (int i = tid; i < kNumDerived; i += blockDim.x) P[i] = (float)A.dparams[i];
+  __syncthreads();
+
+  // Columns of the CTA into its partial row (compensated pairs, in global
+  // memory): at the end, and before a column has taken kColFoldAdds terms.
+  float2* row = reinterpret_cast<float2*>(A.part_bins) + (size_t)blockIdx.x * 2 * dN;
+  bool folded = false;
+  int adds = 0;
+  auto fold = [&]() {
+    __syncthreads();
+    for (int i = tid; i < dN; i += blockDim.x) {
+      const int k = i / d, a = i - k * d;
+      fpair s1, s2;
+      col_sum(columns, warp_bytes, nw, d, hist.P, a, k, s1, s2);
+      float2* r1 = row + a * N + k;
+      float2* r2 = r1 + dN;
+      if (folded) {
+        comp_merge(s1, fpair{r1->x, r1->y});
+        comp_merge(s2, fpair{r2->x, r2->y});
+      }
+      *r1 = make_float2(s1.hi, s1.lo);
+      *r2 = make_float2(s2.hi, s2.lo);
+    }
+    __syncthreads();
+    folded = true;
+    adds = 0;
+  };
+
+  int nonfinite = 0;
+  int cd[DM];
+#pragma unroll
+  for (int a = 0; a < DM; ++a) cd[a] = 0;
+
+  // PIF points of this thread (weights zero where not valid): evaluated while
+  // the previous hand-over is added to the columns, then staged.
+  auto eval = [&](const uint32_t (&s)[PIF], const bool (&v)[PIF], float (&w)[PIF]) {
+    uint32_t kb[PIF][KW];
+    hist.begin();
+#pragma unroll
+    for (int q = 0; q < PIF; ++q) {
+      float x[DM];
+      const float J = col_point<DM, EXACT>(A, d, it, s[q], cd, tab, x, kb[q],
+                                           [&](int a) { hist.advance(q * d + a, PIF * d); });
+      w[q] = F<float, DM>::eval(x, d, P) * J;
+      if (!isfinite(w[q])) {
+        nonfinite += v[q];
+        w[q] = 0.f;
+      }
+      if (!v[q]) w[q] = 0.f;
+    }
+    hist.end();
+    if ((adds += C::steps4(d)) > kColFoldAdds - C::steps4(d)) fold();
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < PIF; ++q) hist.put(q, w[q], kb[q]);
+    __syncwarp();
+  };
+
+  // Totals: sum w, sum w^2, sum of cube means, sum of cube-mean variances.
+  fpair tp[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+  if (!A.strat) {
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    const uint64_t first = (uint64_t)blockIdx.x * blockDim.x;
+    const uint64_t rounds = first < A.ncall ? (A.ncall - first + stride - 1) / stride : 0;
+    uint64_t s = first + tid;
+    for (uint64_t r = 0; r < rounds; r += PIF, s += PIF * stride) {
+      uint32_t sq[PIF];
+      bool v[PIF];
+      float w[PIF];
+#pragma unroll
+      for (int q = 0; q < PIF; ++q) {
+        sq[q] = (uint32_t)(s + q * stride);
+        v[q] = s + q * stride < A.ncall;
+      }
+      eval(sq, v, w);
+#pragma unroll
+      for (int q = 0; q < PIF; ++q) {
+        comp_add(tp[0], w[q]);
+        comp_add(tp[1], w[q] * w[q]);
+      }
+    }
+  } else {
+    // groups of Lw lanes share a hypercube, as in k_sample
+    const int Lw = A.lanes;
+    const int gl = tid & (Lw - 1);
+    const uint32_t groups_per_cta = blockDim.x / Lw;
+    const uint32_t gstride = gridDim.x * groups_per_cta;
+    const uint32_t gfirst = blockIdx.x * groups_per_cta;
+    const uint32_t rounds = gfirst < A.ncubes ? (A.ncubes - gfirst + gstride - 1) / gstride : 0;
+    const uint32_t cmask = A.ncubes - 1u;
+    const uint32_t per_lane = (A.nc + Lw - 1) / Lw;
+    uint32_t gi = gfirst + tid / Lw;
+    for (uint32_t r = 0; r < rounds; ++r, gi += gstride) {
+      const bool live = gi < A.ncubes;  // uniform within a group
+      const uint32_t c = A.cube_mul == 1u ? gi : (gi * A.cube_mul) & cmask;
+      uint32_t rest = live ? c : 0u;
+#pragma unroll
+      for (int a = 0; a < DM; ++a)
+        if (EXACT || a < d) {
+          cd[a] = (int)(rest & (uint32_t)(A.g - 1));
+          rest >>= A.g_log2;
+        }
+      const uint32_t s0 = c * A.nc;
+      float p1 = 0.f, p2 = 0.f;
+      for (uint32_t i = 0; i < per_lane; i += PIF) {
+        uint32_t sq[PIF];
+        bool v[PIF];
+        float w[PIF];
+#pragma unroll
+        for (int q = 0; q < PIF; ++q) {
+          const uint32_t j = gl + (i + q) * Lw;
+          sq[q] = s0 + j;
+          v[q] = live && j < A.nc;
+        }
+        eval(sq, v, w);
+#pragma unroll
+        for (int q = 0; q < PIF; ++q) {
+          p1 += w[q];
+          p2 += w[q] * w[q];
+        }
+      }
+      fpair c1{p1, 0.f}, c2{p2, 0.f};
+      for (int off = Lw >> 1; off > 0; off >>= 1) {
+        fpair o1, o2;
+        o1.hi = __shfl_xor_sync(0xffffffffu, c1.hi, off, Lw);
+        o1.lo = __shfl_xor_sync(0xffffffffu, c1.lo, off, Lw);
+        o2.hi = __shfl_xor_sync(0xffffffffu, c2.hi, off, Lw);
+        o2.lo = __shfl_xor_sync(0xffffffffu, c2.lo, off, Lw);
+        comp_merge(c1, o1);
+        comp_merge(c2, o2);
+      }
+      if (live && gl == 0) cube_totals(A, c, c1, c2, tp);
+    }
+  }
+  hist.drain();
+  fold();
+  store_totals(A, tp, nonfinite);
 }
 
 template <typename T, int ACC>
@@ -1047,9 +1285,14 @@ inline const void* spec_kernel() {
     return nullptr;
 }
 
+template <int DM>
+inline size_t col_smem_bytes(int d, int N, int nwarps) {
+  return ColSmem<DM, false>::total(d, N, nwarps);
+}
+
 template <typename T, int DM, template <typename, int> class F, int ACC, int YB>
 inline KernelEntry make_entry() {
-  KernelEntry e;
+  KernelEntry e{};
   e.sample = (const void*)&k_sample<T, DM, F, ACC, YB, false>;
   e.sample_spec = spec_kernel<T, DM, F, ACC, YB>();
   grad_entry<T, DM, F, YB>(e);
@@ -1059,6 +1302,11 @@ inline KernelEntry make_entry() {
     e.spring_spec = (const void*)&k_spring<T, DM, F, 24, true>;
   else
     e.spring_spec = nullptr;
+  if constexpr (std::is_same<T, float>::value && ACC == 2 && YB == 24) {
+    e.sample_col = (const void*)&k_sample_col<DM, F, false>;
+    e.sample_col_exact = (const void*)&k_sample_col<DM, F, true>;
+    e.smem_col = &col_smem_bytes<DM>;
+  }
   e.smem = &sample_smem_bytes<T, ACC>;
   e.smem_nobins = &sample_smem_nobins<T, ACC>;
   e.dm = DM;
