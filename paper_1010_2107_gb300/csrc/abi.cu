@@ -561,8 +561,9 @@ gv::SampleArgs sample_args(const vegas_ctx* c, int it_override, bool nobins = fa
   return A;
 }
 
-gv::FinArgs fin_args(const vegas_ctx* c, int refine, int record, bool nobins = false) {
+gv::FinArgs fin_args(const vegas_ctx* c, int refine, int record, bool nobins = false, bool combine = true) {
   gv::FinArgs F{};
+  F.combine = combine;
   F.d = c->cfg.ndim;
   F.N = c->cfg.nbins;
   F.nobins = nobins;
@@ -588,15 +589,17 @@ gv::FinArgs fin_args(const vegas_ctx* c, int refine, int record, bool nobins = f
 // One pass of steps 2-6 on the context stream.  A pass that does not
 // refine the grid skips the per-bin histogram, whose sums only step 5
 // reads (`nobins`), unless the caller wants them.
+// `combine`: form the combined result after it (the last pass of a call, and
+// every pass of a call with an ACC target).
 vegas_status launch_pass(vegas_ctx* c, int it_override, int refine, int record, bool record_max = false,
-                         bool nobins = false) {
+                         bool nobins = false, bool combine = true) {
   if (refine) nobins = false;
   gv::SampleArgs A = sample_args(c, it_override, nobins);
   if (record_max) A.cube_max = c->d_cube_max;
   void* args[] = {&A};
   const gv::PassShape& ps = nobins ? c->pass_nobins : c->pass_bins;
   CK(c, cudaLaunchKernel(ps.fn, dim3(ps.ctas), dim3(ps.threads), args, ps.smem, c->stream));
-  gv::FinArgs F = fin_args(c, refine, record, nobins);
+  gv::FinArgs F = fin_args(c, refine, record, nobins, combine);
   CK(c, gv_launch_finish(&F, c->stream));
   return VEGAS_OK;
 }
@@ -623,15 +626,15 @@ vegas_status get_graph(vegas_ctx* c, int shape, int n1, int n2, int refine, doub
   };
   if (shape == 0) {
     ctl(gv::CTL_SET_ACC, acc1);
-    for (int i = 0; i < n1 && !st; ++i) st = launch_pass(c, -1, refine, 1, false, !refine);
+    for (int i = 0; i < n1 && !st; ++i) st = launch_pass(c, -1, refine, 1, false, !refine, acc1 > 0.0 || i == n1 - 1);
   } else {
     ctl(gv::CTL_RESET_WINDOW | gv::CTL_SET_ACC, acc1);
-    for (int i = 0; i < n1 && !st; ++i) st = launch_pass(c, -1, 1, 1);
+    for (int i = 0; i < n1 && !st; ++i) st = launch_pass(c, -1, 1, 1, false, false, acc1 > 0.0 || i == n1 - 1);
     ctl(gv::CTL_SNAPSHOT | gv::CTL_RESET_WINDOW | gv::CTL_SET_ACC, acc2);
     // the integration phase records the per-cube maxima that SPRING uses
     if (!st && cudaMemsetAsync(c->d_cube_max, 0, sizeof(double) * c->ncubes, c->stream) != cudaSuccess)
       st = c->fail(VEGAS_ECUDA, "cube maxima reset");
-    for (int i = 0; i < n2 && !st; ++i) st = launch_pass(c, -1, 0, 1, true, true);
+    for (int i = 0; i < n2 && !st; ++i) st = launch_pass(c, -1, 0, 1, true, true, acc2 > 0.0 || i == n2 - 1);
   }
   cudaError_t e = cudaStreamEndCapture(c->stream, &g);
   if (st != VEGAS_OK) {

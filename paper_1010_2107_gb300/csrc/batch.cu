@@ -269,7 +269,7 @@ __device__ inline void row_sums(const BatchArgs& B, const BatchInst& I, const in
 // Blocks [0, naxes): reduce one axis of one instance (2 N cells) and refine
 // it; blocks [naxes, naxes + n): estimate, history and combination of one
 // instance.
-__global__ void __launch_bounds__(128) k_batch_finalize(const BatchArgs B) {
+__global__ void __launch_bounds__(256) k_batch_finalize(const BatchArgs B) {
   __shared__ double s2[kMaxBins];
   const int b = blockIdx.x;
   if (b < B.naxes) {
@@ -667,12 +667,15 @@ vegas_status launch_sample(vegas_batch* b, BatchArgs& A) {
   return VEGAS_OK;
 }
 
+// Threads per block of k_batch_finalize: one per bin of an axis.
+int finalize_threads(const vegas_batch* b) { return std::max(128, (b->N + 31) / 32 * 32); }
+
 vegas_status launch_iteration(vegas_batch* b, int refine, int record) {
   BatchArgs A = batch_args(b, refine, record);
   vegas_status st = launch_sample(b, A);
   if (st) return st;
   const int blocks = A.naxes + A.n;
-  gv::k_batch_finalize<<<blocks, 128, 0, b->stream>>>(A);
+  gv::k_batch_finalize<<<blocks, finalize_threads(b), 0, b->stream>>>(A);
   BK(b, cudaGetLastError());
   return VEGAS_OK;
 }
@@ -1029,7 +1032,7 @@ vegas_status vegas_batch_profile(vegas_batch* b, int n_pass, double* ms) {
     st = launch_sample(b, A);
     cudaEventRecord(ev[1], b->stream);
     if (!st) {
-      gv::k_batch_finalize<<<A.naxes + A.n, 128, 0, b->stream>>>(A);
+      gv::k_batch_finalize<<<A.naxes + A.n, finalize_threads(b), 0, b->stream>>>(A);
       if (cudaGetLastError() != cudaSuccess) st = b->fail(VEGAS_ECUDA, "finalize launch failed");
     }
     cudaEventRecord(ev[2], b->stream);

@@ -256,6 +256,7 @@ struct SampleArgs {
 // Arguments of the reduction and finalisation kernels (steps 4-6).
 struct FinArgs {
   int d, N, nparts, strat, refine, record;
+  int combine;             // 1: form the combined result (and the ACC test)
   int nobins;              // the pass kept no per-bin histogram: totals only, no refinement
   int pair32;              // part_bins hold float (hi, lo) pairs
   uint64_t ncall;

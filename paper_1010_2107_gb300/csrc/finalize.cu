@@ -155,7 +155,9 @@ __device__ void record_iteration(const FinArgs& F, const double* t) {
     st->samples += (long long)F.ncall;
     st->it += 1;
   }
-  // Inverse-variance combination over the window (Lepage).
+  // Inverse-variance combination over the window (Lepage): in a call without
+  // an ACC target only the last pass's combination can be read.
+  if (!F.combine) return;
   double Ib, sg, chi;
   combine_history(st->hist, h, &Ib, &sg, &chi);
   if (lane == 0) {

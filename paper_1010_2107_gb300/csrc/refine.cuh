@@ -23,127 +23,146 @@ struct Team {
   __device__ __forceinline__ void sync() const { asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory"); }
 };
 
-// Compensated all-reduce over the team (every thread gets the sum).  A
-// thread's values are summed in a fixed tree (xor butterfly within a warp,
-// then the warps in order), each step with TwoSum, so the result is
-// deterministic and its error is that of a twice-as-precise sum.  `buf`:
-// shared scratch of 2 x (warps) doubles; all team threads must call.
-__device__ inline double block_sum(double v, double* buf, Team t) {
-  double s = v, c = 0.0;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const double os = __shfl_xor_sync(0xffffffffu, s, off), oc = __shfl_xor_sync(0xffffffffu, c, off);
-    double t, e;
-    two_sum_d(s, os, t, e);
-    s = t;
-    c = c + oc + e;
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = t.n >> 5;
-  t.sync();  // buf may still be read from an earlier call
-  if (lane == 0) {
-    buf[2 * warp] = s;
-    buf[2 * warp + 1] = c;
-  }
+// Exact sum over the team of 64-bit integers below 2^62 in total: three
+// 22-bit digits per value through the warp's integer reduction, then the
+// warps in order.  `buf`: one entry per warp; all team threads must call.
+__device__ __forceinline__ unsigned long long team_sum(unsigned long long v, unsigned long long* buf, Team t) {
+  constexpr unsigned M = (1u << 22) - 1u;
+  const unsigned d0 = __reduce_add_sync(0xffffffffu, (unsigned)v & M);
+  const unsigned d1 = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 22) & M);
+  const unsigned d2 = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 44));
+  const unsigned long long w = (unsigned long long)d0 + ((unsigned long long)d1 << 22) + ((unsigned long long)d2 << 44);
+  if (t.n == 32) return w;
+  if ((threadIdx.x & 31) == 0) buf[threadIdx.x >> 5] = w;
   t.sync();
-  double S = buf[0], C = buf[1];
-  for (int w = 1; w < nw; ++w) {
-    double t, e;
-    two_sum_d(S, buf[2 * w], t, e);
-    S = t;
-    C = C + buf[2 * w + 1] + e;
-  }
-  return S + C;
+  unsigned long long S = buf[0];
+  for (int i = 1; i < t.n >> 5; ++i) S += buf[i];
+  return S;
 }
 
-// Inclusive prefix sums of x[0..n) into out[0..n) by the team (Hillis-Steele
-// doubling over shared memory).
-__device__ inline void block_prefix(const double* x, double* out, double* tmp, int n, Team t) {
-  const int tid = threadIdx.x;
-  for (int k = tid; k < n; k += t.n) out[k] = x[k];
-  t.sync();
-  for (int off = 1; off < n; off <<= 1) {
-    for (int k = tid; k < n; k += t.n) tmp[k] = k >= off ? out[k] + out[k - off] : out[k];
-    t.sync();
-    for (int k = tid; k < n; k += t.n) out[k] = tmp[k];
-    t.sync();
-  }
-}
-
-// One axis, one team of threads: smooth the per-bin sums of w^2 over
-// neighbours, compress them with r_k = ((1 - d_k/D) / ln(D/d_k))^alpha, and
-// move the edges so that every new bin holds an equal share of sum r, with r
-// spread uniformly inside each old bin.  dd: S2 of the axis (N values);
-// e: its N+1 edges (updated in place); t64 / t32: its (e_k, Delta_k) cells.
-// An axis whose smoothed sum is zero or not finite is left unchanged.
-// The sums D and R are compensated block reductions, and new edge j is
-// found by each thread on its own from the prefix sums C_k = r_0 + ... +
-// r_{k-1}: old bin k_j is the first k with C_{k+1} >= tau_j = j R / N (or
-// the last bin), and the new edge sits at the fraction (tau_j - C_k) / r_k
-// of it.  This is the sequential rebinning walk of Lepage written without
-// its loop-carried dependence; FP64 scalar arithmetic is slow on this GPU,
-// so the serial chains are kept short.
+// One axis, one team of threads (one per bin, N <= t.n): smooth the per-bin
+// sums of w^2 over neighbours, compress them with r_k = ((1 - d_k/D) /
+// ln(D/d_k))^alpha, and move the edges so that every new bin holds an equal
+// share of sum r, with r spread uniformly inside each old bin.  dd: S2 of the
+// axis (N values); ea: its N+1 edges (updated in place); t64 / t32: its (e_k,
+// Delta_k) cells.  An axis whose smoothed sum is zero or not finite is left
+// unchanged.
+//
+// This runs once per refining pass with nothing beside it, so what counts is
+// the length of its dependent chain, and the FP64 pipe (1.65 operations per
+// SM-clock: 19 clocks for a warp's instruction) is all of it.  The sums D
+// and R and the prefix sums C_k = r_0 + ... + r_{k-1} are therefore 64-bit
+// integers: a value enters as a multiple of 2^-58 or less of the largest one
+// (of 1 for r), and the integer sums are exact, so they carry less error
+// than FP64 sums would and cost no FP64 instruction.  Divisions by a common
+// divisor are products with its reciprocal.
+//
+// New edge j is found by each thread on its own: old bin k_j is the first k
+// with C_{k+1} >= tau_j = j R / N (or the last bin), and the new edge sits at
+// the fraction (tau_j - C_k) / r_k of it.  This is the sequential rebinning
+// walk of Lepage written without its loop-carried dependence.
 __device__ inline void refine_axis_core(const double* dd, double* ea, double2* t64, float2* t32, int N,
                                         double alpha, Team t) {
-  __shared__ double dsm[kMaxBins], r[kMaxBins], e[kMaxBins + 1], enew[kMaxBins + 1], C[kMaxBins + 1],
-      tmp[kMaxBins], buf[64];
-  const int tid = threadIdx.x;
-  for (int k = tid; k <= N; k += t.n) e[k] = ea[k];
-  double part = 0.0;
-  for (int k = tid; k < N; k += t.n) {
-    double v;
-    if (N == 2)
-      v = (dd[0] + dd[1]) / 2.0;
-    else if (k == 0)
-      v = (dd[0] + dd[1]) / 2.0;
-    else if (k == N - 1)
-      v = (dd[N - 2] + dd[N - 1]) / 2.0;
-    else
-      v = (dd[k - 1] + dd[k] + dd[k + 1]) / 3.0;
-    dsm[k] = v;
-    part += v;
-  }
-  const double D = block_sum(part, buf, t);
-  if (!(D > 0.0) || !isfinite(D)) return;  // uniform across the team
-  part = 0.0;
-  for (int k = tid; k < N; k += t.n) {
-    const double x = dsm[k];
-    double rk = x <= 0.0 ? 0.0 : 1.0;
-    if (x > 0.0 && x < D) {
-      // y^alpha; the default alpha = 3/2 as y sqrt(y) (a few FP64
-      // instructions instead of a general power)
-      const double y = (1.0 - x / D) / log(D / x);
-      rk = alpha == 1.5 ? y * sqrt(y) : pow(y, alpha);
+  __shared__ double e[kMaxBins + 1], enew[kMaxBins + 1];
+  __shared__ unsigned long long C[kMaxBins + 1], buf[2][8];
+  __shared__ int ibuf[16];
+  const int k = threadIdx.x, lane = k & 31, warp = k >> 5, nw = t.n >> 5;
+  const bool in = k < N;
+  // fixed-point position of the largest value: N values below 2^top sum below 2^62
+  const int top = 62 - (32 - __clz(N - 1));
+  double x = 0.0;
+  if (in) {
+    e[k] = ea[k];
+    if (k == 0) {
+      e[N] = ea[N];
+      enew[0] = 0.0;
+      enew[N] = 1.0;
     }
-    r[k] = rk;
-    part += rk;
+    if (N == 2 || k == 0)
+      x = (dd[0] + dd[1]) * 0.5;
+    else if (k == N - 1)
+      x = (dd[N - 2] + dd[N - 1]) * 0.5;
+    else
+      x = (dd[k - 1] + dd[k] + dd[k + 1]) * (1.0 / 3.0);
   }
-  const double R = block_sum(part, buf, t);
-  // C[k + 1] = r_0 + ... + r_k, C[0] = 0
-  block_prefix(r, C + 1, tmp, N, t);
-  if (tid == 0) {
-    C[0] = 0.0;
-    enew[0] = 0.0;
-    enew[N] = 1.0;
+  // the largest exponent (finite non-negative doubles order as their bits)
+  int hi = __reduce_max_sync(0xffffffffu, __double2hiint(x) & 0x7FFFFFFF);
+  if (nw > 1) {
+    if (lane == 0) ibuf[warp] = hi;
+    t.sync();
+    hi = ibuf[0];
+    for (int i = 1; i < nw; ++i) hi = max(hi, ibuf[i]);
   }
+  const int ex = hi >> 20;  // values below 2^(ex - 1022)
+  if (ex >= 0x7FF) return;  // not finite (uniform across the team)
+  // scale = 2^(top - (ex - 1022)) in two factors, each within range
+  const int sh = top + 1022 - max(ex, 1), h1 = sh / 2, h2 = sh - h1;
+  const double f1 = __hiloint2double((1023 + h1) << 20, 0), f2 = __hiloint2double((1023 + h2) << 20, 0);
+  const unsigned long long Di = team_sum(x > 0.0 ? (unsigned long long)__double2ll_rn(x * f1 * f2) : 0ull, buf[0], t);
+  if (Di == 0ull) return;  // every sum zero (uniform across the team)
+  // q = x / D and r = ((1 - q) / -ln q)^alpha
+  double rk = 0.0;
+  if (x > 0.0) {
+    const double q = (x * f1 * f2) * (1.0 / (double)Di);
+    rk = 1.0;
+    if (q < 1.0) {
+      const double y = (1.0 - q) / -log(q);
+      // the default alpha = 3/2 as y sqrt(y) (a few FP64 instructions
+      // instead of a general power)
+      rk = q > 0.0 ? (alpha == 1.5 ? y * sqrt(y) : pow(y, alpha)) : 0.0;
+    }
+  }
+  // inclusive prefix sums of r 2^top.  With alpha = 3/2 the largest r lies in
+  // [0.06, 1] (q >= 1/N there, N <= 256); for another alpha the values are
+  // scaled by the largest one's exponent first.
+  int re = 0;
+  if (alpha != 1.5) {
+    re = __reduce_max_sync(0xffffffffu, __double2hiint(rk));
+    if (nw > 1) {
+      if (lane == 0) ibuf[8 + warp] = re;
+      t.sync();
+      re = ibuf[8];
+      for (int i = 1; i < nw; ++i) re = max(re, ibuf[8 + i]);
+    }
+    re = max(re >> 20, 64) - 1022;  // r below 2^re
+    if (re < 0) rk *= __hiloint2double((1023 - re) << 20, 0);
+  }
+  const double f = __hiloint2double((1023 + top) << 20, 0);
+  const unsigned long long ri = (unsigned long long)__double2ll_rn(rk * f);
+  unsigned long long run = ri;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const unsigned long long o = __shfl_up_sync(0xffffffffu, run, off);
+    if (lane >= off) run += o;
+  }
+  if (nw > 1) {
+    if (lane == 31) buf[1][warp] = run;
+    t.sync();
+    for (int i = 0; i < warp; ++i) run += buf[1][i];
+  }
+  if (in) C[k + 1] = run;
+  if (k == 0) C[0] = 0ull;
   t.sync();
-  for (int j = 1 + tid; j < N; j += t.n) {
-    const double tau = (double)j * R / (double)N;
-    // first k in [0, N-1) with C[k + 1] >= tau, else N - 1 (C is nondecreasing)
-    int lo = 0, hi = N - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
+  const double share = (double)C[N] * (1.0 / (double)N);
+  const int j = k;
+  if (j > 0 && in) {
+    const unsigned long long tau = (unsigned long long)__double2ll_rn((double)j * share);
+    // first b in [0, N-1) with C[b + 1] >= tau, else N - 1 (C is nondecreasing)
+    int lo = 0, up = N - 1;
+    while (lo < up) {
+      const int mid = (lo + up) >> 1;
       if (C[mid + 1] >= tau)
-        hi = mid;
+        up = mid;
       else
         lo = mid + 1;
     }
-    const int k = lo;
-    enew[j] = e[k] + (tau - C[k]) / r[k] * (e[k + 1] - e[k]);
+    const unsigned long long c0 = C[lo], w = C[lo + 1] - c0;
+    enew[j] = e[lo] + (double)(long long)(tau - c0) / (double)w * (e[lo + 1] - e[lo]);
   }
   t.sync();
-  for (int k = tid; k <= N; k += t.n) ea[k] = enew[k];
-  for (int k = tid; k < N; k += t.n) {
+  if (in) {
     const double lo = enew[k], w = enew[k + 1] - enew[k];
+    if (k > 0) ea[k] = lo;
     t64[k] = make_double2(lo, w);
     t32[k] = make_float2((float)lo, (float)w);
   }
