@@ -106,10 +106,11 @@ __device__ inline void refine_axis_core(const double* dd, double* ea, double2* t
     const double q = (x * f1 * f2) * (1.0 / (double)Di);
     rk = 1.0;
     if (q < 1.0) {
-      const double y = (1.0 - q) / -log(q);
+      // (D / x overflows, and ln with it, for q up to 2^-1024: then y = 0)
+      const double y = q > 0x1p-1024 ? (1.0 - q) / -log(q) : 0.0;
       // the default alpha = 3/2 as y sqrt(y) (a few FP64 instructions
       // instead of a general power)
-      rk = q > 0.0 ? (alpha == 1.5 ? y * sqrt(y) : pow(y, alpha)) : 0.0;
+      rk = alpha == 1.5 ? y * sqrt(y) : pow(y, alpha);
     }
   }
   // inclusive prefix sums of r 2^top.  With alpha = 3/2 the largest r lies in
