@@ -92,6 +92,7 @@ struct vegas_ctx {
   int ybits = 53;
   int g = 1;
   uint64_t ncubes = 1, nc = 0;
+  uint32_t cube_mul = 1;  // order of the cubes (gv::cube_of)
   int strat = 0;
   gv::KernelEntry ke{};
   const void* col = nullptr;  // the column-histogram kernel of this shape, or null
@@ -112,6 +113,8 @@ struct vegas_ctx {
   int part_rows = 0;
   double* d_bins = nullptr;
   double* d_cubes = nullptr;
+  void* d_cube_part = nullptr;   // sums of the hypercubes' parts (16 bytes each)
+  size_t cube_part_len = 0;
   double* d_cube_max = nullptr;  // [G] max(0, largest w) per cube, integration phase
   bool have_max = false;         // a bases_integrate has recorded the maxima
   // SPRING buffers (grown on demand)
@@ -404,7 +407,8 @@ __global__ void k_spring_compact(const uint32_t* counts, uint32_t chunk, int d, 
 // 4M points in 8 dimensions: 64 bins and below columns, see DESIGN).
 constexpr int kColMinWarps = 8;
 bool shape_col(const void* fn, const gv::KernelEntry& ke, int d, int N, int sm_count, int threads, int per_sm_req,
-               uint64_t ncubes, uint64_t nc, uint64_t ncall, int64_t max_rows, gv::PassShape* out, cudaError_t* e) {
+               uint64_t ncubes, uint64_t nc, uint64_t ncall, int64_t max_rows, uint64_t max_parts,
+               gv::PassShape* out, cudaError_t* e) {
   static const int kAuto[] = {512, 384, 256, 192, 128, 64};
   int best_t = 0, best_occ = 0;
   const int one[] = {threads};
@@ -421,6 +425,7 @@ bool shape_col(const void* fn, const gv::KernelEntry& ke, int d, int N, int sm_c
       best_t = list[i];
       best_occ = o;
     }
+    if (best_occ * best_t >= 512) break;  // (16 warps: what the kernels' registers allow)
   }
   if (best_occ * best_t < 32 * kColMinWarps && threads == 0) return false;
   if (best_occ < 1) return false;
@@ -437,8 +442,11 @@ bool shape_col(const void* fn, const gv::KernelEntry& ke, int d, int N, int sm_c
   out->occ = best_occ;
   out->smem = ke.smem_col(d, N, best_t / 32);
   const int64_t most = std::min<int64_t>((int64_t)sm_count * best_occ, max_rows);
-  out->lanes = ncubes > 1 ? gv::balanced_lanes(ncubes, nc, best_t, sm_count, pif) : 1;
-  const uint64_t units = ncubes > 1 ? ncubes * (uint64_t)out->lanes : ncall;
+  const gv::CubeLanes cl =
+      ncubes > 1 ? gv::balanced_lanes(ncubes, nc, best_t, sm_count, pif, max_parts) : gv::CubeLanes{1, 1};
+  out->lanes = cl.lanes;
+  out->parts = cl.parts;
+  const uint64_t units = ncubes > 1 ? ncubes * cl.parts * (uint64_t)cl.lanes : ncall;
   out->ctas = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)((units + best_t - 1) / best_t), most));
   return true;
 }
@@ -449,14 +457,14 @@ vegas_status configure_launch(vegas_ctx* c) {
   gv::PassShape &pb = c->pass_bins, &pn = c->pass_nobins;
   const bool strat = c->strat != 0;
   cudaError_t e = cudaSuccess;
-  auto ctas_for = [&](int lanes, int t, int64_t most) {
-    const uint64_t units = strat ? c->ncubes * (uint64_t)lanes : (uint64_t)c->cfg.ncall;
+  auto ctas_for = [&](const gv::PassShape& s, int t, int64_t most) {
+    const uint64_t units = strat ? c->ncubes * (uint64_t)s.lanes * s.parts : (uint64_t)c->cfg.ncall;
     return (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)((units + t - 1) / t), most));
   };
   int per_sm = 1;
   if (c->col && c->ppt_req == 0 &&
       shape_col(c->col, c->ke, d, N, c->sm_count, c->threads_req, c->ctas_per_sm_req, c->ncubes, c->nc,
-                (uint64_t)c->cfg.ncall, INT64_MAX, &pb, &e)) {
+                (uint64_t)c->cfg.ncall, INT64_MAX, gv::kMaxCubeParts, &pb, &e)) {
     c->cap = 0;
     c->ppt = d <= 8 ? 2 : 1;
     per_sm = std::max(1, pb.occ);
@@ -490,7 +498,12 @@ vegas_status configure_launch(vegas_ctx* c) {
     per_sm = c->ctas_per_sm_req > 0 ? std::min(c->ctas_per_sm_req, t.occ) : t.occ;
     const int64_t most = (int64_t)c->sm_count * per_sm;
     pb.lanes = strat ? gv::choose_lanes(c->ncubes, c->nc, threads, most) : 1;
-    pb.ctas = ctas_for(pb.lanes, threads, most);
+    pb.parts = 1;
+    if (pb.lanes == 32) {  // few cubes: several groups each
+      const gv::CubeLanes cl = gv::balanced_lanes(c->ncubes, c->nc, threads, c->sm_count, c->ppt_min, gv::kMaxCubeParts);
+      pb.parts = cl.parts;
+    }
+    pb.ctas = ctas_for(pb, threads, most);
   }
   // passes without the per-bin histogram (no refinement) need only the
   // grid table and constants in shared memory: more CTAs may be resident
@@ -503,8 +516,22 @@ vegas_status configure_launch(vegas_ctx* c) {
   if (c->ctas_per_sm_req > 0) occ_nb = std::min(occ_nb, std::max(c->ctas_per_sm_req, per_sm));
   pn.occ = std::max(occ_nb, 1);
   const int64_t most_nb = (int64_t)c->sm_count * pn.occ;
-  pn.lanes = strat ? gv::balanced_lanes(c->ncubes, c->nc, threads, c->sm_count, c->ppt_min) : 1;
-  pn.ctas = ctas_for(pn.lanes, threads, most_nb);
+  const gv::CubeLanes cl = strat ? gv::balanced_lanes(c->ncubes, c->nc, threads, c->sm_count, c->ppt_min, gv::kMaxCubeParts)
+                                 : gv::CubeLanes{1, 1};
+  pn.lanes = cl.lanes;
+  pn.parts = cl.parts;
+  pn.ctas = ctas_for(pn, threads, most_nb);
+  // sums of the hypercubes' parts: a refining pass, or the iterations of a
+  // frozen-grid launch
+  const size_t entries = std::max(pb.parts > 1 ? (size_t)c->ncubes * pb.parts : 0,
+                                  pn.parts > 1 ? (size_t)c->ncubes * pn.parts * gv::kMergeIters : 0);
+  if (entries > c->cube_part_len) {
+    cudaFree(c->d_cube_part);
+    c->d_cube_part = nullptr;
+    c->cube_part_len = 0;
+    CK(c, gv_malloc(&c->d_cube_part, 16 * entries));
+    c->cube_part_len = entries;
+  }
   const int rows = std::max(pb.ctas, pn.ctas);
   if (rows > c->part_rows) {
     if (c->d_part_bins) cudaFree(c->d_part_bins);
@@ -513,14 +540,14 @@ vegas_status configure_launch(vegas_ctx* c) {
     c->d_part_tot = nullptr;
     c->part_rows = 0;
     CK(c, gv_malloc(&c->d_part_bins, sizeof(double) * 2 * (size_t)d * N * rows));
-    CK(c, gv_malloc(&c->d_part_tot, sizeof(double) * gv::kTotCols * (size_t)rows));
+    CK(c, gv_malloc(&c->d_part_tot, sizeof(double) * gv::kTotCols * gv::kMergeIters * (size_t)rows));
     c->part_rows = rows;
   }
   destroy_graphs(c);
   return VEGAS_OK;
 }
 
-gv::SampleArgs sample_args(const vegas_ctx* c, int it_override, bool nobins = false) {
+gv::SampleArgs sample_args(const vegas_ctx* c, int it_override, bool nobins = false, int niter = 1) {
   gv::SampleArgs A{};
   const gv::PassShape& ps = nobins ? c->pass_nobins : c->pass_bins;
   A.nobins = nobins;
@@ -529,6 +556,13 @@ gv::SampleArgs sample_args(const vegas_ctx* c, int it_override, bool nobins = fa
   A.g = c->g;
   A.ybits = c->ybits;
   A.lanes = ps.lanes;
+  A.parts = ps.parts;
+  A.niter = niter;
+  {  // the CTAs with a round more than the others
+    const uint64_t lanes = c->strat ? c->ncubes * (uint64_t)ps.lanes * ps.parts : (uint64_t)c->cfg.ncall;
+    A.rot = ps.ctas > 0 ? (uint32_t)((lanes + ps.threads - 1) / ps.threads % ps.ctas) : 0;
+  }
+  A.cube_part = c->d_cube_part;
   A.cap = c->cap;
   A.ppt = c->ppt;
   A.strat = c->strat;
@@ -540,8 +574,7 @@ gv::SampleArgs sample_args(const vegas_ctx* c, int it_override, bool nobins = fa
   A.ncall = (uint64_t)c->cfg.ncall;
   A.nc = (uint32_t)c->nc;
   A.ncubes = (uint32_t)c->ncubes;
-  const bool cubes_pow2 = (c->ncubes & (c->ncubes - 1)) == 0;
-  A.cube_mul = (c->strat && cubes_pow2 && c->ncubes > 1) ? 0x9E3779B1u : 1u;
+  A.cube_mul = c->cube_mul;
   A.g_pow2 = (c->g & (c->g - 1)) == 0;
   A.g_log2 = 0;
   while ((1 << A.g_log2) < c->g) ++A.g_log2;
@@ -561,8 +594,16 @@ gv::SampleArgs sample_args(const vegas_ctx* c, int it_override, bool nobins = fa
   return A;
 }
 
-gv::FinArgs fin_args(const vegas_ctx* c, int refine, int record, bool nobins = false, bool combine = true) {
+gv::FinArgs fin_args(const vegas_ctx* c, int refine, int record, bool nobins = false, bool combine = true,
+                     int niter = 1) {
   gv::FinArgs F{};
+  F.niter = niter;
+  F.parts = (nobins ? c->pass_nobins : c->pass_bins).parts;
+  F.cube_mul = c->cube_mul;
+  F.inv_nc = c->nc > 0 ? 1.0 / (double)c->nc : 0.0;
+  F.inv_nc1 = c->nc > 1 ? 1.0 / (double)(c->nc - 1) : 0.0;
+  F.cube_part = c->d_cube_part;
+  F.cubes = c->d_cubes;
   F.combine = combine;
   F.d = c->cfg.ndim;
   F.N = c->cfg.nbins;
@@ -588,18 +629,19 @@ gv::FinArgs fin_args(const vegas_ctx* c, int refine, int record, bool nobins = f
 
 // One pass of steps 2-6 on the context stream.  A pass that does not
 // refine the grid skips the per-bin histogram, whose sums only step 5
-// reads (`nobins`), unless the caller wants them.
+// reads (`nobins`), unless the caller wants them, and may hold `niter`
+// iterations.
 // `combine`: form the combined result after it (the last pass of a call, and
 // every pass of a call with an ACC target).
 vegas_status launch_pass(vegas_ctx* c, int it_override, int refine, int record, bool record_max = false,
-                         bool nobins = false, bool combine = true) {
+                         bool nobins = false, bool combine = true, int niter = 1) {
   if (refine) nobins = false;
-  gv::SampleArgs A = sample_args(c, it_override, nobins);
+  gv::SampleArgs A = sample_args(c, it_override, nobins, niter);
   if (record_max) A.cube_max = c->d_cube_max;
   void* args[] = {&A};
   const gv::PassShape& ps = nobins ? c->pass_nobins : c->pass_bins;
   CK(c, cudaLaunchKernel(ps.fn, dim3(ps.ctas), dim3(ps.threads), args, ps.smem, c->stream));
-  gv::FinArgs F = fin_args(c, refine, record, nobins, combine);
+  gv::FinArgs F = fin_args(c, refine, record, nobins, combine, niter);
   CK(c, gv_launch_finish(&F, c->stream));
   return VEGAS_OK;
 }
@@ -624,9 +666,22 @@ vegas_status get_graph(vegas_ctx* c, int shape, int n1, int n2, int refine, doub
     cudaError_t e = gv_launch_control(c->d_st, ops, acc, 0u, c->stream);
     if (e != cudaSuccess) st = c->fail(VEGAS_ECUDA, "control: %s", cudaGetErrorString(e));
   };
+  // n iterations on the grid as it stands.  Without an ACC target nothing is
+  // decided between them, so one launch runs up to kMergeIters: no launch
+  // gap and no half-empty last round per iteration.
+  auto frozen = [&](int n, double acc, bool record_max) {
+    for (int i = 0; i < n && !st;) {
+      const int m = acc > 0.0 ? 1 : std::min(gv::kMergeIters, n - i);
+      i += m;
+      st = launch_pass(c, -1, 0, 1, record_max, true, acc > 0.0 || i == n, m);
+    }
+  };
   if (shape == 0) {
     ctl(gv::CTL_SET_ACC, acc1);
-    for (int i = 0; i < n1 && !st; ++i) st = launch_pass(c, -1, refine, 1, false, !refine, acc1 > 0.0 || i == n1 - 1);
+    if (refine)
+      for (int i = 0; i < n1 && !st; ++i) st = launch_pass(c, -1, 1, 1, false, false, acc1 > 0.0 || i == n1 - 1);
+    else
+      frozen(n1, acc1, false);
   } else {
     ctl(gv::CTL_RESET_WINDOW | gv::CTL_SET_ACC, acc1);
     for (int i = 0; i < n1 && !st; ++i) st = launch_pass(c, -1, 1, 1, false, false, acc1 > 0.0 || i == n1 - 1);
@@ -634,7 +689,7 @@ vegas_status get_graph(vegas_ctx* c, int shape, int n1, int n2, int refine, doub
     // the integration phase records the per-cube maxima that SPRING uses
     if (!st && cudaMemsetAsync(c->d_cube_max, 0, sizeof(double) * c->ncubes, c->stream) != cudaSuccess)
       st = c->fail(VEGAS_ECUDA, "cube maxima reset");
-    for (int i = 0; i < n2 && !st; ++i) st = launch_pass(c, -1, 0, 1, true, true, acc2 > 0.0 || i == n2 - 1);
+    if (!st) frozen(n2, acc2, true);
   }
   cudaError_t e = cudaStreamEndCapture(c->stream, &g);
   if (st != VEGAS_OK) {
@@ -752,6 +807,7 @@ vegas_ctx* new_context(const vegas_config* cfg, int ybits, int g, uint64_t G) {
   c->ncubes = G;
   c->nc = (uint64_t)cfg->ncall / G;
   c->strat = G > 1;
+  c->cube_mul = gv::cube_multiplier(G);
   return c;
 }
 
@@ -871,6 +927,7 @@ void vegas_destroy(vegas_ctx* c) {
   cudaFree(c->d_part_tot);
   cudaFree(c->d_bins);
   cudaFree(c->d_cubes);
+  cudaFree(c->d_cube_part);
   cudaFree(c->d_cube_max);
   for (void* p : {(void*)c->d_q, (void*)c->d_mt, (void*)c->d_mt32, (void*)c->d_guide, (void*)c->d_bmax, (void*)c->d_bsum, (void*)c->d_prefix, (void*)c->d_meta, (void*)c->d_stage_x, (void*)c->d_stage_t,
                   (void*)c->d_out_x, (void*)c->d_out_t, (void*)c->d_counts, (void*)c->d_counters})
@@ -1684,7 +1741,7 @@ extern "C" vegas_status vegas_eval_noalloc(const vegas_config* cfg, const vegas_
   gv::PassShape ps;
   int ppt = d <= 8 ? 2 : 1, cap = 0;
   const void* col = pick_col(ke, d, ybits, g, N);
-  if (!col || !shape_col(col, ke, d, N, sms, 0, 0, G, nc, (uint64_t)cfg->ncall, max_rows, &ps, &e)) {
+  if (!col || !shape_col(col, ke, d, N, sms, 0, 0, G, nc, (uint64_t)cfg->ncall, max_rows, 0, &ps, &e)) {
     const int threads = 256;
     auto occ_of = [&](int cp, int) -> int {
       const size_t sm = ke.smem(d, N, cp);
@@ -1747,7 +1804,9 @@ extern "C" vegas_status vegas_eval_noalloc(const vegas_config* cfg, const vegas_
   A.ncall = (uint64_t)cfg->ncall;
   A.nc = (uint32_t)nc;
   A.ncubes = (uint32_t)G;
-  A.cube_mul = (strat && (G & (G - 1)) == 0 && G > 1) ? 0x9E3779B1u : 1u;
+  A.cube_mul = gv::cube_multiplier(G);
+  A.parts = 1;
+  A.niter = 1;
   A.g_pow2 = (g & (g - 1)) == 0;
   A.g_log2 = 0;
   while ((1 << A.g_log2) < g) ++A.g_log2;
@@ -1770,6 +1829,8 @@ extern "C" vegas_status vegas_eval_noalloc(const vegas_config* cfg, const vegas_
   F.d = d;
   F.N = N;
   F.nparts = ctas;
+  F.niter = 1;
+  F.parts = 1;
   F.strat = strat;
   F.refine = 0;
   F.record = 0;

@@ -222,10 +222,61 @@ constexpr int kFinishThreads = 256;
 // Device-side control operations captured into the iteration graphs.
 enum { CTL_RESET_WINDOW = 1, CTL_SET_ACC = 2, CTL_SNAPSHOT = 4, CTL_SET_ITER = 8 };
 
+// Iterations on a frozen grid one sampling launch can run (their points need
+// nothing from one another unless an ACC test may stop between them).
+constexpr int kMergeIters = 8;
+
+// The hypercube in place `slot` of the processing order: an odd or coprime
+// multiplier permutes the n cubes, so that the groups of a CTA sit in
+// unrelated cubes and spread over the bins.
+__host__ __device__ __forceinline__ uint32_t cube_of(uint32_t n, uint32_t mul, uint32_t slot) {
+  return (n & (n - 1u)) == 0u ? (slot * mul) & (n - 1u) : (uint32_t)(((uint64_t)slot * mul) % n);
+}
+
+// Step 4 of one hypercube from its sums (n_c points): the cube mean m = C1 /
+// n_c and variance (C2 / n_c - m^2) / (n_c - 1) into the totals t = (sum w,
+// sum w^2, sum of means, sum of variances).
+// Compensated form: FP32 with the square formed exactly (FMA), pairs kept.
+__device__ __forceinline__ void cube_totals(double inv_nc, double inv_nc1, const fpair& c1, const fpair& c2,
+                                            fpair (&t)[4]) {
+  const float inv = (float)inv_nc, inv1 = (float)inv_nc1;
+  const float mh = c1.hi * inv, ml = c1.lo * inv;
+  const float sq = mh * mh;
+  const float sqe = fmaf(mh, mh, -sq) + 2.0f * mh * ml;
+  const float e2h = c2.hi * inv, e2l = c2.lo * inv;
+  float v = ((e2h - sq) + (e2l - sqe)) * inv1;
+  if (!(v > 0.f)) v = 0.f;
+  comp_merge(t[0], c1);
+  comp_merge(t[1], c2);
+  comp_add(t[2], mh);
+  comp_add(t[2], ml);
+  comp_add(t[3], v);
+}
+__device__ __forceinline__ void cube_totals(double inv_nc, double inv_nc1, double c1, double c2, double (&t)[4]) {
+  const double m = c1 * inv_nc;
+  double v = (c2 * inv_nc - m * m) * inv_nc1;
+  if (v < 0.0) v = 0.0;
+  t[0] += c1;
+  t[1] += c2;
+  t[2] += m;
+  t[3] += v;
+}
+// A hypercube's sums (or a part of them) in memory: (hi, lo, hi, lo) floats
+// or two doubles, 16 bytes.
+__device__ __forceinline__ void cube_store(void* p, size_t i, const fpair& c1, const fpair& c2) {
+  reinterpret_cast<float4*>(p)[i] = make_float4(c1.hi, c1.lo, c2.hi, c2.lo);
+}
+__device__ __forceinline__ void cube_store(void* p, size_t i, double c1, double c2) {
+  reinterpret_cast<double2*>(p)[i] = make_double2(c1, c2);
+}
+
 // Arguments of the sampling kernel (steps 2-4).
 struct SampleArgs {
   int d, N, g, ybits;
-  int lanes;               // lanes per hypercube (stratified mode), power of two <= 32
+  int lanes;               // lanes per group (stratified mode), power of two <= 32
+  uint32_t parts;          // groups per hypercube, each with its share of the cube's points
+  int niter;               // iterations this launch runs (frozen grid; 1 with the histogram)
+  uint32_t rot;            // CTAs by which each iteration's share of the work is turned
   int cap;                 // bucket capacity per (axis, bin) and tile
   int ppt;                 // points per thread per tile (>= 1)
   int strat;
@@ -236,8 +287,7 @@ struct SampleArgs {
   uint64_t ncall;
   uint32_t nc;             // points per hypercube
   uint32_t ncubes;         // number of hypercubes
-  uint32_t cube_mul;       // odd multiplier permuting the cube order (power-of-two
-                           // cube counts; 1 otherwise)
+  uint32_t cube_mul;       // multiplier permuting the cube order (cube_of)
   int g_pow2, g_log2;
   int t32;                 // 24-bit bins fit 32-bit integers (g N <= 256)
   float inv_gb_f;          // 1 / (g 2^ybits)
@@ -248,7 +298,8 @@ struct SampleArgs {
   const double* dparams;   // derived integrand constants
   GState* st;              // the sampling kernel latches st->live
   void* part_bins;         // [nparts][2 d N]: double, or float (hi, lo) pairs (FP32 forms)
-  double* part_tot;        // [kTotCols][nparts]
+  double* part_tot;        // [niter][kTotCols][nparts]
+  void* cube_part;         // [niter][parts][ncubes] sums of the parts (parts > 1), as `cubes`
   void* cubes;             // [ncubes]: double (sum w, sum w^2), or float (hi, lo, hi, lo)
   double* cube_max;        // [ncubes] running max(0, largest w) (integration phase), or null
 };
@@ -266,6 +317,12 @@ struct FinArgs {
   double alpha;
   const void* part_bins;
   const double* part_tot;
+  int niter;               // iterations of the pass (frozen grid)
+  uint32_t parts;          // groups per hypercube; > 1: the totals come from cube_part
+  uint32_t cube_mul;
+  double inv_nc, inv_nc1;  // 1 / nc, 1 / (nc - 1)
+  const void* cube_part;
+  void* cubes;             // per-cube sums of the last iteration (parts > 1), or null
   double* bins;            // [2][d][N] reduced, scaled
   double* edges;           // [d][N+1]
   double2* tab64;          // [d][N]

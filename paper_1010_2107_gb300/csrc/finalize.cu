@@ -117,8 +117,79 @@ __device__ __forceinline__ void reduce_axis(const FinArgs& F, int a, unsigned ra
   cl.sync();  // the first CTA has read the others' sums; s2 is complete
 }
 
+// The totals of iteration j from the hypercubes' part sums, by the whole
+// cluster: each thread adds the parts of its cubes in order, forms their
+// means and variances and writes the last iteration's cube sums; the threads
+// of a warp, the warps and the CTAs are merged in fixed order.  V: a part's
+// two sums (16 bytes), S: running sum.
+__device__ __forceinline__ void cube_load(const float4& v, fpair& c1, fpair& c2) {
+  c1 = fpair{v.x, v.y};
+  c2 = fpair{v.z, v.w};
+}
+__device__ __forceinline__ void cube_load(const double2& v, double& c1, double& c2) {
+  c1 = v.x;
+  c2 = v.y;
+}
+__device__ __forceinline__ fpair psum_xor(const fpair& a, int off) {
+  return fpair{__shfl_xor_sync(0xffffffffu, a.hi, off), __shfl_xor_sync(0xffffffffu, a.lo, off)};
+}
+__device__ __forceinline__ double psum_xor(const double& a, int off) { return __shfl_xor_sync(0xffffffffu, a, off); }
+
+template <typename V, typename S>
+__device__ __forceinline__ void reduce_cubes(const FinArgs& F, int j, unsigned rank, S (*buf)[4], double* tot) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const uint32_t G = (uint32_t)F.ncubes;
+  const V* src = reinterpret_cast<const V*>(F.cube_part) + (size_t)j * F.parts * G;
+  S t[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) psum_zero(t[q]);
+  const bool store = F.cubes && j == F.niter - 1;
+  for (uint32_t i = rank * kFinishThreads + threadIdx.x; i < G; i += kFinishCluster * kFinishThreads) {
+    S c1, c2;
+    psum_zero(c1);
+    psum_zero(c2);
+    for (uint32_t p = 0; p < F.parts; p += 4) {  // (a power of two above one: 2, or fours)
+      V v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (p + u < F.parts) v[u] = __ldcg(src + (size_t)(p + u) * G + i);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (p + u < F.parts) {
+          S a1, a2;
+          cube_load(v[u], a1, a2);
+          psum_merge(c1, a1);
+          psum_merge(c2, a2);
+        }
+    }
+    cube_totals(F.inv_nc, F.inv_nc1, c1, c2, t);
+    if (store) cube_store(F.cubes, cube_of(G, F.cube_mul, i), c1, c2);
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = kFinishThreads / 32;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) psum_merge(t[q], psum_xor(t[q], off));
+    if (lane == 0) buf[warp][q] = t[q];
+  }
+  __syncthreads();
+  if (threadIdx.x < 4) {
+    S a = buf[0][threadIdx.x];
+    for (int w = 1; w < nw; ++w) psum_merge(a, buf[w][threadIdx.x]);
+    buf[0][threadIdx.x] = a;
+  }
+  cl.sync();
+  if (rank == 0 && threadIdx.x < 4) {
+    S a = buf[0][threadIdx.x];
+    for (int r = 1; r < kFinishCluster; ++r) psum_merge(a, cl.map_shared_rank(&buf[0][0], r)[threadIdx.x]);
+    tot[threadIdx.x] = psum_value(a);
+  }
+  cl.sync();  // the others' sums have been read; buf may be used again
+}
+
 // Step 6 for the pass, by one full warp (lane 0 writes the state).
-__device__ void record_iteration(const FinArgs& F, const double* t) {
+__device__ void record_iteration(const FinArgs& F, const double* t, bool combine) {
   GState* st = F.st;
   const int lane = threadIdx.x & 31;
   double I, var;
@@ -157,7 +228,7 @@ __device__ void record_iteration(const FinArgs& F, const double* t) {
   }
   // Inverse-variance combination over the window (Lepage): in a call without
   // an ACC target only the last pass's combination can be read.
-  if (!F.combine) return;
+  if (!combine) return;
   double Ib, sg, chi;
   combine_history(st->hist, h, &Ib, &sg, &chi);
   if (lane == 0) {
@@ -184,7 +255,7 @@ __device__ void record_iteration(const FinArgs& F, const double* t) {
 __global__ void __cluster_dims__(kFinishCluster, 1, 1) __launch_bounds__(kFinishThreads) k_finish(const FinArgs F) {
   __shared__ __align__(16) unsigned char buf[kFinishThreads * 16 > 2 * kMaxBins * 8 ? kFinishThreads * 16 : 2 * kMaxBins * 8];
   __shared__ double s2[kMaxBins];
-  __shared__ double tot[kTotCols];
+  __shared__ double tot[kMergeIters][kTotCols];
   GState* st = F.st;
   if (!st->live) return;  // (uniform over the launch)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -204,16 +275,33 @@ __global__ void __cluster_dims__(kFinishCluster, 1, 1) __launch_bounds__(kFinish
                      F.alpha, t);
     return;
   }
+  // The totals of each iteration: the columns over the partial rows, or,
+  // where several groups share a hypercube, the cubes' own sums over the
+  // cluster (and only the non-finite count from the rows).
+  if (F.parts > 1u) {
+    for (int j = 0; j < F.niter; ++j) {
+      if (F.pair32)
+        reduce_cubes<float4, fpair>(F, j, rank, reinterpret_cast<fpair(*)[4]>(buf), tot[j]);
+      else
+        reduce_cubes<double2, double>(F, j, rank, reinterpret_cast<double(*)[4]>(buf), tot[j]);
+    }
+  }
   if (rank != 0) return;
-  if (warp < 5) {
-    const int q = warp;
-    const double v = total_column(F.part_tot + (size_t)q * F.nparts, F.nparts, lane);
-    const double s1 = *F.scale;
-    const double sc = (q == TOT_SW || q == TOT_SI) ? s1 : (q == TOT_NONFINITE ? 1.0 : s1 * s1);
-    if (lane == 0) tot[q] = v * sc;
+  const double s1 = *F.scale;
+  for (int i = warp; i < 5 * F.niter; i += kFinishThreads / 32) {
+    const int j = i / 5, q = i - 5 * j;
+    if (F.parts > 1u && q != TOT_NONFINITE) continue;
+    const double v = total_column(F.part_tot + ((size_t)j * kTotCols + q) * F.nparts, F.nparts, lane);
+    if (lane == 0) tot[j][q] = v;
   }
   __syncthreads();
-  if (warp == 0) record_iteration(F, tot);
+  if (threadIdx.x < 5 * F.niter) {
+    const int j = threadIdx.x / 5, q = threadIdx.x - 5 * j;
+    tot[j][q] *= (q == TOT_SW || q == TOT_SI) ? s1 : (q == TOT_NONFINITE ? 1.0 : s1 * s1);
+  }
+  __syncthreads();
+  if (warp == 0)
+    for (int j = 0; j < F.niter; ++j) record_iteration(F, tot[j], F.combine && j == F.niter - 1);
 }
 
 // Column sums of a [ncols][nrows] partial block (one warp per column,

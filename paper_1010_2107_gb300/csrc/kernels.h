@@ -81,7 +81,8 @@ int rtc_user_compile(const char* source, int prec, int ybits, int d, bool spec, 
 struct PassShape {
   const void* fn = nullptr;
   int ctas = 0, threads = 256;
-  int lanes = 1;    // lanes per hypercube (stratified sampling)
+  int lanes = 1;    // lanes per group and groups per hypercube (stratified sampling)
+  uint32_t parts = 1;
   int occ = 0;      // CTAs per SM
   size_t smem = 0;  // dynamic shared memory
 };
@@ -163,29 +164,59 @@ inline int choose_lanes(uint64_t G, uint64_t nc, int threads, int64_t ctas) {
 }
 
 // Lanes per hypercube where a tile's crowding does not matter (the column
-// histogram, passes without a histogram): the power of two L <= min(32, nc)
-// of least cost.  A CTA of `threads` threads takes the G L lanes in rounds;
-// a round costs a lane's points (in steps of `pif`) and, in eighths of a
+// histogram, passes without a histogram): the power of two of least cost,
+// L <= min(32, nc) lanes in a group, or 32 lanes in each of `parts` groups of
+// a cube where the cubes are few (a BASES run of 6^3 cubes filled 27 CTAs
+// with one group each).  A CTA of `threads` threads takes the G L lanes in
+// rounds; a round costs a lane's points (in steps of `pif`) and, in eighths of a
 // point, 0.6 per level of the group's butterfly and 3 for the cube's own
 // totals; an SM runs its share of the rounds, and about one more while its
 // last CTAs leave it partly idle.  (Measured, us per pass at 2^22 points:
 // dgauss8, 65 536 cubes of 64, L = 4, 8, 16, 32: 66, 60.5, 63.5, 70.5 with
 // columns and 52, 48, 52, 61 without; wmunu, 32 768 of 128: 72, 73, 66, 70
 // and 61, 62, 57, 61.  The rule takes 8 and 16.)
-inline int balanced_lanes(uint64_t G, uint64_t nc, int threads, int sms, int pif) {
-  int best = 1;
+// Parts cost their round trip through memory (1 per round) and their merge
+// by the finishing kernel's 2048 threads (half a point each).
+struct CubeLanes {
+  int lanes;
+  uint32_t parts;
+};
+constexpr uint64_t kMaxCubeParts = 1u << 17;  // groups of a pass with several per cube (16 bytes each)
+inline CubeLanes balanced_lanes(uint64_t G, uint64_t nc, int threads, int sms, int pif, uint64_t max_parts) {
+  CubeLanes best{1, 1};
   double least = 0.0;
-  for (int L = 1, lg = 0; L <= 32 && (uint64_t)L <= nc; L *= 2, ++lg) {
-    const uint64_t rounds = (G * (uint64_t)L + threads - 1) / threads, per_sm = (rounds + sms - 1) / sms;
+  uint64_t L = 1;
+  for (int lg = 0; L <= nc; L *= 2, ++lg) {
+    const uint64_t parts = L > 32 ? L / 32 : 1;
+    if (parts > 1 && G * parts > max_parts) break;
+    const uint64_t rounds = (G * L + threads - 1) / threads, per_sm = (rounds + sms - 1) / sms;
     uint64_t pts = (nc + L - 1) / L;
     pts = (pts + pif - 1) / pif * pif;
-    const double cost = (double)(per_sm + 1) * (8.0 * (double)pts + 0.6 * lg + 3.0);
+    double cost = (double)(per_sm + 1) * (8.0 * (double)pts + 0.6 * (lg < 5 ? lg : 5) + 3.0 + (parts > 1 ? 1.0 : 0.0));
+    if (parts > 1) cost += 4.0 * (double)((G * parts + 2047) / 2048);
     if (L == 1 || cost < least) {
       least = cost;
-      best = L;
+      best = CubeLanes{(int)(L < 32 ? L : 32), (uint32_t)parts};
     }
   }
   return best;
+}
+
+// Multiplier of the cube order (cube_of) over G cubes: odd for a power of
+// two, else about 0.618 G and coprime to it.
+inline uint32_t cube_multiplier(uint64_t G) {
+  if ((G & (G - 1)) == 0) return 0x9E3779B1u;
+  auto gcd = [](uint64_t a, uint64_t b) {
+    while (b) {
+      const uint64_t r = a % b;
+      a = b;
+      b = r;
+    }
+    return a;
+  };
+  uint64_t m = (uint64_t)(0.6180339887 * (double)G) | 1;
+  while (gcd(m, G) != 1) ++m;
+  return (uint32_t)m;
 }
 
 #endif  // __CUDACC_RTC__

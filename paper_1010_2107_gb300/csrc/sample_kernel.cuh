@@ -377,26 +377,6 @@ __device__ __forceinline__ fpair warp_sum(fpair p) {
   return p;
 }
 
-// Step 4 of one hypercube from its compensated sums: the cube mean m = C1 /
-// nc and variance (C2 / nc - m^2) / (nc - 1) into the totals, in FP32 with
-// the square formed exactly (FMA) and the pairs kept, and the cube's sums.
-__device__ __forceinline__ void cube_totals(const SampleArgs& A, uint32_t c, const fpair& c1, const fpair& c2,
-                                            fpair (&tp)[4]) {
-  const float inv = (float)A.inv_nc, inv1 = (float)A.inv_nc1;
-  const float mh = c1.hi * inv, ml = c1.lo * inv;
-  const float sq = mh * mh;
-  const float sqe = fmaf(mh, mh, -sq) + 2.0f * mh * ml;
-  const float e2h = c2.hi * inv, e2l = c2.lo * inv;
-  float v = ((e2h - sq) + (e2l - sqe)) * inv1;
-  if (!(v > 0.f)) v = 0.f;
-  comp_merge(tp[0], c1);
-  comp_merge(tp[1], c2);
-  comp_add(tp[2], mh);
-  comp_add(tp[2], ml);
-  comp_add(tp[3], v);
-  if (A.cubes) reinterpret_cast<float4*>(A.cubes)[c] = make_float4(c1.hi, c1.lo, c2.hi, c2.lo);
-}
-
 // The CTA's totals (compensated pairs per thread) into its column of
 // part_tot: fixed butterflies, then the warps in order.
 __device__ __forceinline__ void store_totals(const SampleArgs& A, const fpair (&tp)[4], int nonfinite) {
@@ -431,6 +411,7 @@ __device__ __forceinline__ void store_totals(const SampleArgs& A, const fpair (&
 // (their register budget).
 template <bool SPEC>
 constexpr int kSampleMaxThreads = SPEC ? 512 : 256;
+constexpr int kMaxSampleWarps = 16;
 
 template <typename T, int DM, template <typename, int> class F, int ACC, int YB, bool SPEC>
 __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>) k_sample(const SampleArgs A) {
@@ -443,7 +424,7 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>) k_sample(const Sample
   const int stop = A.st->done;
   if (blockIdx.x == 0 && threadIdx.x == 0) A.st->live = !stop;
   if (stop) return;
-  const uint32_t it = A.it_override >= 0 ? (uint32_t)A.it_override : A.st->it;
+  uint32_t it = A.it_override >= 0 ? (uint32_t)A.it_override : A.st->it;
   // SPEC: d equals the compile-time bound DM, 24-bit words and power-of-two
   // hypercube divisions with g N <= 256: every per-axis guard folds away.
   const int d = SPEC ? DM : A.d, N = A.N, dN = d * N, cap = A.cap;
@@ -497,6 +478,13 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>) k_sample(const Sample
   // FP64 (ACC 0/1) or compensated FP32 pairs (ACC 2).
   double t[4] = {0.0, 0.0, 0.0, 0.0};
   fpair tp[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+  // The CTA's place in the order of the work: its row of partial sums.  A
+  // launch of several frozen-grid iterations turns the places by A.rot from
+  // one to the next, so that the CTAs with one round more than the others
+  // change; a place's work and row are the same in every launch.
+  uint32_t place = blockIdx.x;
+  int iter = 0;
+  bool last_iter = true;
   // The pass loop, compiled twice: with the per-bin histogram and without
   // it (a uniform choice per launch; no test inside the loops).
   auto pass = [&](auto with_bins) {
@@ -511,7 +499,7 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>) k_sample(const Sample
       Run<ACC> sw, sw2;
       H pmax = H(0);  // largest weight (integration-phase maximum of the one cube)
       const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-      const uint64_t first = (uint64_t)blockIdx.x * blockDim.x;
+      const uint64_t first = (uint64_t)place * blockDim.x;
       const uint64_t rounds = first < A.ncall ? (A.ncall - first + stride - 1) / stride : 0;
       uint64_t s = first + tid;
       int pend = 0;  // points per thread since the last gather (uniform in the CTA)
@@ -570,25 +558,26 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>) k_sample(const Sample
         t[1] = sw2.value();
       }
     } else {
-      // Groups of Lw lanes share a hypercube; lane j of a group takes the
-      // cube's points j, j + Lw, ... in lock-step with the rest of the CTA
-      // (one tile per step); the group then reduces its sums with a fixed
-      // xor-butterfly (deterministic).  Group i takes cube
-      // (i * cube_mul) mod ncubes, so that the groups of a CTA sit in
-      // unrelated cubes and spread over the bins.
+      // Groups of Lw lanes share a hypercube, or one of its A.parts parts
+      // where the cubes are too few to fill the GPU; of the VL = Lw parts
+      // lanes of a cube, lane j takes its points j, j + VL, ... in lock-step
+      // with the rest of the CTA (one tile per step); the group then reduces
+      // its sums with a fixed xor-butterfly (deterministic).  Group i takes
+      // part i div ncubes of the cube in place i mod ncubes (cube_of).
       const int Lw = A.lanes;
-      const int gl = tid & (Lw - 1);
+      const uint32_t units = A.ncubes * A.parts, VL = (uint32_t)Lw * A.parts;
       const uint32_t groups_per_cta = blockDim.x / Lw;
       const uint32_t gstride = gridDim.x * groups_per_cta;
-      const uint32_t gfirst = blockIdx.x * groups_per_cta;
-      const uint32_t rounds = gfirst < A.ncubes ? (A.ncubes - gfirst + gstride - 1) / gstride : 0;
-      const uint32_t cmask = A.ncubes - 1u;
-      const uint32_t per_lane = (A.nc + Lw - 1) / Lw;
+      const uint32_t gfirst = place * groups_per_cta;
+      const uint32_t rounds = gfirst < units ? (units - gfirst + gstride - 1) / gstride : 0;
+      const uint32_t per_lane = (A.nc + VL - 1) / VL;
       uint32_t gi = gfirst + tid / Lw;
       int pend = 0;  // points per thread since the last gather (uniform in the CTA)
       for (uint32_t r = 0; r < rounds; ++r, gi += gstride) {
-        const bool live = gi < A.ncubes;  // uniform within a group
-        const uint32_t c = A.cube_mul == 1u ? gi : (gi * A.cube_mul) & cmask;
+        const bool live = gi < units;  // uniform within a group
+        const uint32_t part = A.parts > 1u ? gi / A.ncubes : 0u;
+        const uint32_t c = cube_of(A.ncubes, A.cube_mul, gi - part * A.ncubes);
+        const uint32_t gl = part * Lw + (tid & (Lw - 1));
         if (live) {
           uint32_t rest = c;
   #pragma unroll
@@ -610,7 +599,7 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>) k_sample(const Sample
         H p1 = H(0), p2 = H(0), pmax = H(0);
         if constexpr (PAIR) {
           for (uint32_t i = 0; i < per_lane; i += 2) {
-            const uint32_t j0 = gl + i * Lw, j1 = j0 + Lw;
+            const uint32_t j0 = gl + i * VL, j1 = j0 + VL;
             const bool v0 = live && j0 < A.nc, v1 = live && j1 < A.nc;
             int kb0[DM], kb1[DM];
             const H w0 = eval_point(s0 + j0, kb0, v0);
@@ -634,7 +623,7 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>) k_sample(const Sample
           }
         } else {
           for (uint32_t i = 0; i < per_lane; ++i) {
-            const uint32_t j = gl + i * Lw;
+            const uint32_t j = gl + i * VL;
             if (live && j < A.nc) {
               int kb[DM];
               const H w = eval_point(s0 + j, kb);
@@ -649,9 +638,19 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>) k_sample(const Sample
             }
           }
         }
-        if (A.cube_max) {  // integration phase: per-cube maxima (one group per cube)
+        if (A.cube_max) {  // integration phase: per-cube maxima
           for (int off = Lw >> 1; off > 0; off >>= 1) pmax = max(pmax, __shfl_xor_sync(0xffffffffu, pmax, off, Lw));
-          if (live && gl == 0) A.cube_max[c] = fmax(A.cube_max[c], (double)pmax);
+          if (live && (tid & (Lw - 1)) == 0) {
+            // (several parts, or several iterations of one launch, may meet:
+            // non-negative doubles order as their bit patterns)
+            if (A.parts > 1u || A.niter > 1) {
+              if (pmax > H(0))
+                atomicMax(reinterpret_cast<unsigned long long*>(A.cube_max + c),
+                          (unsigned long long)__double_as_longlong((double)pmax));
+            } else {
+              A.cube_max[c] = fmax(A.cube_max[c], (double)pmax);
+            }
+          }
         }
         if constexpr (COMP) {
           fpair c1{p1, 0.f}, c2{p2, 0.f};
@@ -664,8 +663,13 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>) k_sample(const Sample
             comp_merge(c1, o1);
             comp_merge(c2, o2);
           }
-          if (live && gl == 0) {
-            cube_totals(A, c, c1, c2, tp);
+          if (live && (tid & (Lw - 1)) == 0) {
+            if (A.parts > 1u) {
+              cube_store(A.cube_part, (size_t)iter * units + gi, c1, c2);
+            } else {
+              cube_totals(A.inv_nc, A.inv_nc1, c1, c2, tp);
+              if (A.cubes && last_iter) cube_store(A.cubes, c, c1, c2);
+            }
           }
         } else {
           double c1 = p1, c2 = p2;
@@ -673,17 +677,12 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>) k_sample(const Sample
             c1 += __shfl_xor_sync(0xffffffffu, c1, off, Lw);
             c2 += __shfl_xor_sync(0xffffffffu, c2, off, Lw);
           }
-          if (live && gl == 0) {
-            const double m = c1 * A.inv_nc;
-            double v = (c2 * A.inv_nc - m * m) * A.inv_nc1;
-            if (v < 0.0) v = 0.0;
-            t[0] += c1;
-            t[1] += c2;
-            t[2] += m;
-            t[3] += v;
-            if (A.cubes) {
-              reinterpret_cast<double*>(A.cubes)[2 * (size_t)c] = c1;
-              reinterpret_cast<double*>(A.cubes)[2 * (size_t)c + 1] = c2;
+          if (live && (tid & (Lw - 1)) == 0) {
+            if (A.parts > 1u) {
+              cube_store(A.cube_part, (size_t)iter * units + gi, c1, c2);
+            } else {
+              cube_totals(A.inv_nc, A.inv_nc1, c1, c2, t);
+              if (A.cubes && last_iter) cube_store(A.cubes, c, c1, c2);
             }
           }
         }
@@ -691,10 +690,43 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>) k_sample(const Sample
       if (pend) gather();
     }
   };
-  if (bins)
+  // The totals of an iteration, one entry per warp and column: compensated
+  // pairs (COMP) or doubles, and the non-finite count.
+  __shared__ double wone[kMaxSampleWarps][5];
+  double(*wtot)[5] = bins ? wone : reinterpret_cast<double(*)[5]>(smem + L::hist(dN));
+  auto warp_totals = [&]() {
+    double* out = wtot[iter * nw + warp];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if constexpr (COMP) {
+        const fpair v = warp_sum(tp[q]);
+        if (lane == 0) *reinterpret_cast<float2*>(out + q) = make_float2(v.hi, v.lo);
+        tp[q] = fpair{0.f, 0.f};
+      } else {
+        double v = t[q];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if (lane == 0) out[q] = v;
+        t[q] = 0.0;
+      }
+    }
+    int nf = nonfinite;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) nf += __shfl_xor_sync(0xffffffffu, nf, off);
+    if (lane == 0) out[4] = (double)nf;
+    nonfinite = 0;
+  };
+  if (bins) {
     pass(BoolTag<true>{});
-  else
-    pass(BoolTag<false>{});
+    warp_totals();
+  } else {
+    for (; iter < A.niter; ++iter, ++it) {
+      place = (blockIdx.x + (uint32_t)iter * A.rot) % gridDim.x;
+      last_iter = iter == A.niter - 1;
+      pass(BoolTag<false>{});
+      warp_totals();
+    }
+  }
   __syncthreads();
 
   // Partial row of this CTA: histogram cells (FP64, or compensated FP32
@@ -709,27 +741,22 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>) k_sample(const Sample
     }
   }
 
-  if constexpr (COMP) {
-    store_totals(A, tp, nonfinite);
-  } else {
-    __shared__ double wsum[32][5];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      double v = t[q];
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-      if (lane == 0) wsum[warp][q] = v;
+  for (int i = tid; i < 5 * A.niter; i += blockDim.x) {
+    const int j = i / 5, q = i - 5 * j;
+    const double(*v)[5] = wtot + j * nw;
+    double acc = 0.0;
+    if (COMP && q < 4) {
+      fpair p{0.f, 0.f};
+      for (int w = 0; w < nw; ++w) {
+        const float2 u = *reinterpret_cast<const float2*>(&v[w][q]);
+        comp_merge(p, fpair{u.x, u.y});
+      }
+      acc = comp_value(p);
+    } else {
+      for (int w = 0; w < nw; ++w) acc += v[w][q];
     }
-    int nf = nonfinite;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) nf += __shfl_xor_sync(0xffffffffu, nf, off);
-    if (lane == 0) wsum[warp][4] = (double)nf;
-    __syncthreads();
-    if (tid < 5) {
-      double acc = 0.0;
-      for (int w = 0; w < nw; ++w) acc += wsum[w][tid];
-      A.part_tot[(size_t)tid * A.nparts + row] = acc;
-    }
+    const uint32_t at = (blockIdx.x + (uint32_t)j * A.rot) % gridDim.x;
+    A.part_tot[((size_t)j * kTotCols + q) * A.nparts + at] = acc;
   }
 }
 
@@ -890,19 +917,20 @@ __global__ void __launch_bounds__(512, 1) k_sample_col(const SampleArgs A) {
       }
     }
   } else {
-    // groups of Lw lanes share a hypercube, as in k_sample
+    // groups of Lw lanes share a hypercube or a part of it, as in k_sample
     const int Lw = A.lanes;
-    const int gl = tid & (Lw - 1);
+    const uint32_t units = A.ncubes * A.parts, VL = (uint32_t)Lw * A.parts;
     const uint32_t groups_per_cta = blockDim.x / Lw;
     const uint32_t gstride = gridDim.x * groups_per_cta;
     const uint32_t gfirst = blockIdx.x * groups_per_cta;
-    const uint32_t rounds = gfirst < A.ncubes ? (A.ncubes - gfirst + gstride - 1) / gstride : 0;
-    const uint32_t cmask = A.ncubes - 1u;
-    const uint32_t per_lane = (A.nc + Lw - 1) / Lw;
+    const uint32_t rounds = gfirst < units ? (units - gfirst + gstride - 1) / gstride : 0;
+    const uint32_t per_lane = (A.nc + VL - 1) / VL;
     uint32_t gi = gfirst + tid / Lw;
     for (uint32_t r = 0; r < rounds; ++r, gi += gstride) {
-      const bool live = gi < A.ncubes;  // uniform within a group
-      const uint32_t c = A.cube_mul == 1u ? gi : (gi * A.cube_mul) & cmask;
+      const bool live = gi < units;  // uniform within a group
+      const uint32_t part = A.parts > 1u ? gi / A.ncubes : 0u;
+      const uint32_t c = cube_of(A.ncubes, A.cube_mul, gi - part * A.ncubes);
+      const uint32_t gl = part * Lw + (tid & (Lw - 1));
       uint32_t rest = live ? c : 0u;
 #pragma unroll
       for (int a = 0; a < DM; ++a)
@@ -918,7 +946,7 @@ __global__ void __launch_bounds__(512, 1) k_sample_col(const SampleArgs A) {
         float w[PIF];
 #pragma unroll
         for (int q = 0; q < PIF; ++q) {
-          const uint32_t j = gl + (i + q) * Lw;
+          const uint32_t j = gl + (i + q) * VL;
           sq[q] = s0 + j;
           v[q] = live && j < A.nc;
         }
@@ -939,7 +967,14 @@ __global__ void __launch_bounds__(512, 1) k_sample_col(const SampleArgs A) {
         comp_merge(c1, o1);
         comp_merge(c2, o2);
       }
-      if (live && gl == 0) cube_totals(A, c, c1, c2, tp);
+      if (live && (tid & (Lw - 1)) == 0) {
+        if (A.parts > 1u) {
+          cube_store(A.cube_part, gi, c1, c2);
+        } else {
+          cube_totals(A.inv_nc, A.inv_nc1, c1, c2, tp);
+          if (A.cubes) cube_store(A.cubes, c, c1, c2);
+        }
+      }
     }
   }
   hist.drain();
@@ -953,7 +988,8 @@ __host__ __device__ inline size_t sample_smem_bytes(int d, int N, int cap) {
 }
 template <typename T, int ACC>
 __host__ __device__ inline size_t sample_smem_nobins(int d, int N) {
-  return SmemLayout<T, ACC>::hist(d * N);
+  // (behind the table and the constants: the iterations' totals per warp)
+  return SmemLayout<T, ACC>::hist(d * N) + sizeof(double) * 5 * kMaxSampleWarps * kMergeIters;
 }
 
 // Steps 2-3 for a list of sample indices (parity checks and debugging):
@@ -970,8 +1006,14 @@ __host__ __device__ inline size_t sample_smem_nobins(int d, int N) {
 // order).  One thread per trial and round; 256 threads.
 constexpr uint32_t kSpringIt = 0xFFFFFFFFu;
 
+// CTAs per SM the specialised FP32 kernels of low dimension are held to: the
+// cube search waits on L2, so residency counts (d = 8: 54 registers and four
+// CTAs took 452 us per 2^22 trials with their events, 48 and five 442 us).
+template <typename T, int DM, bool SPEC>
+constexpr int kSpringMinBlocks = SPEC && std::is_same<T, float>::value && DM <= 8 ? 5 : 1;
+
 template <typename T, int DM, template <typename, int> class F, int YB, bool SPEC>
-__global__ void __launch_bounds__(256) k_spring(const SpringArgs R) {
+__global__ void __launch_bounds__(256, kSpringMinBlocks<T, DM, SPEC>) k_spring(const SpringArgs R) {
   using T2 = typename Vec2<T>::type;
   const SampleArgs& A = R.S;
   const int d = SPEC ? DM : A.d, N = A.N, dN = d * N;
