@@ -354,11 +354,14 @@ vegas_status vegas_get_launch(vegas_ctx* ctx, int* threads, int* ctas,
  * host code sums the bins): each thread evaluates `points_per_thread`
  * points (1..8; 0 = automatic) between two gathers of the CTA's
  * (axis, bin) buckets; kernels that evaluate two points per thread at a
- * time round it up to even.  Changes only speed and the summation order
- * inside a CTA, never which points are drawn.  get_tile returns the points per
- * thread and the bucket capacity per (axis, bin) in use.  EINVAL outside
- * the range or when the tile does not fit in shared memory (the previous
- * shape then stays). */
+ * time round it up to even.  Automatic: the FP32 form with compensated sums,
+ * 24-bit words and a power-of-two number of divisions (g N <= 256) has no
+ * tiles where its lane-owned columns fit (up to 100 bins); the other forms
+ * choose a tile.  Changes only speed and the summation order inside a CTA,
+ * never which points are drawn.  get_tile returns the points per thread (in
+ * flight) and the bucket capacity per (axis, bin) in use, 0 for columns.
+ * EINVAL outside the range or when the tile does not fit in shared memory
+ * (the previous shape then stays). */
 vegas_status vegas_set_tile(vegas_ctx* ctx, int points_per_thread);
 vegas_status vegas_get_tile(vegas_ctx* ctx, int* points_per_thread, int* cap);
 
@@ -371,7 +374,8 @@ vegas_status vegas_get_tile(vegas_ctx* ctx, int* points_per_thread, int* cap);
  * timed again in three
  * interleaved rounds of five passes, and the one with the best round is
  * kept.  Returns its threads, points
- * per thread and the pass time in ms (any output may be NULL).  The
+ * per thread (the tile itself stays as tuned: automatic where vegas_get_tile
+ * then reports capacity 0) and the pass time in ms (any output may be NULL).  The
  * specialised kernels (d = the compiled bound, 24-bit words, power-of-two
  * strata) accept up to 512 threads, the general ones 256.  Synchronises the
  * stream. */
@@ -453,18 +457,22 @@ vegas_status vegas_batch_get_grid(vegas_batch* batch, int i, double* edges, doub
 vegas_status vegas_batch_get_history(vegas_batch* batch, int i, double* hist, int max_iters, int* n_out);
 
 /* Launch shape: threads per CTA (64..256, multiple of 32) and rounds per
- * work item (an item is threads * rounds points of one instance). */
+ * work item (an item is threads * rounds points of one instance); before the
+ * first call the rounds follow the batch's work. */
 vegas_status vegas_batch_set_launch(vegas_batch* batch, int threads, int rounds);
 vegas_status vegas_batch_get_launch(vegas_batch* batch, int* threads, int* rounds, int* ctas, int* items);
 
 /* Histogram tile of the batched sampling kernels (as vegas_set_tile; no
  * counterpart in the paper): the points each thread evaluates between two
  * gathers of the CTA's buckets, 0 = automatic.  The FP32 form with 24-bit
- * words runs one kernel per dimension (d = 1..16), where this is 1 or 2,
- * the points a thread keeps in flight; the other forms take 0..4.  EINVAL
+ * words runs one kernel per dimension (d = 1..16), automatically with
+ * lane-owned columns instead of buckets where they fit (up to 100 bins);
+ * with 1 or 2, the points a thread keeps in flight, with buckets; the other
+ * forms take 0..4.  EINVAL
  * outside the range or when the tile does not fit (the previous tile then
  * stays).  get_tile returns the points per thread and the bucket capacity
- * (of the widest dimension's kernel for the per-dimension kernels).
+ * (of the widest dimension's kernel for the per-dimension kernels; 0 for
+ * columns).
  * Changes only speed and the summation order inside a CTA. */
 vegas_status vegas_batch_set_tile(vegas_batch* batch, int points_per_thread);
 vegas_status vegas_batch_get_tile(vegas_batch* batch, int* points_per_thread, int* cap);

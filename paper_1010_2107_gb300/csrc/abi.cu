@@ -398,36 +398,34 @@ __global__ void k_spring_compact(const uint32_t* counts, uint32_t chunk, int d, 
   for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) ot[off + i] = st[src + i];
 }
 
-// Shape of the column-histogram pass (col_hist.cuh) for `threads` threads per
-// CTA, or, when 0, for the count that keeps most warps resident (the columns'
-// shared memory bounds them) and, on equal terms, the widest CTA (fewest
-// partial rows); a small pass takes narrower CTAs until every SM has one.
-// False when fewer than kColMinWarps warps would be resident: the columns of
-// many bins are too large and bucketed tiles are the better form (measured at
-// 4M points in 8 dimensions: 64 bins and below columns, see DESIGN).
+// Shape of the column-histogram pass (col_hist.cuh): `threads` threads per
+// CTA, or, when 0, one CTA of as many warps as the columns' shared memory
+// allows (16 at up to 50 bins, the most the registers allow; one wide CTA
+// folds into one partial row: at 72 bins 11 warps in one CTA beat 10 in
+// five, 65 against 70 us at d = 8); a small pass takes narrower CTAs until
+// every SM has one.  False when fewer than kColMinWarps warps fit (from 101
+// bins on): down to that count columns beat bucketed tiles at every measured
+// dimension (us per pass of 2^22 points at 100 bins, columns against the best
+// tile: d = 4 43.9 / 47.1, d = 7 115.6 / 119.6, d = 8 66 / 93, d = 16 119 / 206).
 constexpr int kColMinWarps = 8;
 bool shape_col(const void* fn, const gv::KernelEntry& ke, int d, int N, int sm_count, int threads, int per_sm_req,
                uint64_t ncubes, uint64_t nc, uint64_t ncall, int64_t max_rows, uint64_t max_parts,
                gv::PassShape* out, cudaError_t* e) {
-  static const int kAuto[] = {512, 384, 256, 192, 128, 64};
-  int best_t = 0, best_occ = 0;
-  const int one[] = {threads};
-  const int* list = threads > 0 ? one : kAuto;
-  const int n = threads > 0 ? 1 : (int)(sizeof kAuto / sizeof kAuto[0]);
-  for (int i = 0; i < n; ++i) {
-    const size_t smem = ke.smem_col(d, N, list[i] / 32);
-    if (smem + 2048 > 227 * 1024) continue;  // (2 KB: the kernel's static shared memory)
-    if ((*e = gv_raise_smem_limit(fn, smem)) != cudaSuccess) return false;
-    int o = 0;
-    if ((*e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, fn, list[i], smem)) != cudaSuccess) return false;
-    if (per_sm_req > 0) o = std::min(o, per_sm_req);
-    if (o * list[i] > best_occ * best_t) {
-      best_t = list[i];
-      best_occ = o;
-    }
-    if (best_occ * best_t >= 512) break;  // (16 warps: what the kernels' registers allow)
+  // (2 KB: the kernel's static shared memory)
+  auto fits = [&](int warps) { return ke.smem_col(d, N, warps) + 2048 <= 227 * 1024; };
+  int best_t = threads;
+  if (threads == 0) {
+    int warps = 16;
+    while (warps >= kColMinWarps && !fits(warps)) --warps;
+    best_t = 32 * warps;
+    if (warps < kColMinWarps) return false;
   }
-  if (best_occ * best_t < 32 * kColMinWarps && threads == 0) return false;
+  if (!fits(best_t / 32)) return false;
+  const size_t smem = ke.smem_col(d, N, best_t / 32);
+  if ((*e = gv_raise_smem_limit(fn, smem)) != cudaSuccess) return false;
+  int best_occ = 0;
+  if ((*e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&best_occ, fn, best_t, smem)) != cudaSuccess) return false;
+  if (per_sm_req > 0) best_occ = std::min(best_occ, per_sm_req);
   if (best_occ < 1) return false;
   const int pif = d <= 8 ? 2 : 1;
   if (threads == 0 && ncubes == 1) {

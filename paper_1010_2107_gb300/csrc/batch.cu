@@ -386,6 +386,7 @@ struct vegas_batch {
   int sm_count = 0;
   // launch shape
   int threads = 256, rounds = 32, ctas = 0, cap = 16, ppt = 1, occ = 0;
+  bool launch_set = false;  // by vegas_batch_set_launch (else rounds may be chosen by the work)
   int ppt_req = 0;         // points per thread per tile asked for (0: automatic)
   bool small_cap = false;  // tile capacity policy (gv::choose_tile)
   bool dense_cap = false;  // the dense floor of that policy (per-dimension kernels)
@@ -540,11 +541,56 @@ vegas_status build_items(vegas_batch* b) {
 
 // Dimension kernels: for each dimension present its kernel (points in
 // flight = the tile's points per thread), bucket capacity and CTAs per SM.
+// Automatically (no tile asked for) the column-histogram kernels, where for
+// every dimension present at least kColMinWarps warps per SM fit (up to 100
+// bins; there too they beat the buckets: 64 instances of 2^16..2^20 points
+// 0.423 ms against 0.590, one CTA of eight warps per SM; wider CTAs at 64 to
+// 80 bins gained nothing).  Without a launch shape set, an item's rounds
+// follow the work: about sixteen items per SM, 8 to 128 rounds (a fold per
+// item against an even queue; ms per pass at 16, 32, 64, 128 rounds, 50 bins:
+// 256 instances of 2^16..2^22 points 3.92, 3.41, 3.22, 3.12, 64 of
+// 2^16..2^18 0.172, 0.182, 0.246, 0.354).
+constexpr int kColMinWarps = 8;
+bool configure_cols(vegas_batch* b, const bool (&present)[gv::kBatchDM], cudaError_t* e) {
+  for (int d = 1; d <= gv::kBatchDM; ++d) {
+    auto& c = b->dims[d - 1];
+    c.occ = 0;
+    if (!present[d - 1]) continue;
+    c.fn = d <= 8 ? gv_batch_dim_kernel_lo(d, 0) : gv_batch_dim_kernel_hi(d, 0);
+    c.cap = 0;
+    c.smem = gv::dim_col_smem(d, b->N, b->threads / 32);
+    if (c.smem + 1024 > 227 * 1024) return false;  // (1 KB: the kernel's static shared memory)
+    if ((*e = cudaFuncSetAttribute(c.fn, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                   (int)cudaSharedmemCarveoutMaxShared)) != cudaSuccess)
+      return false;
+    if ((*e = gv_raise_smem_limit(c.fn, c.smem)) != cudaSuccess) return false;
+    if ((*e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c.occ, c.fn, b->threads, c.smem)) != cudaSuccess) return false;
+    if (c.occ * b->threads < 32 * kColMinWarps) return false;
+  }
+  if (!b->launch_set) {
+    double points = 0.0;
+    for (const vegas_config& c : b->cfg) points += (double)c.ncall;
+    b->rounds = 8;
+    while (b->rounds < 128 && (double)b->rounds * 1.5 < points / (256.0 * 16.0 * b->sm_count)) b->rounds *= 2;
+  }
+  return true;
+}
+
 vegas_status configure_dims(vegas_batch* b) {
   const int pif = b->ppt_req == 1 ? 1 : 2;
   b->ppt = pif;
+  if (!b->launch_set) b->rounds = 32;
   bool present[gv::kBatchDM] = {};
   for (int i = 0; i < b->n; ++i) present[b->d[i] - 1] = true;
+  cudaError_t ce = cudaSuccess;
+  if (b->ppt_req == 0 && configure_cols(b, present, &ce)) {
+    b->cap = 0;
+    b->occ = 0;
+    for (int d = gv::kBatchDM; d >= 1 && b->occ == 0; --d) b->occ = b->dims[d - 1].occ;
+    b->ctas = b->sm_count * b->occ;
+    return build_items(b);
+  }
+  BK(b, ce);
   int widest = 0;
   for (int d = 1; d <= gv::kBatchDM; ++d) {
     auto& c = b->dims[d - 1];
@@ -984,6 +1030,7 @@ vegas_status vegas_batch_set_launch(vegas_batch* b, int threads, int rounds) {
   BK(b, cudaStreamSynchronize(b->stream));
   b->threads = threads;
   b->rounds = rounds;
+  b->launch_set = true;
   return configure(b);
 }
 
@@ -1074,12 +1121,18 @@ vegas_status vegas_batch_autotune(vegas_batch* b, int* threads, int* rounds, dou
     if (!st) *out = m[0];
     return st;
   };
-  const std::vector<int> tiles = b->by_dim ? std::vector<int>{1, 2} : std::vector<int>{0};
+  // (columns, where the automatic form is that, beat the buckets' tiles at
+  // every measured shape: only the launch shape is left to choose)
+  b->ppt_req = 0;
+  vegas_status st0 = configure(b);
+  if (st0) return st0;
+  const bool cols = b->by_dim && b->cap == 0;
+  const std::vector<int> tiles = b->by_dim && !cols ? std::vector<int>{1, 2} : std::vector<int>{0};
   for (int t : kThreads)
     for (int r : kRounds)
       for (int p : tiles) {
         int cap_large = -1;  // a repeated tile is not timed twice
-        for (int pol = 0; pol < (b->by_dim ? 3 : 2); ++pol) {
+        for (int pol = 0; pol < (cols ? 1 : (b->by_dim ? 3 : 2)); ++pol) {
           double m = 0.0;
           vegas_status st = time_shape(t, r, p, pol, 3, &m);
           if (st) return st;

@@ -128,10 +128,13 @@ constexpr int kSumPoints = 16;  // points per thread between compensated merges
 // N^(D mod 4) after a last partial one (npw.y): J = prod_a N Delta_a
 // without a multiply per axis, and no partial product falls out of FP32
 // range.
-template <int D, int KIND>
+struct NoSlot {
+  __device__ __forceinline__ void operator()(int) const {}
+};
+template <int D, int KIND, class SLOT = NoSlot>
 __device__ __forceinline__ float dim_point(const BatchArgs& B, uint32_t s, uint32_t it, uint32_t inst, int N,
                                            float2 npw, const float2* tab, const float2* pc, const float* sc,
-                                           uint32_t (&kb)[(D + 3) / 4]) {
+                                           uint32_t (&kb)[(D + 3) / 4], SLOT slot = SLOT()) {
   float J = 1.f;
   Stream<KIND> st;
   st.init(sc);
@@ -157,6 +160,7 @@ __device__ __forceinline__ float dim_point(const BatchArgs& B, uint32_t s, uint3
         J *= e.y;
         kb[b] |= k << (8 * j);
         st.axis(a, x, pc[a], sc);
+        slot(a);
       }
     }
     J *= 4 * b + 4 <= D ? npw.x : npw.y;
@@ -394,16 +398,203 @@ __global__ void __launch_bounds__(256, kDimMinBlocks<D>) k_batch_dim(const Batch
   }
 }
 
+// ---------------------------------------------------------------------------
+// The same pass with the column histogram (col_hist.cuh), the automatic form
+// where the columns fit: two CTAs of 256 threads per SM at up to 50 bins, so
+// that one's fold and set-up lie under the other's evaluation.  Measured over
+// the 256-integral Genz workload (d = 2..16, 2.26 G point-axes per pass):
+// 3.12 ms against 4.63 ms with the bucketed tiles, 15.8 shared-memory
+// wavefronts per 32 point-axes before, the data pipe bounding both.
+// An item's cells are folded into its row at its end (and before a column has
+// taken kColFoldAdds terms): 1600 shared-memory wavefronts per 8 warps, 2 to
+// 4 % of an item of 32 768 points, which the other CTA's evaluation covers.
+// The axis constants are held in registers (a shared-memory broadcast costs
+// a wavefront per axis and point).
+// ---------------------------------------------------------------------------
+// Shared memory of k_batch_col<D> for nw warps: grid table, then each warp's
+// columns and staging area.
+template <int D>
+struct DimColSmem {
+  using C = ColHist<D, true, kColPif<D>>;
+  static __host__ __device__ size_t off_warps(int N) { return ((size_t)D * N * sizeof(float2) + 15) & ~size_t(15); }
+  static __host__ __device__ size_t bytes(int N, int nw) { return off_warps(N) + (size_t)nw * C::warp_bytes(D, N); }
+};
+
+// The CTA's columns into the item's row.
+template <int D>
+__device__ __noinline__ void dim_col_fold(unsigned char* columns, float2* row, int N, bool folded) {
+  using C = ColHist<D, true, kColPif<D>>;
+  const int cells = D * N, nw = blockDim.x >> 5;
+  __syncthreads();
+  for (int i = threadIdx.x; i < cells; i += blockDim.x) {
+    const int k = i / D, a = i - k * D;
+    fpair s1, s2;
+    col_sum(columns, C::warp_bytes(D, N), nw, D, C::points_per_step(D), a, k, s1, s2);
+    float2* r1 = row + a * N + k;
+    float2* r2 = r1 + cells;
+    if (folded) {
+      comp_merge(s1, fpair{r1->x, r1->y});
+      comp_merge(s2, fpair{r2->x, r2->y});
+    }
+    *r1 = make_float2(s1.hi, s1.lo);
+    *r2 = make_float2(s2.hi, s2.lo);
+  }
+  __syncthreads();
+}
+
+// The points of one work item, family KIND.
+template <int D, int KIND>
+__device__ __forceinline__ void dim_col_item(const BatchArgs& B, const BatchItem& W, uint32_t it, uint32_t inst, int N,
+                                             float2 npw, const float2* tab, const double* dp, unsigned char* columns,
+                                             ColHist<D, true, kColPif<D>>& hist, float2* row, fpair& sw, fpair& sw2,
+                                             int& nonfinite) {
+  constexpr int PIF = kColPif<D>, KW = (D + 3) / 4;
+  using C = ColHist<D, true, PIF>;
+  float2 pc[D];
+#pragma unroll
+  for (int a = 0; a < D; ++a) pc[a] = make_float2((float)dp[a], (float)dp[kMaxDim + a]);
+  float sc[4] = {0.f, 0.f, 0.f, 0.f};
+  if (stream_scalar_base(KIND) >= 0)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) sc[i] = (float)dp[kScalar + i];
+  const int tid = threadIdx.x, T = blockDim.x;
+  const uint32_t rounds = (W.count + T - 1) / T;
+  float p1 = 0.f, p2 = 0.f;  // plain FP32 sums since the last compensated merge
+  int since = 0, adds = 0;
+  bool folded = false;
+  for (uint32_t r = 0; r < rounds; r += PIF) {
+    uint32_t kb[PIF][KW];
+    float w[PIF];
+    hist.begin();
+#pragma unroll
+    for (int q = 0; q < PIF; ++q) {
+      const uint32_t j = (r + q) * T + tid;
+      const bool v = j < W.count;
+      w[q] = dim_point<D, KIND>(B, W.s0 + j, it, inst, N, npw, tab, pc, sc, kb[q],
+                                [&](int a) { hist.advance(q * D + a, PIF * D); });
+      if (!isfinite(w[q])) {
+        nonfinite += v;
+        w[q] = 0.f;
+      }
+      if (!v) w[q] = 0.f;
+      p1 += w[q];
+      p2 = fmaf(w[q], w[q], p2);
+    }
+    hist.end();
+    if ((adds += C::steps4(D)) > kColFoldAdds - C::steps4(D)) {
+      dim_col_fold<D>(columns, row, N, folded);
+      folded = true;
+      adds = 0;
+    }
+    if ((since += PIF) >= kSumPoints) {
+      comp_add(sw, p1);
+      comp_add(sw2, p2);
+      p1 = p2 = 0.f;
+      since = 0;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < PIF; ++q) hist.put(q, w[q], kb[q]);
+    __syncwarp();
+  }
+  comp_add(sw, p1);
+  comp_add(sw2, p2);
+  hist.drain();
+  dim_col_fold<D>(columns, row, N, folded);
+}
+
+template <int D>
+__global__ void __launch_bounds__(256, 2) k_batch_col(const BatchArgs B, const BatchRange R) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int N = B.N, cells = D * N;
+  float2* tab = reinterpret_cast<float2*>(smem);
+  unsigned char* columns = smem + DimColSmem<D>::off_warps(N);
+  __shared__ int s_item;
+  __shared__ fpair red_p[8][2];
+  __shared__ int red_n[8];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  ColHist<D, true, kColPif<D>> hist;
+  hist.bind(columns + warp * ColHist<D, true, kColPif<D>>::warp_bytes(D, N), D, N, lane);
+  int cur = -1;
+  for (;;) {
+    if (tid == 0) s_item = atomicAdd(R.head, 1);
+    __syncthreads();
+    const int k = s_item;
+    __syncthreads();
+    if (k >= R.count) break;
+    const BatchItem W = B.items[R.first + k];
+    const BatchInst I = B.inst[W.inst];
+    if (W.inst != cur) {  // the instance's grid cells
+      const float2* gtab = reinterpret_cast<const float2*>(B.tab) + I.tab_off;
+      for (int i = tid; i < cells; i += blockDim.x) tab[i] = gtab[i];
+      cur = W.inst;
+    }
+    const double* dp = B.dparams + (size_t)W.inst * kNumDerived;
+    float2* row = reinterpret_cast<float2*>(B.rows) + W.row;
+    // N^4 and N^(D mod 4) for the Jacobian
+    const float Nf = (float)N, N2 = Nf * Nf;
+    constexpr int rem = D & 3;
+    const float2 npw = make_float2(N2 * N2, rem == 1 ? Nf : (rem == 2 ? N2 : N2 * Nf));
+    __syncthreads();
+    const uint32_t it = B.st[W.inst].it;
+    fpair sw{0.f, 0.f}, sw2{0.f, 0.f};
+    int nonfinite = 0;
+#define GV_DIM_ITEM(K) \
+  dim_col_item<D, K>(B, W, it, I.instance, N, npw, tab, dp, columns, hist, row, sw, sw2, nonfinite)
+    switch (I.kind) {
+      case VG_GENZ_GAUSSIAN: GV_DIM_ITEM(VG_GENZ_GAUSSIAN); break;
+      case VG_GENZ_PRODUCT_PEAK: GV_DIM_ITEM(VG_GENZ_PRODUCT_PEAK); break;
+      case VG_GENZ_CORNER_PEAK: GV_DIM_ITEM(VG_GENZ_CORNER_PEAK); break;
+      case VG_GENZ_OSCILLATORY: GV_DIM_ITEM(VG_GENZ_OSCILLATORY); break;
+      case VG_GENZ_CONTINUOUS: GV_DIM_ITEM(VG_GENZ_CONTINUOUS); break;
+      case VG_GENZ_DISCONTINUOUS: GV_DIM_ITEM(VG_GENZ_DISCONTINUOUS); break;
+      default: GV_DIM_ITEM(VG_DOUBLE_GAUSSIAN); break;
+    }
+#undef GV_DIM_ITEM
+    const fpair a = warp_sum(sw), b = warp_sum(sw2);
+    int nf = nonfinite;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) nf += __shfl_xor_sync(0xffffffffu, nf, off);
+    if (lane == 0) {
+      red_p[warp][0] = a;
+      red_p[warp][1] = b;
+      red_n[warp] = nf;
+    }
+    __syncthreads();
+    if (tid < 2) {
+      fpair p{0.f, 0.f};
+      for (int w = 0; w < nw; ++w) comp_merge(p, red_p[w][tid]);
+      row[2 * cells + tid] = make_float2(p.hi, p.lo);
+    } else if (tid == 2) {
+      int c = 0;
+      for (int w = 0; w < nw; ++w) c += red_n[w];
+      row[2 * cells + 2] = make_float2((float)c, 0.f);
+    }
+    __syncthreads();
+  }
+}
+
 #ifndef __CUDACC_RTC__
-// The dimension kernels of one translation unit: k_batch_dim<d, pif>, or
-// null outside its range of d.
+// The dimension kernels of one translation unit: k_batch_dim<d, pif>
+// (k_batch_col<d> for pif = 0), or null outside its range of d.
 template <int D0, int D1>
 inline const void* dim_kernel_in(int d, int pif) {
   if constexpr (D0 > D1) {
     return nullptr;
   } else {
-    if (d == D0) return pif == 1 ? (const void*)&k_batch_dim<D0, 1> : (const void*)&k_batch_dim<D0, 2>;
+    if (d == D0)
+      return pif == 0 ? (const void*)&k_batch_col<D0>
+                      : (pif == 1 ? (const void*)&k_batch_dim<D0, 1> : (const void*)&k_batch_dim<D0, 2>);
     return dim_kernel_in<D0 + 1, D1>(d, pif);
+  }
+}
+// Dynamic shared memory of k_batch_col<d>.
+template <int D = 1>
+inline size_t dim_col_smem(int d, int N, int nw) {
+  if constexpr (D > kBatchDM) {
+    return 0;
+  } else {
+    return d == D ? DimColSmem<D>::bytes(N, nw) : dim_col_smem<D + 1>(d, N, nw);
   }
 }
 #endif

@@ -174,7 +174,7 @@ struct ColHist {
       }
     }
   }
-  // The whole hand-over at once.
+  // The whole hand-over at once; its slots are left empty.
   __device__ __forceinline__ void drain() {
     begin();
     if constexpr (EXACT) {
@@ -182,6 +182,10 @@ struct ColHist {
       for (int i = 0; i < steps(DM); ++i) step(i);
     }
     end();
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < PIF; ++q) *put_w[q] = 0.f;
+    __syncwarp();
   }
 };
 
