@@ -111,7 +111,7 @@ struct vegas_ctx {
   double* d_part_bins = nullptr;
   double* d_part_tot = nullptr;
   int part_rows = 0;
-  double* d_bins = nullptr;
+  double* d_bins = nullptr;    // behind the edges, in their allocation
   double* d_cubes = nullptr;
   void* d_cube_part = nullptr;   // sums of the hypercubes' parts (16 bytes each)
   size_t cube_part_len = 0;
@@ -569,6 +569,7 @@ gv::SampleArgs sample_args(const vegas_ctx* c, int it_override, bool nobins = fa
   gv::philox_key_schedule(A.key0, A.key1, A.ks);
   A.instance = c->cfg.instance;
   A.it_override = it_override;
+  A.force = it_override >= 0;
   A.ncall = (uint64_t)c->cfg.ncall;
   A.nc = (uint32_t)c->nc;
   A.ncubes = (uint32_t)c->ncubes;
@@ -622,6 +623,7 @@ gv::FinArgs fin_args(const vegas_ctx* c, int refine, int record, bool nobins = f
   F.tab64 = c->d_tab64;
   F.tab32 = c->d_tab32;
   F.st = c->d_st;
+  F.mirror = combine || !record ? c->h_st : nullptr;  // (a pass in the middle of a call: not read)
   return F;
 }
 
@@ -661,7 +663,7 @@ vegas_status get_graph(vegas_ctx* c, int shape, int n1, int n2, int refine, doub
   vegas_status st = VEGAS_OK;
   auto ctl = [&](int ops, double acc) {
     if (st) return;
-    cudaError_t e = gv_launch_control(c->d_st, ops, acc, 0u, c->stream);
+    cudaError_t e = gv_launch_control(c->d_st, ops, acc, 0u, c->h_st, c->stream);
     if (e != cudaSuccess) st = c->fail(VEGAS_ECUDA, "control: %s", cudaGetErrorString(e));
   };
   // n iterations on the grid as it stands.  Without an ACC target nothing is
@@ -705,8 +707,10 @@ vegas_status get_graph(vegas_ctx* c, int shape, int n1, int n2, int refine, doub
   return VEGAS_OK;
 }
 
+// The host's view of the state (c->h_st up to `hist`): pinned memory that the
+// kernels which change the state write themselves, so only the stream is
+// waited for.
 vegas_status read_state(vegas_ctx* c) {
-  CK(c, cudaMemcpyAsync(c->h_st, c->d_st, offsetof(GState, hist), cudaMemcpyDeviceToHost, c->stream));
   CK(c, cudaStreamSynchronize(c->stream));
   return VEGAS_OK;
 }
@@ -745,15 +749,23 @@ vegas_status upload_grid(vegas_ctx* c, const double* edges) {
   return VEGAS_OK;  // stream-ordered; the next host write to the stage synchronises first
 }
 
+// Integrand constants and output scale as a kernel argument: the values
+// travel with the launch, with no staging buffer to wait for.
+struct DerivedBlock {
+  double v[gv::kNumDerived + 1];  // the constants, then the output scale
+};
+
+__global__ void k_derived(const DerivedBlock b, double* dst) {
+  for (int i = threadIdx.x; i <= gv::kNumDerived; i += blockDim.x) dst[i] = b.v[i];
+}
+
 vegas_status upload_derived(vegas_ctx* c) {
-  vegas_status st = stage(c, gv::kNumDerived + 1);
-  if (st) return st;
-  CK(c, cudaStreamSynchronize(c->stream));
-  memcpy(c->h_stage, c->derived, sizeof c->derived);
-  c->h_stage[gv::kNumDerived] = c->scale;  // the output scale follows the constants
-  CK(c, cudaMemcpyAsync(c->d_derived, c->h_stage, sizeof c->derived + sizeof(double), cudaMemcpyHostToDevice,
-                        c->stream));
-  return VEGAS_OK;  // stream-ordered; the next host write to the stage synchronises first
+  DerivedBlock b;
+  memcpy(b.v, c->derived, sizeof c->derived);
+  b.v[gv::kNumDerived] = c->scale;
+  k_derived<<<1, 128, 0, c->stream>>>(b, c->d_derived);
+  CK(c, cudaGetLastError());
+  return VEGAS_OK;  // stream-ordered
 }
 
 bool valid_grid(const double* e, int d, int N) {
@@ -867,11 +879,12 @@ vegas_status finish_create(vegas_ctx* c, vegas_ctx** out) {
     return VEGAS_OK;
   };
   vegas_status st = VEGAS_OK;
-  if (!st) st = alloc((void**)&c->d_edges, sizeof(double) * d * (N + 1));
+  // edges and per-bin sums together: vegas_get_grid reads both in one copy
+  if (!st) st = alloc((void**)&c->d_edges, sizeof(double) * ((size_t)d * (N + 1) + 2 * (size_t)d * N));
   if (!st) st = alloc((void**)&c->d_tab64, sizeof(double2) * d * N);
   if (!st) st = alloc((void**)&c->d_tab32, sizeof(float2) * d * N);
   if (!st) st = alloc((void**)&c->d_derived, sizeof c->derived + sizeof(double));  // + the output scale
-  if (!st) st = alloc((void**)&c->d_bins, sizeof(double) * 2 * d * N);
+  if (!st) c->d_bins = c->d_edges + (size_t)d * (N + 1);
   if (!st && c->strat) st = alloc((void**)&c->d_cubes, sizeof(double) * 2 * G);
   if (!st) st = alloc((void**)&c->d_cube_max, sizeof(double) * G);
   if (!st) st = alloc((void**)&c->d_st, sizeof(GState));
@@ -923,7 +936,6 @@ void vegas_destroy(vegas_ctx* c) {
   cudaFree(c->d_derived);
   cudaFree(c->d_part_bins);
   cudaFree(c->d_part_tot);
-  cudaFree(c->d_bins);
   cudaFree(c->d_cubes);
   cudaFree(c->d_cube_part);
   cudaFree(c->d_cube_max);
@@ -1028,7 +1040,7 @@ vegas_status vegas_iterate(vegas_ctx* c, int n_iter, int refine, vegas_result* o
 
 vegas_status vegas_reset_results(vegas_ctx* c) {
   if (!c) return thread_fail(VEGAS_EINVAL, "ctx is NULL");
-  CK(c, gv_launch_control(c->d_st, gv::CTL_RESET_WINDOW | gv::CTL_SET_ACC, c->cfg.acc, 0u, c->stream));
+  CK(c, gv_launch_control(c->d_st, gv::CTL_RESET_WINDOW | gv::CTL_SET_ACC, c->cfg.acc, 0u, c->h_st, c->stream));
   c->hist_upper = 0;
   return VEGAS_OK;
 }
@@ -1036,8 +1048,7 @@ vegas_status vegas_reset_results(vegas_ctx* c) {
 vegas_status vegas_reset_grid(vegas_ctx* c) {
   if (!c) return thread_fail(VEGAS_EINVAL, "ctx is NULL");
   const int d = c->cfg.ndim, N = c->cfg.nbins;
-  CK(c, gv_launch_uniform_grid(c->d_edges, d, N, c->stream));
-  CK(c, gv_launch_tables(c->d_edges, d, N, c->d_tab64, c->d_tab32, c->stream));
+  CK(c, gv_launch_uniform_grid(c->d_edges, d, N, c->d_tab64, c->d_tab32, c->stream));
   return VEGAS_OK;
 }
 
@@ -1075,9 +1086,10 @@ vegas_status vegas_get_grid(vegas_ctx* c, double* edges, double* bin_sums) {
   const size_t ne = (size_t)d * (N + 1), nb = 2 * (size_t)d * N;
   vegas_status st = stage(c, ne + nb);
   if (st) return st;
-  if (edges) CK(c, cudaMemcpyAsync(c->h_stage, c->d_edges, ne * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  if (bin_sums)
-    CK(c, cudaMemcpyAsync(c->h_stage + ne, c->d_bins, nb * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+  const size_t from = edges ? 0 : ne, upto = bin_sums ? ne + nb : ne;  // (the sums lie behind the edges)
+  if (upto > from)
+    CK(c, cudaMemcpyAsync(c->h_stage + from, c->d_edges + from, (upto - from) * sizeof(double), cudaMemcpyDeviceToHost,
+                          c->stream));
   CK(c, cudaStreamSynchronize(c->stream));
   if (edges) memcpy(edges, c->h_stage, ne * sizeof(double));
   if (bin_sums) memcpy(bin_sums, c->h_stage + ne, nb * sizeof(double));
@@ -1093,17 +1105,18 @@ vegas_status vegas_set_grid(vegas_ctx* c, const double* edges) {
 
 vegas_status vegas_get_history(vegas_ctx* c, double* hist, int max_iters, int* n_out) {
   if (!c) return thread_fail(VEGAS_EINVAL, "ctx is NULL");
-  vegas_status st = read_state(c);
-  if (st) return st;
-  const int n = std::min(c->h_st->nhist, std::max(max_iters, 0));
-  if (n_out) *n_out = c->h_st->nhist;
-  if (n > 0 && hist) {
-    if ((st = stage(c, 2 * (size_t)n))) return st;
-    CK(c, cudaMemcpyAsync(c->h_stage, &c->d_st->hist[0][0], 2 * n * sizeof(double), cudaMemcpyDeviceToHost,
+  // up to the longest window the calls so far can have left, in one go
+  const int most = hist ? std::min(c->hist_upper, std::max(max_iters, 0)) : 0;
+  vegas_status st = VEGAS_OK;
+  if (most > 0) {
+    if ((st = stage(c, 2 * (size_t)most))) return st;
+    CK(c, cudaMemcpyAsync(c->h_stage, &c->d_st->hist[0][0], 2 * most * sizeof(double), cudaMemcpyDeviceToHost,
                           c->stream));
-    CK(c, cudaStreamSynchronize(c->stream));
-    memcpy(hist, c->h_stage, 2 * n * sizeof(double));
   }
+  if ((st = read_state(c))) return st;
+  const int n = std::min(c->h_st->nhist, most);
+  if (n_out) *n_out = c->h_st->nhist;
+  if (n > 0) memcpy(hist, c->h_stage, 2 * (size_t)n * sizeof(double));
   return VEGAS_OK;
 }
 
@@ -1298,7 +1311,7 @@ vegas_status vegas_get_iteration(vegas_ctx* c, uint32_t* it) {
 
 vegas_status vegas_set_iteration(vegas_ctx* c, uint32_t it) {
   if (!c) return thread_fail(VEGAS_EINVAL, "ctx is NULL");
-  CK(c, gv_launch_control(c->d_st, gv::CTL_SET_ITER, 0.0, it, c->stream));
+  CK(c, gv_launch_control(c->d_st, gv::CTL_SET_ITER, 0.0, it, c->h_st, c->stream));
   return VEGAS_OK;
 }
 
@@ -1324,8 +1337,6 @@ vegas_status vegas_set_params(vegas_ctx* c, const double* params, int nparams) {
 vegas_status vegas_eval(vegas_ctx* c, uint32_t it, double* I, double* var) {
   if (!c) return thread_fail(VEGAS_EINVAL, "ctx is NULL");
   if (it > 0x7FFFFFFFu) return c->fail(VEGAS_EINVAL, "iteration index must be < 2^31");
-  int zero = 0;
-  CK(c, cudaMemcpyAsync(&c->d_st->done, &zero, sizeof(int), cudaMemcpyHostToDevice, c->stream));
   vegas_status st = launch_pass(c, (int)it, 0, 0);
   if (st) return st;
   if ((st = read_state(c))) return st;
@@ -1558,8 +1569,6 @@ vegas_status profile_passes(vegas_ctx* c, int n_pass, bool nobins, double* ms) {
   vegas_status st = read_state(c);
   if (st) return st;
   const uint32_t it = c->h_st->it;
-  int zero = 0;
-  CK(c, cudaMemcpyAsync(&c->d_st->done, &zero, sizeof(int), cudaMemcpyHostToDevice, c->stream));
   cudaEvent_t ev[3];
   for (int i = 0; i < 3; ++i) CK(c, cudaEventCreate(&ev[i]));
   double acc[3] = {0, 0, 0};
@@ -1628,20 +1637,19 @@ std::mutex g_noalloc_mutex;
 unsigned char* g_noalloc_ptr[kNoAllocMaxDevices] = {};
 int g_noalloc_sms[kNoAllocMaxDevices] = {};
 
-struct DerivedBlock {
-  double v[gv::kNumDerived + 1];  // the constants, then the output scale
-};
-
-__global__ void k_noalloc_params(DerivedBlock b, double* dst) {
-  for (int i = threadIdx.x; i <= gv::kNumDerived; i += blockDim.x) dst[i] = b.v[i];
-}
-
-__global__ void k_noalloc_result(const GState* st, double* out) {
-  out[0] = st->last_I;
-  out[1] = st->last_var;
-  out[2] = st->last_sw;
-  out[3] = st->last_sw2;
-  out[4] = (double)st->last_nonfinite;
+// Set-up in one launch: the state (it must start cleared; its stop flag gates
+// the kernels), the integrand constants and the grid's tables.
+__global__ void k_noalloc_setup(const DerivedBlock b, double* derived, GState* st, const double* edges, int d, int N,
+                                double2* tab64, float2* tab32) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i <= gv::kNumDerived) derived[i] = b.v[i];
+  const int words = (int)(offsetof(GState, hist) / sizeof(int));
+  if (i < words) reinterpret_cast<int*>(st)[i] = 0;
+  if (i >= d * N) return;
+  const int a = i / N, k = i - a * N;
+  const double lo = edges[(size_t)a * (N + 1) + k], w = edges[(size_t)a * (N + 1) + k + 1] - lo;
+  tab64[i] = make_double2(lo, w);
+  tab32[i] = make_float2((float)lo, (float)w);
 }
 
 size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
@@ -1772,17 +1780,12 @@ extern "C" vegas_status vegas_eval_noalloc(const vegas_config* cfg, const vegas_
   GState* st = reinterpret_cast<GState*>(scratch + off_st);
 
   cudaStream_t s = (cudaStream_t)cfg->stream;
-  // Contents left by the previous call: the pass state must start cleared
-  // (its stop flag gates the kernels); tables, partial rows and totals are
-  // overwritten in full below.
-  e = cudaMemsetAsync(st, 0, offsetof(GState, hist), s);
-  if (e == cudaSuccess) {
-    k_noalloc_params<<<1, 128, 0, s>>>(db, reinterpret_cast<double*>(scratch + off_dp));
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess)
-    e = gv_launch_tables(edges, d, N, reinterpret_cast<double2*>(scratch + off_t64),
-                         reinterpret_cast<float2*>(scratch + off_t32), s);
+  // Contents left by the previous call: the pass state must start cleared;
+  // tables, partial rows and totals are overwritten in full.
+  k_noalloc_setup<<<(std::max(dN, 256) + 255) / 256, 256, 0, s>>>(
+      db, reinterpret_cast<double*>(scratch + off_dp), st, edges, d, N, reinterpret_cast<double2*>(scratch + off_t64),
+      reinterpret_cast<float2*>(scratch + off_t32));
+  e = cudaGetLastError();
   if (e != cudaSuccess) return thread_fail(VEGAS_ECUDA, "no-allocation set-up: %s", cudaGetErrorString(e));
 
   gv::SampleArgs A{};
@@ -1844,11 +1847,8 @@ extern "C" vegas_status vegas_eval_noalloc(const vegas_config* cfg, const vegas_
   F.tab64 = reinterpret_cast<double2*>(scratch + off_t64);
   F.tab32 = reinterpret_cast<float2*>(scratch + off_t32);
   F.st = st;
+  F.result = out + 2 * (size_t)dN;
   if (e == cudaSuccess) e = gv_launch_finish(&F, s);
-  if (e == cudaSuccess) {
-    k_noalloc_result<<<1, 1, 0, s>>>(st, out + 2 * (size_t)dN);
-    e = cudaGetLastError();
-  }
   if (e != cudaSuccess) return thread_fail(VEGAS_ECUDA, "no-allocation pass: %s", cudaGetErrorString(e));
   return VEGAS_OK;
 }

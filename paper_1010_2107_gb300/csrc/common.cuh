@@ -216,6 +216,17 @@ struct GState {
   double hist[kMaxHist][2];
 };
 
+// The state's fields up to the history into its host-visible copy, by one
+// warp (after its writes): the host reads them once the stream has got here,
+// without a copy of its own.
+__device__ __forceinline__ void mirror_state(GState* mirror, const GState* st) {
+  __syncwarp();
+  const int n = (int)((sizeof(GState) - sizeof(st->hist)) / sizeof(int));
+  const int* src = reinterpret_cast<const int*>(st);
+  int* dst = reinterpret_cast<int*>(mirror);
+  for (int i = threadIdx.x & 31; i < n; i += 32) dst[i] = src[i];
+}
+
 // Threads per block of k_finish.
 constexpr int kFinishThreads = 256;
 
@@ -284,6 +295,7 @@ struct SampleArgs {
   uint32_t key0, key1, instance;
   uint32_t ks[kPhiloxKeyWords];  // Philox round keys of (key0, key1)
   int it_override;         // >= 0: use this iteration index
+  int force;               // 1: run even if the ACC test has stopped the last call (evaluation passes)
   uint64_t ncall;
   uint32_t nc;             // points per hypercube
   uint32_t ncubes;         // number of hypercubes
@@ -328,6 +340,8 @@ struct FinArgs {
   double2* tab64;          // [d][N]
   float2* tab32;           // [d][N]
   GState* st;
+  GState* mirror;          // host-visible copy of the state up to `hist`, or null
+  double* result;          // (I, variance, sum w, sum w^2, non-finite count), or null
 };
 
 }  // namespace gv

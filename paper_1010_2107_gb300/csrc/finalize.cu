@@ -210,7 +210,17 @@ __device__ void record_iteration(const FinArgs& F, const double* t, bool combine
     st->last_sw2 = t[TOT_SW2];
     st->last_nonfinite = (long long)t[TOT_NONFINITE];
   }
-  if (!F.record) return;
+  if (F.result && lane == 0) {
+    F.result[0] = I;
+    F.result[1] = var;
+    F.result[2] = t[TOT_SW];
+    F.result[3] = t[TOT_SW2];
+    F.result[4] = t[TOT_NONFINITE];
+  }
+  if (!F.record) {
+    if (F.mirror) mirror_state(F.mirror, st);
+    return;
+  }
   int h = st->nhist;
   if (h < kMaxHist) {
     if (lane == 0) {
@@ -240,6 +250,7 @@ __device__ void record_iteration(const FinArgs& F, const double* t, bool combine
       st->stopped = 1;
     }
   }
+  if (F.mirror) mirror_state(F.mirror, st);
 }
 
 // Steps 4-6 after a sampling pass in one launch.  Cluster a < d reduces the
@@ -317,9 +328,9 @@ __global__ void __launch_bounds__(256) k_colsum(const double* part, int ncols, i
   if (lane == 0) out[col] = acc;
 }
 
-// Window / stop-flag bookkeeping between passes (one thread); CTL_SET_ITER
-// sets the Philox iteration counter.
-__global__ void k_control(GState* st, int ops, double acc, uint32_t it) {
+// Window / stop-flag bookkeeping between passes (one warp; its first lane);
+// CTL_SET_ITER sets the Philox iteration counter.
+__device__ __forceinline__ void control(GState* st, int ops, double acc, uint32_t it) {
   if (ops & CTL_SET_ITER) st->it = it;
   if (ops & CTL_SNAPSHOT) {
     st->ph1_I = st->I;
@@ -343,11 +354,23 @@ __global__ void k_control(GState* st, int ops, double acc, uint32_t it) {
   }
 }
 
-// Uniform grid e_a[k] = k / N (step 1).
-__global__ void k_uniform_grid(double* edges, int d, int N) {
+__global__ void k_control(GState* st, int ops, double acc, uint32_t it, GState* mirror) {
+  if (threadIdx.x == 0) control(st, ops, acc, it);
+  mirror_state(mirror, st);
+}
+
+// Uniform grid e_a[k] = k / N (step 1) and its tables.
+__global__ void k_uniform_grid(double* edges, int d, int N, double2* tab64, float2* tab32) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= d * (N + 1)) return;
-  edges[i] = (double)(i % (N + 1)) / (double)N;
+  const int a = i / (N + 1), k = i - a * (N + 1);
+  const double lo = (double)k / (double)N;
+  edges[i] = lo;
+  if (k < N) {
+    const double w = (double)(k + 1) / (double)N - lo;
+    tab64[a * N + k] = make_double2(lo, w);
+    tab32[a * N + k] = make_float2((float)lo, (float)w);
+  }
 }
 
 // Pure table rebuild (after vegas_set_grid): tab64 / tab32 from edges.
@@ -408,14 +431,14 @@ cudaError_t gv_launch_colsum(const double* part, int ncols, int nrows, double* o
   return cudaGetLastError();
 }
 
-cudaError_t gv_launch_control(gv::GState* st, int ops, double acc, uint32_t it, cudaStream_t s) {
-  gv::k_control<<<1, 1, 0, s>>>(st, ops, acc, it);
+cudaError_t gv_launch_control(gv::GState* st, int ops, double acc, uint32_t it, gv::GState* mirror, cudaStream_t s) {
+  gv::k_control<<<1, 32, 0, s>>>(st, ops, acc, it, mirror);
   return cudaGetLastError();
 }
 
-cudaError_t gv_launch_uniform_grid(double* edges, int d, int N, cudaStream_t s) {
+cudaError_t gv_launch_uniform_grid(double* edges, int d, int N, double2* t64, float2* t32, cudaStream_t s) {
   const int n = d * (N + 1);
-  gv::k_uniform_grid<<<(n + 255) / 256, 256, 0, s>>>(edges, d, N);
+  gv::k_uniform_grid<<<(n + 255) / 256, 256, 0, s>>>(edges, d, N, t64, t32);
   return cudaGetLastError();
 }
 

@@ -412,16 +412,22 @@ __device__ __forceinline__ void store_totals(const SampleArgs& A, const fpair (&
 template <bool SPEC>
 constexpr int kSampleMaxThreads = SPEC ? 512 : 256;
 constexpr int kMaxSampleWarps = 16;
+// CTAs of the largest size that must fit an SM (0: the compiler's choice): 64
+// registers for the specialised kernels of low dimension (four CTAs of 256
+// threads in the frozen-grid passes, 78 registers and three without it), 80
+// for the general FP32 ones (106 and two CTAs without it).
+template <typename T, int DM, bool SPEC>
+constexpr int kSampleMinBlocks = DM > 8 || !std::is_same<T, float>::value ? 0 : (SPEC ? 2 : 3);
 
 template <typename T, int DM, template <typename, int> class F, int ACC, int YB, bool SPEC>
-__global__ void __launch_bounds__(kSampleMaxThreads<SPEC>) k_sample(const SampleArgs A) {
+__global__ void __launch_bounds__(kSampleMaxThreads<SPEC>, kSampleMinBlocks<T, DM, SPEC>) k_sample(const SampleArgs A) {
   using H = typename AccTraits<ACC>::H;
   using T2 = typename Vec2<T>::type;
   using L = SmemLayout<T, ACC>;
   constexpr bool COMP = ACC == 2;  // FP32 throughout, no FP64 in the loop
   // the ACC test stopped this call (device-side): no pass, and k_finish
   // then skips it too (it reads `live`, nothing else here writes it)
-  const int stop = A.st->done;
+  const int stop = A.force ? 0 : A.st->done;
   if (blockIdx.x == 0 && threadIdx.x == 0) A.st->live = !stop;
   if (stop) return;
   uint32_t it = A.it_override >= 0 ? (uint32_t)A.it_override : A.st->it;
@@ -819,7 +825,7 @@ __global__ void __launch_bounds__(512, 1) k_sample_col(const SampleArgs A) {
   constexpr int KW = (DM + 3) / 4;
   using C = ColHist<DM, EXACT, PIF>;
   using L = ColSmem<DM, EXACT>;
-  const int stop = A.st->done;
+  const int stop = A.force ? 0 : A.st->done;
   if (blockIdx.x == 0 && threadIdx.x == 0) A.st->live = !stop;
   if (stop) return;
   const uint32_t it = A.it_override >= 0 ? (uint32_t)A.it_override : A.st->it;
@@ -1010,7 +1016,7 @@ constexpr uint32_t kSpringIt = 0xFFFFFFFFu;
 // cube search waits on L2, so residency counts (d = 8: 54 registers and four
 // CTAs took 452 us per 2^22 trials with their events, 48 and five 442 us).
 template <typename T, int DM, bool SPEC>
-constexpr int kSpringMinBlocks = SPEC && std::is_same<T, float>::value && DM <= 8 ? 5 : 1;
+constexpr int kSpringMinBlocks = !SPEC || !std::is_same<T, float>::value || DM > 8 ? 0 : (DM <= 4 ? 6 : 5);
 
 template <typename T, int DM, template <typename, int> class F, int YB, bool SPEC>
 __global__ void __launch_bounds__(256, kSpringMinBlocks<T, DM, SPEC>) k_spring(const SpringArgs R) {
