@@ -450,7 +450,7 @@ bool shape_col(const void* fn, const gv::KernelEntry& ke, int d, int N, int sm_c
 }
 
 vegas_status configure_launch(vegas_ctx* c) {
-  const int threads = c->threads_req > 0 ? c->threads_req : 256;
+  int threads = c->threads_req > 0 ? c->threads_req : 256;
   const int d = c->cfg.ndim, N = c->cfg.nbins;
   gv::PassShape &pb = c->pass_bins, &pn = c->pass_nobins;
   const bool strat = c->strat != 0;
@@ -480,7 +480,24 @@ vegas_status configure_launch(vegas_ctx* c) {
     int occ_cap = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_cap, c->ke.sample, threads, 0);
     if (e != cudaSuccess) return c->fail(VEGAS_ECUDA, "launch configuration: %s", cudaGetErrorString(e));
-    const gv::TileShape t = gv::choose_tile(threads, N, c->ppt_req, c->ppt_min, occ_cap, occ_of, c->small_cap);
+    gv::TileShape t = gv::choose_tile(threads, N, c->ppt_req, c->ppt_min, occ_cap, occ_of, c->small_cap);
+    // Few points: the same number of rounds with CTAs just wide enough, so
+    // that every SM runs the same number of warps (10^5 points over 456 CTAs:
+    // 224 threads, 21 warps per SM, instead of 391 CTAs of 256, up to 24)
+    if (e == cudaSuccess && c->threads_req == 0 && !strat && t.occ > 0) {
+      const uint64_t n = (uint64_t)c->cfg.ncall, most = (uint64_t)c->sm_count * t.occ;
+      const uint64_t rounds = (n + most * threads - 1) / (most * threads);
+      const int w = (int)(((n + most * rounds - 1) / (most * rounds) + 31) / 32 * 32);
+      if (w >= 64 && w < threads) {
+        const int wide = threads;
+        threads = w;
+        const gv::TileShape u = gv::choose_tile(threads, N, c->ppt_req, c->ppt_min, occ_cap, occ_of, c->small_cap);
+        if (u.occ >= t.occ)
+          t = u;
+        else
+          threads = wide;
+      }
+    }
     if (e != cudaSuccess) return c->fail(VEGAS_ECUDA, "launch configuration: %s", cudaGetErrorString(e));
     if (t.occ < 1) return c->fail(VEGAS_EINVAL, "sampling kernel does not fit: %d threads, %d points per thread",
                                   threads, t.ppt);
@@ -502,6 +519,7 @@ vegas_status configure_launch(vegas_ctx* c) {
       pb.parts = cl.parts;
     }
     pb.ctas = ctas_for(pb, threads, most);
+    threads = c->threads_req > 0 ? c->threads_req : 256;
   }
   // passes without the per-bin histogram (no refinement) need only the
   // grid table and constants in shared memory: more CTAs may be resident

@@ -52,7 +52,7 @@ __device__ __forceinline__ T batch_eval(int kind, const T (&x)[DM], int d, const
 template <typename T, int ACC, int YB, int DMC>
 __device__ __forceinline__ void batch_item_points(const BatchArgs& B, const SampleArgs& A, const BatchItem& W,
                                                   int kind, uint32_t it, int d,
-                                                  const typename Vec2<T>::type* tab, const T* P,
+                                                  const typename Vec2<T>::type* tab, const T* ntab, const T* P,
                                                   TileHist<ACC>& hist, Run<ACC>& sw, Run<ACC>& sw2,
                                                   int& nonfinite) {
   using H = typename AccTraits<ACC>::H;
@@ -66,7 +66,7 @@ __device__ __forceinline__ void batch_item_points(const BatchArgs& B, const Samp
     if (j < W.count) {
       T x[DMC];
       int kb[DMC];
-      const T J = make_point<T, DMC, YB>(A, it, W.s0 + j, cd, tab, x, kb, nullptr);
+      const T J = make_point<T, DMC, YB>(A, it, W.s0 + j, cd, tab, x, kb, nullptr, ntab);
       T w = batch_eval<T, DMC>(kind, x, d, P) * J;
       if (!vfinite(w)) {
         ++nonfinite;
@@ -83,8 +83,11 @@ __device__ __forceinline__ void batch_item_points(const BatchArgs& B, const Samp
 
 template <typename T, int ACC>
 struct BatchSmem {
+  // (the products N Delta_k, as k_sample)
+  static __host__ __device__ bool has_prod(int md, int N) { return std::is_same<T, double>::value && md * N <= kMaxProdCells; }
   static __host__ __device__ size_t a16(size_t b) { return (b + 15) & ~size_t(15); }
-  static __host__ __device__ size_t params(int md, int N) { return (size_t)md * N * sizeof(typename Vec2<T>::type); }
+  static __host__ __device__ size_t prod(int md, int N) { return (size_t)md * N * sizeof(typename Vec2<T>::type); }
+  static __host__ __device__ size_t params(int md, int N) { return prod(md, N) + (has_prod(md, N) ? (size_t)md * N * sizeof(T) : 0); }
   static __host__ __device__ size_t hist(int md, int N) { return a16(params(md, N) + kNumDerived * sizeof(T)); }
   static __host__ __device__ size_t total(int md, int N, int cap) {
     return hist(md, N) + TileHist<ACC>::bytes(md * N, cap);
@@ -101,6 +104,7 @@ __global__ void __launch_bounds__(256) k_batch_sample(const BatchArgs B) {
   extern __shared__ __align__(16) unsigned char smem[];
   T2* tab = reinterpret_cast<T2*>(smem);
   T* P = reinterpret_cast<T*>(smem + L::params(B.maxd, B.N));
+  T* ntab = L::has_prod(B.maxd, B.N) ? reinterpret_cast<T*>(smem + L::prod(B.maxd, B.N)) : nullptr;
   __shared__ int s_item;
   __shared__ double red_d[8][3];
   __shared__ fpair red_p[8][2];
@@ -139,7 +143,10 @@ __global__ void __launch_bounds__(256) k_batch_sample(const BatchArgs B) {
     const int d = I.d, dN = d * N;
     if (W.inst != cur) {  // stage the instance's grid cells and constants
       const T2* gtab = reinterpret_cast<const T2*>(B.tab) + I.tab_off;
-      for (int i = tid; i < dN; i += blockDim.x) tab[i] = gtab[i];
+      for (int i = tid; i < dN; i += blockDim.x) {
+        tab[i] = gtab[i];
+        if (ntab) ntab[i] = T(N) * gtab[i].y;
+      }
       const double* dp = B.dparams + (size_t)W.inst * kNumDerived;
       for (int i = tid; i < kNumDerived; i += blockDim.x) P[i] = (T)dp[i];
       cur = W.inst;
@@ -152,7 +159,7 @@ __global__ void __launch_bounds__(256) k_batch_sample(const BatchArgs B) {
     const uint32_t it = B.st[W.inst].it;
     Run<ACC> sw, sw2;
     int nonfinite = 0;
-    batch_item_points<T, ACC, YB, DM>(B, A, W, I.kind, it, d, tab, P, hist, sw, sw2, nonfinite);
+    batch_item_points<T, ACC, YB, DM>(B, A, W, I.kind, it, d, tab, ntab, P, hist, sw, sw2, nonfinite);
     // the item's partial row: cells, then sum w, sum w^2, non-finite count
     for (int i = tid; i < 2 * dN; i += blockDim.x) {
       if constexpr (COMP) {

@@ -13,7 +13,7 @@ namespace gv {
 // exp of a non-positive Gaussian exponent: the special-function unit for
 // FP32 (relative error ~2^-21 over the range that matters), libm for FP64.
 __device__ __forceinline__ float gexp(float x) { return __expf(x); }
-__device__ __forceinline__ double gexp(double x) { return exp(x); }
+__device__ __forceinline__ double gexp(double x) { return exp64(x); }
 
 // t^e for t > 0: FP32 as exp(e ln t) on the quick forms, FP64 the library.
 __device__ __forceinline__ float qpow_pos(float t, float e) { return __expf(e * __logf(t)); }

@@ -77,7 +77,7 @@ __device__ __forceinline__ void bin_frac(const SampleArgs& A, uint64_t m, int c,
     if (F32)
       fr = T(frac23(r >> A.g_log2));
     else
-      fr = T((double)r * A.inv_gb_d);
+      fr = T(scaled_u64(r, sh));
     return;
   }
   if (YB == 24 && A.t32) {
@@ -87,10 +87,8 @@ __device__ __forceinline__ void bin_frac(const SampleArgs& A, uint64_t m, int c,
       const int sh = 24 + A.g_log2;
       k = (int)(t >> sh);
       r = t & ((1u << sh) - 1u);
-      if (F32) {
-        fr = T(frac23(r >> A.g_log2));
-        return;
-      }
+      fr = F32 ? T(frac23(r >> A.g_log2)) : T(scaled_u64(r, sh));
+      return;
     } else {
       k = (int)((t >> 24) / (uint32_t)A.g);
       r = t - (uint32_t)k * ((uint32_t)A.g << 24);
@@ -98,7 +96,7 @@ __device__ __forceinline__ void bin_frac(const SampleArgs& A, uint64_t m, int c,
     if (F32)
       fr = T((float)r * A.inv_gb_f);
     else
-      fr = T((double)r * A.inv_gb_d);
+      fr = T(scaled_u64(r, 0) * A.inv_gb_d);
     return;
   }
   const uint64_t t = (((uint64_t)c << YB) | m) * (uint64_t)N;
@@ -111,6 +109,8 @@ __device__ __forceinline__ void bin_frac(const SampleArgs& A, uint64_t m, int c,
       fr = T(frac23((uint32_t)(r >> (sh - 24))));
       return;
     }
+    fr = T(scaled_u64(r, sh));
+    return;
   } else {
     k = (int)((uint32_t)(t >> YB) / (uint32_t)A.g);
     r = t - (((uint64_t)k * (uint64_t)A.g) << YB);
@@ -118,16 +118,19 @@ __device__ __forceinline__ void bin_frac(const SampleArgs& A, uint64_t m, int c,
   if (F32)
     fr = T((float)r * A.inv_gb_f);
   else
-    fr = T((double)r * A.inv_gb_d);
+    fr = T(scaled_u64(r, 0) * A.inv_gb_d);
 }
 
 // Point generation for one sample: bins kb[a], point x[a] and the Jacobian.
-// `cd` holds the hypercube digits c_a (zero without stratification).
+// `cd` holds the hypercube digits c_a (zero without stratification); ntab,
+// where given, the products N Delta_k (the FP64 kernels: one operation of the
+// FP64 pipe less per axis, the same bits).
 template <typename T, int DM, int YB, bool SPEC = false>
 __device__ __forceinline__ T make_point(const SampleArgs& A, uint32_t it, uint32_t s,
                                         const int (&cd)[DM],
                                         const typename Vec2<T>::type* tab,
-                                        T (&x)[DM], int (&kb)[DM], uint32_t* words_out) {
+                                        T (&x)[DM], int (&kb)[DM], uint32_t* words_out,
+                                        const T* ntab = nullptr) {
   const int d = SPEC ? DM : A.d, N = A.N;
   const T Nf = T(N);
   T J = T(1);
@@ -171,7 +174,7 @@ __device__ __forceinline__ T make_point(const SampleArgs& A, uint32_t it, uint32
       bin_frac<T, YB, SPEC>(A, m, cd[a], k, fr);
       const typename Vec2<T>::type e = tab[a * N + k];
       x[a] = vfma(fr, e.y, e.x);
-      J *= Nf * e.y;
+      J *= ntab ? ntab[a * N + k] : Nf * e.y;
       kb[a] = k;
     }
   }
@@ -324,8 +327,11 @@ struct TileHist {
             a2 = __ffma2_rn(lo, lo, a2);
             a2 = __ffma2_rn(hi, hi, a2);
           } else {
-            s1 += v[u].x + v[u].y;
-            s2 += v[u].x * v[u].x + v[u].y * v[u].y;
+            // (FP64: four operations per two slots)
+            s1 += v[u].x;
+            s1 += v[u].y;
+            s2 = fma(v[u].x, v[u].x, s2);
+            s2 = fma(v[u].y, v[u].y, s2);
           }
         }
       }
@@ -355,12 +361,20 @@ struct TileHist {
   __device__ __forceinline__ double value(int i) const { return (double)cta[i]; }
 };
 
+// Largest table with a column of products N Delta_k (16 KB; with the smallest
+// buckets such a shape takes 172 KB without it).
+constexpr int kMaxProdCells = 2048;
+
 // Shared memory layout of k_sample (byte offsets): grid table, integrand
 // constants, then the tile histogram.
 template <typename T, int ACC>
 struct SmemLayout {
   static __host__ __device__ size_t a16(size_t b) { return (b + 15) & ~size_t(15); }
-  static __host__ __device__ size_t params(int dN) { return (size_t)dN * sizeof(typename Vec2<T>::type); }
+  // FP64: the products N Delta_k behind the table, up to a size that leaves
+  // every shape room which fits without them
+  static __host__ __device__ bool has_prod(int dN) { return std::is_same<T, double>::value && dN <= kMaxProdCells; }
+  static __host__ __device__ size_t prod(int dN) { return (size_t)dN * sizeof(typename Vec2<T>::type); }
+  static __host__ __device__ size_t params(int dN) { return prod(dN) + (has_prod(dN) ? (size_t)dN * sizeof(T) : 0); }
   static __host__ __device__ size_t hist(int dN) { return a16(params(dN) + kNumDerived * sizeof(T)); }
   static __host__ __device__ size_t total(int dN, int cap) { return hist(dN) + TileHist<ACC>::bytes(dN, cap); }
 };
@@ -415,9 +429,10 @@ constexpr int kMaxSampleWarps = 16;
 // CTAs of the largest size that must fit an SM (0: the compiler's choice): 64
 // registers for the specialised kernels of low dimension (four CTAs of 256
 // threads in the frozen-grid passes, 78 registers and three without it), 80
-// for the general FP32 ones (106 and two CTAs without it).
+// for the general FP32 ones (106 and two CTAs without it; up to 16 axes 128).
 template <typename T, int DM, bool SPEC>
-constexpr int kSampleMinBlocks = DM > 8 || !std::is_same<T, float>::value ? 0 : (SPEC ? 2 : 3);
+constexpr int kSampleMinBlocks =
+    DM > 16 || !std::is_same<T, float>::value ? 0 : (DM > 8 ? (SPEC ? 0 : 2) : (SPEC ? 2 : 3));
 
 template <typename T, int DM, template <typename, int> class F, int ACC, int YB, bool SPEC>
 __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>, kSampleMinBlocks<T, DM, SPEC>) k_sample(const SampleArgs A) {
@@ -444,7 +459,11 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>, kSampleMinBlocks<T, D
 
   // Coalesced, vectorised grid-table load (one 8- or 16-byte cell per bin).
   const T2* gtab = reinterpret_cast<const T2*>(A.tab);
-  for (int i = tid; i < dN; i += blockDim.x) tab[i] = gtab[i];
+  T* ntab = L::has_prod(dN) ? reinterpret_cast<T*>(smem + L::prod(dN)) : nullptr;
+  for (int i = tid; i < dN; i += blockDim.x) {
+    tab[i] = gtab[i];
+    if (ntab) ntab[i] = T(N) * gtab[i].y;
+  }
   for (int i = tid; i < kNumDerived; i += blockDim.x) P[i] = (T)A.dparams[i];
   // Per-bin sums feed only the grid refinement (step 5); a pass that does
   // not refine (the integration phase of BASES, a frozen-grid VEGAS call)
@@ -465,7 +484,7 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>, kSampleMinBlocks<T, D
   // (squares are then formed in H: FP64 unless ACC == 2).
   auto eval_point = [&](uint32_t s, int (&kb)[DM], bool valid = true) -> H {
     T x[DM];
-    const T J = make_point<T, DM, YB, SPEC>(A, it, s, cd, tab, x, kb, nullptr);
+    const T J = make_point<T, DM, YB, SPEC>(A, it, s, cd, tab, x, kb, nullptr, ntab);
     const T f = F<T, DM>::eval(x, d, P);
     T w = f * J;
     if (!vfinite(w)) {
@@ -518,13 +537,13 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>, kSampleMinBlocks<T, D
           if (v0) {
             sw.add(w0);
             sw2.add(w0 * w0);
-            pmax = max(pmax, w0);
+            if (A.cube_max) pmax = max(pmax, w0);
             scatter(kb0, w0);
           }
           if (v1) {
             sw.add(w1);
             sw2.add(w1 * w1);
-            pmax = max(pmax, w1);
+            if (A.cube_max) pmax = max(pmax, w1);
             scatter(kb1, w1);
           }
           if ((pend += 2) >= A.ppt) {
@@ -539,7 +558,7 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>, kSampleMinBlocks<T, D
             const H w = eval_point((uint32_t)s, kb);
             sw.add(w);
             sw2.add(w * w);
-            pmax = max(pmax, w);
+            if (A.cube_max) pmax = max(pmax, w);
             scatter(kb, w);
           }
           if (++pend == A.ppt) {
@@ -613,13 +632,13 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>, kSampleMinBlocks<T, D
             if (v0) {
               p1 += w0;
               p2 += w0 * w0;
-              pmax = max(pmax, w0);
+              if (A.cube_max) pmax = max(pmax, w0);
               scatter(kb0, w0);
             }
             if (v1) {
               p1 += w1;
               p2 += w1 * w1;
-              pmax = max(pmax, w1);
+              if (A.cube_max) pmax = max(pmax, w1);
               scatter(kb1, w1);
             }
             if ((pend += 2) >= A.ppt) {
@@ -635,7 +654,7 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>, kSampleMinBlocks<T, D
               const H w = eval_point(s0 + j, kb);
               p1 += w;
               p2 += w * w;
-              pmax = max(pmax, w);
+              if (A.cube_max) pmax = max(pmax, w);
               scatter(kb, w);
             }
             if (++pend == A.ppt) {
