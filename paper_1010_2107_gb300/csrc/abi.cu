@@ -110,11 +110,10 @@ struct vegas_ctx {
   double* d_derived = nullptr;
   double* d_part_bins = nullptr;
   double* d_part_tot = nullptr;
-  int part_rows = 0;
+  double2* d_cube_part = nullptr;  // sums of the hypercubes' parts
+  size_t part_bins_len = 0, part_tot_len = 0, cube_part_len = 0;  // bytes
   double* d_bins = nullptr;    // behind the edges, in their allocation
   double* d_cubes = nullptr;
-  void* d_cube_part = nullptr;   // sums of the hypercubes' parts (16 bytes each)
-  size_t cube_part_len = 0;
   double* d_cube_max = nullptr;  // [G] max(0, largest w) per cube, integration phase
   bool have_max = false;         // a bases_integrate has recorded the maxima
   // SPRING buffers (grown on demand)
@@ -138,7 +137,8 @@ struct vegas_ctx {
   int grad_ctas = 0;
   size_t grad_smem = 0;
   GState* d_st = nullptr;
-  // host staging (pinned)
+  // pinned host memory: the state's mirror (only the fields before `hist`)
+  // and the staging buffer
   GState* h_st = nullptr;
   double* h_stage = nullptr;
   size_t h_stage_len = 0;
@@ -408,6 +408,8 @@ __global__ void k_spring_compact(const uint32_t* counts, uint32_t chunk, int d, 
 // dimension (us per pass of 2^22 points at 100 bins, columns against the best
 // tile: d = 4 43.9 / 47.1, d = 7 115.6 / 119.6, d = 8 66 / 93, d = 16 119 / 206).
 constexpr int kColMinWarps = 8;
+// Static shared memory of k_sample, at most (its dynamic part must leave room).
+constexpr size_t kSampleStatic = 1024;
 bool shape_col(const void* fn, const gv::KernelEntry& ke, int d, int N, int sm_count, int threads, int per_sm_req,
                uint64_t ncubes, uint64_t nc, uint64_t ncall, int64_t max_rows, uint64_t max_parts,
                gv::PassShape* out, cudaError_t* e) {
@@ -472,7 +474,7 @@ vegas_status configure_launch(vegas_ctx* c) {
     auto occ_of = [&](int cap, int) -> int {
       const size_t smem = c->ke.smem(d, N, cap);
       int o = 0;
-      if (e != cudaSuccess || smem > 227 * 1024) return 0;
+      if (e != cudaSuccess || smem + kSampleStatic > 227 * 1024) return 0;
       e = gv_raise_smem_limit(c->ke.sample, smem);
       if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, c->ke.sample, threads, smem);
       return e == cudaSuccess ? o : 0;
@@ -537,28 +539,27 @@ vegas_status configure_launch(vegas_ctx* c) {
   pn.lanes = cl.lanes;
   pn.parts = cl.parts;
   pn.ctas = ctas_for(pn, threads, most_nb);
-  // sums of the hypercubes' parts: a refining pass, or the iterations of a
-  // frozen-grid launch
-  const size_t entries = std::max(pb.parts > 1 ? (size_t)c->ncubes * pb.parts : 0,
-                                  pn.parts > 1 ? (size_t)c->ncubes * pn.parts * gv::kMergeIters : 0);
-  if (entries > c->cube_part_len) {
-    cudaFree(c->d_cube_part);
-    c->d_cube_part = nullptr;
-    c->cube_part_len = 0;
-    CK(c, gv_malloc(&c->d_cube_part, 16 * entries));
-    c->cube_part_len = entries;
-  }
-  const int rows = std::max(pb.ctas, pn.ctas);
-  if (rows > c->part_rows) {
-    if (c->d_part_bins) cudaFree(c->d_part_bins);
-    if (c->d_part_tot) cudaFree(c->d_part_tot);
-    c->d_part_bins = nullptr;
-    c->d_part_tot = nullptr;
-    c->part_rows = 0;
-    CK(c, gv_malloc(&c->d_part_bins, sizeof(double) * 2 * (size_t)d * N * rows));
-    CK(c, gv_malloc(&c->d_part_tot, sizeof(double) * gv::kTotCols * gv::kMergeIters * (size_t)rows));
-    c->part_rows = rows;
-  }
+  // partial rows (of the passes that keep bins), totals per CTA and
+  // iteration, and the sums of the hypercubes' parts (a refining pass's, or
+  // those of a frozen-grid launch's iterations)
+  auto grow = [&](auto** p, size_t* have, size_t bytes) -> vegas_status {
+    if (bytes <= *have) return VEGAS_OK;
+    cudaFree(*p);
+    *p = nullptr;
+    *have = 0;
+    CK(c, gv_malloc(p, bytes));
+    *have = bytes;
+    return VEGAS_OK;
+  };
+  vegas_status st = grow(&c->d_part_bins, &c->part_bins_len, sizeof(double) * 2 * (size_t)d * N * pb.ctas);
+  if (!st)
+    st = grow(&c->d_part_tot, &c->part_tot_len,
+              sizeof(double) * gv::kTotCols * gv::kMergeIters * (size_t)std::max(pb.ctas, pn.ctas));
+  if (!st)
+    st = grow(&c->d_cube_part, &c->cube_part_len,
+              16 * std::max(pb.parts > 1 ? (size_t)c->ncubes * pb.parts : 0,
+                            pn.parts > 1 ? (size_t)c->ncubes * pn.parts * gv::kMergeIters : 0));
+  if (st) return st;
   destroy_graphs(c);
   return VEGAS_OK;
 }
@@ -907,11 +908,11 @@ vegas_status finish_create(vegas_ctx* c, vegas_ctx** out) {
   if (!st) st = alloc((void**)&c->d_cube_max, sizeof(double) * G);
   if (!st) st = alloc((void**)&c->d_st, sizeof(GState));
   if (st) return bail(st);
-  if (gv_malloc_host(&c->h_st, sizeof(GState)) != cudaSuccess)
-    return bail(c->fail(VEGAS_ENOMEM, "cudaMallocHost(GState)"));
-  memset(c->h_st, 0, sizeof(GState));
-  c->h_st->acc = cfg->acc;
-  if (cudaMemcpyAsync(c->d_st, c->h_st, sizeof(GState), cudaMemcpyHostToDevice, c->stream) != cudaSuccess ||
+  const size_t head = sizeof(GState) - sizeof(c->h_st->hist);
+  if (gv_malloc_host(&c->h_st, head) != cudaSuccess) return bail(c->fail(VEGAS_ENOMEM, "cudaMallocHost(state)"));
+  memset(c->h_st, 0, head);
+  if ((st = stage(c, (size_t)d * (N + 1) + 2 * (size_t)d * N))) return bail(st);  // (what vegas_get_grid reads)
+  if (cudaMemsetAsync(c->d_st, 0, sizeof(GState), c->stream) != cudaSuccess ||
       cudaMemsetAsync(c->d_bins, 0, sizeof(double) * 2 * d * N, c->stream) != cudaSuccess)
     return bail(c->fail(VEGAS_ECUDA, "state initialisation failed"));
   if ((st = configure_launch(c))) return bail(st);
@@ -926,10 +927,8 @@ vegas_status finish_create(vegas_ctx* c, vegas_ctx** out) {
     if ((st = alloc((void**)&c->d_gpart, sizeof(double) * (size_t)(c->ke.grad_nt + 2) * (c->grad_ctas + 1))))
       return bail(st);
   }
-  std::vector<double> e0((size_t)d * (N + 1));
-  for (int a = 0; a < d; ++a)
-    for (int k = 0; k <= N; ++k) e0[(size_t)a * (N + 1) + k] = (double)k / (double)N;
-  if ((st = upload_grid(c, e0.data()))) return bail(st);
+  e = gv_launch_uniform_grid(c->d_edges, d, N, c->d_tab64, c->d_tab32, c->stream);
+  if (e != cudaSuccess) return bail(c->fail(VEGAS_ECUDA, "uniform grid: %s", cudaGetErrorString(e)));
   if ((st = upload_derived(c))) return bail(st);
   *out = c;
   return VEGAS_OK;
@@ -954,8 +953,8 @@ void vegas_destroy(vegas_ctx* c) {
   cudaFree(c->d_derived);
   cudaFree(c->d_part_bins);
   cudaFree(c->d_part_tot);
-  cudaFree(c->d_cubes);
   cudaFree(c->d_cube_part);
+  cudaFree(c->d_cubes);
   cudaFree(c->d_cube_max);
   for (void* p : {(void*)c->d_q, (void*)c->d_mt, (void*)c->d_mt32, (void*)c->d_guide, (void*)c->d_bmax, (void*)c->d_bsum, (void*)c->d_prefix, (void*)c->d_meta, (void*)c->d_stage_x, (void*)c->d_stage_t,
                   (void*)c->d_out_x, (void*)c->d_out_t, (void*)c->d_counts, (void*)c->d_counters})
@@ -1770,7 +1769,7 @@ extern "C" vegas_status vegas_eval_noalloc(const vegas_config* cfg, const vegas_
     auto occ_of = [&](int cp, int) -> int {
       const size_t sm = ke.smem(d, N, cp);
       int o = 0;
-      if (e != cudaSuccess || sm > 227 * 1024) return 0;
+      if (e != cudaSuccess || sm + kSampleStatic > 227 * 1024) return 0;
       e = gv_raise_smem_limit(ke.sample, sm);
       if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, ke.sample, threads, sm);
       return e == cudaSuccess ? o : 0;

@@ -1062,7 +1062,7 @@ __global__ void __launch_bounds__(256, kSpringMinBlocks<T, DM, SPEC>) k_spring(c
   // the second block only when they run past the first
   const int o = W & 3;
   const bool two_blocks = o + (YB == 24 ? 3 : 4) > 4;
-  unsigned long long ov = 0, np = 0;
+  uint32_t ov = 0, np = 0;
   for (uint32_t chunk = blockIdx.x; chunk < R.nchunks; chunk += gridDim.x) {
     uint32_t chunk_count = 0;  // the same in every thread
     const uint32_t base = chunk * R.chunk;
@@ -1172,8 +1172,8 @@ __global__ void __launch_bounds__(256, kSpringMinBlocks<T, DM, SPEC>) k_spring(c
     np += __shfl_xor_sync(0xffffffffu, np, off);
   }
   if (lane == 0) {
-    if (ov) atomicAdd(R.counters, ov);
-    if (np) atomicAdd(R.counters + 1, np);
+    if (ov) atomicAdd(R.counters, (unsigned long long)ov);
+    if (np) atomicAdd(R.counters + 1, (unsigned long long)np);
   }
 }
 
