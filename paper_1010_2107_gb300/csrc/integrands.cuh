@@ -269,15 +269,21 @@ struct RamboBW {
   };
 
   // Momenta -> (pT, eta, transverse direction) and the cyclic invariants.
-  // Returns false for a zero-weight point.
+  // Returns false for a zero-weight point (a zero uniform; the event is then
+  // not meaningful).
   static __device__ __forceinline__ bool kinematics(const T (&x)[DM], int n, Event& ev) {
     T E[NM], nx[NM], ny[NM], nz[NM];
+    bool pos = true;
     T Q0 = T(0), Qx = T(0), Qy = T(0), Qz = T(0);
 #pragma unroll
     for (int i = 0; i < NM; ++i)
       if (i < n) {
         const T r1 = x[4 * i], r2 = x[4 * i + 1], r3 = x[4 * i + 2], r4 = x[4 * i + 3];
-        if (!(r1 > T(0) && r2 > T(0))) return false;
+        // (a zero uniform: FP64 leaves; FP32 goes on without a branch, and the
+        // caller drops whatever comes out)
+        pos = pos & (r1 > T(0)) & (r2 > T(0));
+        if constexpr (!std::is_same<T, float>::value)
+          if (!pos) return false;
         const T q0 = -qlog_rel(r1 * r2);  // energy density q0 e^{-q0}: one logarithm
         const T sn = T(2) * qsqrt(r3 * (T(1) - r3));
         T sp, cp;
@@ -332,7 +338,7 @@ struct RamboBW {
         ev.ux[i] = qx * ipt;
         ev.uy[i] = qy * ipt;
       }
-    return true;
+    return pos;
   }
 
   // |u_i - u_j|^2 = 4 sin^2(dphi / 2)
@@ -368,39 +374,80 @@ struct RamboBW {
     return chord2(ev, i, j) > T(4) * h * h;
   }
 
+  // The cuts of a point.  FP32: every test evaluated, without a branch (a
+  // warp of 32 points seldom fails one as a whole, so leaving early saved
+  // nothing and its branches cost issue slots and resolving); FP64: left at
+  // the first failure (its pipe is the scarce one).
+  static __device__ __forceinline__ bool pt_pass(const Event& ev, int n, const T* P) {
+    bool ok = true;
+#pragma unroll
+    for (int i = 0; i < NM; ++i)
+      if (i < n) {
+        ok = ok & (ev.pt[i] > P[RB_PTMIN]);
+        if constexpr (!std::is_same<T, float>::value)
+          if (!ok) return false;
+      }
+    return ok;
+  }
+  static __device__ __forceinline__ bool all_dr_pass(const Event& ev, int n, const T* P) {
+    if constexpr (std::is_same<T, float>::value) {
+      if (P[RB_DR2] <= T(0.25)) {
+        bool ok = true;
+#pragma unroll
+        for (int i = 0; i < NM; ++i)
+#pragma unroll
+          for (int j = i + 1; j < NM; ++j)
+            if (j < n) {
+              // (dr_pass's series; for t <= 0 it is not above zero, and the
+              // pair passes)
+              const T de = ev.eta[i] - ev.eta[j];
+              const T t = P[RB_DR2] - de * de;
+              const T b = t * vfma(-t * T(1.0 / 12.0), vfma(-t * T(1.0 / 30.0), vfma(-t, T(1.0 / 56.0), T(1)), T(1)), T(1));
+              ok = ok & (!(t > T(0)) | (chord2(ev, i, j) > b));
+            }
+        return ok;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NM; ++i)
+#pragma unroll
+      for (int j = i + 1; j < NM; ++j)
+        if (j < n && !dr_pass(ev, i, j, P)) return false;
+    return true;
+  }
+
   static __device__ __forceinline__ T eval(const T (&x)[DM], int d, const T* P) {
     const int obs = (int)P[RB_OBS];
     if (obs == 1) return T(1);
     const int n = d >> 2;
     Event ev;
-    if (!kinematics(x, n, ev)) return T(0);
+    bool ok = kinematics(x, n, ev);
+    if constexpr (!std::is_same<T, float>::value)
+      if (!ok) return T(0);
     const int cut = (int)P[RB_CUT];
     T cw = T(1);
     if (obs == 0 && cut == 0) {
-#pragma unroll
-      for (int i = 0; i < NM; ++i)
-        if (i < n && !(ev.pt[i] > P[RB_PTMIN])) return T(0);
+      ok = ok & pt_pass(ev, n, P);
+      if constexpr (!std::is_same<T, float>::value)
+        if (!ok) return T(0);
     } else if (obs == 0 && cut == 1) {
 #pragma unroll
       for (int i = 0; i < NM; ++i)
         if (i < n) cw *= qdiv(T(1), T(1) + qexp(-(ev.pt[i] - P[RB_T]) * P[RB_INVWC]));
     }
-    if (obs == 0 && cut != 2) {
-#pragma unroll
-      for (int i = 0; i < NM; ++i)
-#pragma unroll
-        for (int j = i + 1; j < NM; ++j)
-          if (j < n && !dr_pass(ev, i, j, P)) return T(0);
-    }
+    if (obs == 0 && cut != 2) ok = ok & all_dr_pass(ev, n, P);
+    if constexpr (!std::is_same<T, float>::value)
+      if (!ok) return T(0);
     const T s12 = ev.s[0];
-    if (obs == 2) return s12;
+    if (obs == 2) return ok ? s12 : T(0);
     const T b = bw(s12, P);
-    if (obs == 3) return b;
+    if (obs == 3) return ok ? b : T(0);
     T den = s12;
 #pragma unroll
     for (int i = 1; i < NM; ++i)
       if (i < n) den *= ev.s[i];
-    return qdiv(cw * b, den);
+    const T f = qdiv(cw * b, den);
+    return ok ? f : T(0);
   }
 
   // theta = (M, Gamma, T) in GeV for the full integrand (obs 0).  The Breit-
@@ -414,13 +461,15 @@ struct RamboBW {
     if (obs != 0) return eval(x, d, P);
     const int n = d >> 2;
     Event ev;
-    if (!kinematics(x, n, ev)) return T(0);
+    bool ok = kinematics(x, n, ev);
+    if constexpr (!std::is_same<T, float>::value)
+      if (!ok) return T(0);
     const int cut = (int)P[RB_CUT];
     T cw = T(1), dlc = T(0);
     if (cut == 0) {
-#pragma unroll
-      for (int i = 0; i < NM; ++i)
-        if (i < n && !(ev.pt[i] > P[RB_PTMIN])) return T(0);
+      ok = ok & pt_pass(ev, n, P);
+      if constexpr (!std::is_same<T, float>::value)
+        if (!ok) return T(0);
     } else if (cut == 1) {
 #pragma unroll
       for (int i = 0; i < NM; ++i)
@@ -430,13 +479,9 @@ struct RamboBW {
           dlc -= (T(1) - sg) * P[RB_INVWC_GEV];
         }
     }
-    if (cut != 2) {
-#pragma unroll
-      for (int i = 0; i < NM; ++i)
-#pragma unroll
-        for (int j = i + 1; j < NM; ++j)
-          if (j < n && !dr_pass(ev, i, j, P)) return T(0);
-    }
+    if (cut != 2) ok = ok & all_dr_pass(ev, n, P);
+    if constexpr (!std::is_same<T, float>::value)
+      if (!ok) return T(0);
     const T s12 = ev.s[0];
     T den = s12;
 #pragma unroll
@@ -455,6 +500,11 @@ struct RamboBW {
     g[1] = pre * (P[RB_DMUG_DG] * tm) * iD * iD;
     const T f = pre * b;
     g[2] = f * dlc;
+    if constexpr (std::is_same<T, float>::value)
+      if (!ok) {
+        g[0] = g[1] = g[2] = T(0);
+        return T(0);
+      }
     return f;
   }
 };
