@@ -131,7 +131,8 @@ struct vegas_ctx {
   uint64_t* d_out_t = nullptr;
   uint32_t* d_counts = nullptr;
   unsigned long long* d_counters = nullptr;
-  uint32_t spring_cap = 0, spring_chunks_cap = 0;
+  uint32_t spring_cap = 0, spring_out_cap = 0;
+  void* h_spring = nullptr;  // SpringOutcome (pinned)
   cudaEvent_t spring_timer[2] = {nullptr, nullptr};  // set by spring_profile around the trial kernel
   double* d_gpart = nullptr;  // adjoint partials [grad_nt + 2][grad_ctas] then totals
   int grad_ctas = 0;
@@ -379,10 +380,21 @@ __global__ void __launch_bounds__(256) k_spring_guide(const uint64_t* prefix, ui
   guide[j] = lo;
 }
 
+// What the host reads of a SPRING call (pinned memory, written by the
+// compaction kernel's last block).
+struct SpringOutcome {
+  unsigned long long events, overflow, nonpos;
+  double status;  // meta[2]
+};
+
 // SPRING compaction: block k copies chunk k's kept points behind those of
-// chunks 0 .. k-1 (trial order).
+// chunks 0 .. k-1 (trial order).  ox and ot, either of which may be null, are
+// the caller's own buffers where the GPU can write them (pinned memory): the
+// events then cross to the host once, while they are compacted, and nothing
+// waits for their number first.
 __global__ void k_spring_compact(const uint32_t* counts, uint32_t chunk, int d, const double* sx, const uint64_t* st,
-                                 double* ox, uint64_t* ot) {
+                                 double* ox, uint64_t* ot, const double* meta, const unsigned long long* counters,
+                                 SpringOutcome* outcome) {
   __shared__ unsigned long long part[32];
   const uint32_t k = blockIdx.x;
   unsigned long long o = 0;
@@ -394,8 +406,35 @@ __global__ void k_spring_compact(const uint32_t* counts, uint32_t chunk, int d, 
   for (uint32_t w = 0; w < blockDim.x / 32; ++w) off += part[w];
   const uint32_t n = counts[k];
   const size_t src = (size_t)k * chunk;
-  for (uint32_t i = threadIdx.x; i < n * (uint32_t)d; i += blockDim.x) ox[off * d + i] = sx[src * d + i];
-  for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) ot[off + i] = st[src + i];
+  if (meta[2] == 0.0) {
+    if (ox)
+      for (uint32_t i = threadIdx.x; i < n * (uint32_t)d; i += blockDim.x) ox[off * d + i] = sx[src * d + i];
+    if (ot)
+      for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) ot[off + i] = st[src + i];
+  }
+  if (k == gridDim.x - 1 && threadIdx.x == 0) {
+    outcome->events = off + n;
+    outcome->overflow = counters[0];
+    outcome->nonpos = counters[1];
+    outcome->status = meta[2];
+  }
+}
+
+// The address under which the GPU writes the caller's host buffer [p, p +
+// bytes), or null when it cannot (pageable memory).
+void* device_view(void* p, size_t bytes) {
+  void* first = nullptr;
+  for (size_t at : {size_t(0), bytes - 1}) {
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, static_cast<unsigned char*>(p) + at) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    if (a.type != cudaMemoryTypeHost || !a.devicePointer) return nullptr;
+    if (at == 0) first = a.devicePointer;
+    else if (static_cast<unsigned char*>(a.devicePointer) != static_cast<unsigned char*>(first) + at) return nullptr;
+  }
+  return first;
 }
 
 // Shape of the column-histogram pass (col_hist.cuh): `threads` threads per
@@ -962,6 +1001,7 @@ void vegas_destroy(vegas_ctx* c) {
   cudaFree(c->d_gpart);
   cudaFree(c->d_st);
   if (c->h_st) cudaFreeHost(c->h_st);
+  if (c->h_spring) cudaFreeHost(c->h_spring);
   if (c->h_stage) cudaFreeHost(c->h_stage);
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
   delete c;
@@ -1210,20 +1250,33 @@ vegas_status spring_generate(vegas_ctx* c, uint64_t trial0, uint32_t n_trials, d
     if (!st) st = grow((void**)&c->d_meta, sizeof(double) * 3);
     if (!st) st = grow((void**)&c->d_counters, sizeof(unsigned long long) * 2);
   }
+  if (!st && !c->h_spring && gv_malloc_host(&c->h_spring, sizeof(SpringOutcome)) != cudaSuccess) {
+    c->h_spring = nullptr;
+    st = c->fail(VEGAS_ENOMEM, "cudaMallocHost(SPRING outcome)");
+  }
   if (!st && n_trials > c->spring_cap) {
     if (!st) st = grow((void**)&c->d_stage_x, sizeof(double) * d * (size_t)n_trials);
-    if (!st) st = grow((void**)&c->d_out_x, sizeof(double) * d * (size_t)n_trials);
     if (!st) st = grow((void**)&c->d_stage_t, sizeof(uint64_t) * (size_t)n_trials);
-    if (!st) st = grow((void**)&c->d_out_t, sizeof(uint64_t) * (size_t)n_trials);
     if (!st) st = grow((void**)&c->d_counts, sizeof(uint32_t) * nchunks);
-    if (!st) {
-      c->spring_cap = n_trials;
-      c->spring_chunks_cap = nchunks;
-    }
+    if (!st) c->spring_cap = n_trials;
+  }
+  // where the compacted events go: the caller's buffers, or, when the GPU
+  // cannot write those, device buffers that are copied
+  double* ox = x_out ? static_cast<double*>(device_view(x_out, sizeof(double) * d * (size_t)n_trials)) : nullptr;
+  uint64_t* ot = trial_out ? static_cast<uint64_t*>(device_view(trial_out, sizeof(uint64_t) * (size_t)n_trials)) : nullptr;
+  const bool copy = (x_out && !ox) || (trial_out && !ot);
+  if (!st && copy && n_trials > c->spring_out_cap) {
+    if (!st) st = grow((void**)&c->d_out_x, sizeof(double) * d * (size_t)n_trials);
+    if (!st) st = grow((void**)&c->d_out_t, sizeof(uint64_t) * (size_t)n_trials);
+    c->spring_out_cap = st ? 0 : n_trials;
   }
   if (st) {
     c->spring_cap = 0;
     return st;
+  }
+  if (copy) {
+    ox = x_out ? c->d_out_x : nullptr;
+    ot = trial_out ? c->d_out_t : nullptr;
   }
   // integer cube table from the recorded maxima (in the integrand's units)
   {
@@ -1267,28 +1320,23 @@ vegas_status spring_generate(vegas_ctx* c, uint64_t trial0, uint32_t n_trials, d
   if (c->spring_timer[0]) CK(c, cudaEventRecord(c->spring_timer[0], c->stream));
   CK(c, cudaLaunchKernel(fn, dim3(blocks), dim3(256), args, smem, c->stream));
   if (c->spring_timer[1]) CK(c, cudaEventRecord(c->spring_timer[1], c->stream));
-  k_spring_compact<<<nchunks, 256, 0, c->stream>>>(c->d_counts, chunk, d, c->d_stage_x, c->d_stage_t, c->d_out_x,
-                                                  c->d_out_t);
+  SpringOutcome* oc = static_cast<SpringOutcome*>(c->h_spring);
+  k_spring_compact<<<nchunks, 256, 0, c->stream>>>(c->d_counts, chunk, d, c->d_stage_x, c->d_stage_t, ox, ot,
+                                                  c->d_meta, c->d_counters, oc);
   CK(c, cudaGetLastError());
-  // status, counts and counters back to the host
-  std::vector<uint32_t> counts(nchunks);
-  double meta[3];
-  unsigned long long ctr[2];
-  CK(c, cudaMemcpyAsync(meta, c->d_meta, sizeof meta, cudaMemcpyDeviceToHost, c->stream));
-  CK(c, cudaMemcpyAsync(counts.data(), c->d_counts, sizeof(uint32_t) * nchunks, cudaMemcpyDeviceToHost, c->stream));
-  CK(c, cudaMemcpyAsync(ctr, c->d_counters, sizeof ctr, cudaMemcpyDeviceToHost, c->stream));
   CK(c, cudaStreamSynchronize(c->stream));
-  if (meta[2] != 0.0) return c->fail(VEGAS_ESTATE, "every recorded cube maximum is zero");
-  uint64_t total = 0;
-  for (uint32_t k : counts) total += k;
+  if (oc->status != 0.0) return c->fail(VEGAS_ESTATE, "every recorded cube maximum is zero");
+  const uint64_t total = oc->events;
   *n_events = (uint32_t)total;
-  if (n_overflow) *n_overflow = (uint32_t)ctr[0];
-  if (n_nonpos) *n_nonpos = (uint32_t)ctr[1];
-  if (x_out && total)
-    CK(c, cudaMemcpyAsync(x_out, c->d_out_x, sizeof(double) * d * total, cudaMemcpyDeviceToHost, c->stream));
-  if (trial_out && total)
-    CK(c, cudaMemcpyAsync(trial_out, c->d_out_t, sizeof(uint64_t) * total, cudaMemcpyDeviceToHost, c->stream));
-  if ((x_out || trial_out) && total) CK(c, cudaStreamSynchronize(c->stream));
+  if (n_overflow) *n_overflow = (uint32_t)oc->overflow;
+  if (n_nonpos) *n_nonpos = (uint32_t)oc->nonpos;
+  if (copy && total) {
+    if (x_out)
+      CK(c, cudaMemcpyAsync(x_out, c->d_out_x, sizeof(double) * d * total, cudaMemcpyDeviceToHost, c->stream));
+    if (trial_out)
+      CK(c, cudaMemcpyAsync(trial_out, c->d_out_t, sizeof(uint64_t) * total, cudaMemcpyDeviceToHost, c->stream));
+    CK(c, cudaStreamSynchronize(c->stream));
+  }
   return VEGAS_OK;
 }
 
