@@ -65,10 +65,10 @@ ALGO_OPS = {
 # DRAM bytes per launch of the sampling kernel from the committed ncu
 # capture (profiles/), per pass kind (refining, frozen grid); a workload
 # whose kernel changed since its capture has no entry.
-TRAFFIC = {"dgauss8": (83968, 614528), "rambo5": (108032,), "wmunu": (80896, 352512),
-           "rambo4_adjoint": (45504,), "spring_dgauss8": (1017088 + 3060992,),
+TRAFFIC = {"dgauss8": (56832, 79872), "rambo5": (99328,), "wmunu": (57856, 78336),
+           "rambo4_adjoint": (55296,), "spring_dgauss8": (1009408 + 3294208,),
            # one batched pass: the sum over its fifteen dimension kernels
-           "genz256": (3620992,)}
+           "genz256": (2594000,)}
 
 
 def _workload(name):
@@ -494,20 +494,20 @@ class Runner:
         # kernels of this library per step (memset nodes not counted):
         # batched: one reset, then per iteration the sampling kernels (FP32
         # form: one per dimension present; otherwise one) and k_batch_finalize;
-        # BASES: grid reset (2), iteration set (1), control (2), then k_sample
-        # + k_finish per pass; VEGAS: grid reset (2), window reset (1),
-        # iteration set (1), control (1), then the passes; adjoint: k_grad +
-        # k_colsum
+        # BASES: grid reset (1), iteration set (1), control (2), then a sampling
+        # kernel + k_finish per refining pass and per up to eight frozen-grid
+        # iterations; VEGAS: grid reset (1), window reset (1), iteration set
+        # (1), control (1), then the passes; adjoint: k_grad + k_colsum
         if self.mode == "batched":
             per_it = len({i["ndim"] for i in self.insts}) if self.prec_name == "fp32" else 1
             return 1 + (per_it + 1) * w["itmx"]
         if self.mode == "bases":
-            return 2 + 1 + 2 + 2 * (w["itmx1"] + w["itmx2"])
+            return 1 + 1 + 2 + 2 * (w["itmx1"] + (w["itmx2"] + 7) // 8)
         if self.mode == "adjoint":
             return 2
         if self.mode == "spring":  # cube table and guide (5 kernels), trials, compaction
             return 7
-        return 2 + 1 + 1 + 1 + 2 * w["itmx"]
+        return 1 + 1 + 1 + 1 + 2 * w["itmx"]
 
     def estimates(self, h):
         """The results the step produced, as (I, sigma) pairs: one per
@@ -565,8 +565,8 @@ class Runner:
         gv = self.gv
         if self.mode == "batched":
             p = gv.vegas_batch_profile(h, 5)
-            name = ("k_batch_dim (one kernel per dimension, concurrent)" if self.prec_name == "fp32"
-                    else "k_batch_sample")
+            form = "k_batch_col" if gv.vegas_batch_get_tile(h)["cap"] == 0 else "k_batch_dim"
+            name = f"{form} (one kernel per dimension, concurrent)" if self.prec_name == "fp32" else "k_batch_sample"
             return name, p["sample"], sum(i["ncall"] for i in self.insts), {"finalize_ms": p["finalize"]}
         if self.mode == "adjoint":
             import torch
@@ -583,9 +583,12 @@ class Runner:
             return "k_spring", gv.spring_profile(h, self.w["ntrials"], 5), self.w["ntrials"], {}
         p = gv.vegas_profile_pass(h, 20)
         other = {"finish_ms": p["finish"]}
+        # refining passes: the column-histogram kernel, or the bucketed one
+        name = "k_sample_col" if gv.vegas_get_tile(h)["cap"] == 0 else "k_sample"
         if self.mode == "bases":
             # the step's mix: ITMX1 refining passes with the per-bin histogram,
-            # ITMX2 frozen-grid passes without it
+            # ITMX2 frozen-grid iterations without it (timed one to a launch; a
+            # run's share a launch and take less each)
             q = gv.vegas_profile_frozen_pass(h, 20)
             n1, n2 = self.w["itmx1"], self.w["itmx2"]
             ops = ALGO_OPS.get(self.name, {})
@@ -595,8 +598,8 @@ class Runner:
                 {"kind": "frozen-grid pass", "launches_per_step": n2, "ms_per_launch": q["sample"],
                  "ops_per_point": off}]
             other["finish_ms_frozen"] = q["finish"]
-            return "k_sample", (n1 * p["sample"] + n2 * q["sample"]) / (n1 + n2), self.w["ncall"], other
-        return "k_sample", p["sample"], self.w["ncall"], other
+            return name, (n1 * p["sample"] + n2 * q["sample"]) / (n1 + n2), self.w["ncall"], other
+        return name, p["sample"], self.w["ncall"], other
 
     def ops_per_point(self):
         if self.mode == "batched":
