@@ -363,17 +363,15 @@ __device__ __forceinline__ void cube_store(void* p, size_t i, double c1, double 
 struct SampleArgs {
   int d, N, g, ybits;
   int lanes;               // lanes per group (stratified mode), power of two <= 32
-  uint32_t parts;          // groups per hypercube, each with its share of the cube's points
-  int niter;               // iterations this launch runs (frozen grid; 1 with the histogram)
-  uint32_t rot;            // CTAs by which each iteration's share of the work is turned
   int cap;                 // bucket capacity per (axis, bin) and tile
   int ppt;                 // points per thread per tile (>= 1)
   int strat;
   int nobins;              // 1: no per-bin histogram (a pass whose grid is not refined)
   uint32_t key0, key1, instance;
-  uint32_t ks[kPhiloxKeyWords];  // Philox round keys of (key0, key1)
+  // Philox round keys of (key0, key1).  On a 16-byte boundary: off it the
+  // compiler reads them word by word (k_spring, d = 8: 52 registers, not 48)
+  alignas(16) uint32_t ks[kPhiloxKeyWords];
   int it_override;         // >= 0: use this iteration index
-  int force;               // 1: run even if the ACC test has stopped the last call (evaluation passes)
   uint64_t ncall;
   uint32_t nc;             // points per hypercube
   uint32_t ncubes;         // number of hypercubes
@@ -389,9 +387,13 @@ struct SampleArgs {
   GState* st;              // the sampling kernel latches st->live
   void* part_bins;         // [nparts][2 d N]: double, or float (hi, lo) pairs (FP32 forms)
   double* part_tot;        // [niter][kTotCols][nparts]
-  void* cube_part;         // [niter][parts][ncubes] sums of the parts (parts > 1), as `cubes`
   void* cubes;             // [ncubes]: double (sum w, sum w^2), or float (hi, lo, hi, lo)
   double* cube_max;        // [ncubes] running max(0, largest w) (integration phase), or null
+  void* cube_part;         // [niter][parts][ncubes] sums of the parts (parts > 1), as `cubes`
+  uint32_t parts;          // groups per hypercube, each with its share of the cube's points
+  int niter;               // iterations this launch runs (frozen grid; 1 with the histogram)
+  uint32_t rot;            // CTAs by which each iteration's share of the work is turned
+  int force;               // 1: run even if the ACC test has stopped the last call (evaluation passes)
 };
 
 // Arguments of the reduction and finalisation kernels (steps 4-6).
