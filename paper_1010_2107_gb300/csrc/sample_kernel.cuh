@@ -1031,14 +1031,11 @@ __host__ __device__ inline size_t sample_smem_nobins(int d, int N) {
 // order).  One thread per trial and round; 256 threads.
 constexpr uint32_t kSpringIt = 0xFFFFFFFFu;
 
-// CTAs per SM the specialised FP32 kernels of low dimension are held to: the
-// cube search waits on L2, so residency counts (d = 8: 54 registers and four
-// CTAs took 452 us per 2^22 trials with their events, 48 and five 442 us).
-template <typename T, int DM, bool SPEC>
-constexpr int kSpringMinBlocks = !SPEC || !std::is_same<T, float>::value || DM > 8 ? 0 : (DM <= 4 ? 6 : 5);
-
+// No minimum of CTAs per SM is asked for: held to five at d = 8 the kernels
+// spilled up to 28 bytes (two-peak Gaussian, 2^24 trials: 387 us, 374 without;
+// both run five CTAs of 48 registers).
 template <typename T, int DM, template <typename, int> class F, int YB, bool SPEC>
-__global__ void __launch_bounds__(256, kSpringMinBlocks<T, DM, SPEC>) k_spring(const SpringArgs R) {
+__global__ void __launch_bounds__(256) k_spring(const SpringArgs R) {
   using T2 = typename Vec2<T>::type;
   const SampleArgs& A = R.S;
   const int d = SPEC ? DM : A.d, N = A.N, dN = d * N;
