@@ -23,8 +23,9 @@
 // while the table lookups and constants around them stay free to move.)
 //
 // What it costs per 32 point-axes, in shared-memory wavefronts: bin byte 1,
-// cell load 2, cell store 2, weight 1/4, about 5.5 with the staging writes,
-// against 11 for bucketed tiles (claim atomic 3.8, slot store 3.6, gather);
+// cell load 2, cell store 2, weight 1/4, about 5.5 with the staging writes
+// (6.9 measured with the folds, d = 8), against 11.2 for bucketed tiles (claim
+// atomic 3.8, slot store 3.6, gather);
 // and about 6 issue slots against 16.  The price is memory: 256 N bytes per
 // warp (12.8 KB at 50 bins), which bounds the warps per SM (16 at 50 bins).
 #pragma once
