@@ -233,7 +233,8 @@ struct SpringArgs {
   const uint32_t* guide;    // [2^gk + 1] guide table of the cube search (Chen and Asau):
                             // guide[j] = the last cube c with prefix[c] <= floor(j Q / 2^gk)
   uint32_t gk;              // log2 of the number of guide intervals
-  const double* meta;       // {Q, scale} written by the table kernel
+  const double* meta;       // {Q, scale, status} written by the table kernels (status 1: no positive
+                            // maximum, and the tables above are not formed)
   double out_scale;         // integrand output scale: weights in the integrand's units
   uint32_t trial0, n, chunk, nchunks;
   double* stage_x;

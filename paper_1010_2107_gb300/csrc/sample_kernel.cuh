@@ -1039,6 +1039,13 @@ __global__ void __launch_bounds__(256) k_spring(const SpringArgs R) {
   using T2 = typename Vec2<T>::type;
   const SampleArgs& A = R.S;
   const int d = SPEC ? DM : A.d, N = A.N, dN = d * N;
+  // No positive cube maximum: the table kernels have formed no prefix sums
+  // and no guide, so there is no cube to draw (what those arrays hold then is
+  // no valid index).  The host reports it; the chunks stay empty.
+  if (R.meta[2] != 0.0) {
+    for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < R.nchunks; k += gridDim.x * blockDim.x) R.counts[k] = 0u;
+    return;
+  }
   extern __shared__ __align__(16) unsigned char smem[];
   T2* tab = reinterpret_cast<T2*>(smem);
   T* P = reinterpret_cast<T*>(smem + (size_t)dN * sizeof(T2));
