@@ -2,6 +2,7 @@
 // lifetime, derived integrand constants, launch geometry, the per-iteration
 // kernel sequence (captured once into a CUDA graph per call shape) and the
 // result read-back.
+#include <cuda.h>  // types only: the driver is reached through the runtime
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -420,21 +421,37 @@ __global__ void k_spring_compact(const uint32_t* counts, uint32_t chunk, int d, 
   }
 }
 
-// The address under which the GPU writes the caller's host buffer [p, p +
-// bytes), or null when it cannot (pageable memory).
-void* device_view(void* p, size_t bytes) {
-  void* first = nullptr;
-  for (size_t at : {size_t(0), bytes - 1}) {
-    cudaPointerAttributes a{};
-    if (cudaPointerGetAttributes(&a, static_cast<unsigned char*>(p) + at) != cudaSuccess) {
-      cudaGetLastError();
-      return nullptr;
-    }
-    if (a.type != cudaMemoryTypeHost || !a.devicePointer) return nullptr;
-    if (at == 0) first = a.devicePointer;
-    else if (static_cast<unsigned char*>(a.devicePointer) != static_cast<unsigned char*>(first) + at) return nullptr;
+// The address under which the GPU may write the caller's host buffer [p, p +
+// bytes), or null where the events must go through device memory and a copy:
+// pageable memory, a start that is not a multiple of `align` (the kernel
+// stores whole elements; a copy takes any address), or a buffer that does not
+// lie inside one pinned allocation.  The driver names the allocation's range:
+// under unified addressing two separate pinned allocations can have pageable
+// memory between them at addresses that look contiguous.
+void* device_view(void* p, size_t bytes, size_t align) {
+  using Query = CUresult (*)(void*, CUpointer_attribute, CUdeviceptr);
+  static const Query query = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult r;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault, &r);
+    if (e != cudaSuccess) cudaGetLastError();
+    return reinterpret_cast<Query>(e == cudaSuccess && r == cudaDriverEntryPointSuccess ? f : nullptr);
+  }();
+  if (!query || reinterpret_cast<uintptr_t>(p) % align != 0) return nullptr;
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
   }
-  return first;
+  if (a.type != cudaMemoryTypeHost || !a.devicePointer || reinterpret_cast<uintptr_t>(a.devicePointer) % align != 0)
+    return nullptr;
+  const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(a.devicePointer);
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  if (query(&base, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, at) != CUDA_SUCCESS ||
+      query(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, at) != CUDA_SUCCESS)
+    return nullptr;
+  return at >= base && bytes <= size && at - base <= size - bytes ? a.devicePointer : nullptr;
 }
 
 // Shape of the column-histogram pass (col_hist.cuh): `threads` threads per
@@ -1262,8 +1279,10 @@ vegas_status spring_generate(vegas_ctx* c, uint64_t trial0, uint32_t n_trials, d
   }
   // where the compacted events go: the caller's buffers, or, when the GPU
   // cannot write those, device buffers that are copied
-  double* ox = x_out ? static_cast<double*>(device_view(x_out, sizeof(double) * d * (size_t)n_trials)) : nullptr;
-  uint64_t* ot = trial_out ? static_cast<uint64_t*>(device_view(trial_out, sizeof(uint64_t) * (size_t)n_trials)) : nullptr;
+  double* ox = x_out ? static_cast<double*>(device_view(x_out, sizeof(double) * d * (size_t)n_trials, sizeof(double)))
+                     : nullptr;
+  uint64_t* ot = trial_out ? static_cast<uint64_t*>(device_view(trial_out, sizeof(uint64_t) * (size_t)n_trials, sizeof(uint64_t)))
+                           : nullptr;
   const bool copy = (x_out && !ox) || (trial_out && !ot);
   if (!st && copy && n_trials > c->spring_out_cap) {
     if (!st) st = grow((void**)&c->d_out_x, sizeof(double) * d * (size_t)n_trials);

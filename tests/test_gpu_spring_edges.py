@@ -41,3 +41,52 @@ def test_no_positive_maximum_is_an_error_and_draws_nothing(gv, precision, ybits,
         with pytest.raises(gv.VegasError) as e:
             gv.spring_generate(ctx, 0, 5000)
         assert e.value.status == gv.ESTATE
+
+
+def _spring_into(gv, ctx, n, x_ptr, t_ptr):
+    """spring_generate through the C ABI with raw addresses (None: not asked for)."""
+    import ctypes
+    k, ov, npos = ctypes.c_uint32(), ctypes.c_uint32(), ctypes.c_uint32()
+    st = gv.lib().spring_generate(
+        ctx.handle, 0, n, None if x_ptr is None else ctypes.cast(x_ptr, ctypes.POINTER(ctypes.c_double)),
+        None if t_ptr is None else ctypes.cast(t_ptr, ctypes.POINTER(ctypes.c_uint64)),
+        ctypes.byref(k), ctypes.byref(ov), ctypes.byref(npos))
+    assert st == gv.OK
+    return k.value, ov.value, npos.value
+
+
+def _buffer(nbytes, kind):
+    """A host byte buffer filled with 0xA5 and the offset to use in it."""
+    import torch
+    off = {"pageable": 16, "pinned": 16, "pinned-odd": 20, "pageable-odd": 3}[kind]
+    b = torch.empty(nbytes + off + 64, dtype=torch.uint8, pin_memory=kind.startswith("pinned"))
+    b.fill_(0xA5)
+    return b, off
+
+
+@pytest.mark.parametrize("kx,kt", [("pinned", "pinned"), ("pageable", "pinned"), ("pinned", "pageable"),
+                                   ("pinned-odd", "pinned"), ("pinned", "pinned-odd"),
+                                   ("pageable-odd", "pageable-odd"), ("pinned", None), (None, "pinned"),
+                                   ("pageable", None), (None, "pageable")])
+def test_events_do_not_depend_on_the_callers_buffers(gv, kx, kt):
+    """Pinned buffers (written by the GPU), pageable ones (copied), one of each,
+    one alone, and addresses off the elements' alignment (copied): the same
+    events and counts byte for byte, and nothing past them, for one trial, sizes
+    around a chunk of 4096, and a larger call after smaller ones."""
+    d = 4
+    with gv.vegas_create(wl.DOUBLE_GAUSSIAN, d, wl.double_gaussian_params(w=0.15), ncall=4 ** d * 32, nstrat=4,
+                         precision="fp32") as ctx:
+        gv.bases_integrate(ctx, 2, 0.0, 2, 0.0)
+        for n in (1, 4095, 4097, 30011):
+            ref = gv.spring_generate(ctx, 0, n)
+            m = ref["n_events"]
+            assert n == 1 or 0 < m < n
+            bx, ox = _buffer(8 * d * n, kx) if kx else (None, 0)
+            bt, ot = _buffer(8 * n, kt) if kt else (None, 0)
+            got = _spring_into(gv, ctx, n, bx.data_ptr() + ox if kx else None, bt.data_ptr() + ot if kt else None)
+            assert got == (m, ref["overflow"], ref["nonpos"])
+            for b, o, want in ((bx, ox, ref["x"]), (bt, ot, ref["trial"])):
+                if b is not None:
+                    raw = np.ascontiguousarray(want).tobytes()
+                    assert b.numpy()[o:o + len(raw)].tobytes() == raw
+                    assert np.all(b.numpy()[:o] == 0xA5) and np.all(b.numpy()[o + len(raw):] == 0xA5)
