@@ -507,10 +507,15 @@ bool shape_col(const void* fn, const gv::KernelEntry& ke, int d, int N, int sm_c
   return true;
 }
 
+// Launch shapes of both kinds of pass and the buffers they need.  The context
+// changes only where all of it succeeds: new buffers are allocated before the
+// old ones go, and the graphs, which hold the old addresses, go first.  (The
+// stream is idle here.)
 vegas_status configure_launch(vegas_ctx* c) {
   int threads = c->threads_req > 0 ? c->threads_req : 256;
   const int d = c->cfg.ndim, N = c->cfg.nbins;
-  gv::PassShape &pb = c->pass_bins, &pn = c->pass_nobins;
+  gv::PassShape pb, pn;
+  int cap = 0, ppt = 1;
   const bool strat = c->strat != 0;
   cudaError_t e = cudaSuccess;
   auto ctas_for = [&](const gv::PassShape& s, int t, int64_t most) {
@@ -521,14 +526,13 @@ vegas_status configure_launch(vegas_ctx* c) {
   if (c->col && c->ppt_req == 0 &&
       shape_col(c->col, c->ke, d, N, c->sm_count, c->threads_req, c->ctas_per_sm_req, c->ncubes, c->nc,
                 (uint64_t)c->cfg.ncall, INT64_MAX, gv::kMaxCubeParts, &pb, &e)) {
-    c->cap = 0;
-    c->ppt = d <= 8 ? 2 : 1;
+    ppt = d <= 8 ? 2 : 1;
     per_sm = std::max(1, pb.occ);
   } else {
     // Histogram tile (gv::choose_tile): points per thread between gathers and
     // bucket capacity, against the CTAs per SM each leaves resident.
-    auto occ_of = [&](int cap, int) -> int {
-      const size_t smem = c->ke.smem(d, N, cap);
+    auto occ_of = [&](int cp, int) -> int {
+      const size_t smem = c->ke.smem(d, N, cp);
       int o = 0;
       if (e != cudaSuccess || smem + kSampleStatic > 227 * 1024) return 0;
       e = gv_raise_smem_limit(c->ke.sample, smem);
@@ -566,8 +570,8 @@ vegas_status configure_launch(vegas_ctx* c) {
     pb.smem = c->ke.smem(d, N, t.cap);
     e = gv_raise_smem_limit(c->ke.sample, pb.smem);
     if (e != cudaSuccess) return c->fail(VEGAS_ECUDA, "launch configuration: %s", cudaGetErrorString(e));
-    c->cap = t.cap;
-    c->ppt = t.ppt;
+    cap = t.cap;
+    ppt = t.ppt;
     per_sm = c->ctas_per_sm_req > 0 ? std::min(c->ctas_per_sm_req, t.occ) : t.occ;
     const int64_t most = (int64_t)c->sm_count * per_sm;
     pb.lanes = strat ? gv::choose_lanes(c->ncubes, c->nc, threads, most) : 1;
@@ -598,25 +602,36 @@ vegas_status configure_launch(vegas_ctx* c) {
   // partial rows (of the passes that keep bins), totals per CTA and
   // iteration, and the sums of the hypercubes' parts (a refining pass's, or
   // those of a frozen-grid launch's iterations)
-  auto grow = [&](auto** p, size_t* have, size_t bytes) -> vegas_status {
-    if (bytes <= *have) return VEGAS_OK;
-    cudaFree(*p);
-    *p = nullptr;
-    *have = 0;
-    CK(c, gv_malloc(p, bytes));
-    *have = bytes;
-    return VEGAS_OK;
-  };
-  vegas_status st = grow(&c->d_part_bins, &c->part_bins_len, sizeof(double) * 2 * (size_t)d * N * pb.ctas);
-  if (!st)
-    st = grow(&c->d_part_tot, &c->part_tot_len,
-              sizeof(double) * gv::kTotCols * gv::kMergeIters * (size_t)std::max(pb.ctas, pn.ctas));
-  if (!st)
-    st = grow(&c->d_cube_part, &c->cube_part_len,
-              16 * std::max(pb.parts > 1 ? (size_t)c->ncubes * pb.parts : 0,
-                            pn.parts > 1 ? (size_t)c->ncubes * pn.parts * gv::kMergeIters : 0));
-  if (st) return st;
+  struct Buffer {
+    void** p;
+    size_t* have;
+    size_t need;
+    void* fresh;
+  } buffers[3] = {
+      {(void**)&c->d_part_bins, &c->part_bins_len, sizeof(double) * 2 * (size_t)d * N * pb.ctas, nullptr},
+      {(void**)&c->d_part_tot, &c->part_tot_len,
+       sizeof(double) * gv::kTotCols * gv::kMergeIters * (size_t)std::max(pb.ctas, pn.ctas), nullptr},
+      {(void**)&c->d_cube_part, &c->cube_part_len,
+       16 * std::max(pb.parts > 1 ? (size_t)c->ncubes * pb.parts : 0,
+                     pn.parts > 1 ? (size_t)c->ncubes * pn.parts * gv::kMergeIters : 0),
+       nullptr}};
+  for (Buffer& b : buffers) {
+    if (b.need <= *b.have || (e = gv_dev_malloc(&b.fresh, b.need)) == cudaSuccess) continue;
+    for (Buffer& o : buffers) cudaFree(o.fresh);
+    return c->fail(e == cudaErrorMemoryAllocation ? VEGAS_ENOMEM : VEGAS_ECUDA, "cudaMalloc(%zu): %s", b.need,
+                   cudaGetErrorString(e));
+  }
   destroy_graphs(c);
+  for (Buffer& b : buffers)
+    if (b.fresh) {
+      cudaFree(*b.p);
+      *b.p = b.fresh;
+      *b.have = b.need;
+    }
+  c->pass_bins = pb;
+  c->pass_nobins = pn;
+  c->cap = cap;
+  c->ppt = ppt;
   return VEGAS_OK;
 }
 
@@ -1502,10 +1517,9 @@ vegas_status vegas_set_launch(vegas_ctx* c, int threads, int ctas_per_sm) {
   c->threads_req = threads;
   c->ctas_per_sm_req = ctas_per_sm;
   vegas_status st = configure_launch(c);
-  if (st) {
+  if (st) {  // (the shape and its buffers are as before)
     c->threads_req = t0;
     c->ctas_per_sm_req = p0;
-    configure_launch(c);
   }
   return st;
 }
@@ -1518,10 +1532,7 @@ vegas_status vegas_set_tile(vegas_ctx* c, int points_per_thread) {
   const int p0 = c->ppt_req;
   c->ppt_req = points_per_thread;
   vegas_status st = configure_launch(c);
-  if (st) {
-    c->ppt_req = p0;
-    configure_launch(c);
-  }
+  if (st) c->ppt_req = p0;  // (the shape and its buffers are as before)
   return st;
 }
 
