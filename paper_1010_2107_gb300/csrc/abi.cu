@@ -1270,7 +1270,7 @@ vegas_status spring_generate(vegas_ctx* c, uint64_t trial0, uint32_t n_trials, d
   vegas_status st = VEGAS_OK;
   uint32_t gk = 0;  // 2^gk guide intervals: about one per cube, at most 2^22 (16 MB)
   while (gk < 22 && (1ull << gk) < c->ncubes) ++gk;
-  if (!c->d_q) {
+  if (!c->d_counters) {  // the tables (all of them again where an earlier call got only some: the counters come last)
     if (!st) st = grow((void**)&c->d_q, sizeof(uint64_t) * c->ncubes);
     if (!st) st = grow((void**)&c->d_mt, sizeof(double) * c->ncubes);
     if (!st) st = grow((void**)&c->d_mt32, sizeof(float) * c->ncubes);

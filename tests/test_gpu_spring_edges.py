@@ -90,3 +90,32 @@ def test_events_do_not_depend_on_the_callers_buffers(gv, kx, kt):
                     raw = np.ascontiguousarray(want).tobytes()
                     assert b.numpy()[o:o + len(raw)].tobytes() == raw
                     assert np.all(b.numpy()[:o] == 0xA5) and np.all(b.numpy()[o + len(raw):] == 0xA5)
+
+
+def test_every_failed_allocation_of_the_first_call(gv):
+    """Each allocation of a context's first SPRING call fails in turn (on the
+    host), on one context: every call answers ENOMEM, none leaves tables half
+    there, and the first that gets all of them draws the events of an untouched
+    context; so does a larger call after its own failures."""
+    d = 3
+    kw = dict(ncall=4 ** d * 50, nstrat=4, precision="fp64", ybits=24, seed=3)
+    mk = lambda: gv.vegas_create(wl.GENZ_GAUSSIAN, d, wl.genz_gaussian_params(d, a=4.0), **kw)
+    with mk() as ref, mk() as ctx:
+        for c in (ref, ctx):  # no refining iteration: the same grid and maxima bit for bit in both
+            gv.bases_integrate(c, 0, 0.0, 2, 0.0)
+        for n, least in ((4096, 10), (9000, 3)):
+            want, failed = gv.spring_generate(ref, 0, n), 0
+            for j in range(32):
+                gv.vegas_fail_alloc_after(j)
+                try:
+                    got = gv.spring_generate(ctx, 0, n)
+                    break
+                except gv.VegasError as e:
+                    assert e.status == gv.ENOMEM
+                    failed += 1
+                finally:
+                    gv.vegas_fail_alloc_after(-1)
+            assert failed >= least
+            assert got["n_events"] == want["n_events"] > 0
+            np.testing.assert_array_equal(got["trial"], want["trial"])
+            np.testing.assert_array_equal(got["x"], want["x"])
