@@ -382,7 +382,23 @@ thread_local std::string g_batch_err;
 
 }  // namespace
 
-struct vegas_batch {
+// Launch shape of a batch: what was asked for and what configure() made of it.
+struct BatchShape {
+  int threads = 256, rounds = 32, ctas = 0, cap = 16, ppt = 1, occ = 0;
+  bool launch_set = false;  // by vegas_batch_set_launch (else rounds may be chosen by the work)
+  int ppt_req = 0;         // points per thread per tile asked for (0: automatic)
+  bool small_cap = false;  // tile capacity policy (gv::choose_tile)
+  bool dense_cap = false;  // the dense floor of that policy (per-dimension kernels)
+  struct Dim {
+    int first = 0, count = 0, cap = 4, ctas = 0, occ = 0;
+    size_t smem = 0;
+    const void* fn = nullptr;
+  } dims[gv::kBatchDM];
+  size_t smem = 0;
+  const void* kernel = nullptr;
+};
+
+struct vegas_batch : BatchShape {
   int n = 0, N = 50, prec = VG_FP32_ACCCOMP, ybits = 24;
   int maxd = 1;  // widest instance
   uint64_t seed = 1;
@@ -391,26 +407,13 @@ struct vegas_batch {
   std::vector<std::vector<double>> params;
   std::vector<double> derived;  // [n][kNumDerived]
   int sm_count = 0;
-  // launch shape
-  int threads = 256, rounds = 32, ctas = 0, cap = 16, ppt = 1, occ = 0;
-  bool launch_set = false;  // by vegas_batch_set_launch (else rounds may be chosen by the work)
-  int ppt_req = 0;         // points per thread per tile asked for (0: automatic)
-  bool small_cap = false;  // tile capacity policy (gv::choose_tile)
-  bool dense_cap = false;  // the dense floor of that policy (per-dimension kernels)
   // FP32 form with 24-bit words: one kernel per exact dimension d = 1..16,
   // each with its item range, tile and launch shape, run concurrently on
   // the auxiliary streams (forked from and joined to `stream`)
   bool by_dim = false;
-  struct Dim {
-    int first = 0, count = 0, cap = 4, ctas = 0, occ = 0;
-    size_t smem = 0;
-    const void* fn = nullptr;
-  } dims[gv::kBatchDM];
   static constexpr int kAux = 4;
   cudaStream_t aux[kAux] = {};
   cudaEvent_t fork = nullptr, join[kAux] = {};
-  size_t smem = 0;
-  const void* kernel = nullptr;
   // host copies of the tables
   std::vector<BatchInst> inst;
   std::vector<BatchItem> items;
@@ -484,7 +487,8 @@ size_t batch_smem(int prec, int md, int N, int cap) {
 
 // Items of `threads * rounds` points, instances in decreasing NCALL order so
 // that the small items come last (grouped by dimension first, widest first,
-// when the dimension kernels run); rows laid out in item order.
+// when the dimension kernels run); rows laid out in item order.  The batch's
+// items, buffers and graphs change only once every buffer is there.
 vegas_status build_items(vegas_batch* b) {
   const uint64_t tile = (uint64_t)b->threads * b->rounds;
   std::vector<int> order(b->n);
@@ -493,19 +497,20 @@ vegas_status build_items(vegas_batch* b) {
     if (b->by_dim && b->d[x] != b->d[y]) return b->d[x] > b->d[y];
     return b->cfg[x].ncall > b->cfg[y].ncall;
   });
-  b->items.clear();
+  std::vector<BatchItem> items;
+  std::vector<BatchInst> inst = b->inst;
   for (auto& c : b->dims) c.first = c.count = 0;
   size_t row = 0;
   for (int i : order) {
-    BatchInst& I = b->inst[i];
+    BatchInst& I = inst[i];
     if (b->by_dim) {
       auto& c = b->dims[I.d - 1];
-      if (c.count == 0) c.first = (int)b->items.size();
+      if (c.count == 0) c.first = (int)items.size();
     }
     // an instance's items are consecutive and so are their rows, each
     // 2 d N + kRowTail entries long: k_batch_finalize addresses them by
     // that stride from the first item's row
-    I.first_item = (int)b->items.size();
+    I.first_item = (int)items.size();
     const uint64_t n = (uint64_t)b->cfg[i].ncall;
     for (uint64_t s0 = 0; s0 < n; s0 += tile) {
       BatchItem it;
@@ -514,35 +519,41 @@ vegas_status build_items(vegas_batch* b) {
       it.count = (uint32_t)std::min<uint64_t>(tile, n - s0);
       it.row = (uint32_t)row;
       row += 2 * (size_t)I.d * b->N + gv::kRowTail;
-      b->items.push_back(it);
+      items.push_back(it);
     }
-    I.nitems = (int)b->items.size() - I.first_item;
+    I.nitems = (int)items.size() - I.first_item;
     if (b->by_dim) b->dims[I.d - 1].count += I.nitems;
   }
   for (auto& c : b->dims) c.ctas = std::min(c.count, b->sm_count * std::max(c.occ, 1));
   if (row > 0xFFFFFFFFull) return b->fail(VEGAS_EINVAL, "batch too large for the partial-row index");
   const size_t esz = b->prec == VG_FP64 ? sizeof(double) : sizeof(float2);
-  if (row > b->rows_cap) {
+  void* rows = nullptr;
+  BatchItem* ditems = nullptr;
+  if (row > b->rows_cap) BK(b, gv_dev_malloc(&rows, row * esz));
+  if (items.size() > b->items_cap) {
+    const cudaError_t e = gv_malloc(&ditems, items.size() * sizeof(BatchItem));
+    if (e != cudaSuccess) cudaFree(rows);
+    BK(b, e);
+  }
+  drop_graphs(b);  // they hold the old addresses
+  if (rows) {
     cudaFree(b->d_rows);
-    b->d_rows = nullptr;
-    b->rows_cap = 0;
-    BK(b, gv_dev_malloc(&b->d_rows, row * esz));
+    b->d_rows = rows;
     b->rows_cap = row;
   }
-  b->row_entries = row;
-  if (b->items.size() > b->items_cap) {
+  if (ditems) {
     cudaFree(b->d_items);
-    b->d_items = nullptr;
-    b->items_cap = 0;
-    BK(b, gv_malloc(&b->d_items, b->items.size() * sizeof(BatchItem)));
-    b->items_cap = b->items.size();
+    b->d_items = ditems;
+    b->items_cap = items.size();
   }
+  b->row_entries = row;
+  b->items.swap(items);
+  b->inst.swap(inst);
   BK(b, cudaMemcpyAsync(b->d_items, b->items.data(), b->items.size() * sizeof(BatchItem),
                         cudaMemcpyHostToDevice, b->stream));
   BK(b, cudaMemcpyAsync(b->d_inst, b->inst.data(), b->n * sizeof(BatchInst), cudaMemcpyHostToDevice,
                         b->stream));
   BK(b, cudaStreamSynchronize(b->stream));
-  drop_graphs(b);
   return VEGAS_OK;
 }
 
@@ -633,8 +644,7 @@ vegas_status configure_dims(vegas_batch* b) {
   return build_items(b);
 }
 
-vegas_status configure(vegas_batch* b) {
-  if (b->by_dim) return configure_dims(b);
+vegas_status configure_general(vegas_batch* b) {
   b->kernel = pick_batch_kernel(b->prec, b->ybits);
   BK(b, cudaFuncSetAttribute(b->kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                              (int)cudaSharedmemCarveoutMaxShared));
@@ -660,6 +670,16 @@ vegas_status configure(vegas_batch* b) {
   const int occ = t.occ;
   b->ctas = b->sm_count * occ;
   return build_items(b);
+}
+
+// Kernels, shapes and items for the shape `want` (its requests); a batch that
+// cannot have it keeps the shape it has.
+vegas_status configure(vegas_batch* b, const BatchShape& want) {
+  const BatchShape had = *b;
+  static_cast<BatchShape&>(*b) = want;
+  const vegas_status st = b->by_dim ? configure_dims(b) : configure_general(b);
+  if (st) static_cast<BatchShape&>(*b) = had;
+  return st;
 }
 
 BatchArgs batch_args(const vegas_batch* b, int refine, int record) {
@@ -915,7 +935,7 @@ vegas_status vegas_batch_create(int n, const vegas_config* cfgs, const vegas_int
       return bail(VEGAS_ECUDA);
     }
   }
-  vegas_status st = configure(b);
+  vegas_status st = configure(b, *b);
   if (st) return bail(st);
   *out = b;
   return VEGAS_OK;
@@ -1035,10 +1055,11 @@ vegas_status vegas_batch_set_launch(vegas_batch* b, int threads, int rounds) {
   if (threads < 64 || threads > 256 || threads % 32 || rounds < 1 || rounds > 4096)
     return b->fail(VEGAS_EINVAL, "threads must be 64..256 (multiple of 32), rounds 1..4096");
   BK(b, cudaStreamSynchronize(b->stream));
-  b->threads = threads;
-  b->rounds = rounds;
-  b->launch_set = true;
-  return configure(b);
+  BatchShape want = *b;
+  want.threads = threads;
+  want.rounds = rounds;
+  want.launch_set = true;
+  return configure(b, want);
 }
 
 vegas_status vegas_batch_set_tile(vegas_batch* b, int points_per_thread) {
@@ -1047,14 +1068,9 @@ vegas_status vegas_batch_set_tile(vegas_batch* b, int points_per_thread) {
   if (points_per_thread < 0 || points_per_thread > hi)
     return b->fail(VEGAS_EINVAL, "points_per_thread must be in 0..%d (0: automatic)", hi);
   BK(b, cudaStreamSynchronize(b->stream));
-  const int p0 = b->ppt_req;
-  b->ppt_req = points_per_thread;
-  vegas_status st = configure(b);
-  if (st) {
-    b->ppt_req = p0;
-    configure(b);
-  }
-  return st;
+  BatchShape want = *b;
+  want.ppt_req = points_per_thread;
+  return configure(b, want);
 }
 
 vegas_status vegas_batch_get_tile(vegas_batch* b, int* points_per_thread, int* cap) {
@@ -1117,11 +1133,19 @@ vegas_status vegas_batch_autotune(vegas_batch* b, int* threads, int* rounds, dou
   // (the per-dimension kernels: points in flight) and capacity policy pol
   // (0: the largest capacity of the range, 1: the smallest, 2: the dense
   // floor, per-dimension kernels only)
+  auto set_shape = [&](int t, int r, int p, int pol) -> vegas_status {
+    BatchShape want = *b;
+    want.threads = t;
+    want.rounds = r;
+    want.launch_set = true;
+    want.ppt_req = p;
+    want.small_cap = pol >= 1;
+    want.dense_cap = pol == 2;
+    BK(b, cudaStreamSynchronize(b->stream));
+    return configure(b, want);
+  };
   auto time_shape = [&](int t, int r, int p, int pol, int n, double* out) -> vegas_status {
-    b->small_cap = pol >= 1;
-    b->dense_cap = pol == 2;
-    b->ppt_req = p;
-    vegas_status st = vegas_batch_set_launch(b, t, r);
+    vegas_status st = set_shape(t, r, p, pol);
     double m[2];
     if (!st) st = vegas_batch_profile(b, 1, m);
     if (!st) st = vegas_batch_profile(b, n, m);
@@ -1130,8 +1154,10 @@ vegas_status vegas_batch_autotune(vegas_batch* b, int* threads, int* rounds, dou
   };
   // (columns, where the automatic form is that, beat the buckets' tiles at
   // every measured shape: only the launch shape is left to choose)
-  b->ppt_req = 0;
-  vegas_status st0 = configure(b);
+  BatchShape automatic = *b;
+  automatic.ppt_req = 0;
+  BK(b, cudaStreamSynchronize(b->stream));
+  vegas_status st0 = configure(b, automatic);
   if (st0) return st0;
   const bool cols = b->by_dim && b->cap == 0;
   const std::vector<int> tiles = b->by_dim && !cols ? std::vector<int>{1, 2} : std::vector<int>{0};
@@ -1160,10 +1186,7 @@ vegas_status vegas_batch_autotune(vegas_batch* b, int* threads, int* rounds, dou
     }
   const Cand best = *std::min_element(cands.begin(), cands.end(),
                                       [](const Cand& a, const Cand& c) { return a.ms < c.ms; });
-  b->small_cap = best.pol >= 1;
-  b->dense_cap = best.pol == 2;
-  b->ppt_req = best.p;
-  vegas_status st = vegas_batch_set_launch(b, best.t, best.r);
+  vegas_status st = set_shape(best.t, best.r, best.p, best.pol);
   if (st) return st;
   if (threads) *threads = best.t;
   if (rounds) *rounds = best.r;

@@ -56,3 +56,41 @@ def test_failed_shape_change_keeps_the_context(gv, change):
         assert (gv.vegas_get_launch(ctx), gv.vegas_get_tile(ctx)) != shape
         r, w = gv.bases_integrate(ctx, 2, 0.0, 3, 0.0)[0], want[0][0]
         assert r["I"] == pytest.approx(w["I"], rel=1e-5)
+
+
+@pytest.mark.parametrize("change", ["launch", "tile"])
+@pytest.mark.parametrize("precision,ybits", [("fp32", 24), ("fp64", 53)])
+def test_failed_shape_change_keeps_the_batch(gv, precision, ybits, change):
+    """As above for a batch: items and partial rows grow with fewer rounds per
+    item (or, where a tile brings buckets with fewer rounds, with the tile);
+    shape, graphs, frozen passes and results stay."""
+    insts = wl.genz_batch(6, seed=5, log2n_min=17, log2n_max=18)
+    if change == "tile":  # work enough for 128 rounds with columns
+        insts = wl.genz_batch(40, seed=5, log2n_min=22, log2n_max=22) if precision == "fp32" else insts
+    mk = lambda: gv.vegas_batch_create(insts, nbins=50, seed=1, precision=precision, ybits=ybits)
+
+    def calls(b):
+        gv.vegas_batch_reset(b)
+        return [r["I"] for r in gv.vegas_batch_iterate(b, 2, refine=False)]
+
+    with mk() as b:
+        want = calls(b)
+        shape = gv.vegas_batch_get_launch(b), gv.vegas_batch_get_tile(b)
+        failed = 0
+        for j in range(4):
+            n0 = gv.vegas_alloc_count()
+            gv.vegas_fail_alloc_after(j)
+            try:
+                gv.vegas_batch_set_launch(b, 64, 4) if change == "launch" else gv.vegas_batch_set_tile(b, 2)
+                break
+            except gv.VegasError as e:
+                assert e.status == gv.ENOMEM
+            finally:
+                gv.vegas_fail_alloc_after(-1)
+            failed += 1
+            assert gv.vegas_alloc_count() - n0 == j + 1
+            assert (gv.vegas_batch_get_launch(b), gv.vegas_batch_get_tile(b)) == shape
+            assert calls(b) == want
+        if change == "launch":
+            assert failed == 2 and gv.vegas_batch_get_launch(b)["threads"] == 64
+        assert calls(b) == pytest.approx(want, rel=1e-5)
