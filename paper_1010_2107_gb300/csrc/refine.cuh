@@ -100,6 +100,7 @@ __device__ inline void refine_axis_core(const double* dd, double* ea, double2* t
   const double f1 = __hiloint2double((1023 + h1) << 20, 0), f2 = __hiloint2double((1023 + h2) << 20, 0);
   const unsigned long long Di = team_sum(x > 0.0 ? (unsigned long long)__double2ll_rn(x * f1 * f2) : 0ull, buf[0], t);
   if (Di == 0ull) return;  // every sum zero (uniform across the team)
+  if (64 - __clzll((long long)Di) - sh > 1024) return;  // D = Di 2^-sh not finite, though its terms are
   // q = x / D and r = ((1 - q) / -ln q)^alpha
   double rk = 0.0;
   if (x > 0.0) {

@@ -45,3 +45,21 @@ def test_batched_refinement_of_many_bins(gv, orc):
         gv.vegas_batch_iterate(b, 1)
         edges, bins = gv.vegas_batch_get_grid(b, 0, bin_sums=True)
     assert np.max(np.abs(edges - orc.refine(bins[1], e0))) <= 1e-13
+
+
+@pytest.mark.parametrize("scale,moves", [(1e152, True), (1e153, False)])
+def test_sums_that_overflow_together_leave_the_grid(gv, orc, scale, moves):
+    """Every bin's sum of squares finite, their total past the largest double:
+    the axis is left as it is, as the oracle does; a tenth of it still refines."""
+    src = """
+template <typename T>
+__device__ T vegas_user_f(const T* x, int d, const T* p) { return x[0] < T(0.5) ? p[0] : T(0.1) * p[0]; }
+"""
+    with gv.vegas_create_user(src, 1, [scale], nbins=50, ncall=2000) as ctx:
+        e0 = gv.vegas_get_grid(ctx)
+        gv.vegas_iterate(ctx, 1)
+        edges, bins = gv.vegas_get_grid(ctx, bin_sums=True)
+    assert np.all(np.isfinite(bins[1]))
+    ref = orc.refine(bins[1], e0)
+    assert np.array_equal(ref, e0) == (not moves)
+    assert np.max(np.abs(edges - ref)) <= (1e-13 if moves else 0.0)
