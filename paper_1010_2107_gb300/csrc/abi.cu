@@ -585,14 +585,18 @@ vegas_status configure_launch(vegas_ctx* c) {
   }
   // passes without the per-bin histogram (no refinement) need only the
   // grid table and constants in shared memory: more CTAs may be resident
-  pn.fn = c->ke.sample;
+  pn.fn = c->ke.frozen;
   pn.threads = threads;
   pn.smem = c->ke.smem_nobins(d, N);
   int occ_nb = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_nb, c->ke.sample, threads, pn.smem);
+  e = gv_raise_smem_limit(pn.fn, pn.smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_nb, pn.fn, threads, pn.smem);
   if (e != cudaSuccess) return c->fail(VEGAS_ECUDA, "launch configuration: %s", cudaGetErrorString(e));
   if (c->ctas_per_sm_req > 0) occ_nb = std::min(occ_nb, std::max(c->ctas_per_sm_req, per_sm));
-  pn.occ = std::max(occ_nb, 1);
+  // 32 warps hide the latencies; more CTAs only add rows of totals (each
+  // ends in dependent reductions) and set-up (64 threads, d = 7, 72 bins: 36.0 us
+  // per pass against 40.0 with all that fit)
+  pn.occ = std::max(1, std::min(occ_nb, std::max(32 * 32 / threads, per_sm)));
   const int64_t most_nb = (int64_t)c->sm_count * pn.occ;
   const gv::CubeLanes cl = strat ? gv::balanced_lanes(c->ncubes, c->nc, threads, c->sm_count, c->ppt_min, gv::kMaxCubeParts)
                                  : gv::CubeLanes{1, 1};
@@ -638,18 +642,16 @@ vegas_status configure_launch(vegas_ctx* c) {
 gv::SampleArgs sample_args(const vegas_ctx* c, int it_override, bool nobins = false, int niter = 1) {
   gv::SampleArgs A{};
   const gv::PassShape& ps = nobins ? c->pass_nobins : c->pass_bins;
-  A.nobins = nobins;
   A.d = c->cfg.ndim;
   A.N = c->cfg.nbins;
   A.g = c->g;
   A.ybits = c->ybits;
   A.lanes = ps.lanes;
   A.parts = ps.parts;
+  A.units = (uint32_t)c->ncubes * ps.parts;
+  A.vl = (uint32_t)ps.lanes * ps.parts;
+  A.per_lane = c->strat ? (uint32_t)((c->nc + A.vl - 1) / A.vl) : 0;
   A.niter = niter;
-  {  // the CTAs with a round more than the others
-    const uint64_t lanes = c->strat ? c->ncubes * (uint64_t)ps.lanes * ps.parts : (uint64_t)c->cfg.ncall;
-    A.rot = ps.ctas > 0 ? (uint32_t)((lanes + ps.threads - 1) / ps.threads % ps.ctas) : 0;
-  }
   A.cube_part = c->d_cube_part;
   A.cap = c->cap;
   A.ppt = c->ppt;
@@ -730,7 +732,7 @@ vegas_status launch_pass(vegas_ctx* c, int it_override, int refine, int record, 
   if (record_max) A.cube_max = c->d_cube_max;
   void* args[] = {&A};
   const gv::PassShape& ps = nobins ? c->pass_nobins : c->pass_bins;
-  CK(c, cudaLaunchKernel(ps.fn, dim3(ps.ctas), dim3(ps.threads), args, ps.smem, c->stream));
+  CK(c, cudaLaunchKernel(ps.fn, dim3(ps.ctas, A.niter), dim3(ps.threads), args, ps.smem, c->stream));
   gv::FinArgs F = fin_args(c, refine, record, nobins, combine, niter);
   CK(c, gv_launch_finish(&F, c->stream));
   return VEGAS_OK;
@@ -934,6 +936,8 @@ vegas_status finish_create(vegas_ctx* c, vegas_ctx** out) {
   // the specialised kernel when the shape allows it (see kernels.h)
   if (c->ke.sample_spec && spec_shape(d, c->ke.dm, c->ybits, c->g, N)) {
     c->ke.sample = c->ke.sample_spec;
+    c->ke.frozen = c->ke.frozen_spec;
+    c->ke.max_threads = gv::kSampleMaxThreads<true>;
     c->ppt_min = c->ke.spec_ppt_min;
     if (c->ke.grad_spec) c->ke.grad = c->ke.grad_spec;
   }
@@ -948,12 +952,9 @@ vegas_status finish_create(vegas_ctx* c, vegas_ctx** out) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return bail(c->fail(VEGAS_ECUDA, "no CUDA device: %s", cudaGetErrorString(e)));
   e = gv_prepare_aux_kernels();
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(c->ke.sample, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-  if (e == cudaSuccess && c->col)
-    e = cudaFuncSetAttribute(c->col, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
+  for (const void* f : {c->ke.sample, c->ke.frozen, c->col})
+    if (e == cudaSuccess && f)
+      e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return bail(c->fail(VEGAS_ECUDA, "kernel attributes: %s", cudaGetErrorString(e)));
   if (cfg->stream) {
     c->stream = (cudaStream_t)cfg->stream;
@@ -1507,10 +1508,8 @@ vegas_status vegas_sample_dump(vegas_ctx* c, uint32_t it, const uint64_t* s, int
 
 vegas_status vegas_set_launch(vegas_ctx* c, int threads, int ctas_per_sm) {
   if (!c) return thread_fail(VEGAS_EINVAL, "ctx is NULL");
-  cudaFuncAttributes fa{};
-  CK(c, cudaFuncGetAttributes(&fa, c->ke.sample));
-  if (threads < 64 || threads > fa.maxThreadsPerBlock || threads % 32 != 0)
-    return c->fail(VEGAS_EINVAL, "threads must be a multiple of 32 in 64..%d", fa.maxThreadsPerBlock);
+  if (threads < 64 || threads > c->ke.max_threads || threads % 32 != 0)
+    return c->fail(VEGAS_EINVAL, "threads must be a multiple of 32 in 64..%d", c->ke.max_threads);
   if (ctas_per_sm < 0) return c->fail(VEGAS_EINVAL, "ctas_per_sm < 0");
   CK(c, cudaStreamSynchronize(c->stream));
   const int t0 = c->threads_req, p0 = c->ctas_per_sm_req;
@@ -1902,6 +1901,9 @@ extern "C" vegas_status vegas_eval_noalloc(const vegas_config* cfg, const vegas_
   A.ncubes = (uint32_t)G;
   A.cube_mul = gv::cube_multiplier(G);
   A.parts = 1;
+  A.units = (uint32_t)G;
+  A.vl = (uint32_t)ps.lanes;
+  A.per_lane = (uint32_t)((nc + A.vl - 1) / A.vl);
   A.niter = 1;
   A.g_pow2 = (g & (g - 1)) == 0;
   A.g_log2 = 0;

@@ -366,7 +366,6 @@ struct SampleArgs {
   int cap;                 // bucket capacity per (axis, bin) and tile
   int ppt;                 // points per thread per tile (>= 1)
   int strat;
-  int nobins;              // 1: no per-bin histogram (a pass whose grid is not refined)
   uint32_t key0, key1, instance;
   // Philox round keys of (key0, key1).  On a 16-byte boundary: off it the
   // compiler reads them word by word (k_spring, d = 8: 52 registers, not 48)
@@ -391,8 +390,8 @@ struct SampleArgs {
   double* cube_max;        // [ncubes] running max(0, largest w) (integration phase), or null
   void* cube_part;         // [niter][parts][ncubes] sums of the parts (parts > 1), as `cubes`
   uint32_t parts;          // groups per hypercube, each with its share of the cube's points
-  int niter;               // iterations this launch runs (frozen grid; 1 with the histogram)
-  uint32_t rot;            // CTAs by which each iteration's share of the work is turned
+  uint32_t units, vl, per_lane;  // groups of a pass (hypercubes x parts), lanes of a cube, points per lane
+  int niter;               // iterations this launch runs, one per blockIdx.y (frozen grid; 1 with the histogram)
   int force;               // 1: run even if the ACC test has stopped the last call (evaluation passes)
 };
 
@@ -409,6 +408,7 @@ struct FinArgs {
   double alpha;
   const void* part_bins;
   const double* part_tot;
+  uint32_t units, vl, per_lane;  // groups of a pass (hypercubes x parts), lanes of a cube, points per lane
   int niter;               // iterations of the pass (frozen grid)
   uint32_t parts;          // groups per hypercube; > 1: the totals come from cube_part
   uint32_t cube_mul;

@@ -14,13 +14,20 @@
 
 namespace gv {
 
+// Threads per CTA a sampling kernel may be launched with: the specialised
+// kernels up to 512 (larger tiles for many cells), the general ones 256
+// (their register budget).
+template <bool SPEC>
+constexpr int kSampleMaxThreads = SPEC ? 512 : 256;
+
 #ifndef __CUDACC_RTC__  // host side only (run-time compiled kernels see the argument blocks)
 
 // One compiled sampling kernel and its companions for a (kind, precision, DM).
 struct KernelEntry {
-  const void* sample;                 // k_sample<T, DM, F, ACC, YB, false> (any d <= DM)
-  const void* sample_spec;            // k_sample<..., true>: d == DM, 24-bit, power-of-two
-                                      // divisions with g N <= 256; may be null
+  const void* sample;                 // k_sample<T, DM, F, ACC, YB, false, true> (any d <= DM)
+  const void* frozen;                 // ... <..., false, false>: passes without the per-bin sums
+  const void* sample_spec;            // <..., true, true> and <..., true, false>: d == DM, 24-bit,
+  const void* frozen_spec;            // power-of-two divisions with g N <= 256; may be null
   const void* sample_col;             // k_sample_col<DM, F, false>: the FP32 form with 24-bit words,
                                       // column histogram (any d <= DM, the divisions of sample_spec); or null
   const void* sample_col_exact;       // k_sample_col<DM, F, true>: d == DM
@@ -30,6 +37,7 @@ struct KernelEntry {
                                           // with bucket capacity cap
   size_t (*smem_nobins)(int d, int N);    // ... of a pass without the histogram
   int dm;                             // compile-time dimension bound
+  int max_threads;                    // threads per CTA `sample` and `frozen` may be launched with
   int spec_ppt_min;                   // `sample_spec` evaluates this many points per
                                       // thread at a time: tiles are multiples of it
   const void* grad;                   // k_grad<T, DM, F, YB> or null

@@ -83,7 +83,7 @@ const Nvrtc* nvrtc(std::string* why) {
 }
 
 // Kernels of one program: which are built and their names.
-enum { K_SAMPLE = 0, K_SPRING = 1, K_DUMP = 2, K_COL = 3, K_COUNT = 4 };
+enum { K_SAMPLE = 0, K_FROZEN = 1, K_SPRING = 2, K_DUMP = 3, K_COL = 4, K_COUNT = 5 };
 
 struct Shape {
   int prec, ybits, d;
@@ -111,8 +111,9 @@ std::string name_expr(int k, const Shape& s) {
   const std::string sp = s.spec ? "true" : "false";
   switch (k) {
     case K_SAMPLE:
+    case K_FROZEN:
       return "&gv::k_sample<" + T + ", " + D + ", gv::UserIntegrand, " + std::to_string(acc_of(s.prec)) + ", " + Y +
-             ", " + sp + ">";
+             ", " + sp + (k == K_SAMPLE ? ", true>" : ", false>");
     case K_COL:
       return "&gv::k_sample_col<" + D + ", gv::UserIntegrand, true>";
     case K_SPRING:
@@ -304,7 +305,9 @@ int rtc_user_entry(const char* source, int prec, int ybits, int d, bool spec, Ke
   }
   KernelEntry ke{};
   ke.sample = (const void*)k[K_SAMPLE];
+  ke.frozen = (const void*)k[K_FROZEN];
   ke.sample_spec = s.spec ? ke.sample : nullptr;
+  ke.frozen_spec = s.spec ? ke.frozen : nullptr;
   ke.spring = (const void*)k[K_SPRING];
   ke.spring_spec = s.spec ? ke.spring : nullptr;
   ke.dump = (const void*)k[K_DUMP];
@@ -316,6 +319,7 @@ int rtc_user_entry(const char* source, int prec, int ybits, int d, bool spec, Ke
                                    : (prec == VG_FP32_ACC64 ? &sample_smem_nobins<float, 1>
                                                             : &sample_smem_nobins<float, 2>);
   ke.dm = d;
+  ke.max_threads = s.spec ? kSampleMaxThreads<true> : kSampleMaxThreads<false>;
   ke.spec_ppt_min = spec_ppt_min(s);
   ke.grad = ke.grad_spec = nullptr;
   ke.grad_nt = 0;

@@ -391,16 +391,29 @@ __device__ __forceinline__ fpair warp_sum(fpair p) {
   return p;
 }
 
-// The CTA's totals (compensated pairs per thread) into its column of
-// part_tot: fixed butterflies, then the warps in order.
-__device__ __forceinline__ void store_totals(const SampleArgs& A, const fpair (&tp)[4], int nonfinite) {
-  __shared__ double wnf[32];
-  __shared__ fpair wpair[32][4];
+// Warps of a sampling kernel's CTA, at most.
+constexpr int kMaxSampleWarps = 16;
+
+// The CTA's totals (compensated pairs or doubles per thread) into its column
+// of part_tot: fixed butterflies, then the warps in order.
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  return v;
+}
+__device__ __forceinline__ void tot_merge(fpair& a, const fpair& b) { comp_merge(a, b); }
+__device__ __forceinline__ void tot_merge(double& a, double b) { a += b; }
+__device__ __forceinline__ double tot_value(const fpair& a) { return comp_value(a); }
+__device__ __forceinline__ double tot_value(double a) { return a; }
+template <typename S>  // fpair or double
+__device__ __forceinline__ void store_totals(const SampleArgs& A, double* part_tot, const S (&t)[4], int nonfinite) {
+  __shared__ double wnf[kMaxSampleWarps];
+  __shared__ S wtot[kMaxSampleWarps][4];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const fpair v = warp_sum(tp[q]);
-    if (lane == 0) wpair[warp][q] = v;
+  for (int q = 0; q < 4; ++q) {  // (the hypercubes' two are zero without strata: no butterfly for them)
+    const S v = q < 2 || A.strat ? warp_sum(t[q]) : S{};
+    if (lane == 0) wtot[warp][q] = v;
   }
   int nf = nonfinite;
 #pragma unroll
@@ -410,46 +423,73 @@ __device__ __forceinline__ void store_totals(const SampleArgs& A, const fpair (&
   if (tid < 5) {
     double acc = 0.0;
     if (tid < 4) {
-      fpair p{0.f, 0.f};
-      for (int w = 0; w < nw; ++w) comp_merge(p, wpair[w][tid]);
-      acc = comp_value(p);
+      S p{};
+      for (int w = 0; w < nw; ++w) tot_merge(p, wtot[w][tid]);
+      acc = tot_value(p);
     } else {
       for (int w = 0; w < nw; ++w) acc += wnf[w];
     }
-    A.part_tot[(size_t)tid * A.nparts + blockIdx.x] = acc;
+    part_tot[(size_t)tid * A.nparts + blockIdx.x] = acc;
   }
 }
 
-// Threads per CTA a sampling kernel may be launched with: the specialised
-// kernels up to 512 (larger tiles for many cells), the general ones 256
-// (their register budget).
-template <bool SPEC>
-constexpr int kSampleMaxThreads = SPEC ? 512 : 256;
-constexpr int kMaxSampleWarps = 16;
-// CTAs of the largest size that must fit an SM (0: the compiler's choice): 64
-// registers for the specialised kernels of low dimension (four CTAs of 256
-// threads in the frozen-grid passes, 78 registers and three without it), 80
-// for the general FP32 ones (106 and two CTAs without it; up to 16 axes 128).
-template <typename T, int DM, bool SPEC>
-constexpr int kSampleMinBlocks =
-    DM > 16 || !std::is_same<T, float>::value ? 0 : (DM > 8 ? (SPEC ? 0 : 2) : (SPEC ? 2 : 3));
+// CTAs of the largest size that must fit an SM (0: the compiler's choice), for
+// the light integrands; RAMBO needs up to 255 registers and a user's integrand
+// what it needs.
+// FP64, up to 16 axes: two (128 registers).  Left to itself the compiler holds
+// some of these kernels to 64 or 80 and spills for a third CTA, which the FP64
+// pipe has no use for.
+template <template <typename, int> class F> constexpr bool kLight = false;
+template <> constexpr bool kLight<GenzGaussian> = true;
+template <> constexpr bool kLight<GenzProductPeak> = true;
+template <> constexpr bool kLight<GenzCornerPeak> = true;
+template <> constexpr bool kLight<GenzOscillatory> = true;
+template <> constexpr bool kLight<GenzContinuous> = true;
+template <> constexpr bool kLight<GenzDiscontinuous> = true;
+template <> constexpr bool kLight<DoubleGaussian> = true;
+template <> constexpr bool kLight<WMuNu> = true;
+template <typename T, int DM, template <typename, int> class F, bool SPEC>
+constexpr int kSampleMinBlocks = std::is_same<T, double>::value && DM <= 16 && kLight<F> ? (SPEC ? 1 : 2) : 0;
 
-template <typename T, int DM, template <typename, int> class F, int ACC, int YB, bool SPEC>
-__global__ void __launch_bounds__(kSampleMaxThreads<SPEC>, kSampleMinBlocks<T, DM, SPEC>) k_sample(const SampleArgs A) {
+// Threads a kernel is compiled for: kSampleMaxThreads, but 336 for the FP32
+// form with 53-bit words and the histogram in 5 to 8 dimensions.  Compiled for
+// 256 it takes 92 to 95 registers and two CTAs per SM, for 336 73 to 79 and
+// three (it is launched with 256 at most).  Two-peak Gaussian, 2^20 points, us
+// at (d, N) = (6, 50), (8, 20), (8, 50), (8, 200): 33.7, 40.4, 41.3, 66.4
+// against 36.9, 43.8, 43.5, 65.5; with three CTAs as launch bounds 35.4, 41.8,
+// 42.0, 70.
+template <int DM, template <typename, int> class F, int ACC, int YB, bool SPEC, bool BINS>
+constexpr int kSampleBound = ACC == 2 && YB == 53 && DM == 8 && BINS && kLight<F> ? 336 : kSampleMaxThreads<SPEC>;
+
+// BINS: with the per-bin sums, which feed only the grid refinement (step 5).  A
+// pass that does not refine (the integration phase of BASES, a frozen-grid
+// VEGAS call) keeps its estimate, cube sums and maxima alone, and several
+// such iterations may share a launch, one per blockIdx.y: the CTAs of the next
+// fill the SMs as those of one end.  A kernel each, because the two need
+// registers of their own: one kernel for both, with a loop over the iterations
+// that share a launch, spilled and held the frozen pass to the histogram's
+// occupancy (us per single frozen pass of 2^20 points, one kernel -> two: Genz
+// Gaussian d = 8 19.8 -> 17.2, RAMBO 2 -> 3 with FP64 sums 70 -> 52, d = 8 with
+// 53 bits 46 -> 40).
+template <typename T, int DM, template <typename, int> class F, int ACC, int YB, bool SPEC, bool BINS>
+__global__ void __launch_bounds__(kSampleBound<DM, F, ACC, YB, SPEC, BINS>, kSampleMinBlocks<T, DM, F, SPEC>)
+    k_sample(const SampleArgs A) {
   using H = typename AccTraits<ACC>::H;
   using T2 = typename Vec2<T>::type;
   using L = SmemLayout<T, ACC>;
   constexpr bool COMP = ACC == 2;  // FP32 throughout, no FP64 in the loop
+  const bool maxima = !BINS && A.cube_max;  // the integration phase of BASES
   // the ACC test stopped this call (device-side): no pass, and k_finish
   // then skips it too (it reads `live`, nothing else here writes it)
   const int stop = A.force ? 0 : A.st->done;
-  if (blockIdx.x == 0 && threadIdx.x == 0) A.st->live = !stop;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) A.st->live = !stop;
   if (stop) return;
-  uint32_t it = A.it_override >= 0 ? (uint32_t)A.it_override : A.st->it;
+  // (a launch of several frozen-grid iterations: one per blockIdx.y)
+  const uint32_t it = (A.it_override >= 0 ? (uint32_t)A.it_override : A.st->it) + blockIdx.y;
   // SPEC: d equals the compile-time bound DM, 24-bit words and power-of-two
   // hypercube divisions with g N <= 256: every per-axis guard folds away.
   const int d = SPEC ? DM : A.d, N = A.N, dN = d * N, cap = A.cap;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
 
   extern __shared__ __align__(16) unsigned char smem[];
   T2* tab = reinterpret_cast<T2*>(smem);
@@ -465,11 +505,7 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>, kSampleMinBlocks<T, D
     if (ntab) ntab[i] = T(N) * gtab[i].y;
   }
   for (int i = tid; i < kNumDerived; i += blockDim.x) P[i] = (T)A.dparams[i];
-  // Per-bin sums feed only the grid refinement (step 5); a pass that does
-  // not refine (the integration phase of BASES, a frozen-grid VEGAS call)
-  // keeps its estimate, cube sums and maxima and skips the histogram.
-  const bool bins = !A.nobins;
-  if (bins) {
+  if constexpr (BINS) {
     hist.zero_buckets(tid, blockDim.x, dN);
     hist.zero(tid, blockDim.x);
   }
@@ -503,47 +539,130 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>, kSampleMinBlocks<T, D
   // FP64 (ACC 0/1) or compensated FP32 pairs (ACC 2).
   double t[4] = {0.0, 0.0, 0.0, 0.0};
   fpair tp[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-  // The CTA's place in the order of the work: its row of partial sums.  A
-  // launch of several frozen-grid iterations turns the places by A.rot from
-  // one to the next, so that the CTAs with one round more than the others
-  // change; a place's work and row are the same in every launch.
-  uint32_t place = blockIdx.x;
-  int iter = 0;
-  bool last_iter = true;
-  // The pass loop, compiled twice: with the per-bin histogram and without
-  // it (a uniform choice per launch; no test inside the loops).
-  auto pass = [&](auto with_bins) {
-    constexpr bool B = decltype(with_bins)::value;
-    auto scatter = [&](const int (&kb)[DM], H w) {
-      if constexpr (B) hist.template scatter<DM>(kb, d, w);
-    };
-    auto gather = [&]() {
-      if constexpr (B) hist.gather(tid, blockDim.x);
-    };
-    if (!A.strat) {
-      Run<ACC> sw, sw2;
-      H pmax = H(0);  // largest weight (integration-phase maximum of the one cube)
-      const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-      const uint64_t first = (uint64_t)place * blockDim.x;
-      const uint64_t rounds = first < A.ncall ? (A.ncall - first + stride - 1) / stride : 0;
-      uint64_t s = first + tid;
-      int pend = 0;  // points per thread since the last gather (uniform in the CTA)
+  auto scatter = [&](const int (&kb)[DM], H w) {
+    if constexpr (BINS) hist.template scatter<DM>(kb, d, w);
+  };
+  auto gather = [&]() {
+    if constexpr (BINS) hist.gather(tid, blockDim.x);
+  };
+  if (!A.strat) {
+    Run<ACC> sw, sw2;
+    H pmax = H(0);  // largest weight (integration-phase maximum of the one cube)
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    const uint64_t first = (uint64_t)blockIdx.x * blockDim.x;
+    const uint64_t rounds = first < A.ncall ? (A.ncall - first + stride - 1) / stride : 0;
+    uint64_t s = first + tid;
+    int pend = 0;  // points per thread since the last gather (uniform in the CTA)
+    if constexpr (PAIR) {
+      for (uint64_t r = 0; r < rounds; r += 2, s += 2 * stride) {
+        const bool v0 = s < A.ncall, v1 = s + stride < A.ncall;
+        int kb0[DM], kb1[DM];
+        const H w0 = eval_point((uint32_t)s, kb0, v0);
+        const H w1 = eval_point((uint32_t)(s + stride), kb1, v1);
+        if (v0) {
+          sw.add(w0);
+          sw2.add(w0 * w0);
+          if (maxima) pmax = max(pmax, w0);
+          scatter(kb0, w0);
+        }
+        if (v1) {
+          sw.add(w1);
+          sw2.add(w1 * w1);
+          if (maxima) pmax = max(pmax, w1);
+          scatter(kb1, w1);
+        }
+        if ((pend += 2) >= A.ppt) {
+          gather();
+          pend = 0;
+        }
+      }
+    } else {
+      for (uint64_t r = 0; r < rounds; ++r, s += stride) {
+        if (s < A.ncall) {
+          int kb[DM];
+          const H w = eval_point((uint32_t)s, kb);
+          sw.add(w);
+          sw2.add(w * w);
+          if (maxima) pmax = max(pmax, w);
+          scatter(kb, w);
+        }
+        if (++pend == A.ppt) {
+          gather();
+          pend = 0;
+        }
+      }
+    }
+    if (pend) gather();
+    if (maxima) {  // non-negative doubles order as their bit patterns
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) pmax = max(pmax, __shfl_xor_sync(0xffffffffu, pmax, off));
+      if (lane == 0 && pmax > H(0))
+        atomicMax(reinterpret_cast<unsigned long long*>(A.cube_max),
+                  (unsigned long long)__double_as_longlong((double)pmax));
+    }
+    if constexpr (COMP) {
+      tp[0] = sw.p;
+      tp[1] = sw2.p;
+    } else {
+      t[0] = sw.value();
+      t[1] = sw2.value();
+    }
+  } else {
+    // Groups of Lw lanes share a hypercube, or one of its A.parts parts
+    // where the cubes are too few to fill the GPU; of the A.vl = Lw parts
+    // lanes of a cube, lane j takes its points j, j + A.vl, ... in lock-step
+    // with the rest of the CTA (one tile per step); the group then reduces
+    // its sums with a fixed xor-butterfly (deterministic).  Group i takes
+    // part i div ncubes of the cube in place i mod ncubes (cube_of).
+    const int Lw = A.lanes;
+    const uint32_t groups_per_cta = blockDim.x / Lw;
+    const uint32_t gstride = gridDim.x * groups_per_cta;
+    const uint32_t gfirst = blockIdx.x * groups_per_cta;
+    const uint32_t rounds = gfirst < A.units ? (A.units - gfirst + gstride - 1) / gstride : 0;
+    uint32_t gi = gfirst + tid / Lw;
+    int pend = 0;  // points per thread since the last gather (uniform in the CTA)
+    for (uint32_t r = 0; r < rounds; ++r, gi += gstride) {
+      const bool live = gi < A.units;  // uniform within a group
+      // (SPEC: a power of two of cubes, so that both are bit fields of gi)
+      const uint32_t part = SPEC ? gi >> __popc(A.ncubes - 1u) : (A.parts > 1u ? gi / A.ncubes : 0u);
+      const uint32_t c = SPEC ? (gi * A.cube_mul) & (A.ncubes - 1u) : cube_of(A.ncubes, A.cube_mul, gi - part * A.ncubes);
+      const uint32_t gl = part * Lw + (tid & (Lw - 1));
+      if (live) {
+        uint32_t rest = c;
+#pragma unroll
+        for (int a = 0; a < DM; ++a)
+          if (a < d) {
+            if (A.g_pow2) {
+              cd[a] = (int)(rest & (uint32_t)(A.g - 1));
+              rest >>= A.g_log2;
+            } else {
+              cd[a] = (int)(rest % (uint32_t)A.g);
+              rest /= (uint32_t)A.g;
+            }
+          }
+      }
+      const uint32_t s0 = c * A.nc;
+      // a lane's chain of points in one cube is short: plain sums in H,
+      // compensated merges across the group; pmax: the largest weight (for
+      // the per-cube maxima of the integration phase)
+      H p1 = H(0), p2 = H(0), pmax = H(0);
       if constexpr (PAIR) {
-        for (uint64_t r = 0; r < rounds; r += 2, s += 2 * stride) {
-          const bool v0 = s < A.ncall, v1 = s + stride < A.ncall;
+        for (uint32_t i = 0; i < A.per_lane; i += 2) {
+          const uint32_t j0 = gl + i * A.vl, j1 = j0 + A.vl;
+          const bool v0 = live && j0 < A.nc, v1 = live && j1 < A.nc;
           int kb0[DM], kb1[DM];
-          const H w0 = eval_point((uint32_t)s, kb0, v0);
-          const H w1 = eval_point((uint32_t)(s + stride), kb1, v1);
+          const H w0 = eval_point(s0 + j0, kb0, v0);
+          const H w1 = eval_point(s0 + j1, kb1, v1);
           if (v0) {
-            sw.add(w0);
-            sw2.add(w0 * w0);
-            if (A.cube_max) pmax = max(pmax, w0);
+            p1 += w0;
+            p2 += w0 * w0;
+            if (maxima) pmax = max(pmax, w0);
             scatter(kb0, w0);
           }
           if (v1) {
-            sw.add(w1);
-            sw2.add(w1 * w1);
-            if (A.cube_max) pmax = max(pmax, w1);
+            p1 += w1;
+            p2 += w1 * w1;
+            if (maxima) pmax = max(pmax, w1);
             scatter(kb1, w1);
           }
           if ((pend += 2) >= A.ppt) {
@@ -552,13 +671,14 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>, kSampleMinBlocks<T, D
           }
         }
       } else {
-        for (uint64_t r = 0; r < rounds; ++r, s += stride) {
-          if (s < A.ncall) {
+        uint32_t j = gl;
+        for (uint32_t i = 0; i < A.per_lane; ++i, j += A.vl) {
+          if (live && j < A.nc) {
             int kb[DM];
-            const H w = eval_point((uint32_t)s, kb);
-            sw.add(w);
-            sw2.add(w * w);
-            if (A.cube_max) pmax = max(pmax, w);
+            const H w = eval_point(s0 + j, kb);
+            p1 += w;
+            p2 += w * w;
+            if (maxima) pmax = max(pmax, w);
             scatter(kb, w);
           }
           if (++pend == A.ppt) {
@@ -567,222 +687,73 @@ __global__ void __launch_bounds__(kSampleMaxThreads<SPEC>, kSampleMinBlocks<T, D
           }
         }
       }
-      if (pend) gather();
-      if (A.cube_max) {  // non-negative doubles order as their bit patterns
-  #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) pmax = max(pmax, __shfl_xor_sync(0xffffffffu, pmax, off));
-        if (lane == 0 && pmax > H(0))
-          atomicMax(reinterpret_cast<unsigned long long*>(A.cube_max),
-                    (unsigned long long)__double_as_longlong((double)pmax));
+      if (maxima) {  // integration phase: per-cube maxima
+        for (int off = Lw >> 1; off > 0; off >>= 1) pmax = max(pmax, __shfl_xor_sync(0xffffffffu, pmax, off, Lw));
+        if (live && (tid & (Lw - 1)) == 0) {
+          // (several parts, or several iterations of one launch, may meet:
+          // non-negative doubles order as their bit patterns)
+          if (A.parts > 1u || A.niter > 1) {
+            if (pmax > H(0))
+              atomicMax(reinterpret_cast<unsigned long long*>(A.cube_max + c),
+                        (unsigned long long)__double_as_longlong((double)pmax));
+          } else {
+            A.cube_max[c] = fmax(A.cube_max[c], (double)pmax);
+          }
+        }
       }
       if constexpr (COMP) {
-        tp[0] = sw.p;
-        tp[1] = sw2.p;
+        fpair c1{p1, 0.f}, c2{p2, 0.f};
+        for (int off = Lw >> 1; off > 0; off >>= 1) {
+          fpair o1, o2;
+          o1.hi = __shfl_xor_sync(0xffffffffu, c1.hi, off, Lw);
+          o1.lo = __shfl_xor_sync(0xffffffffu, c1.lo, off, Lw);
+          o2.hi = __shfl_xor_sync(0xffffffffu, c2.hi, off, Lw);
+          o2.lo = __shfl_xor_sync(0xffffffffu, c2.lo, off, Lw);
+          comp_merge(c1, o1);
+          comp_merge(c2, o2);
+        }
+        if (live && (tid & (Lw - 1)) == 0) {
+          if (A.parts > 1u) {
+            cube_store(A.cube_part, (size_t)blockIdx.y * A.units + gi, c1, c2);
+          } else {
+            cube_totals(A.inv_nc, A.inv_nc1, c1, c2, tp);
+            if (A.cubes && blockIdx.y == gridDim.y - 1) cube_store(A.cubes, c, c1, c2);
+          }
+        }
       } else {
-        t[0] = sw.value();
-        t[1] = sw2.value();
-      }
-    } else {
-      // Groups of Lw lanes share a hypercube, or one of its A.parts parts
-      // where the cubes are too few to fill the GPU; of the VL = Lw parts
-      // lanes of a cube, lane j takes its points j, j + VL, ... in lock-step
-      // with the rest of the CTA (one tile per step); the group then reduces
-      // its sums with a fixed xor-butterfly (deterministic).  Group i takes
-      // part i div ncubes of the cube in place i mod ncubes (cube_of).
-      const int Lw = A.lanes;
-      const uint32_t units = A.ncubes * A.parts, VL = (uint32_t)Lw * A.parts;
-      const uint32_t groups_per_cta = blockDim.x / Lw;
-      const uint32_t gstride = gridDim.x * groups_per_cta;
-      const uint32_t gfirst = place * groups_per_cta;
-      const uint32_t rounds = gfirst < units ? (units - gfirst + gstride - 1) / gstride : 0;
-      const uint32_t per_lane = (A.nc + VL - 1) / VL;
-      uint32_t gi = gfirst + tid / Lw;
-      int pend = 0;  // points per thread since the last gather (uniform in the CTA)
-      for (uint32_t r = 0; r < rounds; ++r, gi += gstride) {
-        const bool live = gi < units;  // uniform within a group
-        const uint32_t part = A.parts > 1u ? gi / A.ncubes : 0u;
-        const uint32_t c = cube_of(A.ncubes, A.cube_mul, gi - part * A.ncubes);
-        const uint32_t gl = part * Lw + (tid & (Lw - 1));
-        if (live) {
-          uint32_t rest = c;
-  #pragma unroll
-          for (int a = 0; a < DM; ++a)
-            if (a < d) {
-              if (A.g_pow2) {
-                cd[a] = (int)(rest & (uint32_t)(A.g - 1));
-                rest >>= A.g_log2;
-              } else {
-                cd[a] = (int)(rest % (uint32_t)A.g);
-                rest /= (uint32_t)A.g;
-              }
-            }
+        double c1 = p1, c2 = p2;
+        for (int off = Lw >> 1; off > 0; off >>= 1) {
+          c1 += __shfl_xor_sync(0xffffffffu, c1, off, Lw);
+          c2 += __shfl_xor_sync(0xffffffffu, c2, off, Lw);
         }
-        const uint32_t s0 = c * A.nc;
-        // a lane's chain of points in one cube is short: plain sums in H,
-        // compensated merges across the group; pmax: the largest weight (for
-        // the per-cube maxima of the integration phase)
-        H p1 = H(0), p2 = H(0), pmax = H(0);
-        if constexpr (PAIR) {
-          for (uint32_t i = 0; i < per_lane; i += 2) {
-            const uint32_t j0 = gl + i * VL, j1 = j0 + VL;
-            const bool v0 = live && j0 < A.nc, v1 = live && j1 < A.nc;
-            int kb0[DM], kb1[DM];
-            const H w0 = eval_point(s0 + j0, kb0, v0);
-            const H w1 = eval_point(s0 + j1, kb1, v1);
-            if (v0) {
-              p1 += w0;
-              p2 += w0 * w0;
-              if (A.cube_max) pmax = max(pmax, w0);
-              scatter(kb0, w0);
-            }
-            if (v1) {
-              p1 += w1;
-              p2 += w1 * w1;
-              if (A.cube_max) pmax = max(pmax, w1);
-              scatter(kb1, w1);
-            }
-            if ((pend += 2) >= A.ppt) {
-              gather();
-              pend = 0;
-            }
-          }
-        } else {
-          for (uint32_t i = 0; i < per_lane; ++i) {
-            const uint32_t j = gl + i * VL;
-            if (live && j < A.nc) {
-              int kb[DM];
-              const H w = eval_point(s0 + j, kb);
-              p1 += w;
-              p2 += w * w;
-              if (A.cube_max) pmax = max(pmax, w);
-              scatter(kb, w);
-            }
-            if (++pend == A.ppt) {
-              gather();
-              pend = 0;
-            }
-          }
-        }
-        if (A.cube_max) {  // integration phase: per-cube maxima
-          for (int off = Lw >> 1; off > 0; off >>= 1) pmax = max(pmax, __shfl_xor_sync(0xffffffffu, pmax, off, Lw));
-          if (live && (tid & (Lw - 1)) == 0) {
-            // (several parts, or several iterations of one launch, may meet:
-            // non-negative doubles order as their bit patterns)
-            if (A.parts > 1u || A.niter > 1) {
-              if (pmax > H(0))
-                atomicMax(reinterpret_cast<unsigned long long*>(A.cube_max + c),
-                          (unsigned long long)__double_as_longlong((double)pmax));
-            } else {
-              A.cube_max[c] = fmax(A.cube_max[c], (double)pmax);
-            }
-          }
-        }
-        if constexpr (COMP) {
-          fpair c1{p1, 0.f}, c2{p2, 0.f};
-          for (int off = Lw >> 1; off > 0; off >>= 1) {
-            fpair o1, o2;
-            o1.hi = __shfl_xor_sync(0xffffffffu, c1.hi, off, Lw);
-            o1.lo = __shfl_xor_sync(0xffffffffu, c1.lo, off, Lw);
-            o2.hi = __shfl_xor_sync(0xffffffffu, c2.hi, off, Lw);
-            o2.lo = __shfl_xor_sync(0xffffffffu, c2.lo, off, Lw);
-            comp_merge(c1, o1);
-            comp_merge(c2, o2);
-          }
-          if (live && (tid & (Lw - 1)) == 0) {
-            if (A.parts > 1u) {
-              cube_store(A.cube_part, (size_t)iter * units + gi, c1, c2);
-            } else {
-              cube_totals(A.inv_nc, A.inv_nc1, c1, c2, tp);
-              if (A.cubes && last_iter) cube_store(A.cubes, c, c1, c2);
-            }
-          }
-        } else {
-          double c1 = p1, c2 = p2;
-          for (int off = Lw >> 1; off > 0; off >>= 1) {
-            c1 += __shfl_xor_sync(0xffffffffu, c1, off, Lw);
-            c2 += __shfl_xor_sync(0xffffffffu, c2, off, Lw);
-          }
-          if (live && (tid & (Lw - 1)) == 0) {
-            if (A.parts > 1u) {
-              cube_store(A.cube_part, (size_t)iter * units + gi, c1, c2);
-            } else {
-              cube_totals(A.inv_nc, A.inv_nc1, c1, c2, t);
-              if (A.cubes && last_iter) cube_store(A.cubes, c, c1, c2);
-            }
+        if (live && (tid & (Lw - 1)) == 0) {
+          if (A.parts > 1u) {
+            cube_store(A.cube_part, (size_t)blockIdx.y * A.units + gi, c1, c2);
+          } else {
+            cube_totals(A.inv_nc, A.inv_nc1, c1, c2, t);
+            if (A.cubes && blockIdx.y == gridDim.y - 1) cube_store(A.cubes, c, c1, c2);
           }
         }
       }
-      if (pend) gather();
     }
-  };
-  // The totals of an iteration, one entry per warp and column: compensated
-  // pairs (COMP) or doubles, and the non-finite count.
-  __shared__ double wone[kMaxSampleWarps][5];
-  double(*wtot)[5] = bins ? wone : reinterpret_cast<double(*)[5]>(smem + L::hist(dN));
-  auto warp_totals = [&]() {
-    double* out = wtot[iter * nw + warp];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if constexpr (COMP) {
-        const fpair v = warp_sum(tp[q]);
-        if (lane == 0) *reinterpret_cast<float2*>(out + q) = make_float2(v.hi, v.lo);
-        tp[q] = fpair{0.f, 0.f};
-      } else {
-        double v = t[q];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if (lane == 0) out[q] = v;
-        t[q] = 0.0;
-      }
-    }
-    int nf = nonfinite;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) nf += __shfl_xor_sync(0xffffffffu, nf, off);
-    if (lane == 0) out[4] = (double)nf;
-    nonfinite = 0;
-  };
-  if (bins) {
-    pass(BoolTag<true>{});
-    warp_totals();
-  } else {
-    for (; iter < A.niter; ++iter, ++it) {
-      place = (blockIdx.x + (uint32_t)iter * A.rot) % gridDim.x;
-      last_iter = iter == A.niter - 1;
-      pass(BoolTag<false>{});
-      warp_totals();
-    }
+    if (pend) gather();
   }
-  __syncthreads();
 
   // Partial row of this CTA: histogram cells (FP64, or compensated FP32
   // pairs) including the overflow cells, then the totals.
-  const int row = blockIdx.x;
-  for (int i = tid; bins && i < 2 * dN; i += blockDim.x) {
+  for (int i = tid; BINS && i < 2 * dN; i += blockDim.x) {
     if constexpr (COMP) {
       const fpair p = hist.pair(i);
-      reinterpret_cast<float2*>(A.part_bins)[(size_t)row * 2 * dN + i] = make_float2(p.hi, p.lo);
+      reinterpret_cast<float2*>(A.part_bins)[(size_t)blockIdx.x * 2 * dN + i] = make_float2(p.hi, p.lo);
     } else {
-      reinterpret_cast<double*>(A.part_bins)[(size_t)row * 2 * dN + i] = hist.value(i);
+      reinterpret_cast<double*>(A.part_bins)[(size_t)blockIdx.x * 2 * dN + i] = hist.value(i);
     }
   }
-
-  for (int i = tid; i < 5 * A.niter; i += blockDim.x) {
-    const int j = i / 5, q = i - 5 * j;
-    const double(*v)[5] = wtot + j * nw;
-    double acc = 0.0;
-    if (COMP && q < 4) {
-      fpair p{0.f, 0.f};
-      for (int w = 0; w < nw; ++w) {
-        const float2 u = *reinterpret_cast<const float2*>(&v[w][q]);
-        comp_merge(p, fpair{u.x, u.y});
-      }
-      acc = comp_value(p);
-    } else {
-      for (int w = 0; w < nw; ++w) acc += v[w][q];
-    }
-    const uint32_t at = (blockIdx.x + (uint32_t)j * A.rot) % gridDim.x;
-    A.part_tot[((size_t)j * kTotCols + q) * A.nparts + at] = acc;
-  }
+  double* part_tot = A.part_tot + (size_t)blockIdx.y * kTotCols * A.nparts;
+  if constexpr (COMP)
+    store_totals(A, part_tot, tp, nonfinite);
+  else
+    store_totals(A, part_tot, t, nonfinite);
 }
 
 // ---------------------------------------------------------------------------
@@ -944,15 +915,13 @@ __global__ void __launch_bounds__(512, 1) k_sample_col(const SampleArgs A) {
   } else {
     // groups of Lw lanes share a hypercube or a part of it, as in k_sample
     const int Lw = A.lanes;
-    const uint32_t units = A.ncubes * A.parts, VL = (uint32_t)Lw * A.parts;
     const uint32_t groups_per_cta = blockDim.x / Lw;
     const uint32_t gstride = gridDim.x * groups_per_cta;
     const uint32_t gfirst = blockIdx.x * groups_per_cta;
-    const uint32_t rounds = gfirst < units ? (units - gfirst + gstride - 1) / gstride : 0;
-    const uint32_t per_lane = (A.nc + VL - 1) / VL;
+    const uint32_t rounds = gfirst < A.units ? (A.units - gfirst + gstride - 1) / gstride : 0;
     uint32_t gi = gfirst + tid / Lw;
     for (uint32_t r = 0; r < rounds; ++r, gi += gstride) {
-      const bool live = gi < units;  // uniform within a group
+      const bool live = gi < A.units;  // uniform within a group
       const uint32_t part = A.parts > 1u ? gi / A.ncubes : 0u;
       const uint32_t c = cube_of(A.ncubes, A.cube_mul, gi - part * A.ncubes);
       const uint32_t gl = part * Lw + (tid & (Lw - 1));
@@ -965,13 +934,13 @@ __global__ void __launch_bounds__(512, 1) k_sample_col(const SampleArgs A) {
         }
       const uint32_t s0 = c * A.nc;
       float p1 = 0.f, p2 = 0.f;
-      for (uint32_t i = 0; i < per_lane; i += PIF) {
+      for (uint32_t i = 0; i < A.per_lane; i += PIF) {
         uint32_t sq[PIF];
         bool v[PIF];
         float w[PIF];
 #pragma unroll
         for (int q = 0; q < PIF; ++q) {
-          const uint32_t j = gl + (i + q) * VL;
+          const uint32_t j = gl + (i + q) * A.vl;
           sq[q] = s0 + j;
           v[q] = live && j < A.nc;
         }
@@ -1004,7 +973,7 @@ __global__ void __launch_bounds__(512, 1) k_sample_col(const SampleArgs A) {
   }
   hist.drain();
   fold();
-  store_totals(A, tp, nonfinite);
+  store_totals(A, A.part_tot, tp, nonfinite);
 }
 
 template <typename T, int ACC>
@@ -1013,8 +982,7 @@ __host__ __device__ inline size_t sample_smem_bytes(int d, int N, int cap) {
 }
 template <typename T, int ACC>
 __host__ __device__ inline size_t sample_smem_nobins(int d, int N) {
-  // (behind the table and the constants: the iterations' totals per warp)
-  return SmemLayout<T, ACC>::hist(d * N) + sizeof(double) * 5 * kMaxSampleWarps * kMergeIters;
+  return SmemLayout<T, ACC>::hist(d * N);
 }
 
 // Steps 2-3 for a list of sample indices (parity checks and debugging):
@@ -1348,10 +1316,10 @@ inline void grad_entry(KernelEntry& e) {
   }
 }
 
-template <typename T, int DM, template <typename, int> class F, int ACC, int YB>
+template <typename T, int DM, template <typename, int> class F, int ACC, int YB, bool BINS>
 inline const void* spec_kernel() {
   if constexpr (YB == 24 && ACC != 1)
-    return (const void*)&k_sample<T, DM, F, ACC, 24, true>;
+    return (const void*)&k_sample<T, DM, F, ACC, 24, true, BINS>;
   else
     return nullptr;
 }
@@ -1364,8 +1332,10 @@ inline size_t col_smem_bytes(int d, int N, int nwarps) {
 template <typename T, int DM, template <typename, int> class F, int ACC, int YB>
 inline KernelEntry make_entry() {
   KernelEntry e{};
-  e.sample = (const void*)&k_sample<T, DM, F, ACC, YB, false>;
-  e.sample_spec = spec_kernel<T, DM, F, ACC, YB>();
+  e.sample = (const void*)&k_sample<T, DM, F, ACC, YB, false, true>;
+  e.frozen = (const void*)&k_sample<T, DM, F, ACC, YB, false, false>;
+  e.sample_spec = spec_kernel<T, DM, F, ACC, YB, true>();
+  e.frozen_spec = spec_kernel<T, DM, F, ACC, YB, false>();
   grad_entry<T, DM, F, YB>(e);
   e.dump = (const void*)&k_dump<T, DM, F, YB>;
   e.spring = (const void*)&k_spring<T, DM, F, YB, false>;
@@ -1381,6 +1351,7 @@ inline KernelEntry make_entry() {
   e.smem = &sample_smem_bytes<T, ACC>;
   e.smem_nobins = &sample_smem_nobins<T, ACC>;
   e.dm = DM;
+  e.max_threads = kSampleMaxThreads<false>;
   e.spec_ppt_min = kPairPoints<T, DM, true> ? 2 : 1;
   return e;
 }
