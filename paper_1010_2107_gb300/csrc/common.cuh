@@ -305,8 +305,8 @@ __device__ __forceinline__ void mirror_state(GState* mirror, const GState* st) {
   for (int i = threadIdx.x & 31; i < n; i += 32) dst[i] = src[i];
 }
 
-// Threads per block of k_finish.
-constexpr int kFinishThreads = 256;
+// Threads per block of k_finish: up to 64 bins (and in passes without bins), and beyond.
+constexpr int kFinishThreads = 256, kMaxFinishThreads = 512;
 
 // Device-side control operations captured into the iteration graphs.
 enum { CTL_RESET_WINDOW = 1, CTL_SET_ACC = 2, CTL_SNAPSHOT = 4, CTL_SET_ITER = 8 };
