@@ -545,16 +545,24 @@ vegas_status configure_launch(vegas_ctx* c) {
     gv::TileShape t = gv::choose_tile(threads, N, c->ppt_req, c->ppt_min, occ_cap, occ_of, c->small_cap);
     // Few points: the same number of rounds with CTAs just wide enough, so
     // that every SM runs the same number of warps (10^5 points over 456 CTAs:
-    // 224 threads, 21 warps per SM, instead of 391 CTAs of 256, up to 24)
+    // 224 threads, 21 warps per SM, instead of 391 CTAs of 256, up to 24).
+    // Where warps are what an SM runs short of, that is FP64 points and FP64
+    // sums of 8 or more axes, and only a little narrower: set-up and
+    // finishing go by CTAs (us per pass with 256 threads -> so: FP64 53 bits
+    // d = 8, 2 10^5 points, 224 threads 65.9 -> 57.5; d = 16, 10^5, 224 69.3 ->
+    // 59.8; d = 6, 10^5, 192 41.9 -> 39.5; but 3 10^4, 128 27.0 -> 28.7; FP64 sums
+    // d = 8, 2 10^5, 224 44.1 -> 39.7, but d = 4 33.0 -> 35.8; FP32 sums 53 bits
+    // d = 16, 4 10^5, 224 47.9 -> 52.9).
+    const int narrowest = c->prec == VG_FP64 ? 160 : (c->prec == VG_FP32_ACC64 && d >= 8 ? 224 : 256);
     if (e == cudaSuccess && c->threads_req == 0 && !strat && t.occ > 0) {
       const uint64_t n = (uint64_t)c->cfg.ncall, most = (uint64_t)c->sm_count * t.occ;
       const uint64_t rounds = (n + most * threads - 1) / (most * threads);
       const int w = (int)(((n + most * rounds - 1) / (most * rounds) + 31) / 32 * 32);
-      if (w >= 64 && w < threads) {
+      if (w >= narrowest && w < threads) {
         const int wide = threads;
         threads = w;
         const gv::TileShape u = gv::choose_tile(threads, N, c->ppt_req, c->ppt_min, occ_cap, occ_of, c->small_cap);
-        if (u.occ >= t.occ)
+        if (u.occ >= t.occ && u.ppt == t.ppt)  // (a shorter tile costs more than even rounds give)
           t = u;
         else
           threads = wide;

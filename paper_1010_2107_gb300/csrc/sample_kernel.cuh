@@ -436,9 +436,9 @@ __device__ __forceinline__ void store_totals(const SampleArgs& A, double* part_t
 // CTAs of the largest size that must fit an SM (0: the compiler's choice), for
 // the light integrands; RAMBO needs up to 255 registers and a user's integrand
 // what it needs.
-// FP64, up to 16 axes: two (128 registers).  Left to itself the compiler holds
-// some of these kernels to 64 or 80 and spills for a third CTA, which the FP64
-// pipe has no use for.
+// FP64: three up to 4 axes (80 registers; 10^5 points in one even round), two up
+// to 16 (128).  Left to itself the compiler holds some of these kernels to 64 or
+// 80 and spills for one CTA more, which the FP64 pipe has no use for.
 template <template <typename, int> class F> constexpr bool kLight = false;
 template <> constexpr bool kLight<GenzGaussian> = true;
 template <> constexpr bool kLight<GenzProductPeak> = true;
@@ -449,7 +449,7 @@ template <> constexpr bool kLight<GenzDiscontinuous> = true;
 template <> constexpr bool kLight<DoubleGaussian> = true;
 template <> constexpr bool kLight<WMuNu> = true;
 template <typename T, int DM, template <typename, int> class F, bool SPEC>
-constexpr int kSampleMinBlocks = std::is_same<T, double>::value && DM <= 16 && kLight<F> ? (SPEC ? 1 : 2) : 0;
+constexpr int kSampleMinBlocks = std::is_same<T, double>::value && DM <= 16 && kLight<F> ? (SPEC ? 1 : (DM <= 4 ? 3 : 2)) : 0;
 
 // Threads a kernel is compiled for: kSampleMaxThreads, but 336 for the FP32
 // form with 53-bit words and the histogram in 5 to 8 dimensions.  Compiled for
