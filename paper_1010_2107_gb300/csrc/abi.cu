@@ -458,21 +458,43 @@ void* device_view(void* p, size_t bytes, size_t align) {
 // CTA, or, when 0, one CTA of as many warps as the columns' shared memory
 // allows (16 at up to 50 bins, the most the registers allow; one wide CTA
 // folds into one partial row: at 72 bins 11 warps in one CTA beat 10 in
-// five, 65 against 70 us at d = 8); a small pass takes narrower CTAs until
-// every SM has one.  False when fewer than kColMinWarps warps fit (from 101
-// bins on): down to that count columns beat bucketed tiles at every measured
-// dimension (us per pass of 2^22 points at 100 bins, columns against the best
-// tile: d = 4 43.9 / 47.1, d = 7 115.6 / 119.6, d = 8 66 / 93, d = 16 119 / 206).
+// five, 65 against 70 us at d = 8).  A small pass takes narrower CTAs until
+// every SM has one, but wide enough that the CTA's threads cover the cells they
+// clear and fold, 128 or 256 (us per pass of 1000 points with 64 threads -> so:
+// d = 4, 50 bins 17.7 -> 16.9, d = 15, 50 bins 25.9 -> 23.2, d = 20, 80 bins
+// 38.0 -> 33.0).
+//
+// False, and the pass takes bucketed tiles, when threads == 0 and fewer than
+// kColMinWarps warps of columns fit an SM (8 fit up to 109 bins at d = 2, 105 at
+// 8, 103 at 16, 95 at 32): us per pass of 2^22 points at 100 bins, columns
+// against the best tile: d = 4 43.9 / 47.1, d = 7 115.6 / 119.6, d = 8 66 / 93,
+// d = 16 119 / 206.  And, unstratified with more than 50 bins (fewer than 16
+// warps), for passes too small to pay for clearing and folding the columns (one
+// or two axes have little to fold).  Columns over tiles, measured at 80 bins:
+//   d (exact)      4     8    16   |  d (run-time) 3     6     7    9    12    15
+//   10^5 points   .98  1.08  1.12  |             1.09  1.10  1.18 1.17  1.15  1.09
+//   4 10^5        .95  1.00   .98  |             1.00  1.08  1.04 1.08  1.01   .87
+//   2^20          .92   .87   .84  |             1.09  1.04   .97 1.01   .97   .76
+//   2^22                .79   .76  |             1.09  1.04   .93       .92   .69
+// so from n d = 2 10^6 on where the kernel knows the dimension, and from 6 10^6
+// with at least 7 axes where it does not.
 constexpr int kColMinWarps = 8;
 // Static shared memory of k_sample, at most (its dynamic part must leave room).
 constexpr size_t kSampleStatic = 1024;
+bool cols_pay(bool exact, int d, int N, uint64_t ncubes, uint64_t ncall) {
+  if (ncubes > 1 || N <= 50 || d <= 2) return true;
+  return exact ? ncall * (uint64_t)d >= 2000000u : d >= 7 && ncall * (uint64_t)d >= 6000000u;
+}
 bool shape_col(const void* fn, const gv::KernelEntry& ke, int d, int N, int sm_count, int threads, int per_sm_req,
                uint64_t ncubes, uint64_t nc, uint64_t ncall, int64_t max_rows, uint64_t max_parts,
                gv::PassShape* out, cudaError_t* e) {
+  // A shape whose smallest buckets do not fit has columns or nothing.
+  const bool tiles = ke.smem(d, N, 4) + kSampleStatic <= 227 * 1024;
   // (2 KB: the kernel's static shared memory)
   auto fits = [&](int warps) { return ke.smem_col(d, N, warps) + 2048 <= 227 * 1024; };
   int best_t = threads;
   if (threads == 0) {
+    if (tiles && !cols_pay(fn == ke.sample_col_exact, d, N, ncubes, ncall)) return false;
     int warps = 16;
     while (warps >= kColMinWarps && !fits(warps)) --warps;
     best_t = 32 * warps;
@@ -489,7 +511,8 @@ bool shape_col(const void* fn, const gv::KernelEntry& ke, int d, int N, int sm_c
   if (threads == 0 && ncubes == 1) {
     const uint64_t per = (ncall + (uint64_t)sm_count * pif - 1) / ((uint64_t)sm_count * pif);
     if (per < (uint64_t)best_t) {
-      best_t = (int)std::max<uint64_t>(64, (per + 31) / 32 * 32);
+      const uint64_t least = d * N <= 400 ? 128 : 256;
+      best_t = (int)std::min<uint64_t>(best_t, (std::max(per, least) + 31) / 32 * 32);
       best_occ = 1;
     }
   }
