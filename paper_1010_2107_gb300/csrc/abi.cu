@@ -508,7 +508,7 @@ bool shape_col(const void* fn, const gv::KernelEntry& ke, int d, int N, int sm_c
   if (per_sm_req > 0) best_occ = std::min(best_occ, per_sm_req);
   if (best_occ < 1) return false;
   const int pif = d <= 8 ? 2 : 1;
-  if (threads == 0 && ncubes == 1) {
+  if (threads == 0) {
     const uint64_t per = (ncall + (uint64_t)sm_count * pif - 1) / ((uint64_t)sm_count * pif);
     if (per < (uint64_t)best_t) {
       const uint64_t least = d * N <= 400 ? 128 : 256;
@@ -629,7 +629,11 @@ vegas_status configure_launch(vegas_ctx* c) {
   // per pass against 40.0 with all that fit)
   pn.occ = std::max(1, std::min(occ_nb, std::max(32 * 32 / threads, per_sm)));
   const int64_t most_nb = (int64_t)c->sm_count * pn.occ;
-  const gv::CubeLanes cl = strat ? gv::balanced_lanes(c->ncubes, c->nc, threads, c->sm_count, c->ppt_min, gv::kMaxCubeParts)
+  // (without the histogram a cube's parts cost more, in their merge and in the
+  // groups' own reductions, than even rounds give, until half the SMs would
+  // idle: 6561 cubes of 300, d = 8, 85.6 us per call with parts, 78.4 without)
+  const uint64_t max_parts = c->ncubes * 32 < (uint64_t)threads * c->sm_count / 2 ? gv::kMaxCubeParts : 0;
+  const gv::CubeLanes cl = strat ? gv::balanced_lanes(c->ncubes, c->nc, threads, c->sm_count, c->ppt_min, max_parts)
                                  : gv::CubeLanes{1, 1};
   pn.lanes = cl.lanes;
   pn.parts = cl.parts;
