@@ -356,8 +356,10 @@ vegas_status vegas_get_launch(vegas_ctx* ctx, int* threads, int* ctas,
  * (axis, bin) buckets; kernels that evaluate two points per thread at a
  * time round it up to even.  Automatic: the FP32 form with compensated sums,
  * 24-bit words and a power-of-two number of divisions (g N <= 256) has no
- * tiles where its lane-owned columns fit (up to 100 bins); the other forms
- * choose a tile.  Changes only speed and the summation order inside a CTA,
+ * tiles where its lane-owned columns fit (eight warps of them on an SM: up to
+ * 107 to 109 bins in low dimensions, 105 at d = 8, 103 at 16, 95 at 32) and,
+ * unstratified with more than 50 bins, the pass is large enough to pay for
+ * them; the other forms choose a tile.  Changes only speed and the summation order inside a CTA,
  * never which points are drawn.  get_tile returns the points per thread (in
  * flight) and the bucket capacity per (axis, bin) in use, 0 for columns.
  * EINVAL outside the range or when the tile does not fit in shared memory
@@ -367,18 +369,20 @@ vegas_status vegas_get_tile(vegas_ctx* ctx, int* points_per_thread, int* cap);
 
 /* Launch-shape autotuner (the paper tunes nBlockSize by hand, Appendix A):
  * times evaluation passes (as vegas_profile_pass: no refinement, window
- * untouched) for threads per CTA in {128, 256, 384, 512} and histogram
- * tiles in {automatic, 1, 2, 4} points per thread, each with the largest
- * and with the smallest bucket capacity that reaches the tile's best
- * occupancy, skipping shapes the kernel cannot take; the three fastest are
- * timed again in three
- * interleaved rounds of five passes, and the one with the best round is
- * kept.  Returns its threads, points
- * per thread (the tile itself stays as tuned: automatic where vegas_get_tile
- * then reports capacity 0) and the pass time in ms (any output may be NULL).  The
- * specialised kernels (d = the compiled bound, 24-bit words, power-of-two
- * strata) accept up to 512 threads, the general ones 256.  Synchronises the
- * stream. */
+ * untouched) for the automatic shape and for threads per CTA in {128, 256,
+ * 384, 512} with histogram tiles in {automatic, 1, 2, 4} points per thread,
+ * each with the largest and with the smallest bucket capacity that reaches
+ * the tile's best occupancy, skipping shapes the kernel cannot take; the three
+ * fastest are timed again in three interleaved rounds of five passes, and the
+ * one with the best round is kept.  The passes that leave the grid unchanged
+ * then get the fastest of the same threads per CTA for themselves
+ * (vegas_set_launch sets both kinds).  Returns the threads and points per
+ * thread in use (the tile itself stays as tuned: automatic where
+ * vegas_get_tile then reports capacity 0) and the pass time in ms (any output
+ * may be NULL).  The specialised kernels (d = the compiled bound, 24-bit words,
+ * power-of-two strata) accept up to 512 threads, the general ones 256; the
+ * automatic shape may use more.  A pass that fails leaves the shape as it was.
+ * Synchronises the stream. */
 vegas_status vegas_autotune(vegas_ctx* ctx, int* threads, int* points_per_thread, double* ms);
 
 /* Measurement (the paper times whole programs, Sec. 3.3; this times each

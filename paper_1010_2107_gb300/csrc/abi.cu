@@ -98,8 +98,9 @@ struct vegas_ctx {
   gv::KernelEntry ke{};
   const void* col = nullptr;  // the column-histogram kernel of this shape, or null
   int sm_count = 0;
-  // launch geometry: threads per CTA asked for (0: automatic) and CTAs per SM
-  int threads_req = 0, ctas_per_sm_req = 0;
+  // launch geometry: threads per CTA asked for (0: automatic) and CTAs per SM;
+  // those of the passes without bins, where the autotuner set them apart
+  int threads_req = 0, ctas_per_sm_req = 0, frozen_req = 0;
   int cap = 0;  // histogram bucket capacity (see sample_kernel.cuh; 0: column histogram)
   int ppt = 1, ppt_req = 0, ppt_min = 1;  // points per thread per histogram tile
   bool small_cap = false;                 // tile capacity policy (gv::choose_tile)
@@ -612,8 +613,8 @@ vegas_status configure_launch(vegas_ctx* c) {
       pb.parts = cl.parts;
     }
     pb.ctas = ctas_for(pb, threads, most);
-    threads = c->threads_req > 0 ? c->threads_req : 256;
   }
+  threads = c->frozen_req > 0 ? c->frozen_req : (c->threads_req > 0 ? c->threads_req : 256);
   // passes without the per-bin histogram (no refinement) need only the
   // grid table and constants in shared memory: more CTAs may be resident
   pn.fn = c->ke.frozen;
@@ -1547,13 +1548,15 @@ vegas_status vegas_set_launch(vegas_ctx* c, int threads, int ctas_per_sm) {
     return c->fail(VEGAS_EINVAL, "threads must be a multiple of 32 in 64..%d", c->ke.max_threads);
   if (ctas_per_sm < 0) return c->fail(VEGAS_EINVAL, "ctas_per_sm < 0");
   CK(c, cudaStreamSynchronize(c->stream));
-  const int t0 = c->threads_req, p0 = c->ctas_per_sm_req;
+  const int t0 = c->threads_req, p0 = c->ctas_per_sm_req, f0 = c->frozen_req;
   c->threads_req = threads;
   c->ctas_per_sm_req = ctas_per_sm;
+  c->frozen_req = 0;
   vegas_status st = configure_launch(c);
   if (st) {  // (the shape and its buffers are as before)
     c->threads_req = t0;
     c->ctas_per_sm_req = p0;
+    c->frozen_req = f0;
   }
   return st;
 }
@@ -1572,56 +1575,94 @@ vegas_status vegas_set_tile(vegas_ctx* c, int points_per_thread) {
 
 vegas_status vegas_autotune(vegas_ctx* c, int* threads, int* points_per_thread, double* ms) {
   if (!c) return thread_fail(VEGAS_EINVAL, "ctx is NULL");
-  static const int kThreads[] = {128, 256, 384, 512};
+  // (0: the automatic shape, which has CTA widths of its own)
+  static const int kThreads[] = {0, 128, 256, 384, 512};
   static const int kTiles[] = {0, 1, 2, 4};
-  struct Cand {
-    int t, p;
+  struct Shape {  // requests of configure_launch
+    int t, per_sm, f, p;
     bool small;
+  };
+  struct Cand {
+    Shape s;
     double ms;
   };
-  std::vector<Cand> cands;
-  // one pass of warm-up, then the mean of n passes, for shape (t, p) and
-  // capacity policy `small`
-  auto time_shape = [&](int t, int p, bool small, int n, double* out) -> vegas_status {
-    c->small_cap = small;
-    if (vegas_set_launch(c, t, 0) != VEGAS_OK || vegas_set_tile(c, p) != VEGAS_OK) return VEGAS_EINVAL;
+  auto get = [&]() { return Shape{c->threads_req, c->ctas_per_sm_req, c->frozen_req, c->ppt_req, c->small_cap}; };
+  auto put = [&](const Shape& s) {
+    c->threads_req = s.t;
+    c->ctas_per_sm_req = s.per_sm;
+    c->frozen_req = s.f;
+    c->ppt_req = s.p;
+    c->small_cap = s.small;
+  };
+  auto set_shape = [&](const Shape& s) -> vegas_status {
+    CK(c, cudaStreamSynchronize(c->stream));
+    const Shape had = get();
+    put(s);
+    const vegas_status st = configure_launch(c);
+    if (st) put(had);
+    return st;
+  };
+  // one pass of warm-up, then the mean of n passes, for shape s
+  auto time_shape = [&](const Shape& s, bool frozen, int n, double* out) -> vegas_status {
+    if (set_shape(s) != VEGAS_OK) return VEGAS_EINVAL;
     double m[3];
-    vegas_status st = vegas_profile_pass(c, 1, m);
-    if (!st) st = vegas_profile_pass(c, n, m);
+    vegas_status st = VEGAS_OK;
+    for (int k : {1, n})
+      if (!st) st = frozen ? vegas_profile_frozen_pass(c, k, m) : vegas_profile_pass(c, k, m);
     if (!st) *out = m[2];
     return st == VEGAS_OK ? VEGAS_OK : VEGAS_ECUDA;
   };
+  const Shape before = get();
+  auto give_up = [&]() -> vegas_status {  // a pass failed: back to the shape it came with
+    const std::string why = c->err;
+    set_shape(before);
+    return c->fail(VEGAS_ECUDA, "%s", why.empty() ? "autotune: pass failed" : why.c_str());
+  };
   // screening: every shape the kernel takes (the others are skipped)
+  std::vector<Cand> cands;
   for (int t : kThreads)
     for (int p : kTiles) {
+      if (t > c->ke.max_threads || (t == 0 && p > 0)) continue;
       int cap_large = -1;  // the tile of the largest-capacity policy (a repeat is not timed twice)
       for (bool small : {false, true}) {
+        const Shape s{t, 0, 0, p, small};
         double m = 0.0;
-        const vegas_status st = time_shape(t, p, small, 3, &m);
-        if (st == VEGAS_ECUDA) return c->err.empty() ? c->fail(st, "autotune: pass failed") : st;
+        const vegas_status st = time_shape(s, false, 3, &m);
+        if (st == VEGAS_ECUDA) return give_up();
         if (st != VEGAS_OK || (small && c->cap == cap_large)) continue;
         if (!small) cap_large = c->cap;
-        cands.push_back({t, p, small, m});
+        cands.push_back({s, m});
       }
     }
   if (cands.empty()) return c->fail(VEGAS_EINVAL, "autotune: no launch shape fits");
   // the three fastest again, in interleaved rounds, keeping each one's best
   // round (shapes a few percent apart are within one screening's noise)
-  std::sort(cands.begin(), cands.end(), [](const Cand& a, const Cand& b) { return a.ms < b.ms; });
+  auto faster = [](const Cand& a, const Cand& b) { return a.ms < b.ms; };
+  auto finals = [&](std::vector<Cand>& v, bool frozen, int rounds) -> vegas_status {
+    for (int r = 0; r < rounds; ++r)
+      for (Cand& k : v) {
+        double m = 0.0;
+        if (time_shape(k.s, frozen, 5, &m) != VEGAS_OK) return VEGAS_ECUDA;
+        k.ms = r == 0 ? m : std::min(k.ms, m);
+      }
+    return VEGAS_OK;
+  };
+  std::sort(cands.begin(), cands.end(), faster);
   cands.resize(std::min<size_t>(cands.size(), 3));
-  for (int r = 0; r < 3; ++r)
-    for (Cand& k : cands) {
-      double m = 0.0;
-      if (time_shape(k.t, k.p, k.small, 5, &m) != VEGAS_OK) return c->fail(VEGAS_ECUDA, "autotune: pass failed");
-      k.ms = r == 0 ? m : std::min(k.ms, m);
+  if (finals(cands, false, 3) != VEGAS_OK) return give_up();
+  const Cand best = *std::min_element(cands.begin(), cands.end(), faster);
+  // the passes without bins have a width of their own
+  std::vector<Cand> widths;
+  for (int f : {128, 256, 384, 512})
+    if (f <= c->ke.max_threads) {
+      widths.push_back({best.s, 0.0});
+      widths.back().s.f = f;
     }
-  const Cand best = *std::min_element(cands.begin(), cands.end(),
-                                      [](const Cand& a, const Cand& b) { return a.ms < b.ms; });
-  c->small_cap = best.small;
-  vegas_status st = vegas_set_launch(c, best.t, 0);
-  if (!st) st = vegas_set_tile(c, best.p);
+  if (finals(widths, true, 3) != VEGAS_OK) return give_up();
+  const Cand width = *std::min_element(widths.begin(), widths.end(), faster);
+  const vegas_status st = set_shape(width.s);
   if (st) return st;
-  if (threads) *threads = best.t;
+  if (threads) *threads = c->pass_bins.threads;
   if (points_per_thread) *points_per_thread = c->ppt;
   if (ms) *ms = best.ms;
   return VEGAS_OK;
