@@ -470,7 +470,8 @@ vegas_status vegas_batch_get_launch(vegas_batch* batch, int* threads, int* round
  * counterpart in the paper): the points each thread evaluates between two
  * gathers of the CTA's buckets, 0 = automatic.  The FP32 form with 24-bit
  * words runs one kernel per dimension (d = 1..16), automatically with
- * lane-owned columns instead of buckets where they fit (up to 100 bins);
+ * lane-owned columns instead of buckets where eight warps of them fit an SM
+ * (about 100 bins, with 256 threads per CTA);
  * with 1 or 2, the points a thread keeps in flight, with buckets; the other
  * forms take 0..4.  EINVAL
  * outside the range or when the tile does not fit (the previous tile then

@@ -560,14 +560,23 @@ vegas_status build_items(vegas_batch* b) {
 // Dimension kernels: for each dimension present its kernel (points in
 // flight = the tile's points per thread), bucket capacity and CTAs per SM.
 // Automatically (no tile asked for) the column-histogram kernels, where for
-// every dimension present at least kColMinWarps warps per SM fit (up to 100
-// bins; there too they beat the buckets: 64 instances of 2^16..2^20 points
-// 0.423 ms against 0.590, one CTA of eight warps per SM; wider CTAs at 64 to
-// 80 bins gained nothing).  Without a launch shape set, an item's rounds
-// follow the work: about sixteen items per SM, 8 to 128 rounds (a fold per
-// item against an even queue; ms per pass at 16, 32, 64, 128 rounds, 50 bins:
-// 256 instances of 2^16..2^22 points 3.92, 3.41, 3.22, 3.12, 64 of
-// 2^16..2^18 0.172, 0.182, 0.246, 0.354).
+// every dimension present at least kColMinWarps warps per SM fit (64 instances
+// of 2^18..2^20 points at 100 bins, one CTA of eight warps per SM: 0.69 ms
+// against 0.92; wider CTAs at 64 to 80 bins gained nothing).
+//
+// Without a launch shape set, an item's rounds follow the work.  A fold costs
+// as much as F rounds: F = 5 + 15 / d (d: the points' mean dimension) where two
+// CTAs' worth of warps share an SM, and 1.6 sqrt(N / 64) times that where one
+// CTA's fold has nothing beside it; with W rounds of work per resident CTA the
+// folds add F / R of it, the uneven end of the queue about R / W.  So R = sqrt(F
+// W), the nearest power of two in 2..128.  us per pass with finalisation at R =
+// 2, 8, 16, 32, 64 (the rule's marked; 256 instances take 128):
+//   16 of 2^10..13, d <= 16, 50 bins      55*   62    66    74    74
+//   64 of 2^14..18, d <= 16, 50 bins     379   169   146*  159   215
+//   64 of 2^14..18, d <= 16, 100 bins    723   263   195   178*  231
+//   64 of 2^14..19, d <= 4, 50 bins      361   133    96    78*   72
+//   64 of 2^14..19, d <= 4, 100 bins     651   215   141   107    89*
+//   64 of 2^18..20, d <= 16, 50 bins    2026   855   631   539   511*
 constexpr int kColMinWarps = 8;
 bool configure_cols(vegas_batch* b, const bool (&present)[gv::kBatchDM], cudaError_t* e) {
   for (int d = 1; d <= gv::kBatchDM; ++d) {
@@ -586,10 +595,18 @@ bool configure_cols(vegas_batch* b, const bool (&present)[gv::kBatchDM], cudaErr
     if (c.occ * b->threads < 32 * kColMinWarps) return false;
   }
   if (!b->launch_set) {
-    double points = 0.0;
-    for (const vegas_config& c : b->cfg) points += (double)c.ncall;
-    b->rounds = 8;
-    while (b->rounds < 128 && (double)b->rounds * 1.5 < points / (256.0 * 16.0 * b->sm_count)) b->rounds *= 2;
+    double points = 0.0, axes = 0.0;
+    int occ = 64;
+    for (int i = 0; i < b->n; ++i) {
+      points += (double)b->cfg[i].ncall;
+      axes += (double)b->cfg[i].ncall * b->d[i];
+      occ = std::min(occ, b->dims[b->d[i] - 1].occ);
+    }
+    double fold = 5.0 + 15.0 * points / axes;
+    if (occ * b->threads < 512) fold *= 1.6 * std::sqrt(std::max(b->N, 64) / 64.0);
+    const double best = std::sqrt(fold * points / ((double)b->threads * b->sm_count * occ));
+    b->rounds = 2;
+    while (b->rounds < 128 && b->rounds * 1.4142 < best) b->rounds *= 2;
   }
   return true;
 }
