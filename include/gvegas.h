@@ -482,11 +482,14 @@ vegas_status vegas_batch_get_launch(vegas_batch* batch, int* threads, int* round
 vegas_status vegas_batch_set_tile(vegas_batch* batch, int points_per_thread);
 vegas_status vegas_batch_get_tile(vegas_batch* batch, int* points_per_thread, int* cap);
 
-/* Autotuner: times every (threads, rounds) candidate, each with the largest
- * and the smallest bucket capacity that reach its occupancy, on the batch's
- * own workload (an evaluation pass, nothing recorded), times the three fastest
- * again in three interleaved rounds and keeps the one with the best round;
- * returns it and its sampling-kernel milliseconds. */
+/* Autotuner: times the automatic shape and every (threads, rounds) candidate
+ * on the batch's own workload (an evaluation pass, nothing recorded): with
+ * columns where they fit, with buckets (points in flight, capacity policies)
+ * where two of their better shapes come within 15 % of the best columns, or
+ * where there are no columns.  The three fastest are timed again in three
+ * interleaved rounds and the one with the best round is kept; returns it and
+ * its sampling-kernel milliseconds.  A pass that fails leaves the shape as it
+ * was. */
 vegas_status vegas_batch_autotune(vegas_batch* batch, int* threads, int* rounds, double* ms);
 
 /* Mean milliseconds of the sampling kernel (ms[0]) and the finalisation

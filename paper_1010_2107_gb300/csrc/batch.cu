@@ -1143,71 +1143,95 @@ vegas_status vegas_batch_autotune(vegas_batch* b, int* threads, int* rounds, dou
   static const int kRounds[] = {8, 16, 32, 64, 128};
   struct Cand {
     int t, r, p, pol;
-    double ms;
+    double ms, sample;  // of a pass, and of its sampling kernels
   };
   std::vector<Cand> cands;
-  // one warm-up pass, then the mean of n passes, for shape (t, r), tile p
-  // (the per-dimension kernels: points in flight) and capacity policy pol
-  // (0: the largest capacity of the range, 1: the smallest, 2: the dense
-  // floor, per-dimension kernels only)
-  auto set_shape = [&](int t, int r, int p, int pol) -> vegas_status {
-    BatchShape want = *b;
-    want.threads = t;
-    want.rounds = r;
-    want.launch_set = true;
-    want.ppt_req = p;
-    want.small_cap = pol >= 1;
-    want.dense_cap = pol == 2;
+  const BatchShape before = *b;
+  auto put = [&](const BatchShape& want) -> vegas_status {
     BK(b, cudaStreamSynchronize(b->stream));
     return configure(b, want);
   };
-  auto time_shape = [&](int t, int r, int p, int pol, int n, double* out) -> vegas_status {
-    vegas_status st = set_shape(t, r, p, pol);
+  // one warm-up pass, then the mean of n passes, for shape (t, r) (r = 0: the
+  // rounds that follow the work), tile p (the per-dimension kernels: 0 columns,
+  // else points in flight) and capacity policy pol (0: the largest capacity of
+  // the range, 1: the smallest, 2: the dense floor, per-dimension kernels only)
+  auto set_shape = [&](int t, int r, int p, int pol) -> vegas_status {
+    BatchShape want = *b;
+    want.threads = t;
+    if (r > 0) want.rounds = r;
+    want.launch_set = r > 0;
+    want.ppt_req = p;
+    want.small_cap = pol >= 1;
+    want.dense_cap = pol == 2;
+    return put(want);
+  };
+  auto time_shape = [&](Cand& c, int n, bool first) -> vegas_status {
+    vegas_status st = set_shape(c.t, c.r, c.p, c.pol);
     double m[2];
     if (!st) st = vegas_batch_profile(b, 1, m);
     if (!st) st = vegas_batch_profile(b, n, m);
-    if (!st) *out = m[0];
+    if (!st && (first || m[0] + m[1] < c.ms)) {  // (the finalisation reads a row per item)
+      c.ms = m[0] + m[1];
+      c.sample = m[0];
+    }
     return st;
   };
-  // (columns, where the automatic form is that, beat the buckets' tiles at
-  // every measured shape: only the launch shape is left to choose)
-  BatchShape automatic = *b;
-  automatic.ppt_req = 0;
-  BK(b, cudaStreamSynchronize(b->stream));
-  vegas_status st0 = configure(b, automatic);
-  if (st0) return st0;
-  const bool cols = b->by_dim && b->cap == 0;
-  const std::vector<int> tiles = b->by_dim && !cols ? std::vector<int>{1, 2} : std::vector<int>{0};
-  for (int t : kThreads)
-    for (int r : kRounds)
-      for (int p : tiles) {
-        int cap_large = -1;  // a repeated tile is not timed twice
-        for (int pol = 0; pol < (cols ? 1 : (b->by_dim ? 3 : 2)); ++pol) {
-          double m = 0.0;
-          vegas_status st = time_shape(t, r, p, pol, 3, &m);
-          if (st) return st;
-          if (pol == 1 && b->cap == cap_large) continue;
-          if (pol == 0) cap_large = b->cap;
-          cands.push_back({t, r, p, pol, m});
-        }
-      }
+  auto give_up = [&](vegas_status st) {
+    const std::string why = b->err;
+    put(before);
+    return b->fail(st, "%s", why.c_str());
+  };
+  vegas_status st = VEGAS_OK;
+  double fastest = 0.0;
+  auto add = [&](int t, int r, int p, int pol) -> bool {  // false: a pass failed
+    Cand c{t, r, p, pol, 0.0, 0.0};
+    if ((st = time_shape(c, 3, true)) != VEGAS_OK) return false;
+    if (cands.empty() || c.ms < fastest) fastest = c.ms;
+    cands.push_back(c);
+    return true;
+  };
+  if (b->by_dim) {
+    // columns, at every shape whose columns fit
+    auto columns = [&](int t, int r) -> bool {
+      if ((st = set_shape(t, r, 0, 0)) != VEGAS_OK) return false;
+      return b->cap != 0 || add(t, r, 0, 0);
+    };
+    if (!columns(256, 0)) return give_up(st);
+    for (int t : kThreads)
+      for (int r : kRounds)
+        if (!columns(t, r)) return give_up(st);
+    // buckets: the whole range only where two of its better shapes come near
+    const bool any = !cands.empty();
+    const double near = 1.15 * fastest;
+    bool screen = !any;
+    for (int r : {8, 32}) {
+      if (!any) break;
+      if (!add(256, r, 2, 2)) return give_up(st);
+      screen = screen || cands.back().ms < near;
+    }
+    for (int t : kThreads)
+      for (int r : kRounds)
+        for (int p : {1, 2})
+          for (int pol = 0; pol < 3 && screen; ++pol)
+            if (!add(t, r, p, pol)) return give_up(st);
+  } else {
+    for (int t : kThreads)
+      for (int r : kRounds)
+        for (int pol : {0, 1})
+          if (!add(t, r, 0, pol)) return give_up(st);
+  }
   // the three fastest again in interleaved rounds, keeping each one's best
   std::sort(cands.begin(), cands.end(), [](const Cand& a, const Cand& c) { return a.ms < c.ms; });
   cands.resize(std::min<size_t>(cands.size(), 3));
   for (int k = 0; k < 3; ++k)
-    for (Cand& c : cands) {
-      double m = 0.0;
-      vegas_status st = time_shape(c.t, c.r, c.p, c.pol, 3, &m);
-      if (st) return st;
-      c.ms = k == 0 ? m : std::min(c.ms, m);
-    }
+    for (Cand& c : cands)
+      if ((st = time_shape(c, 3, k == 0)) != VEGAS_OK) return give_up(st);
   const Cand best = *std::min_element(cands.begin(), cands.end(),
                                       [](const Cand& a, const Cand& c) { return a.ms < c.ms; });
-  vegas_status st = set_shape(best.t, best.r, best.p, best.pol);
-  if (st) return st;
-  if (threads) *threads = best.t;
-  if (rounds) *rounds = best.r;
-  if (ms) *ms = best.ms;
+  if ((st = set_shape(best.t, best.r, best.p, best.pol)) != VEGAS_OK) return give_up(st);
+  if (threads) *threads = b->threads;
+  if (rounds) *rounds = b->rounds;
+  if (ms) *ms = best.sample;
   return VEGAS_OK;
 }
 

@@ -40,3 +40,19 @@ def test_automatic_rounds_beat_buckets(gv, count, dmax, lo, hi, nbins):
         gv.vegas_batch_reset(b)
         r1 = gv.vegas_batch_iterate(b, 1, refine=False)
         np.testing.assert_allclose([r["I"] for r in r0], [r["I"] for r in r1], rtol=2e-5, atol=1e-7)
+
+
+@pytest.mark.parametrize("count,dmax,lo,hi,nbins", CASES)
+@pytest.mark.parametrize("threads", [None, 128])
+def test_tuning_does_not_slow_a_batch(gv, count, dmax, lo, hi, nbins, threads):
+    """Whatever shape was set before: at 100 bins with 128 threads columns do not
+    fit, with 256 they do, and both are tried."""
+    ins = wl.genz_batch(count, seed=5, dmax=dmax, log2n_min=lo, log2n_max=hi)
+    with gv.vegas_batch_create(ins, nbins=nbins, seed=1, precision="fp32", ybits=24) as b:
+        auto = _ms(gv, b)
+        if threads:
+            gv.vegas_batch_set_launch(b, threads, 32)
+        tuned = gv.vegas_batch_autotune(b)
+        shape = gv.vegas_batch_get_launch(b)
+        assert (tuned["threads"], tuned["rounds"]) == (shape["threads"], shape["rounds"])
+        assert _ms(gv, b) <= 1.03 * auto
