@@ -18,9 +18,14 @@
 // next one, so the load's latency lies under the evaluation's arithmetic
 // (two-peak Gaussian, d = 8, 2^22 points: 70.5 -> 61.4 us per pass; with a
 // run-time dimension the steps' own bookkeeping costs more than it hides,
-// 78.7 -> 85.2 us at d = 7, so there they run together after it).  (The cells are accessed through volatile inline assembly
-// without a memory clobber: the accesses keep their order among themselves,
-// while the table lookups and constants around them stay free to move.)
+// 78.7 -> 85.2 us at d = 7, so there they run together after it).
+//
+// The cells are accessed through volatile inline assembly without a memory
+// clobber: these accesses keep their order among themselves, while the table
+// lookups and constants around them stay free to move.  Ordinary accesses to
+// the cells (bind clears them, col_sum folds and clears) are not ordered
+// against them by the compiler, so a barrier has to stand wherever the two meet:
+// bind ends in __syncwarp, a fold begins and ends in __syncthreads.
 //
 // What it costs per 32 point-axes, in shared-memory wavefronts: bin byte 1,
 // cell load 2, cell store 2, weight 1/4, about 5.5 with the staging writes

@@ -164,9 +164,11 @@ __device__ __forceinline__ double scaled_u64(uint64_t r, int bits) {
 
 // exp in FP64 for the integrands: Tang's table method (Tang, ACM TOMS 15,
 // 1989): x = (64 m + j) ln2 / 64 + r, |r| <= ln2 / 128, exp x = 2^m 2^(j/64)
-// (1 + p(r)) with a degree-5 polynomial (truncation r^6 / 720 < 2^-54) and
-// the table 2^(j/64) in two doubles, so the error stays near 0.53 ulp
-// (CUDA's exp: 1 ulp).  11 FP64 operations instead of the library's 16 or so:
+// (1 + p(r)) with a degree-5 polynomial and the table 2^(j/64) in two
+// doubles.  The error stays below 0.84 ulp: half from the last rounding, up to
+// 0.31 from the polynomial's end (r^6 / 720 <= 3.5e-17 of a value below 2), the
+// rest from the roundings of p (largest measured 0.80, mean 0.254; CUDA's exp
+// 0.85 and 0.258).  11 FP64 operations instead of the library's 16 or so:
 // the FP64 kernels are bound by that pipe.  Arguments whose result is not a
 // normal number go to the library.
 static __device__ const double2 kExpTable[64] = {
@@ -224,8 +226,8 @@ __device__ __forceinline__ double exp64(double x) {
 // Quick FP32 forms for the FP32 integrands: the special-function unit's
 // approximations (__logf, __expf, __sincosf, __fdividef, sqrt.approx),
 // a few parts in 2^22 on the ranges used; arguments of the trigonometric
-// forms are kept in [-pi, pi] by their callers.  The FP64 overloads are the
-// correctly rounded library functions, so FP64 kernels are unchanged.
+// forms are kept in [-pi, pi] by their callers.  The FP64 overloads are CUDA's
+// library functions, except for exp, which is exp64.
 __device__ __forceinline__ float qlog(float x) { return __logf(x); }
 __device__ __forceinline__ double qlog(double x) { return log(x); }
 // ln x with a small relative error also near x = 1, where __logf's

@@ -11,7 +11,7 @@
 namespace gv {
 
 // exp of a non-positive Gaussian exponent: the special-function unit for
-// FP32 (relative error ~2^-21 over the range that matters), libm for FP64.
+// FP32 (relative error ~2^-21 over the range that matters), exp64 for FP64.
 __device__ __forceinline__ float gexp(float x) { return __expf(x); }
 __device__ __forceinline__ double gexp(double x) { return exp64(x); }
 
