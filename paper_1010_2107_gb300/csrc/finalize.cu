@@ -59,11 +59,11 @@ __device__ __forceinline__ void psum_zero(double& a) { a = 0.0; }
 // by the cluster's first CTA.  The rows are stored [CTA][2 d N], so a warp
 // reads consecutive columns of a row.  V: stored element, S: running sum.
 // Returns in the first CTA's s2[] the scaled S2 sums.
-template <typename V, typename S>
+template <int T, typename V, typename S>
 __device__ __forceinline__ void reduce_axis(const FinArgs& F, int a, unsigned rank, S* buf, double* s2) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
-  const int N = F.N, dN = F.d * N, C = 2 * N, np = F.nparts, T = blockDim.x;
+  const int N = F.N, dN = F.d * N, C = 2 * N, np = F.nparts;
   const int nsl = min(kFinishSlices, max(1, T / C));
   const int j = threadIdx.x % C, sl = threadIdx.x / C;  // column and slice (C <= T: one column per thread)
   const size_t stride = 2 * (size_t)dN;
@@ -74,13 +74,6 @@ __device__ __forceinline__ void reduce_axis(const FinArgs& F, int a, unsigned ra
     int r = (int)rank + kFinishCluster * slice;
     S acc;
     psum_zero(acc);
-    for (; r + 15 * step < np; r += 16 * step) {
-      V v[16];
-#pragma unroll
-      for (int u = 0; u < 16; ++u) v[u] = __ldcg(src + (size_t)(r + u * step) * stride);
-#pragma unroll
-      for (int u = 0; u < 16; ++u) psum_add(acc, v[u]);
-    }
     for (; r + 7 * step < np; r += 8 * step) {
       V v[8];
 #pragma unroll
@@ -142,7 +135,7 @@ __device__ __forceinline__ fpair psum_xor(const fpair& a, int off) {
 }
 __device__ __forceinline__ double psum_xor(const double& a, int off) { return __shfl_xor_sync(0xffffffffu, a, off); }
 
-template <typename V, typename S>
+template <int T, typename V, typename S>
 __device__ __forceinline__ void reduce_cubes(const FinArgs& F, int j, unsigned rank, S (*buf)[4], double* tot) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
@@ -152,7 +145,7 @@ __device__ __forceinline__ void reduce_cubes(const FinArgs& F, int j, unsigned r
 #pragma unroll
   for (int q = 0; q < 4; ++q) psum_zero(t[q]);
   const bool store = F.cubes && j == F.niter - 1;
-  for (uint32_t i = rank * blockDim.x + threadIdx.x; i < G; i += kFinishCluster * blockDim.x) {
+  for (uint32_t i = rank * T + threadIdx.x; i < G; i += kFinishCluster * T) {
     S c1, c2;
     psum_zero(c1);
     psum_zero(c2);
@@ -173,7 +166,7 @@ __device__ __forceinline__ void reduce_cubes(const FinArgs& F, int j, unsigned r
     cube_totals(F.inv_nc, F.inv_nc1, c1, c2, t);
     if (store) cube_store(F.cubes, cube_of(G, F.cube_mul, i), c1, c2);
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = T / 32;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
 #pragma unroll
@@ -271,13 +264,15 @@ __device__ void record_iteration(const FinArgs& F, const double* t, bool combine
 // distributed shared memory, without a memory fence and an arrival counter,
 // and what remains is the dependent FP64 chain of the refinement.
 //
-// Threads: two to eight slices of an axis's 2 N columns, so 256 up to 64 bins and
-// twice that beyond (one column each at 256 bins), and up to 16 rows per thread
-// in flight (d = 4, us of this kernel, with 256 threads and 8 rows for every
-// shape -> now: 160 bins, 456 rows 14.7 -> 11.6; 256 bins, 304 rows 13.8 -> 11.7).
-__global__ void __cluster_dims__(kFinishCluster, 1, 1) __launch_bounds__(kMaxFinishThreads) k_finish(const FinArgs F) {
+// T threads: two to eight slices of an axis's 2 N columns, so 256 up to 64 bins
+// and 512 beyond (one column each at 256 bins), two CTAs of which fit an SM, as
+// the clusters of 16 and more axes need (d = 4, us of this kernel, 256 threads ->
+// 512: 160 bins, 456 rows 15.0 -> 11.9; 256 bins, 304 rows 13.9 -> 11.65; d = 8, 200
+// bins 11.9 -> 9.85).
+template <int T>
+__global__ void __cluster_dims__(kFinishCluster, 1, 1) __launch_bounds__(T, T > kFinishThreads ? 2 : 0) k_finish(const FinArgs F) {
   // (the slices' partial sums, 8 bytes per thread, or the cubes', 64 per warp)
-  __shared__ __align__(16) unsigned char buf[kMaxFinishThreads * 8];
+  __shared__ __align__(16) unsigned char buf[T * 16];
   __shared__ double s2[kMaxBins];
   __shared__ double tot[kMergeIters][kTotCols];
   GState* st = F.st;
@@ -287,13 +282,13 @@ __global__ void __cluster_dims__(kFinishCluster, 1, 1) __launch_bounds__(kMaxFin
   const int group = F.nobins ? F.d : (int)(blockIdx.x / kFinishCluster);
   if (group < F.d) {
     if (F.pair32)
-      reduce_axis<float2, fpair>(F, group, rank, reinterpret_cast<fpair*>(buf), s2);
+      reduce_axis<T, float2, fpair>(F, group, rank, reinterpret_cast<fpair*>(buf), s2);
     else
-      reduce_axis<double, double>(F, group, rank, reinterpret_cast<double*>(buf), s2);
+      reduce_axis<T, double, double>(F, group, rank, reinterpret_cast<double*>(buf), s2);
     if (rank != 0 || !F.refine) return;
     // one thread per bin (whole warps) refines; the other warps leave
     const int N = F.N, a = group;
-    const Team t{min((int)blockDim.x, (N + 31) / 32 * 32)};
+    const Team t{min(T, (N + 31) / 32 * 32)};
     if ((int)threadIdx.x >= t.n) return;
     refine_axis_core(s2, F.edges + (size_t)a * (N + 1), F.tab64 + (size_t)a * N, F.tab32 + (size_t)a * N, N,
                      F.alpha, t);
@@ -305,14 +300,14 @@ __global__ void __cluster_dims__(kFinishCluster, 1, 1) __launch_bounds__(kMaxFin
   if (F.parts > 1u) {
     for (int j = 0; j < F.niter; ++j) {
       if (F.pair32)
-        reduce_cubes<float4, fpair>(F, j, rank, reinterpret_cast<fpair(*)[4]>(buf), tot[j]);
+        reduce_cubes<T, float4, fpair>(F, j, rank, reinterpret_cast<fpair(*)[4]>(buf), tot[j]);
       else
-        reduce_cubes<double2, double>(F, j, rank, reinterpret_cast<double(*)[4]>(buf), tot[j]);
+        reduce_cubes<T, double2, double>(F, j, rank, reinterpret_cast<double(*)[4]>(buf), tot[j]);
     }
   }
   if (rank != 0) return;
   const double s1 = *F.scale;
-  for (int i = warp; i < 5 * F.niter; i += (int)blockDim.x / 32) {
+  for (int i = warp; i < 5 * F.niter; i += T / 32) {
     const int j = i / 5, q = i - 5 * j;
     if (F.parts > 1u && q != TOT_NONFINITE) continue;
     const double v = total_column(F.part_tot + ((size_t)j * kTotCols + q) * F.nparts, F.nparts, lane);
@@ -404,7 +399,7 @@ extern "C" {
 // shared memory; the small kernels between them ask for the same split, so
 // that an SM need not change its partition (and drain) at every boundary.
 cudaError_t gv_prepare_aux_kernels(void) {
-  const void* fns[] = {(const void*)gv::k_finish, (const void*)gv::k_colsum,
+  const void* fns[] = {(const void*)gv::k_finish<gv::kFinishThreads>, (const void*)gv::k_finish<gv::kMaxFinishThreads>, (const void*)gv::k_colsum,
                        (const void*)gv::k_control, (const void*)gv::k_uniform_grid, (const void*)gv::k_tables};
   for (const void* f : fns) {
     const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -435,7 +430,10 @@ cudaError_t gv_raise_smem_limit(const void* fn, size_t bytes) {
 
 cudaError_t gv_launch_finish(const gv::FinArgs* F, cudaStream_t s) {
   const int blocks = gv::kFinishCluster * (F->nobins ? 1 : F->d + 1);
-  gv::k_finish<<<blocks, F->N <= 64 || F->nobins ? gv::kFinishThreads : gv::kMaxFinishThreads, 0, s>>>(*F);
+  if (F->N <= 64 || F->nobins)
+    gv::k_finish<gv::kFinishThreads><<<blocks, gv::kFinishThreads, 0, s>>>(*F);
+  else
+    gv::k_finish<gv::kMaxFinishThreads><<<blocks, gv::kMaxFinishThreads, 0, s>>>(*F);
   return cudaGetLastError();
 }
 
