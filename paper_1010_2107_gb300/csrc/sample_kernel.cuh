@@ -396,23 +396,39 @@ constexpr int kMaxSampleWarps = 16;
 
 // The CTA's totals (compensated pairs or doubles per thread) into its column
 // of part_tot: fixed butterflies, then the warps in order.
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+// GROUPS: in stratified runs only the groups' first lanes hold sums, and the
+// butterfly's steps within a group, which would add zeros, are left out (the same
+// bits; an FP64 step costs the pipe 19 SM-clocks a warp, and every CTA has 20 of
+// them per warp).  The columns' kernel does without: its sums are FP32 pairs, and
+// the loop's bound costs the heavy kernels registers (RAMBO 2 -> 5, 2^22 points:
+// 219.2 -> 222.9 us).
+__device__ __forceinline__ fpair warp_sum_from(fpair p, int width) {
+  for (int off = 16; off >= width; off >>= 1)
+    comp_merge(p, fpair{__shfl_xor_sync(0xffffffffu, p.hi, off), __shfl_xor_sync(0xffffffffu, p.lo, off)});
+  return p;
+}
+__device__ __forceinline__ double warp_sum_from(double v, int width) {
+  for (int off = 16; off >= width; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
   return v;
 }
 __device__ __forceinline__ void tot_merge(fpair& a, const fpair& b) { comp_merge(a, b); }
 __device__ __forceinline__ void tot_merge(double& a, double b) { a += b; }
 __device__ __forceinline__ double tot_value(const fpair& a) { return comp_value(a); }
 __device__ __forceinline__ double tot_value(double a) { return a; }
-template <typename S>  // fpair or double
+template <bool GROUPS, typename S>  // S: fpair or double
 __device__ __forceinline__ void store_totals(const SampleArgs& A, double* part_tot, const S (&t)[4], int nonfinite) {
   __shared__ double wnf[kMaxSampleWarps];
   __shared__ S wtot[kMaxSampleWarps][4];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {  // (the hypercubes' two are zero without strata: no butterfly for them)
-    const S v = q < 2 || A.strat ? warp_sum(t[q]) : S{};
+    S v{};
+    if (q < 2 || A.strat) {
+      if constexpr (GROUPS)
+        v = warp_sum_from(t[q], A.strat ? A.lanes : 1);
+      else
+        v = warp_sum(t[q]);
+    }
     if (lane == 0) wtot[warp][q] = v;
   }
   int nf = nonfinite;
@@ -751,9 +767,9 @@ __global__ void __launch_bounds__(kSampleBound<DM, F, ACC, YB, SPEC, BINS>, kSam
   }
   double* part_tot = A.part_tot + (size_t)blockIdx.y * kTotCols * A.nparts;
   if constexpr (COMP)
-    store_totals(A, part_tot, tp, nonfinite);
+    store_totals<true>(A, part_tot, tp, nonfinite);
   else
-    store_totals(A, part_tot, t, nonfinite);
+    store_totals<true>(A, part_tot, t, nonfinite);
 }
 
 // ---------------------------------------------------------------------------
@@ -973,7 +989,7 @@ __global__ void __launch_bounds__(512, 1) k_sample_col(const SampleArgs A) {
   }
   hist.drain();
   fold();
-  store_totals(A, A.part_tot, tp, nonfinite);
+  store_totals<false>(A, A.part_tot, tp, nonfinite);
 }
 
 template <typename T, int ACC>
