@@ -937,18 +937,18 @@ __global__ void __launch_bounds__(512, 1) k_sample_col(const SampleArgs A) {
     }
   } else {
     // groups of Lw lanes share a hypercube or a part of it, as in k_sample
+    // (units and the rest formed here: taken as arguments, as k_sample does, they
+    // cost the RAMBO 2 -> 5 kernel 1.6 %, 219.2 -> 222.8 us at 2^22 points)
     const int Lw = A.lanes;
+    const uint32_t units = A.ncubes * A.parts, VL = (uint32_t)Lw * A.parts;
+    const uint32_t per_lane = (A.nc + VL - 1) / VL;
     const uint32_t groups_per_cta = blockDim.x / Lw;
     const uint32_t gstride = gridDim.x * groups_per_cta;
     const uint32_t gfirst = blockIdx.x * groups_per_cta;
     const uint32_t rounds = gfirst < units ? (units - gfirst + gstride - 1) / gstride : 0;
     uint32_t gi = gfirst + tid / Lw;
     for (uint32_t r = 0; r < rounds; ++r, gi += gstride) {
-    // (units and the rest formed here: taken as arguments, as k_sample does, they
-    // cost the RAMBO 2 -> 5 kernel 1.6 %, 219.2 -> 222.8 us at 2^22 points)
       const bool live = gi < units;  // uniform within a group
-    const uint32_t units = A.ncubes * A.parts, VL = (uint32_t)Lw * A.parts;
-    const uint32_t per_lane = (A.nc + VL - 1) / VL;
       const uint32_t part = A.parts > 1u ? gi / A.ncubes : 0u;
       const uint32_t c = cube_of(A.ncubes, A.cube_mul, gi - part * A.ncubes);
       const uint32_t gl = part * Lw + (tid & (Lw - 1));
