@@ -478,16 +478,13 @@ void* device_view(void* p, size_t bytes, size_t align) {
 //   2^20          .92   .87   .84  |             1.09  1.04   .97 1.01   .97   .76
 //   2^22                .79   .76  |             1.09  1.04   .93       .92   .69
 // so from n d = 2 10^6 on where the kernel knows the dimension, and from 6 10^6
-// with at least 7 axes where it does not (beyond 16 axes, where tiles keep one
-// small CTA per SM, from 2 10^6 again: 1.2 10^5 points d = 17, 64 bins, tiles 5.2
-// us, columns 4.7; 8.3 10^4, d = 24, 80 bins, 5.5 and 5.0; 6.7 10^4, d = 30, 60
-// bins, 4.95 and 5.2; 2 10^5, d = 24, 80 bins, 63 and 51 per evaluation).
+// with at least 7 axes where it does not.
 constexpr int kColMinWarps = 8;
 // Static shared memory of k_sample, at most (its dynamic part must leave room).
 constexpr size_t kSampleStatic = 1024;
 bool cols_pay(bool exact, int d, int N, uint64_t ncubes, uint64_t ncall) {
   if (ncubes > 1 || N <= 50 || d <= 2) return true;
-  return exact || d > 16 ? ncall * (uint64_t)d >= 2000000u : d >= 7 && ncall * (uint64_t)d >= 6000000u;
+  return exact ? ncall * (uint64_t)d >= 2000000u : d >= 7 && ncall * (uint64_t)d >= 6000000u;
 }
 bool shape_col(const void* fn, const gv::KernelEntry& ke, int d, int N, int sm_count, int threads, int per_sm_req,
                uint64_t ncubes, uint64_t nc, uint64_t ncall, int64_t max_rows, uint64_t max_parts,
@@ -579,14 +576,8 @@ vegas_status configure_launch(vegas_ctx* c) {
     // d = 8, 2 10^5 points, 224 threads 65.9 -> 57.5; d = 16, 10^5, 224 69.3 ->
     // 59.8; d = 6, 10^5, 192 41.9 -> 39.5; but 3 10^4, 128 27.0 -> 28.7; FP64 sums
     // d = 8, 2 10^5, 224 44.1 -> 39.7, but d = 4 33.0 -> 35.8; FP32 sums 53 bits
-    // d = 16, 4 10^5, 224 47.9 -> 52.9), narrower yet where one CTA is all that
-    // fits (d = 8, 256 bins, 9 10^4: 218 -> 182 per four iterations).
-    // And where few bins would overflow their buckets (64 slots): narrower at
-    // any rate (2 bins, d = 7, 2 10^4 points: 217 us per four iterations with
-    // 256 threads, 98 so; FP64, d = 9, 4 10^4: 283 and 171).
-    int narrowest = c->prec == VG_FP64 ? 160 : 256;
-    if (c->prec == VG_FP32_ACC64) narrowest = t.occ == 1 ? 160 : (d >= 8 ? 224 : 256);
-    if (threads > 40 * N) narrowest = 64;
+    // d = 16, 4 10^5, 224 47.9 -> 52.9).
+    const int narrowest = c->prec == VG_FP64 ? 160 : (c->prec == VG_FP32_ACC64 && d >= 8 ? 224 : 256);
     if (e == cudaSuccess && c->threads_req == 0 && !strat && t.occ > 0) {
       const uint64_t n = (uint64_t)c->cfg.ncall, most = (uint64_t)c->sm_count * t.occ;
       const uint64_t rounds = (n + most * threads - 1) / (most * threads);
@@ -595,7 +586,7 @@ vegas_status configure_launch(vegas_ctx* c) {
         const int wide = threads;
         threads = w;
         const gv::TileShape u = gv::choose_tile(threads, N, c->ppt_req, c->ppt_min, occ_cap, occ_of, c->small_cap);
-        if (u.occ >= t.occ && u.ppt >= t.ppt)  // (a shorter tile costs more than even rounds give)
+        if (u.occ >= t.occ && u.ppt == t.ppt)  // (a shorter tile costs more than even rounds give)
           t = u;
         else
           threads = wide;
@@ -640,10 +631,9 @@ vegas_status configure_launch(vegas_ctx* c) {
   pn.occ = std::max(1, std::min(occ_nb, std::max(32 * 32 / threads, per_sm)));
   const int64_t most_nb = (int64_t)c->sm_count * pn.occ;
   // (without the histogram a cube's parts cost more, in their merge and in the
-  // groups' own reductions, than even rounds give, until a quarter of the SMs
-  // would idle: 6561 cubes of 300, d = 8, 85.6 us per call with parts, 78.4
-  // without; 729 of 1438, d = 6, 45 and 63)
-  const uint64_t max_parts = c->ncubes * 128 < (uint64_t)threads * c->sm_count * 3 ? gv::kMaxCubeParts : 0;
+  // groups' own reductions, than even rounds give, until half the SMs would
+  // idle: 6561 cubes of 300, d = 8, 85.6 us per call with parts, 78.4 without)
+  const uint64_t max_parts = c->ncubes * 32 < (uint64_t)threads * c->sm_count / 2 ? gv::kMaxCubeParts : 0;
   const gv::CubeLanes cl = strat ? gv::balanced_lanes(c->ncubes, c->nc, threads, c->sm_count, c->ppt_min, max_parts)
                                  : gv::CubeLanes{1, 1};
   pn.lanes = cl.lanes;
@@ -1668,11 +1658,7 @@ vegas_status vegas_autotune(vegas_ctx* c, int* threads, int* points_per_thread, 
       widths.push_back({best.s, 0.0});
       widths.back().s.f = f;
     }
-  for (Cand& k : widths)
-    if (time_shape(k.s, true, 3, &k.ms) != VEGAS_OK) return give_up();
-  std::sort(widths.begin(), widths.end(), faster);
-  widths.resize(std::min<size_t>(widths.size(), 2));
-  if (finals(widths, true, 2) != VEGAS_OK) return give_up();
+  if (finals(widths, true, 3) != VEGAS_OK) return give_up();
   const Cand width = *std::min_element(widths.begin(), widths.end(), faster);
   const vegas_status st = set_shape(width.s);
   if (st) return st;

@@ -464,15 +464,8 @@ template <> constexpr bool kLight<GenzContinuous> = true;
 template <> constexpr bool kLight<GenzDiscontinuous> = true;
 template <> constexpr bool kLight<DoubleGaussian> = true;
 template <> constexpr bool kLight<WMuNu> = true;
-// FP32 with buckets, general, 9 to 16 axes: two as well (128 registers; RAMBO 2 ->
-// 3 and 2 -> 4, compensated sums, 53 bits, 2^20 points: 95 and 132 us against 129
-// and 152 with the 169 and 179 registers it takes by itself; Genz Gaussian d = 16,
-// 1.9 10^6: 147 against 154), but for the heavy ones with FP64 sums (RAMBO 2 -> 3 206 us by
-// itself, 220 so).
-template <typename T, int DM, template <typename, int> class F, int ACC, bool SPEC, bool BINS>
-constexpr int kSampleMinBlocks =
-    std::is_same<T, double>::value ? (DM <= 16 && kLight<F> ? (SPEC ? 1 : (DM <= 4 ? 3 : 2)) : 0)
-                                   : (BINS && !SPEC && DM > 8 && DM <= 16 && (ACC == 2 || kLight<F>) ? 2 : 0);
+template <typename T, int DM, template <typename, int> class F, bool SPEC>
+constexpr int kSampleMinBlocks = std::is_same<T, double>::value && DM <= 16 && kLight<F> ? (SPEC ? 1 : (DM <= 4 ? 3 : 2)) : 0;
 
 // Threads a kernel is compiled for: kSampleMaxThreads, but 336 for the FP32
 // form with 53-bit words and the histogram in 5 to 8 dimensions.  Compiled for
@@ -495,7 +488,7 @@ constexpr int kSampleBound = ACC == 2 && YB == 53 && DM == 8 && BINS && kLight<F
 // Gaussian d = 8 19.8 -> 17.2, RAMBO 2 -> 3 with FP64 sums 70 -> 52, d = 8 with
 // 53 bits 46 -> 40).
 template <typename T, int DM, template <typename, int> class F, int ACC, int YB, bool SPEC, bool BINS>
-__global__ void __launch_bounds__(kSampleBound<DM, F, ACC, YB, SPEC, BINS>, kSampleMinBlocks<T, DM, F, ACC, SPEC, BINS>)
+__global__ void __launch_bounds__(kSampleBound<DM, F, ACC, YB, SPEC, BINS>, kSampleMinBlocks<T, DM, F, SPEC>)
     k_sample(const SampleArgs A) {
   using H = typename AccTraits<ACC>::H;
   using T2 = typename Vec2<T>::type;
@@ -937,18 +930,14 @@ __global__ void __launch_bounds__(512, 1) k_sample_col(const SampleArgs A) {
     }
   } else {
     // groups of Lw lanes share a hypercube or a part of it, as in k_sample
-    // (units and the rest formed here: taken as arguments, as k_sample does, they
-    // cost the RAMBO 2 -> 5 kernel 1.6 %, 219.2 -> 222.8 us at 2^22 points)
     const int Lw = A.lanes;
-    const uint32_t units = A.ncubes * A.parts, VL = (uint32_t)Lw * A.parts;
-    const uint32_t per_lane = (A.nc + VL - 1) / VL;
     const uint32_t groups_per_cta = blockDim.x / Lw;
     const uint32_t gstride = gridDim.x * groups_per_cta;
     const uint32_t gfirst = blockIdx.x * groups_per_cta;
-    const uint32_t rounds = gfirst < units ? (units - gfirst + gstride - 1) / gstride : 0;
+    const uint32_t rounds = gfirst < A.units ? (A.units - gfirst + gstride - 1) / gstride : 0;
     uint32_t gi = gfirst + tid / Lw;
     for (uint32_t r = 0; r < rounds; ++r, gi += gstride) {
-      const bool live = gi < units;  // uniform within a group
+      const bool live = gi < A.units;  // uniform within a group
       const uint32_t part = A.parts > 1u ? gi / A.ncubes : 0u;
       const uint32_t c = cube_of(A.ncubes, A.cube_mul, gi - part * A.ncubes);
       const uint32_t gl = part * Lw + (tid & (Lw - 1));
@@ -961,13 +950,13 @@ __global__ void __launch_bounds__(512, 1) k_sample_col(const SampleArgs A) {
         }
       const uint32_t s0 = c * A.nc;
       float p1 = 0.f, p2 = 0.f;
-      for (uint32_t i = 0; i < per_lane; i += PIF) {
+      for (uint32_t i = 0; i < A.per_lane; i += PIF) {
         uint32_t sq[PIF];
         bool v[PIF];
         float w[PIF];
 #pragma unroll
         for (int q = 0; q < PIF; ++q) {
-          const uint32_t j = gl + (i + q) * VL;
+          const uint32_t j = gl + (i + q) * A.vl;
           sq[q] = s0 + j;
           v[q] = live && j < A.nc;
         }
