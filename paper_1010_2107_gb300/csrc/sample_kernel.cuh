@@ -930,14 +930,18 @@ __global__ void __launch_bounds__(512, 1) k_sample_col(const SampleArgs A) {
     }
   } else {
     // groups of Lw lanes share a hypercube or a part of it, as in k_sample
+    // (units and the rest formed here: taken as arguments, as k_sample does, they
+    // cost the RAMBO 2 -> 5 kernel 1.6 %, 219.2 -> 222.8 us at 2^22 points)
     const int Lw = A.lanes;
+    const uint32_t units = A.ncubes * A.parts, VL = (uint32_t)Lw * A.parts;
+    const uint32_t per_lane = (A.nc + VL - 1) / VL;
     const uint32_t groups_per_cta = blockDim.x / Lw;
     const uint32_t gstride = gridDim.x * groups_per_cta;
     const uint32_t gfirst = blockIdx.x * groups_per_cta;
-    const uint32_t rounds = gfirst < A.units ? (A.units - gfirst + gstride - 1) / gstride : 0;
+    const uint32_t rounds = gfirst < units ? (units - gfirst + gstride - 1) / gstride : 0;
     uint32_t gi = gfirst + tid / Lw;
     for (uint32_t r = 0; r < rounds; ++r, gi += gstride) {
-      const bool live = gi < A.units;  // uniform within a group
+      const bool live = gi < units;  // uniform within a group
       const uint32_t part = A.parts > 1u ? gi / A.ncubes : 0u;
       const uint32_t c = cube_of(A.ncubes, A.cube_mul, gi - part * A.ncubes);
       const uint32_t gl = part * Lw + (tid & (Lw - 1));
@@ -950,13 +954,13 @@ __global__ void __launch_bounds__(512, 1) k_sample_col(const SampleArgs A) {
         }
       const uint32_t s0 = c * A.nc;
       float p1 = 0.f, p2 = 0.f;
-      for (uint32_t i = 0; i < A.per_lane; i += PIF) {
+      for (uint32_t i = 0; i < per_lane; i += PIF) {
         uint32_t sq[PIF];
         bool v[PIF];
         float w[PIF];
 #pragma unroll
         for (int q = 0; q < PIF; ++q) {
-          const uint32_t j = gl + (i + q) * A.vl;
+          const uint32_t j = gl + (i + q) * VL;
           sq[q] = s0 + j;
           v[q] = live && j < A.nc;
         }
