@@ -464,8 +464,15 @@ template <> constexpr bool kLight<GenzContinuous> = true;
 template <> constexpr bool kLight<GenzDiscontinuous> = true;
 template <> constexpr bool kLight<DoubleGaussian> = true;
 template <> constexpr bool kLight<WMuNu> = true;
-template <typename T, int DM, template <typename, int> class F, bool SPEC>
-constexpr int kSampleMinBlocks = std::is_same<T, double>::value && DM <= 16 && kLight<F> ? (SPEC ? 1 : (DM <= 4 ? 3 : 2)) : 0;
+// FP32 with buckets, general, 9 to 16 axes: two as well (128 registers; RAMBO 2 ->
+// 3 and 2 -> 4, compensated sums, 53 bits, 2^20 points: 95 and 132 us against 129
+// and 152 with the 169 and 179 registers it takes by itself; Genz Gaussian d = 16,
+// 1.9 10^6: 147 against 154), but for the heavy ones with FP64 sums (RAMBO 2 -> 3 206 us by
+// itself, 220 so).
+template <typename T, int DM, template <typename, int> class F, int ACC, bool SPEC, bool BINS>
+constexpr int kSampleMinBlocks =
+    std::is_same<T, double>::value ? (DM <= 16 && kLight<F> ? (SPEC ? 1 : (DM <= 4 ? 3 : 2)) : 0)
+                                   : (BINS && !SPEC && DM > 8 && DM <= 16 && (ACC == 2 || kLight<F>) ? 2 : 0);
 
 // Threads a kernel is compiled for: kSampleMaxThreads, but 336 for the FP32
 // form with 53-bit words and the histogram in 5 to 8 dimensions.  Compiled for
@@ -488,7 +495,7 @@ constexpr int kSampleBound = ACC == 2 && YB == 53 && DM == 8 && BINS && kLight<F
 // Gaussian d = 8 19.8 -> 17.2, RAMBO 2 -> 3 with FP64 sums 70 -> 52, d = 8 with
 // 53 bits 46 -> 40).
 template <typename T, int DM, template <typename, int> class F, int ACC, int YB, bool SPEC, bool BINS>
-__global__ void __launch_bounds__(kSampleBound<DM, F, ACC, YB, SPEC, BINS>, kSampleMinBlocks<T, DM, F, SPEC>)
+__global__ void __launch_bounds__(kSampleBound<DM, F, ACC, YB, SPEC, BINS>, kSampleMinBlocks<T, DM, F, ACC, SPEC, BINS>)
     k_sample(const SampleArgs A) {
   using H = typename AccTraits<ACC>::H;
   using T2 = typename Vec2<T>::type;
