@@ -576,8 +576,14 @@ vegas_status configure_launch(vegas_ctx* c) {
     // d = 8, 2 10^5 points, 224 threads 65.9 -> 57.5; d = 16, 10^5, 224 69.3 ->
     // 59.8; d = 6, 10^5, 192 41.9 -> 39.5; but 3 10^4, 128 27.0 -> 28.7; FP64 sums
     // d = 8, 2 10^5, 224 44.1 -> 39.7, but d = 4 33.0 -> 35.8; FP32 sums 53 bits
-    // d = 16, 4 10^5, 224 47.9 -> 52.9).
-    const int narrowest = c->prec == VG_FP64 ? 160 : (c->prec == VG_FP32_ACC64 && d >= 8 ? 224 : 256);
+    // d = 16, 4 10^5, 224 47.9 -> 52.9), narrower yet where one CTA is all that
+    // fits (d = 8, 256 bins, 9 10^4: 218 -> 182 per four iterations).
+    // And where few bins would overflow their buckets (64 slots): narrower at
+    // any rate (2 bins, d = 7, 2 10^4 points: 217 us per four iterations with
+    // 256 threads, 98 so; FP64, d = 9, 4 10^4: 283 and 171).
+    int narrowest = c->prec == VG_FP64 ? 160 : 256;
+    if (c->prec == VG_FP32_ACC64) narrowest = t.occ == 1 ? 160 : (d >= 8 ? 224 : 256);
+    if (threads > 40 * N) narrowest = 64;
     if (e == cudaSuccess && c->threads_req == 0 && !strat && t.occ > 0) {
       const uint64_t n = (uint64_t)c->cfg.ncall, most = (uint64_t)c->sm_count * t.occ;
       const uint64_t rounds = (n + most * threads - 1) / (most * threads);
@@ -586,7 +592,7 @@ vegas_status configure_launch(vegas_ctx* c) {
         const int wide = threads;
         threads = w;
         const gv::TileShape u = gv::choose_tile(threads, N, c->ppt_req, c->ppt_min, occ_cap, occ_of, c->small_cap);
-        if (u.occ >= t.occ && u.ppt == t.ppt)  // (a shorter tile costs more than even rounds give)
+        if (u.occ >= t.occ && u.ppt >= t.ppt)  // (a shorter tile costs more than even rounds give)
           t = u;
         else
           threads = wide;
