@@ -637,9 +637,10 @@ vegas_status configure_launch(vegas_ctx* c) {
   pn.occ = std::max(1, std::min(occ_nb, std::max(32 * 32 / threads, per_sm)));
   const int64_t most_nb = (int64_t)c->sm_count * pn.occ;
   // (without the histogram a cube's parts cost more, in their merge and in the
-  // groups' own reductions, than even rounds give, until half the SMs would
-  // idle: 6561 cubes of 300, d = 8, 85.6 us per call with parts, 78.4 without)
-  const uint64_t max_parts = c->ncubes * 32 < (uint64_t)threads * c->sm_count / 2 ? gv::kMaxCubeParts : 0;
+  // groups' own reductions, than even rounds give, until a quarter of the SMs
+  // would idle: 6561 cubes of 300, d = 8, 85.6 us per call with parts, 78.4
+  // without; 729 of 1438, d = 6, 45 and 63)
+  const uint64_t max_parts = c->ncubes * 128 < (uint64_t)threads * c->sm_count * 3 ? gv::kMaxCubeParts : 0;
   const gv::CubeLanes cl = strat ? gv::balanced_lanes(c->ncubes, c->nc, threads, c->sm_count, c->ppt_min, max_parts)
                                  : gv::CubeLanes{1, 1};
   pn.lanes = cl.lanes;
