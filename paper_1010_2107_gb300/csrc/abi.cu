@@ -478,13 +478,16 @@ void* device_view(void* p, size_t bytes, size_t align) {
 //   2^20          .92   .87   .84  |             1.09  1.04   .97 1.01   .97   .76
 //   2^22                .79   .76  |             1.09  1.04   .93       .92   .69
 // so from n d = 2 10^6 on where the kernel knows the dimension, and from 6 10^6
-// with at least 7 axes where it does not.
+// with at least 7 axes where it does not (beyond 16 axes, where tiles keep one
+// small CTA per SM, from 2 10^6 again: 1.2 10^5 points d = 17, 64 bins, tiles 5.2
+// us, columns 4.7; 8.3 10^4, d = 24, 80 bins, 5.5 and 5.0; 6.7 10^4, d = 30, 60
+// bins, 4.95 and 5.2; 2 10^5, d = 24, 80 bins, 63 and 51 per evaluation).
 constexpr int kColMinWarps = 8;
 // Static shared memory of k_sample, at most (its dynamic part must leave room).
 constexpr size_t kSampleStatic = 1024;
 bool cols_pay(bool exact, int d, int N, uint64_t ncubes, uint64_t ncall) {
   if (ncubes > 1 || N <= 50 || d <= 2) return true;
-  return exact ? ncall * (uint64_t)d >= 2000000u : d >= 7 && ncall * (uint64_t)d >= 6000000u;
+  return exact || d > 16 ? ncall * (uint64_t)d >= 2000000u : d >= 7 && ncall * (uint64_t)d >= 6000000u;
 }
 bool shape_col(const void* fn, const gv::KernelEntry& ke, int d, int N, int sm_count, int threads, int per_sm_req,
                uint64_t ncubes, uint64_t nc, uint64_t ncall, int64_t max_rows, uint64_t max_parts,

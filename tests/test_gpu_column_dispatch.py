@@ -53,7 +53,7 @@ def test_where_no_bucket_fits_columns_take_any_work(gv, orc, ncall, threads):
 
 
 @pytest.mark.parametrize("d,N,least", [(4, 51, 500_000), (8, 64, 250_000), (16, 100, 125_000), (32, 51, 62_500),
-                                       (7, 51, 857_143), (9, 80, 666_667), (20, 64, 300_000)])
+                                       (7, 51, 857_143), (9, 80, 666_667), (20, 64, 100_000)])
 def test_least_work_beyond_50_bins(gv, orc, d, N, least):
     _check(gv, orc, d, N, least, True)
     _check(gv, orc, d, N, least - 1, False)
