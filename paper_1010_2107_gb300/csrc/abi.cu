@@ -1668,7 +1668,11 @@ vegas_status vegas_autotune(vegas_ctx* c, int* threads, int* points_per_thread, 
       widths.push_back({best.s, 0.0});
       widths.back().s.f = f;
     }
-  if (finals(widths, true, 3) != VEGAS_OK) return give_up();
+  for (Cand& k : widths)
+    if (time_shape(k.s, true, 3, &k.ms) != VEGAS_OK) return give_up();
+  std::sort(widths.begin(), widths.end(), faster);
+  widths.resize(std::min<size_t>(widths.size(), 2));
+  if (finals(widths, true, 2) != VEGAS_OK) return give_up();
   const Cand width = *std::min_element(widths.begin(), widths.end(), faster);
   const vegas_status st = set_shape(width.s);
   if (st) return st;

@@ -1183,9 +1183,9 @@ vegas_status vegas_batch_autotune(vegas_batch* b, int* threads, int* rounds, dou
   };
   vegas_status st = VEGAS_OK;
   double fastest = 0.0;
-  auto add = [&](int t, int r, int p, int pol) -> bool {  // false: a pass failed
+  auto add = [&](int t, int r, int p, int pol, int n = 3) -> bool {  // false: a pass failed
     Cand c{t, r, p, pol, 0.0, 0.0};
-    if ((st = time_shape(c, 3, true)) != VEGAS_OK) return false;
+    if ((st = time_shape(c, n, true)) != VEGAS_OK) return false;
     if (cands.empty() || c.ms < fastest) fastest = c.ms;
     cands.push_back(c);
     return true;
@@ -1206,7 +1206,7 @@ vegas_status vegas_batch_autotune(vegas_batch* b, int* threads, int* rounds, dou
     bool screen = !any;
     for (int r : {8, 32}) {
       if (!any) break;
-      if (!add(256, r, 2, 2)) return give_up(st);
+      if (!add(256, r, 2, 2, 1)) return give_up(st);
       screen = screen || cands.back().ms < near;
     }
     for (int t : kThreads)
